@@ -79,8 +79,8 @@ KERNEL_OF_STAGE["chain_o_ffn_lm"] = "k_umma_chain (o, gate|up, down, LM head)"
 
 
 def kernel_of_stage(stage, rows):
-    if stage == "lm_head" and rows > 32:   # logits stored by the GEMM, statistics by one block per row
-        return "k_umma_gemm<STORE> + k_row_stats"
+    if stage == "lm_head" and rows > 16:   # logits stored by the GEMM, statistics by a pass of their own
+        return "k_umma_gemm<STORE> + k_logit_stats"
     return KERNEL_OF_STAGE.get(stage, stage)
 
 

@@ -2091,7 +2091,7 @@ ps_status umma_draft_step(ps_ctx* c, const UmmaMaps& u, const SeqMap& sm, int B,
     a.ssq_out = f.ssq[2];
     a.out_hi = f.hdnp.hi; a.out_lo = f.hdnp.lo; a.ld_plane = H; a.gain_next = (BP)w.g_final;
   }
-  const bool stats_pass = M > 32 && logits_out;
+  const bool stats_pass = M > 16 && logits_out;
   {
     StageDesc& x = d[n++];
     x = StageDesc{stats_pass ? EPI_STORE : EPI_LMHEAD, &u.w_lm, &u.w_lm, &u.w_lm, &u.hdn_hi, &u.hdn_lo, UArgs{}, "lm_head"};
@@ -2099,9 +2099,9 @@ ps_status umma_draft_step(ps_ctx* c, const UmmaMaps& u, const SeqMap& sm, int B,
     a.N = V; a.K = H; a.M = M; a.n_mats = 1; a.mat_rows[0] = V; a.lo = 1;
     a.ssq_in = f.ssq[2]; a.ssq_n = tiles_h; a.eps = g.rms_eps;
     if (stats_pass) {
-      // S6 with many rows and the logits kept: the row statistics in the tile epilogue cost more
-      // than the weights' streaming then (they are serial in the rows), so the GEMM only stores
-      // the logits and one block per row reads them back from L2
+      // S6 with more than 16 rows and the logits kept: the statistics in the tile epilogue are serial
+      // in the rows (20 rows of the 13B shape with sampling: 140 us), so the GEMM only stores the
+      // logits and a kernel of its own reads them back from L2 (83 us together)
       a.out = logits_out; a.ldo = V;
       x.name = nullptr;   // (timed together with the statistics pass below)
     } else {  // S6 logits = W_lm rms(hdn), softmax statistics and top-n without a second pass over logits
@@ -2114,8 +2114,7 @@ ps_status umma_draft_step(ps_ctx* c, const UmmaMaps& u, const SeqMap& sm, int B,
   if ((s = run_stages(c, d, n, chain, 1, f, st))) return s;
   if (chain) prof_mark(c, st, "chain_o_ffn_lm");
   if (stats_pass) {
-    if ((s = launch_row_stats(c, logits_out, M, V, top_n, top_ids, top_logit, row_max, row_lse, st))) return s;
-    if (sa && (s = launch_gumbel_argmax(c, logits_out, M, V, R, *sa, st))) return s;
+    if ((s = launch_logit_stats(c, logits_out, M, V, R, top_n, top_ids, top_logit, row_max, row_lse, sa, st))) return s;
     prof_mark(c, st, "lm_head");
   }
   return PS_OK;
@@ -2291,7 +2290,7 @@ ps_status fused_draft_step(ps_ctx* c, const SeqMap& sm, int B, const void* hidde
     a.top_n = top_n; a.top_ids = top_ids; a.top_logit = top_logit; a.row_max = row_max; a.row_lse = row_lse;
     if ((s = launch_gemm<false, EPI_LMHEAD>(c, a, st))) return s;
   }
-  if (sa && (s = launch_gumbel_argmax(c, logits_out, M, V, R, *sa, st))) return s;
+  if (sa && (s = launch_logit_stats(c, logits_out, M, V, R, 0, nullptr, nullptr, nullptr, nullptr, sa, st))) return s;
   prof_mark(c, st, "lm_head");
   return PS_OK;
 }

@@ -271,100 +271,6 @@ __global__ void k_silu_mul(const float* gate, const float* up, float* out, size_
   }
 }
 
-// Per-row max, log-sum-exp and top-n (descending logit, ties to the lower id).  One block per
-// row; top-n by n selection passes, each picking the best entry that ranks after the last pick.
-__global__ void __launch_bounds__(256) k_row_stats(const float* logits, int V, int top_n,
-                                                   int* top_ids, float* top_logit, float* row_max,
-                                                   float* row_lse) {
-  __shared__ float s_v[8];
-  __shared__ int s_i[8];
-  __shared__ float s_f[8];
-  const float* row = logits + (size_t)blockIdx.x * V;
-  const int nv4 = (reinterpret_cast<uintptr_t>(row) & 15) == 0 ? V / 4 : 0;   // float4 part of the row
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float prev_v = FLT_MAX;
-  int prev_i = -1;
-  float rmax = 0.f;
-  int passes = top_n > 0 ? top_n : 1;
-  for (int t = 0; t < passes; ++t) {
-    float bv = -FLT_MAX;
-    int bi = 0x7fffffff;
-    auto consider = [&](float x, int v) {
-      const bool after = (x < prev_v) || (x == prev_v && v > prev_i);   // ranks after the last pick
-      if (after && (x > bv || (x == bv && v < bi))) { bv = x; bi = v; }
-    };
-#pragma unroll 4
-    for (int i = threadIdx.x; i < nv4; i += blockDim.x) {   // 16-byte loads, several in flight
-      const float4 x = __ldg(reinterpret_cast<const float4*>(row) + i);
-      consider(x.x, 4 * i); consider(x.y, 4 * i + 1); consider(x.z, 4 * i + 2); consider(x.w, 4 * i + 3);
-    }
-    for (int v = 4 * nv4 + threadIdx.x; v < V; v += blockDim.x) consider(row[v], v);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-    }
-    if (lane == 0) { s_v[warp] = bv; s_i[warp] = bi; }
-    __syncthreads();
-    bv = s_v[0]; bi = s_i[0];
-    for (int w = 1; w < 8; ++w)
-      if (s_v[w] > bv || (s_v[w] == bv && s_i[w] < bi)) { bv = s_v[w]; bi = s_i[w]; }
-    __syncthreads();
-    if (t == 0) rmax = bv;
-    if (top_n > 0 && threadIdx.x == 0) {
-      top_ids[(size_t)blockIdx.x * top_n + t] = bi;
-      top_logit[(size_t)blockIdx.x * top_n + t] = bv;
-    }
-    prev_v = bv; prev_i = bi;
-  }
-  float s = 0.f;
-#pragma unroll 4
-  for (int i = threadIdx.x; i < nv4; i += blockDim.x) {
-    const float4 x = __ldg(reinterpret_cast<const float4*>(row) + i);
-    s += (expf(x.x - rmax) + expf(x.y - rmax)) + (expf(x.z - rmax) + expf(x.w - rmax));
-  }
-  for (int v = 4 * nv4 + threadIdx.x; v < V; v += blockDim.x) s += expf(row[v] - rmax);
-  s = warp_sum(s);
-  if (lane == 0) s_f[warp] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float tot = 0.f;
-    for (int w = 0; w < 8; ++w) tot += s_f[w];
-    if (row_max) row_max[blockIdx.x] = rmax;
-    if (row_lse) row_lse[blockIdx.x] = rmax + logf(tot);
-  }
-}
-
-// Gumbel-max token of each row of stored logits (draft sampling on the paths that keep logits
-// in memory).  One block per row.
-__global__ void __launch_bounds__(256) k_gumbel_argmax(const float* logits, int V, int R, SampleArgs sa) {
-  __shared__ float s_v[8];
-  __shared__ int s_i[8];
-  const int m = blockIdx.x, b = m / R, j = m - b * R;
-  const uint32_t row_id = ((uint32_t)b + sa.b_base) | ((uint32_t)j << 8);
-  const float* row = logits + (size_t)m * V;
-  float bv = -FLT_MAX;
-  int bi = 0x7fffffff;
-  for (int v = threadIdx.x; v < V; v += blockDim.x) {
-    const float y = row[v] * sa.inv_temp + gumbel_noise(sa, (uint32_t)v, row_id);
-    if (y > bv || (y == bv && v < bi)) { bv = y; bi = v; }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-  }
-  if ((threadIdx.x & 31) == 0) { s_v[threadIdx.x >> 5] = bv; s_i[threadIdx.x >> 5] = bi; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w)
-      if (s_v[w] > bv || (s_v[w] == bv && s_i[w] < bi)) { bv = s_v[w]; bi = s_i[w]; }
-    sa.sampled[m] = bi;
-  }
-}
-
 template <typename WT>
 __global__ void k_kv_copy(WT* kcache, WT* vcache, WT* K, WT* V, int slot, int len, int n_kv_heads,
                           int d, int max_ctx, int to_cache) {
@@ -466,8 +372,8 @@ ps_status draft_impl(ps_ctx* c, const SeqMap& sm, int B, const void* hidden_last
   c->launches++;
   float* logits = logits_out ? logits_out : c->logits;
   if ((s = linear<WT>(c, c->hn, H, w.w_lm, nullptr, nullptr, 0, logits, V, M, V, H, st))) return s;
-  if ((s = launch_row_stats(c, logits, M, V, top_n, top_ids, top_logit, row_max, row_lse, st))) return s;
-  if (sa && (s = launch_gumbel_argmax(c, logits, M, V, g.k_masks + 1, *sa, st))) return s;
+  if ((s = launch_logit_stats(c, logits, M, V, g.k_masks + 1, top_n, top_ids, top_logit, row_max, row_lse, sa, st)))
+    return s;
   prof_mark(c, st, "lm_head");
   return cuda_check(c, cudaGetLastError(), "draft_step");
 }
@@ -504,21 +410,6 @@ ps_status launch_rope_store_kv(ps_ctx* c, const SeqMap& sm, int rows, cudaStream
         g.n_kv_heads, g.head_dim, g.max_ctx, g.rope_base);
   c->launches++;
   return cuda_check(c, cudaGetLastError(), "k_rope_store");
-}
-
-ps_status launch_row_stats(ps_ctx* c, const float* logits, int M, int V, int top_n, int* top_ids,
-                           float* top_logit, float* row_max, float* row_lse, cudaStream_t st) {
-  if (top_n <= 0 && !row_max && !row_lse) return PS_OK;
-  k_row_stats<<<M, 256, 0, st>>>(logits, V, top_n, top_ids, top_logit, row_max, row_lse);
-  c->launches++;
-  return cuda_check(c, cudaGetLastError(), "k_row_stats");
-}
-
-ps_status launch_gumbel_argmax(ps_ctx* c, const float* logits, int M, int V, int R, const SampleArgs& sa,
-                               cudaStream_t st) {
-  k_gumbel_argmax<<<M, 256, 0, st>>>(logits, V, R, sa);
-  c->launches++;
-  return cuda_check(c, cudaGetLastError(), "k_gumbel_argmax");
 }
 
 ps_status launch_kv_copy(ps_ctx* c, int slot, int len, void* K, void* V, bool to_cache,

@@ -88,17 +88,19 @@ struct SampleArgs {
   int* sampled;   // [B][k+1]
   uint32_t b_base;   // index, in the caller's batch, of the first sequence of this launch
 };
-__device__ __forceinline__ float gumbel_noise(const SampleArgs& sa, uint32_t v, uint32_t row_id) {
-  uint32_t c[4] = {v, row_id, sa.off_lo, sa.off_hi};
-  philox4x32_10(sa.key0, sa.key1, c);
-  // e = -ln u in single precision without losing u's distance from 1 (u can sit within 2^-25
-  // of it): below one half from u itself, above from 1 - u = (2^24 - w - 0.5) / 2^24, which like
-  // w + 0.5 is exact in fp32 on its half of the range.
-  const uint32_t w = c[0] >> 8;
+// G of the 24-bit word w: e = -ln u in single precision without losing u's distance from 1 (u can
+// sit within 2^-25 of it): below one half from u itself, above from 1 - u = (2^24 - w - 0.5) / 2^24,
+// which like w + 0.5 is exact in fp32 on its half of the range.
+__device__ __forceinline__ float gumbel_of_word(uint32_t w) {
   float e;
   if (w < (1u << 23)) e = -__logf(((float)w + 0.5f) * (1.0f / 16777216.0f));
   else e = -log1pf(-((float)(16777216u - w) - 0.5f) * (1.0f / 16777216.0f));
   return -__logf(e);
+}
+__device__ __forceinline__ float gumbel_noise(const SampleArgs& sa, uint32_t v, uint32_t row_id) {
+  uint32_t c[4] = {v, row_id, sa.off_lo, sa.off_hi};
+  philox4x32_10(sa.key0, sa.key1, c);
+  return gumbel_of_word(c[0] >> 8);
 }
 
 // Device status word values (bit flags).
@@ -175,12 +177,10 @@ ps_status plain_draft_step(ps_ctx* c, const SeqMap& sm, int B, const void* hidde
                            const int* token_last, int top_n, int* top_ids, float* top_logit,
                            float* row_max, float* row_lse, float* logits_out, float* feat_out,
                            const SampleArgs* sa, cudaStream_t st);
-// One block per row of stored logits [M][V]: max, log-sum-exp and top-n of the row.
-ps_status launch_row_stats(ps_ctx* c, const float* logits, int M, int V, int top_n, int* top_ids,
-                           float* top_logit, float* row_max, float* row_lse, cudaStream_t st);
-// One block per row of stored logits [M][V]: the Gumbel-max token of the row (R rows per sequence).
-ps_status launch_gumbel_argmax(ps_ctx* c, const float* logits, int M, int V, int R, const SampleArgs& sa,
-                               cudaStream_t st);
+// One pass over stored logits [M][V] (R rows per sequence): max, log-sum-exp, top-n and, with sa, the
+// Gumbel-max token of every row (row_stats.cu).
+ps_status launch_logit_stats(ps_ctx* c, const float* logits, int M, int V, int R, int top_n, int* top_ids,
+                             float* top_logit, float* row_max, float* row_lse, const SampleArgs* sa, cudaStream_t st);
 // ---- fused bf16 kernels for small M ---------------------------------------------------------
 bool fused_supported(ps_ctx* c, int M);
 int fused_kv_rows(ps_ctx* c);     // rows per pass of fused_kv_append (0: not available)
