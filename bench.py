@@ -78,13 +78,20 @@ KERNEL_OF_STAGE["chain_fc_qkv"] = "k_gather_x + k_umma_chain (fc, q|k|v)"
 KERNEL_OF_STAGE["chain_o_ffn_lm"] = "k_umma_chain (o, gate|up, down, LM head)"
 
 
+KERNEL_OF_STAGE_PAIR = {   # more than 16 rows
+    "fc_norm": "k_gather_x + k_pair_gemm + k_row_norm", "qkv_rope": "k_pair_gemm + k_finish_shared",
+    "o_proj": "k_pair_gemm + k_row_norm", "ffn_gate_up": "k_pair_gemm + k_finish_shared",
+    "ffn_down": "k_pair_gemm + k_row_norm", "lm_head": "k_pair_gemm + k_finish_shared + k_logit_stats",
+}
+
+
 def kernel_of_stage(stage, rows):
-    if stage == "lm_head" and rows > 16:   # logits stored by the GEMM, statistics by a pass of their own
-        return "k_umma_gemm<STORE> + k_logit_stats"
+    if rows > 16 and stage in KERNEL_OF_STAGE_PAIR:
+        return KERNEL_OF_STAGE_PAIR[stage]
     return KERNEL_OF_STAGE.get(stage, stage)
 
 
-GEMM_SOURCES = ("fused_kernels.cu", "umma_gemm.cuh", "ws_gemm.cuh", "ps_internal.cuh")
+GEMM_SOURCES = ("fused_kernels.cu", "pair_gemm.cu", "pair_gemm.cuh", "umma_gemm.cuh", "ws_gemm.cuh", "ps_internal.cuh")
 
 
 def kernel_sources_digest():

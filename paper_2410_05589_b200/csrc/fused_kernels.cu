@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cfloat>
 
+#include "pair_gemm.cuh"
 #include "umma_gemm.cuh"
 #include "ws_gemm.cuh"
 
@@ -412,51 +413,76 @@ struct FusedScratch {
   float* ssq[3];            // partial sums of squares of x0, a and hdn rows: [kMaxSm][kMaxM] each
   Planes x0p, ap, hdnp, attnp, actp;
   // tensor-core path
-  __nv_bfloat16* xin;       // [kMaxM][2H] gathered fc input (exact bf16: one plane)
-  float* partials;          // [kMaxSm][2][16][128] partial tiles of CTAs that share a tile
+  __nv_bfloat16* xin;       // [rows][2H] gathered fc input (exact bf16: one plane)
+  float* partials;          // [kMaxSm][2][16][128] partial tiles of CTAs that share a tile (up to 16 rows)
+  float* slots; size_t slot_floats;   // partial tiles of the CTA-pair GEMM
+  float* kv;                // [append rows][2 Hkv] k | v of appended positions before RoPE
   unsigned* tile_tickets;   // one per tile of the widest stage, zero between launches
   unsigned* chain_ctr;      // chained stages: finished-tile and passed-CTA counts, zero between launches
   int n_part_rows;          // rows of `parts` and of each ssq array
+  size_t counter_bytes;     // the counters, which start at zero, lie at the front
   size_t bytes;
 };
 
+// Rows of a draft step of this context (16 at least: what the small kernels round up to), and rows
+// of one pass of ps_kv_append: enough that the weights are streamed for long runs of rows, half
+// of all cache rows at most (a prompt longer than that is rare, and the scratch stays in
+// proportion to the cache).
+int draft_rows_cap(const ps_config& g) { return std::max(kMaxM, g.max_batch * (g.k_masks + 1)); }
+int append_rows_cap(const ps_config& g) {
+  return (int)std::min<long long>(2048, std::max<long long>(128, (long long)g.max_batch * g.max_ctx / 2));
+}
+
 // One carve-up for sizing (base == nullptr) and for use; always the largest row and CTA counts.
 FusedScratch carve_fused(const ps_config& g, char* base) {
-  constexpr int kRows = umma::kMaxRows;   // rows the tensor-core path can take (the mma.sync kernels: kMaxM)
   const size_t Hq = (size_t)g.n_heads * g.head_dim, Hkv = (size_t)g.n_kv_heads * g.head_dim;
+  const size_t rd = draft_rows_cap(g), ra = append_rows_cap(g), rx = std::max(rd, ra);
   size_t off = 0;
   auto take = [&](size_t bytes) {
     size_t at = off;
     off += (bytes + 255) & ~(size_t)255;
     return base ? base + at : nullptr;
   };
-  auto planes = [&](size_t width) {
+  auto planes = [&](size_t rows, size_t width) {
     Planes p;
-    p.hi = (__nv_bfloat16*)take((size_t)kRows * width * 2);
-    p.lo = (__nv_bfloat16*)take((size_t)kRows * width * 2);
+    p.hi = (__nv_bfloat16*)take(rows * width * 2);
+    p.lo = (__nv_bfloat16*)take(rows * width * 2);
     return p;
   };
   FusedScratch s;
-  s.qkv = (float*)take((size_t)kRows * (Hq + 2 * Hkv) * 4);
-  // (rows x splits is bounded: the attention launcher takes fewer splits when there are more rows)
-  s.att_ml = (float*)take((size_t)kMaxM * g.n_heads * kAttnMaxSplit * 2 * 4);
-  s.att_o = (float*)take((size_t)kMaxM * g.n_heads * kAttnMaxSplit * g.head_dim * 4);
-  s.act = (float*)take((size_t)kRows * g.ffn * 4);
-  // per-CTA (mma.sync path) or per-tile (tensor-core path) summaries
+  if (g.dtype != PS_DTYPE_BF16) {   // fp32 models run on the plain kernels
+    s = FusedScratch{};
+    s.bytes = 256;
+    return s;
+  }
   const int tiles_v = (g.vocab + 127) / 128, tiles_h = (g.hidden + 127) / 128;
-  s.n_part_rows = std::max(kMaxSm, std::max(tiles_v, tiles_h));
-  s.parts = (LmPart*)take((size_t)s.n_part_rows * kRows * sizeof(LmPart));
-  s.ticket = (unsigned*)take(256);
-  s.attn_tickets = (unsigned*)take((size_t)PS_MAX_BATCH * g.n_heads * 4);
-  for (int i = 0; i < 3; ++i) s.ssq[i] = (float*)take((size_t)s.n_part_rows * kRows * 4);
-  s.xin = (__nv_bfloat16*)take((size_t)kRows * 2 * g.hidden * 2);
-  s.partials = (float*)take((size_t)kMaxSm * 2 * kRows * 128 * 4);
   const size_t max_tiles = std::max<size_t>({(size_t)tiles_v, (size_t)(g.ffn + 63) / 64,
                                              (Hq + 127) / 128 + 2 * ((Hkv + 127) / 128), (size_t)tiles_h});
+  s.ticket = (unsigned*)take(256);
+  s.attn_tickets = (unsigned*)take((size_t)PS_MAX_BATCH * g.n_heads * 4);
   s.tile_tickets = (unsigned*)take(max_tiles * 4);
   s.chain_ctr = (unsigned*)take(256);
-  s.x0p = planes(g.hidden); s.ap = planes(g.hidden); s.hdnp = planes(g.hidden);
-  s.attnp = planes(Hq); s.actp = planes(g.ffn);
+  s.counter_bytes = off;
+  s.qkv = (float*)take(rd * (Hq + 2 * Hkv) * 4);
+  // (rows x splits is bounded: the attention launcher takes fewer splits when there are more rows)
+  const size_t att = std::max<size_t>((size_t)kMaxM * kAttnMaxSplit, rd) * g.n_heads;
+  s.att_ml = (float*)take(att * 2 * 4);
+  s.att_o = (float*)take(att * g.head_dim * 4);
+  s.act = (float*)take(rd * g.ffn * 4);
+  // per-CTA (mma.sync path) or per-tile (tensor-core path) summaries
+  s.n_part_rows = std::max(kMaxSm, std::max(tiles_v, tiles_h));
+  s.parts = (LmPart*)take((size_t)s.n_part_rows * kMaxM * sizeof(LmPart));
+  for (int i = 0; i < 3; ++i) s.ssq[i] = (float*)take((size_t)s.n_part_rows * kMaxM * 4);
+  s.xin = (__nv_bfloat16*)take(rx * 2 * g.hidden * 2);
+  s.partials = (float*)take((size_t)kMaxSm * 2 * kMaxM * 128 * 4);
+  // room for one contributor of every pair of a 148-SM chip at the largest tile twice over, and for
+  // two contributors of every row of a hidden-wide stage
+  const size_t h_pad = ((size_t)g.hidden + 511) / 512 * 512, r_pad = (rx + 511) / 256 * 256;
+  s.slot_floats = std::max<size_t>((size_t)2 * (kMaxSm / 2) * 256 * pg::kMaxNp / 4 * 3, 2 * r_pad * h_pad);
+  s.slots = (float*)take(s.slot_floats * 4);
+  s.kv = (float*)take(ra * 2 * Hkv * 4);
+  s.x0p = planes(rx, g.hidden); s.ap = planes(rd, g.hidden); s.hdnp = planes(rd, g.hidden);
+  s.attnp = planes(rd, Hq); s.actp = planes(rd, g.ffn);
   s.bytes = off;
   return s;
 }
@@ -467,9 +493,7 @@ FusedScratch carve_fused(const ps_config& g, char* base) {
 // =============================================================================================
 struct UArgs {
   int N, K, M;
-  int Mp;                  // M padded to 16, 32, 48, 64, 96 or 128: rows of a plane box, half the MMA's N
   int n_tiles, KB;         // tiles of 128 weight rows (64 features when zipped), k-blocks of 64
-  int split;               // blocks a tile's k range is dealt in, 1..KB (see cta_begin)
   int zip;                 // 1: a tile is 64 rows of matrix 0 (gate) over 64 rows of matrix 1 (up)
   int lo;                  // 0: the activation operand is exact bf16 (no lo plane)
   int n_mats;              // concatenated matrices (q|k|v): tiles never straddle two of them
@@ -496,24 +520,6 @@ __device__ __forceinline__ int unit_owner(int u, int U, int G) {
 __device__ __forceinline__ int unit_begin(int c, int U, int G) {
   return (int)((unsigned)U * (unsigned)c / (unsigned)G);
 }
-// Units are dealt in blocks: the KB k-blocks of a tile are cut into a.split contiguous blocks
-// (block j of a tile starts at its k-block j KB / split) and CTA c owns blocks
-// [S c / G, S (c+1) / G) of the S = n_tiles * split blocks.  split = KB deals single units
-// (every CTA streams the same bytes: the choice for few activation rows, where streaming is
-// all that counts); split = 1 deals whole tiles (no tile is shared, nothing to reduce: the
-// choice once a tile's epilogue and reduction cost more than an uneven load).
-__device__ __forceinline__ int block_first_unit(const UArgs& a, int x) {
-  const int t = x / a.split, j = x - t * a.split;
-  return t * a.KB + (j * a.KB) / a.split;
-}
-__device__ __forceinline__ int cta_begin(const UArgs& a, int c, int G) {
-  return block_first_unit(a, unit_begin(c, a.n_tiles * a.split, G));
-}
-__device__ __forceinline__ int cta_of_unit(const UArgs& a, int u, int G) {
-  const int t = u / a.KB, w = u - t * a.KB;
-  return unit_owner(t * a.split + ((w + 1) * a.split - 1) / a.KB, a.n_tiles * a.split, G);
-}
-
 // The tiles a CTA's unit range [u0, u1) touches, in the order the CTA works through them.  A
 // range that ends inside a tile starts with that tail: the tiles a CTA shares with its
 // neighbours are then reduced while the rest of its range still streams, and the last thing it
@@ -581,12 +587,10 @@ __device__ __forceinline__ int tile_feature(const UArgs& a, int t, int r, bool& 
 // 128 epilogue threads after each has put its accumulator row r (= 32 * q + lane) of those
 // rows into ctl.acc[(m - m0) * 128 + r].  A dry call executes the same instructions and writes
 // nothing to global memory.  res_pre: the caller has put the rows' residual values into
-// ctl.land[m * 128 + r] already (m0 = 0).  With UNR = 1
-// the loops over m are rolled on purpose: for up to 16 rows this code runs once or twice per
-// CTA, so what it costs is the fetch of its instructions, not their execution.  With more rows
-// it runs once per 16 rows of every tile and its single warp per scheduler is bound by the
-// latency of dependent instructions: UNR = 4 interleaves four rows.
-template <int EPI, int UNR>
+// ctl.land[m * 128 + r] already (m0 = 0).  The loops over m
+// are rolled on purpose: this code runs once or twice per CTA, so what it costs is the fetch of
+// its instructions, not their execution.
+template <int EPI>
 __device__ __forceinline__ void tile_epilogue(const UArgs& a, umma::Ctl& ctl, int t, int r, int q, int lane,
                                               int m0, int mc, bool dry, bool res_pre = false) {
   using namespace umma;
@@ -638,12 +642,12 @@ __device__ __forceinline__ void tile_epilogue(const UArgs& a, umma::Ctl& ctl, in
     }
   } else if (EPI == EPI_SWIGLU) {
     if (r >= 64) {
-#pragma unroll UNR
+#pragma unroll 1
       for (int m = 0; m < mc; ++m) ctl.xch[m * 64 + (r - 64)] = acc[m * 128] * ctl.scale[m0 + m];
     }
     epi_sync();
     if (r < 64 && valid && !dry) {
-#pragma unroll UNR
+#pragma unroll 1
       for (int m = 0; m < mc; ++m) {
         const float gv = acc[m * 128] * ctl.scale[m0 + m], uv = ctl.xch[m * 64 + r];
         const float act = gv / (1.f + __expf(-gv)) * uv;
@@ -653,7 +657,7 @@ __device__ __forceinline__ void tile_epilogue(const UArgs& a, umma::Ctl& ctl, in
     }
     epi_sync();
   } else {  // EPI_LMHEAD: logits, and the tile's softmax / top-n summary per row
-#pragma unroll UNR
+#pragma unroll 1
     for (int m = 0; m < mc; ++m) {
       const float x = acc[m * 128] * ctl.scale[m0 + m];
       if (valid && a.logits_out && !dry) a.logits_out[(size_t)(m0 + m) * a.N + n] = x;
@@ -663,7 +667,7 @@ __device__ __forceinline__ void tile_epilogue(const UArgs& a, umma::Ctl& ctl, in
       if (lane == 0) ctl.red[q][m] = mx;
     }
     epi_sync();
-#pragma unroll UNR
+#pragma unroll 1
     for (int m = 0; m < mc; ++m) {
       const float bmax = fmaxf(fmaxf(ctl.red[0][m], ctl.red[1][m]), fmaxf(ctl.red[2][m], ctl.red[3][m]));
       const float s = warp_sum(valid ? __expf(acc[m * 128] * ctl.scale[m0 + m] - bmax) : 0.f);
@@ -678,7 +682,7 @@ __device__ __forceinline__ void tile_epilogue(const UArgs& a, umma::Ctl& ctl, in
     // top-n per row: repeated block arg-max over the values after the previous pick
 #pragma unroll 1
     for (int tn = 0; tn < a.top_n; ++tn) {
-#pragma unroll UNR
+#pragma unroll 1
       for (int m = 0; m < mc; ++m) {
         const float x = acc[m * 128] * ctl.scale[m0 + m];
         const float pv = tn ? ctl.prev_v[m] : FLT_MAX;
@@ -712,7 +716,7 @@ __device__ __forceinline__ void tile_epilogue(const UArgs& a, umma::Ctl& ctl, in
       epi_sync();
     }
     if (a.sample) {   // Gumbel-max candidate of this vocabulary range per row
-#pragma unroll UNR
+#pragma unroll 1
       for (int m = 0; m < mc; ++m) {
         const int sb = (m0 + m) / a.R;
         const uint32_t row_id = ((uint32_t)sb + a.sa.b_base) | ((uint32_t)(m0 + m - sb * a.R) << 8);
@@ -745,70 +749,6 @@ __device__ __forceinline__ void tile_epilogue(const UArgs& a, umma::Ctl& ctl, in
       }
     }
     epi_sync();   // red / red2 / cand are free again
-  }
-}
-
-// Epilogue of 16 activation rows [m0, m0 + mc) of a tile for launches of more than 16 rows
-// (EPI_STORE and EPI_SWIGLU): the thread of accumulator row r holds the rows' sums in v[] (no
-// detour through shared memory) and their residual values in rv[] (loaded by the caller before the
-// sums were ready).  With that many rows the epilogue runs eight times per tile and is what a
-// launch costs beyond its weight stream, so the per-row work is kept free of cross-lane steps:
-// the rows' sums of squares go through a [16][128] tile in shared memory (ctl.acc) and are added
-// by 8 threads per row, instead of a shuffle reduction per row and warp.
-template <int EPI>
-__device__ __forceinline__ void big_chunk_epilogue(const UArgs& a, umma::Ctl& ctl, int n, bool valid, int pidx, int r,
-                                                   int m0, int mc, const float (&v)[16], float bias, float gain,
-                                                   const float (&rv)[16], bool dry) {
-  using namespace umma;
-  constexpr int kSqLd = 132;   // row pitch of the squares' tile: the 8 x 4 threads of a warp read different banks
-  static_assert(16 * kSqLd <= 2 * kN * 128, "the squares' tile fits ctl.acc + ctl.land");
-  if (EPI == EPI_STORE) {
-    float sq[16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      sq[j] = 0.f;
-      if (j < mc && valid) {
-        const float x = v[j] * ctl.scale[m0 + j] + bias + rv[j];
-        sq[j] = x * x;
-        if (!dry) {
-          a.out[(size_t)(m0 + j) * a.ldo + n] = x;
-          if (a.out_hi)
-            split_store(a.out_hi + (size_t)(m0 + j) * a.ld_plane + n, a.out_lo + (size_t)(m0 + j) * a.ld_plane + n, x * gain);
-        }
-      }
-    }
-    if (a.ssq_out) {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) ctl.acc[j * kSqLd + r] = sq[j];   // (runs on into ctl.land, unused here)
-      epi_sync();
-      const int row = r >> 3, part = r & 7;   // 8 threads per row, every 8th feature each
-      float sum = 0.f;
-#pragma unroll
-      for (int i = 0; i < 16; ++i) sum += ctl.acc[row * kSqLd + i * 8 + part];
-      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-      sum += __shfl_xor_sync(0xffffffffu, sum, 4);
-      if (part == 0 && row < mc && !dry) a.ssq_out[(size_t)pidx * a.M + m0 + row] = sum;
-      epi_sync();
-    }
-  } else {   // EPI_SWIGLU: rows 0..63 of the tile are gate features, rows 64..127 the same features of up
-    if (r >= 64) {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) ctl.xch[j * 64 + (r - 64)] = v[j] * ctl.scale[min(m0 + j, kMaxRows - 1)];
-    }
-    epi_sync();
-    if (r < 64 && valid && !dry) {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        if (j < mc) {
-          const float gv = v[j] * ctl.scale[m0 + j], uv = ctl.xch[j * 64 + r];
-          const float act = gv / (1.f + __expf(-gv)) * uv;
-          if (a.out) a.out[(size_t)(m0 + j) * a.ldo + n] = act;
-          split_store(a.out_hi + (size_t)(m0 + j) * a.ld_plane + n, a.out_lo + (size_t)(m0 + j) * a.ld_plane + n, act);
-        }
-      }
-    }
-    epi_sync();
   }
 }
 
@@ -921,7 +861,7 @@ __device__ __forceinline__ void lm_merge(const UArgs& a, umma::Ctl& ctl, unsigne
 
 static_assert(umma::kMaxCtas >= kMaxSm, "contributor table covers every CTA of a launch");
 
-template <int EPI, int MP>
+template <int EPI>
 __global__ void __launch_bounds__(umma::kThreads, 1)
 k_umma_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUtensorMap tA1,
             const __grid_constant__ CUtensorMap tA2, const __grid_constant__ CUtensorMap tBh,
@@ -943,7 +883,7 @@ k_umma_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
   }
   if (warp == 1) {   // tensor memory for two accumulators
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl.tmem_base)),
-                 "r"(tmem_cols(MP))
+                 "r"(kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -953,14 +893,11 @@ k_umma_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
   const uint32_t tmem = *(volatile uint32_t*)&ctl.tmem_base;
 
   const int G = gridDim.x, U = a.n_tiles * a.KB;
-  // (up to 16 rows single units are dealt: split = KB, and the block arithmetic drops out)
-  auto begin_of = [&](int c) { return MP <= 16 ? unit_begin(c, U, G) : cta_begin(a, c, G); };
-  auto owner_of = [&](int u) { return MP <= 16 ? unit_owner(u, U, G) : cta_of_unit(a, u, G); };
-  const int u0 = begin_of(blockIdx.x), u1 = begin_of(blockIdx.x + 1);
+  const int u0 = unit_begin(blockIdx.x, U, G), u1 = unit_begin(blockIdx.x + 1, U, G);
   const Segs segs(u0, u1, a.KB);
   volatile int* abort_flag = &ctl.abort_flag;
-  constexpr int Mp = MP, sbytes = stage_bytes(Mp), nst = n_stages(Mp), ksplit = k_split(Mp), acols = acc_cols(Mp);
-  constexpr int plane_bytes = Mp * kBK * 2;
+  constexpr int Mp = kMaxRows, sbytes = kStageBytes, nst = kStages, ksplit = kSplit, acols = kAccCols;
+  constexpr int plane_bytes = kBBytes;
 
   if (warp == 0) {
     if (lane == 0) {   // ---- TMA producer
@@ -1045,26 +982,15 @@ k_umma_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
       const bool dry = seg < 0;
       if (seg == 0) {
         pdl_wait();   // everything below reads or writes what the kernel before this one touches
-        if (MP <= 16) {
-          for (int m = warp - 2; m < a.M; m += 4) {   // RMSNorm row scales of the input
-            float sc = 1.f;
-            if (a.ssq_in) {
-              float ss = 0.f;
-              for (int c = lane; c < a.ssq_n; c += 32) ss += a.ssq_in[(size_t)c * a.M + m];
-              ss = warp_sum(ss);
-              sc = rsqrtf(ss / (float)a.K + a.eps);
-            }
-            if (lane == 0) ctl.scale[m] = sc;
-          }
-        } else if (et < a.M) {   // many rows: one thread per row, its loads independent of each other
+        for (int m = warp - 2; m < a.M; m += 4) {   // RMSNorm row scales of the input
           float sc = 1.f;
           if (a.ssq_in) {
             float ss = 0.f;
-#pragma unroll 8
-            for (int c = 0; c < a.ssq_n; ++c) ss += a.ssq_in[(size_t)c * a.M + et];
+            for (int c = lane; c < a.ssq_n; c += 32) ss += a.ssq_in[(size_t)c * a.M + m];
+            ss = warp_sum(ss);
             sc = rsqrtf(ss / (float)a.K + a.eps);
           }
-          ctl.scale[et] = sc;
+          if (lane == 0) ctl.scale[m] = sc;
         }
         epi_sync();
       }
@@ -1094,35 +1020,24 @@ k_umma_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
       float* P = a.partials + ((size_t)blockIdx.x * 2 + slot) * kMaxRows * 128;
       bool finish = whole || dry;   // this CTA runs the tile's epilogue
       int c_first = blockIdx.x, c_last = blockIdx.x;
-      // (launches of more than 16 rows keep a partial as [accumulator row][activation row]: a
-      // thread writes and reads its 16 rows of a chunk as four 16-byte vectors)
-      constexpr bool kBig = MP > 16 && EPI != EPI_LMHEAD;
       if (!whole && !dry) {
         for (int m0 = 0; m0 < a.M; m0 += 16) {
           float v[16];
           load_chunk(m0, v);
-          if (kBig) {
-            float4* d4 = reinterpret_cast<float4*>(P + (size_t)r * kMaxRows + m0);
-            d4[0] = make_float4(v[0], v[1], v[2], v[3]);
-            d4[1] = make_float4(v[4], v[5], v[6], v[7]);
-            d4[2] = make_float4(v[8], v[9], v[10], v[11]);
-            d4[3] = make_float4(v[12], v[13], v[14], v[15]);
-          } else {
 #pragma unroll
-            for (int m = 0; m < 16; ++m)
-              if (m0 + m < a.M) P[(m0 + m) * 128 + r] = v[m];
-          }
+          for (int m = 0; m < 16; ++m)
+            if (m0 + m < a.M) P[(m0 + m) * 128 + r] = v[m];
         }
         fence_before_sync();
         mbar_arrive(&ctl.acc_empty[buf]);
         epi_sync();
-        c_first = owner_of(t_begin);
-        c_last = owner_of(t_end - 1);
+        c_first = unit_owner(t_begin, U, G);
+        c_last = unit_owner(t_end - 1, U, G);
         if (et == 0) {
           // one thread publishes the block's partial (the barrier above ordered the other
           // threads' stores before this release) and, if it came last, acquires the others'
           int n_contrib = 0;   // CTAs between the owners of the tile's ends that hold any unit
-          for (int c = c_first; c <= c_last; ++c) n_contrib += begin_of(c) < begin_of(c + 1);
+          for (int c = c_first; c <= c_last; ++c) n_contrib += unit_begin(c, U, G) < unit_begin(c + 1, U, G);
           unsigned old;
           asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(&a.tile_tickets[t]) : "memory");
           const int last = old == (unsigned)(n_contrib - 1);
@@ -1135,9 +1050,9 @@ k_umma_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
       }
       if (finish && !whole) {   // where each contributor's partial lies (a CTA without units has none)
         for (int j = et; j <= c_last - c_first; j += kEpiThreads) {
-          const int c = c_first + j, cb = begin_of(c);
+          const int c = c_first + j, cb = unit_begin(c, U, G);
           int off = -1;
-          if (cb < begin_of(c + 1)) {
+          if (cb < unit_begin(c + 1, U, G)) {
             const int sl = (c == c_first && cb / a.KB != t) ? 1 : 0;
             off = (c * 2 + sl) * kMaxRows * 128;
           }
@@ -1145,54 +1060,7 @@ k_umma_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
         }
         epi_sync();
       }
-      if (finish && kBig) {
-        // many rows: the sums stay in registers from tensor memory (or from the partials, added in
-        // CTA order with all of a contributor's vectors in flight together) to the stores
-        bool valid;
-        const int n = tile_feature(a, t, r, valid);
-        const float bias = (EPI == EPI_STORE && a.bias && valid) ? __bfloat162float(a.bias[n]) : 0.f;
-        const float gain = (EPI == EPI_STORE && a.gain_next && valid) ? __bfloat162float(a.gain_next[n]) : 1.f;
-        const int nc = c_last - c_first + 1;
-        const int m_end = dry ? min(a.M, 16) : a.M;   // the rehearsal takes one chunk
-        for (int m0 = 0; m0 < m_end; m0 += 16) {
-          const int mc = min(16, a.M - m0);
-          float rv[16];
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            rv[j] = (EPI == EPI_STORE && a.res && valid && j < mc && !dry) ? __ldcg(a.res + (size_t)(m0 + j) * a.ldr + n) : 0.f;
-          float v[16];
-          if (whole) {
-            load_chunk(m0, v);
-            if (m0 + 16 >= a.M) {   // the accumulator is read: the MMA warp may reuse it
-              fence_before_sync();
-              mbar_arrive(&ctl.acc_empty[buf]);
-            }
-          } else {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = 0.f;
-            const float* Pr = a.partials + (size_t)r * kMaxRows + m0;
-#pragma unroll 1
-            for (int j0 = 0; j0 < nc; j0 += 2) {   // two contributors' vectors in flight at a time
-              const int o0 = ctl.coff[j0], o1 = j0 + 1 < nc ? ctl.coff[j0 + 1] : -1;
-              float4 x0[4], x1[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                x0[i] = o0 >= 0 ? __ldcg(reinterpret_cast<const float4*>(Pr + o0) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-                x1[i] = o1 >= 0 ? __ldcg(reinterpret_cast<const float4*>(Pr + o1) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-              }
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                v[4 * i] += x0[i].x; v[4 * i + 1] += x0[i].y; v[4 * i + 2] += x0[i].z; v[4 * i + 3] += x0[i].w;
-              }
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                v[4 * i] += x1[i].x; v[4 * i + 1] += x1[i].y; v[4 * i + 2] += x1[i].z; v[4 * i + 3] += x1[i].w;
-              }
-            }
-          }
-          big_chunk_epilogue<EPI>(a, ctl, n, valid, t, r, m0, mc, v, bias, gain, rv, dry);
-        }
-      } else if (finish) {
+      if (finish) {
         // 16 activation rows at a time: the tile's sums into ctl.acc (from tensor memory, or the
         // partials added in CTA order, which does not depend on who came last), then the epilogue
         const int m_end = dry ? min(a.M, 16) : a.M;   // the rehearsal takes one chunk
@@ -1239,7 +1107,7 @@ k_umma_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
               }
             }
           }
-          tile_epilogue<EPI, (MP > 16 ? 4 : 1)>(a, ctl, t, r, q, lane, m0, mc, dry);
+          tile_epilogue<EPI>(a, ctl, t, r, q, lane, m0, mc, dry);
         }
       }
     }
@@ -1256,7 +1124,7 @@ k_umma_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
   }
   if (warp == 1) {
     fence_after_sync();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols(MP)) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
   }
 }
 
@@ -1298,10 +1166,8 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
 }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
 
-template <int MP>
 __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_constant__ ChainParams p) {
   using namespace umma;
-  static_assert(MP == 16, "chained stages take up to 16 rows");
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -1318,7 +1184,7 @@ __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_c
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl.tmem_base)),
-                 "r"(tmem_cols(MP))
+                 "r"(kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -1329,8 +1195,8 @@ __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_c
 
   const int G = gridDim.x;
   volatile int* abort_flag = &ctl.abort_flag;
-  constexpr int sbytes = stage_bytes(MP), nst = n_stages(MP), ksplit = k_split(MP), acols = acc_cols(MP);
-  constexpr int plane_bytes = MP * kBK * 2;
+  constexpr int MP = kMaxRows, sbytes = kStageBytes, nst = kStages, ksplit = kSplit, acols = kAccCols;
+  constexpr int plane_bytes = kBBytes;
   auto stage_segs = [&](const UArgs& a) {
     const int U = a.n_tiles * a.KB;
     return Segs(unit_begin(blockIdx.x, U, G), unit_begin(blockIdx.x + 1, U, G), a.KB);
@@ -1655,9 +1521,9 @@ __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_c
           }
 #pragma unroll
           for (int m = 0; m < 16; ++m) ctl.acc[m * 128 + r] = v[m];
-          if (epi == EPI_STORE) tile_epilogue<EPI_STORE, 1>(a, ctl, t, r, q, lane, 0, mc, dry, res_pre);
-          else if (epi == EPI_SWIGLU) tile_epilogue<EPI_SWIGLU, 1>(a, ctl, t, r, q, lane, 0, mc, dry);
-          else tile_epilogue<EPI_LMHEAD, 1>(a, ctl, t, r, q, lane, 0, mc, dry);
+          if (epi == EPI_STORE) tile_epilogue<EPI_STORE>(a, ctl, t, r, q, lane, 0, mc, dry, res_pre);
+          else if (epi == EPI_SWIGLU) tile_epilogue<EPI_SWIGLU>(a, ctl, t, r, q, lane, 0, mc, dry);
+          else tile_epilogue<EPI_LMHEAD>(a, ctl, t, r, q, lane, 0, mc, dry);
           if (!dry && s + 1 < p.n) {   // one more tile of this stage is complete
             fence_proxy_async();
             epi_sync();
@@ -1682,7 +1548,7 @@ __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_c
   }
   if (warp == 1) {
     fence_after_sync();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols(MP)) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
   }
 }
 
@@ -1712,14 +1578,15 @@ __global__ void k_gather_x(const __nv_bfloat16* __restrict__ embed, const __nv_b
 }
 
 // Embedding-only input (PS_FLAG_NO_FC): x0 = embedding(token) for a sequence's first row, the
-// learned [MASK] embeddings after it; also the planes of x0 * g_in and each row's sum of
-// squares (one partial per row).  One block per row.
+// learned [MASK] embeddings after it; also the planes of x0 * g_in (with `normalise`: of the row's
+// RMS-normalised values) and each row's sum of squares (one partial per row).  One block per row.
+// (Normalised rows need no sums of squares.)
 __global__ void __launch_bounds__(256) k_embed_x0(const __nv_bfloat16* __restrict__ embed,
                                                   const __nv_bfloat16* __restrict__ mask_embed,
                                                   const int* __restrict__ tokens, const __nv_bfloat16* __restrict__ g_in,
                                                   int H, int V, int R, float* __restrict__ x0,
                                                   __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
-                                                  float* __restrict__ ssq) {
+                                                  float* __restrict__ ssq, int normalise, float eps) {
   __shared__ float s_part[8];
   pdl_launch_dependents();
   pdl_wait();
@@ -1729,17 +1596,23 @@ __global__ void __launch_bounds__(256) k_embed_x0(const __nv_bfloat16* __restric
   for (int n = threadIdx.x; n < H; n += blockDim.x) {
     const float x = __bfloat162float(e[n]);
     x0[(size_t)m * H + n] = x;
-    split_store(hi + (size_t)m * H + n, lo + (size_t)m * H + n, x * __bfloat162float(g_in[n]));
     ss += x * x;
   }
   ss = warp_sum(ss);
   if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = ss;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    float tot = 0.f;
-    for (int w = 0; w < 8; ++w) tot += s_part[w];
-    ssq[m] = tot;
-  }
+  float tot = 0.f;
+  for (int w = 0; w < 8; ++w) tot += s_part[w];
+  if (threadIdx.x == 0 && !normalise) ssq[m] = tot;
+  const float sc = normalise ? rsqrtf(tot / (float)H + eps) : 1.f;
+  for (int n = threadIdx.x; n < H; n += blockDim.x)
+    split_store(hi + (size_t)m * H + n, lo + (size_t)m * H + n, __bfloat162float(e[n]) * sc * __bfloat162float(g_in[n]));
+}
+
+// act = hi + lo (test helper: the rows of the last draft step as floats).
+__global__ void k_join_planes(const __nv_bfloat16* hi, const __nv_bfloat16* lo, float* out, size_t n) {
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+    out[i] = __bfloat162float(hi[i]) + __bfloat162float(lo[i]);
 }
 
 // The bounded wait of the GEMM kernels on a barrier that nothing ever completes: what a lost
@@ -1787,17 +1660,25 @@ bool make_map(CUtensorMap* m, const void* base, size_t rows, size_t cols, int bo
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-struct PlaneMaps {   // one activation plane with boxes of every padded row count (umma::kRowPads)
-  CUtensorMap m[umma::kNumRowPads];
+struct PlaneMaps {   // one activation plane: boxes of 16 rows, and of every size the CTA-pair GEMM takes
+  CUtensorMap m16;
+  pg::PlaneMaps pair;
 };
+constexpr int kPairStages = 8;   // fc, q|k|v, o, gate|up, down, LM head of a draft step; fc, k|v of an append
 struct UmmaMaps {
   CUtensorMap w_fc, w_q, w_k, w_v, w_o, w_gate, w_up, w_down, w_lm;
+  CUtensorMap w_gate128, w_up128;   // 128-row boxes (the others' gate / up boxes: 64 rows)
   PlaneMaps xin, x0_hi, x0_lo, attn_hi, attn_lo, a_hi, a_lo, act_hi, act_lo, hdn_hi, hdn_lo;
+  // how each stage was last dealt (a function of the shapes and the row count alone)
+  pg::Plan plan[kPairStages] = {};
 };
 
-bool make_plane_maps(PlaneMaps* pm, const void* base, size_t cols) {
-  for (int i = 0; i < umma::kNumRowPads; ++i)
-    if (!make_map(&pm->m[i], base, umma::kMaxRows, cols, umma::kRowPads[i])) return false;
+bool make_plane_maps(PlaneMaps* pm, const void* base, size_t rows, size_t cols) {
+  if (!make_map(&pm->m16, base, rows, cols, 16)) return false;
+  for (int i = 0; i < pg::kMaxNp / pg::kNpStep; ++i) {
+    if (i > 0 && (size_t)i * pg::kNpStep >= rows) { pm->pair.m[i] = pm->pair.m[i - 1]; continue; }   // never that many rows
+    if (!make_map(&pm->pair.m[i], base, rows, cols, (i + 1) * pg::kNpStep / 2)) return false;
+  }
   return true;
 }
 
@@ -1815,12 +1696,14 @@ UmmaMaps* build_maps(const ps_ctx* c, const FusedScratch& f) {
             make_map(&u->w_o, w.w_o, H, Hq, 128) && make_map(&u->w_gate, w.w_gate, F, H, 64) &&
             make_map(&u->w_up, w.w_up, F, H, 64) && make_map(&u->w_down, w.w_down, H, F, 128) &&
             make_map(&u->w_lm, w.w_lm, V, H, 128);
-  ok = ok && make_plane_maps(&u->xin, f.xin, 2 * H) && make_plane_maps(&u->x0_hi, f.x0p.hi, H) &&
-       make_plane_maps(&u->x0_lo, f.x0p.lo, H) && make_plane_maps(&u->attn_hi, f.attnp.hi, Hq) &&
-       make_plane_maps(&u->attn_lo, f.attnp.lo, Hq) && make_plane_maps(&u->a_hi, f.ap.hi, H) &&
-       make_plane_maps(&u->a_lo, f.ap.lo, H) && make_plane_maps(&u->act_hi, f.actp.hi, F) &&
-       make_plane_maps(&u->act_lo, f.actp.lo, F) && make_plane_maps(&u->hdn_hi, f.hdnp.hi, H) &&
-       make_plane_maps(&u->hdn_lo, f.hdnp.lo, H);
+  const size_t rd = draft_rows_cap(g), rx = std::max<size_t>(rd, append_rows_cap(g));
+  ok = ok && make_map(&u->w_gate128, w.w_gate, F, H, 128) && make_map(&u->w_up128, w.w_up, F, H, 128);
+  ok = ok && make_plane_maps(&u->xin, f.xin, rx, 2 * H) && make_plane_maps(&u->x0_hi, f.x0p.hi, rx, H) &&
+       make_plane_maps(&u->x0_lo, f.x0p.lo, rx, H) && make_plane_maps(&u->attn_hi, f.attnp.hi, rd, Hq) &&
+       make_plane_maps(&u->attn_lo, f.attnp.lo, rd, Hq) && make_plane_maps(&u->a_hi, f.ap.hi, rd, H) &&
+       make_plane_maps(&u->a_lo, f.ap.lo, rd, H) && make_plane_maps(&u->act_hi, f.actp.hi, rd, F) &&
+       make_plane_maps(&u->act_lo, f.actp.lo, rd, F) && make_plane_maps(&u->hdn_hi, f.hdnp.hi, rd, H) &&
+       make_plane_maps(&u->hdn_lo, f.hdnp.lo, rd, H);
   if (!ok) {
     delete u;
     return nullptr;
@@ -1828,38 +1711,9 @@ UmmaMaps* build_maps(const ps_ctx* c, const FusedScratch& f) {
   return u;
 }
 
-// Blocks per tile (UArgs::split) for a launch of M rows on G CTAs.  Up to 16 rows single units
-// are dealt (split = KB).  Beyond, a tile shared between CTAs costs more the more rows there
-// are (its partial sums come back 16 rows x one contributor at a time), so a model of the
-// slowest CTA picks the split.  Its constants are fitted on a B200 with 80 to 144 rows: 0.3 us
-// per unit, 2 us of epilogue per 16 rows of a finished tile, 1 us per contributor and 16 rows
-// of a shared tile plus 0.5 us per 16 rows to publish a partial.  (At these row counts a unit
-// brings 32 KB of activation planes from L2 beside its 16 KB of weights, and the launches are
-// bound by that traffic rather than by HBM: the split moves their time by a tenth at most.)
-static int choose_split(int M, int Mp, int n_tiles, int KB, int G) {
-  if (Mp <= 16) return KB;
-  const double t_unit = 0.3, t_epi = 2.0, t_trip = 1.0, t_part = 0.5;   // microseconds
-  const int chunks = (M + 15) / 16, finished = (n_tiles + G - 1) / G;
-  int best = 1;
-  double best_cost = 1e30;
-  for (int s = 1; s <= KB; s = (s < 16 ? s + 1 : (s < KB ? KB : KB + 1))) {
-    const long long S = (long long)n_tiles * s;
-    const int blocks = (int)((S + G - 1) / G), units = blocks * ((KB + s - 1) / s);
-    // contributors of a shared tile: its blocks lie on ceil(s / blocks) CTAs, one more when unaligned
-    const int contrib = std::min(s, (s + blocks - 1) / blocks + 1);
-    const double cost = units * t_unit + finished * chunks * t_epi +
-                        (s > 1 ? chunks * (contrib * t_trip + t_part) : 0.0);
-    if (cost < best_cost) { best_cost = cost; best = s; }
-  }
-  return best;
-}
-
-// Geometry of one GEMM stage: padded rows, tiles, k-blocks, the split, the shared scratch.
-// *mi = index of the padded row count in umma::kRowPads.
-ps_status prep_uargs(ps_ctx* c, UArgs& a, const FusedScratch& f, int* mi) {
-  *mi = 0;
-  while (umma::kRowPads[*mi] < a.M) ++*mi;
-  a.Mp = umma::kRowPads[*mi];
+// Geometry of one GEMM stage of up to 16 rows: tiles, k-blocks, the shared scratch.
+ps_status prep_uargs(ps_ctx* c, UArgs& a, const FusedScratch& f) {
+  if (a.M > umma::kMaxRows) return fail(c, PS_ERR_INVALID_ARG, "these stages take up to 16 rows");
   a.KB = (a.K + umma::kBK - 1) / umma::kBK;
   if (a.zip) {
     a.n_tiles = (a.N + 63) / 64;
@@ -1874,7 +1728,6 @@ ps_status prep_uargs(ps_ctx* c, UArgs& a, const FusedScratch& f, int* mi) {
     }
   }
   if ((long long)a.n_tiles * a.KB * (c->n_sm + 1) >= (1ll << 31)) return fail(c, PS_ERR_UNSUPPORTED, "too many GEMM units");
-  a.split = choose_split(a.M, a.Mp, a.n_tiles, a.KB, c->n_sm);
   a.partials = f.partials; a.tile_tickets = f.tile_tickets; a.status = c->dev_status;
   return PS_OK;
 }
@@ -1883,19 +1736,12 @@ template <int EPI>
 ps_status launch_umma(ps_ctx* c, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& a2,
                       const PlaneMaps& ph, const PlaneMaps& pl, UArgs& a, const FusedScratch& f,
                       cudaStream_t st) {
-  int mi;
-  ps_status s = prep_uargs(c, a, f, &mi);
+  ps_status s = prep_uargs(c, a, f);
   if (s) return s;
-  const CUtensorMap &bh = ph.m[mi], &bl = pl.m[mi];
-  auto kern = mi == 0   ? k_umma_gemm<EPI, 16>
-              : mi == 1 ? k_umma_gemm<EPI, 32>
-              : mi == 2 ? k_umma_gemm<EPI, 48>
-              : mi == 3 ? k_umma_gemm<EPI, 64>
-              : mi == 4 ? k_umma_gemm<EPI, 96>
-                        : k_umma_gemm<EPI, 128>;
+  auto kern = k_umma_gemm<EPI>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, umma::kSmemBytes);
   if (e != cudaSuccess) return cuda_check(c, e, "umma smem attribute");
-  e = launch_after(kern, dim3(c->n_sm), dim3(umma::kThreads), umma::kSmemBytes, st, !c->prof, a0, a1, a2, bh, bl, a);
+  e = launch_after(kern, dim3(c->n_sm), dim3(umma::kThreads), umma::kSmemBytes, st, !c->prof, a0, a1, a2, ph.m16, pl.m16, a);
   c->launches++;
   return cuda_check(c, e, "k_umma_gemm");
 }
@@ -1934,9 +1780,7 @@ ps_status run_stages(ps_ctx* c, StageDesc* d, int n, bool chain, int chain_id, c
   int nm = 0;
   for (int i = 0; i < n; ++i) {
     StageDesc& x = d[i];
-    int mi;
-    if ((s = prep_uargs(c, x.a, f, &mi))) return s;
-    if (mi != 0) return fail(c, PS_ERR_INVALID_ARG, "chained stages take up to 16 rows");
+    if ((s = prep_uargs(c, x.a, f))) return s;
     p.a[i] = x.a;
     p.epi[i] = x.epi;
     const CUtensorMap* am[3] = {x.a0, x.a1, x.a2};
@@ -1948,11 +1792,11 @@ ps_status run_stages(ps_ctx* c, StageDesc* d, int n, bool chain, int chain_id, c
     }
     if (nm + 2 > kChainMaps + (x.a.lo ? 0 : 1)) return fail(c, PS_ERR_INVALID_ARG, "too many tensor maps in a chain");
     p.map_bh[i] = nm;
-    p.maps[nm++] = x.ph->m[0];
+    p.maps[nm++] = x.ph->m16;
     p.map_bl[i] = p.map_bh[i];
-    if (x.a.lo) { p.map_bl[i] = nm; p.maps[nm++] = x.pl->m[0]; }
+    if (x.a.lo) { p.map_bl[i] = nm; p.maps[nm++] = x.pl->m16; }
   }
-  auto kern = k_umma_chain<16>;
+  auto kern = k_umma_chain;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, umma::kSmemBytes);
   if (e != cudaSuccess) return cuda_check(c, e, "chain smem attribute");
   // A dependent launch like the others.  Its CTAs wait for one another: the grid is one CTA per
@@ -1966,11 +1810,134 @@ ps_status run_stages(ps_ctx* c, StageDesc* d, int n, bool chain, int chain_id, c
   return cuda_check(c, e, "k_umma_chain");
 }
 
+// One stage on the CTA-pair GEMM (more than 16 rows) with the kernel that finishes its shared tiles.
+// `id` names the stage's place in the plan cache.
+ps_status pair_stage(ps_ctx* c, UmmaMaps& u, int id, pg::Mode mode, int M, int K, int planes, const pg::Weights& w,
+                     const PlaneMaps& hi, const PlaneMaps& lo, const FusedScratch& f, pg::Args& a, cudaStream_t st) {
+  pg::Plan& plan = u.plan[id];
+  if (plan.T == 0 || plan.M != M) plan = pg::make_plan(M, w, K, planes, mode, f.slot_floats, c->n_sm);
+  a.p = plan;
+  a.planes = planes;
+  a.part = f.slots;
+  ps_status s = pg::launch_gemm(c, w, hi.pair, lo.pair, a, mode, st);
+  if (s == PS_OK && mode != pg::MODE_RAW) s = pg::launch_finish_shared(c, a, mode, st);
+  return s;
+}
+
+ps_status pair_kv_append(ps_ctx* c, UmmaMaps& u, const SeqMap& sm, int rows, const void* hidden, const int* tokens,
+                         cudaStream_t st) {
+  const ps_config& g = c->cfg;
+  const ps_weights& w = c->w;
+  const int H = g.hidden, Hkv = g.n_kv_heads * g.head_dim, V = g.vocab;
+  typedef const __nv_bfloat16* BP;
+  const FusedScratch f = carve_fused(g, (char*)c->fused_scratch);
+  ps_status s;
+  prof_mark(c, st, "begin");
+  const cudaError_t ge = launch_after(k_gather_x, dim3(rows), dim3(256), 0, st, !c->prof, (BP)w.embed, (BP)w.mask_embed,
+                                      (BP)w.mask_feat, (BP)hidden + (size_t)sm.row_base * H, tokens + sm.row_base, H, V, 1,
+                                      f.xin);
+  c->launches++;
+  if (ge != cudaSuccess) return cuda_check(c, ge, "k_gather_x");
+  pg::Args a{};
+  if ((s = pair_stage(c, u, 6, pg::MODE_RAW, rows, 2 * H, 1, pg::Weights{{&u.w_fc}, {H}, 1, false}, u.xin, u.xin, f, a, st)))
+    return s;
+  if ((s = pg::launch_row_norm(c, a, H, (g.flags & PS_FLAG_FC_BIAS) ? (BP)w.b_fc : nullptr, nullptr, (BP)w.g_in, nullptr,
+                               f.x0p.hi, f.x0p.lo, st)))
+    return s;
+  prof_mark(c, st, "fc_norm");
+  pg::Args b{};
+  b.out = f.kv; b.ldo = 2 * Hkv;
+  if ((s = pair_stage(c, u, 7, pg::MODE_STORE, rows, H, 2, pg::Weights{{&u.w_k, &u.w_v}, {Hkv, Hkv}, 2, false}, u.x0_hi,
+                      u.x0_lo, f, b, st)))
+    return s;
+  if ((s = launch_rope_store_kv(c, sm, rows, f.kv, st))) return s;
+  prof_mark(c, st, "qkv_rope");
+  return PS_OK;
+}
+
+// The draft step with more than 16 rows: every GEMM stage is one launch over all rows, and its
+// row kernel (norm and planes) or shared-tile kernel follows.
+ps_status pair_draft_step(ps_ctx* c, UmmaMaps& u, const SeqMap& sm, int B, const void* hidden_last,
+                          const int* token_last, int top_n, int* top_ids, float* top_logit, float* row_max,
+                          float* row_lse, float* logits_out, float* feat_out, const SampleArgs* sa, cudaStream_t st) {
+  const ps_config& g = c->cfg;
+  const ps_weights& w = c->w;
+  const int H = g.hidden, Hq = g.n_heads * g.head_dim, Hkv = g.n_kv_heads * g.head_dim, F = g.ffn, V = g.vocab,
+            R = g.k_masks + 1, M = B * R;
+  typedef const __nv_bfloat16* BP;
+  const FusedScratch f = carve_fused(g, (char*)c->fused_scratch);
+  ps_status s;
+  prof_mark(c, st, "begin");
+  if (g.flags & PS_FLAG_NO_FC) {
+    const cudaError_t e = launch_after(k_embed_x0, dim3(M), dim3(256), 0, st, !c->prof, (BP)w.embed, (BP)w.mask_embed,
+                                       token_last, (BP)w.g_in, H, V, R, c->x0, f.x0p.hi, f.x0p.lo, f.ssq[0], 1, g.rms_eps);
+    c->launches++;
+    if (e != cudaSuccess) return cuda_check(c, e, "k_embed_x0");
+  } else {   // S1 x0 = W_fc [e ; f] (+ b), planes of rms(x0) * g_in
+    const cudaError_t e = launch_after(k_gather_x, dim3(M), dim3(256), 0, st, !c->prof, (BP)w.embed, (BP)w.mask_embed,
+                                       (BP)w.mask_feat, (BP)hidden_last, token_last, H, V, R, f.xin);
+    c->launches++;
+    if (e != cudaSuccess) return cuda_check(c, e, "k_gather_x");
+    pg::Args a{};
+    if ((s = pair_stage(c, u, 0, pg::MODE_RAW, M, 2 * H, 1, pg::Weights{{&u.w_fc}, {H}, 1, false}, u.xin, u.xin, f, a, st)))
+      return s;
+    if ((s = pg::launch_row_norm(c, a, H, (g.flags & PS_FLAG_FC_BIAS) ? (BP)w.b_fc : nullptr, nullptr, (BP)w.g_in, c->x0,
+                                 f.x0p.hi, f.x0p.lo, st)))
+      return s;
+  }
+  prof_mark(c, st, "fc_norm");
+  {  // S2 q|k|v
+    pg::Args a{};
+    a.out = f.qkv; a.ldo = Hq + 2 * Hkv;
+    if ((s = pair_stage(c, u, 1, pg::MODE_STORE, M, H, 2, pg::Weights{{&u.w_q, &u.w_k, &u.w_v}, {Hq, Hkv, Hkv}, 3, false},
+                        u.x0_hi, u.x0_lo, f, a, st)))
+      return s;
+  }
+  prof_mark(c, st, "qkv_rope");
+  if ((s = launch_attn_split(c, sm, B, f.qkv, f.att_ml, f.att_o, f.attn_tickets, f.attnp.hi, f.attnp.lo, st))) return s;
+  prof_mark(c, st, "attention");
+  {  // S4 a = x0 + W_o attn, planes of rms(a) * g_post
+    pg::Args a{};
+    if ((s = pair_stage(c, u, 2, pg::MODE_RAW, M, Hq, 2, pg::Weights{{&u.w_o}, {H}, 1, false}, u.attn_hi, u.attn_lo, f, a, st)))
+      return s;
+    if ((s = pg::launch_row_norm(c, a, H, nullptr, c->x0, (BP)w.g_post, c->a, f.ap.hi, f.ap.lo, st))) return s;
+  }
+  prof_mark(c, st, "o_proj");
+  {  // S5a act = silu(gate) * up
+    pg::Args a{};
+    a.hi = f.actp.hi; a.lo = f.actp.lo; a.ld_plane = F;
+    if ((s = pair_stage(c, u, 3, pg::MODE_SWIGLU, M, H, 2, pg::Weights{{&u.w_gate128, &u.w_up128}, {F, F}, 2, true}, u.a_hi,
+                        u.a_lo, f, a, st)))
+      return s;
+    c->act_rows = M;
+  }
+  prof_mark(c, st, "ffn_gate_up");
+  {  // S5b hdn = a + W_d act, planes of rms(hdn) * g_final
+    pg::Args a{};
+    if ((s = pair_stage(c, u, 4, pg::MODE_RAW, M, F, 2, pg::Weights{{&u.w_down}, {H}, 1, false}, u.act_hi, u.act_lo, f, a, st)))
+      return s;
+    if ((s = pg::launch_row_norm(c, a, H, nullptr, c->a, (BP)w.g_final, feat_out ? feat_out : c->hdn, f.hdnp.hi, f.hdnp.lo, st)))
+      return s;
+  }
+  prof_mark(c, st, "ffn_down");
+  {  // S6 logits, then their statistics in one pass (from L2)
+    float* logits = logits_out ? logits_out : c->logits;
+    pg::Args a{};
+    a.out = logits; a.ldo = V;
+    if ((s = pair_stage(c, u, 5, pg::MODE_STORE, M, H, 2, pg::Weights{{&u.w_lm}, {V}, 1, false}, u.hdn_hi, u.hdn_lo, f, a, st)))
+      return s;
+    if ((s = launch_logit_stats(c, logits, M, V, R, top_n, top_ids, top_logit, row_max, row_lse, sa, st))) return s;
+  }
+  prof_mark(c, st, "lm_head");
+  return PS_OK;
+}
+
 // ps_kv_append on the tensor-core GEMM: rows [sm.row_base, sm.row_base + rows) of the call's real
 // (token, feature) pairs: gather, fc (+ the planes of its normalised output), k | v projection,
 // then RoPE and the store into the cache rows (the kernel the plain path uses).
-ps_status umma_kv_append(ps_ctx* c, const UmmaMaps& u, const SeqMap& sm, int rows, const void* hidden,
+ps_status umma_kv_append(ps_ctx* c, UmmaMaps& u, const SeqMap& sm, int rows, const void* hidden,
                          const int* tokens, cudaStream_t st) {
+  if (rows > umma::kMaxRows) return pair_kv_append(c, u, sm, rows, hidden, tokens, st);
   const ps_config& g = c->cfg;
   const ps_weights& w = c->w;
   const int H = g.hidden, Hkv = g.n_kv_heads * g.head_dim, V = g.vocab;
@@ -2004,12 +1971,12 @@ ps_status umma_kv_append(ps_ctx* c, const UmmaMaps& u, const SeqMap& sm, int row
     a.out = c->kv_tmp; a.ldo = 2 * Hkv;
   }
   if ((s = run_stages(c, d, 2, chain, 0, f, st))) return s;
-  if ((s = launch_rope_store_kv(c, sm, rows, st))) return s;
+  if ((s = launch_rope_store_kv(c, sm, rows, c->kv_tmp, st))) return s;
   prof_mark(c, st, "qkv_rope");
   return PS_OK;
 }
 
-ps_status umma_draft_step(ps_ctx* c, const UmmaMaps& u, const SeqMap& sm, int B, const void* hidden_last,
+ps_status umma_draft_step(ps_ctx* c, UmmaMaps& u, const SeqMap& sm, int B, const void* hidden_last,
                           const int* token_last, int top_n, int* top_ids, float* top_logit, float* row_max,
                           float* row_lse, float* logits_out, float* feat_out, const SampleArgs* sa,
                           cudaStream_t st) {
@@ -2020,9 +1987,13 @@ ps_status umma_draft_step(ps_ctx* c, const UmmaMaps& u, const SeqMap& sm, int B,
   typedef const __nv_bfloat16* BP;
   const FusedScratch f = carve_fused(g, (char*)c->fused_scratch);
   const int tiles_h = (H + umma::kTile - 1) / umma::kTile;
-  // up to 16 rows the stages on either side of the attention run as one launch each (the stage
-  // timers need a launch per stage)
-  const bool chain = M <= 16 && (!c->prof || c->prof_launches) && !(g.flags & PS_FLAG_STAGE_LAUNCHES);
+  if (M > umma::kMaxRows)
+    return pair_draft_step(c, u, sm, B, hidden_last, token_last, top_n, top_ids, top_logit, row_max, row_lse, logits_out,
+                           feat_out, sa, st);
+  c->act_rows = 0;
+  // the stages on either side of the attention run as one launch each (the stage timers need a
+  // launch per stage)
+  const bool chain = (!c->prof || c->prof_launches) && !(g.flags & PS_FLAG_STAGE_LAUNCHES);
   ps_status s;
   prof_mark(c, st, "begin");
   const bool no_fc = (g.flags & PS_FLAG_NO_FC) != 0;
@@ -2030,7 +2001,7 @@ ps_status umma_draft_step(ps_ctx* c, const UmmaMaps& u, const SeqMap& sm, int B,
   int n = 0;
   if (no_fc) {   // embedding-only input: x0 and its planes come straight from the embedding rows
     cudaError_t ee = launch_after(k_embed_x0, dim3(M), dim3(256), 0, st, !c->prof, (BP)w.embed, (BP)w.mask_embed,
-                                  token_last, (BP)w.g_in, H, V, R, c->x0, f.x0p.hi, f.x0p.lo, f.ssq[0]);
+                                  token_last, (BP)w.g_in, H, V, R, c->x0, f.x0p.hi, f.x0p.lo, f.ssq[0], 0, g.rms_eps);
     c->launches++;
     if (ee != cudaSuccess) return cuda_check(c, ee, "k_embed_x0");
     prof_mark(c, st, "fc_norm");
@@ -2091,32 +2062,19 @@ ps_status umma_draft_step(ps_ctx* c, const UmmaMaps& u, const SeqMap& sm, int B,
     a.ssq_out = f.ssq[2];
     a.out_hi = f.hdnp.hi; a.out_lo = f.hdnp.lo; a.ld_plane = H; a.gain_next = (BP)w.g_final;
   }
-  const bool stats_pass = M > 16 && logits_out;
-  {
+  {  // S6 logits = W_lm rms(hdn), softmax statistics and top-n without a second pass over logits
     StageDesc& x = d[n++];
-    x = StageDesc{stats_pass ? EPI_STORE : EPI_LMHEAD, &u.w_lm, &u.w_lm, &u.w_lm, &u.hdn_hi, &u.hdn_lo, UArgs{}, "lm_head"};
+    x = StageDesc{EPI_LMHEAD, &u.w_lm, &u.w_lm, &u.w_lm, &u.hdn_hi, &u.hdn_lo, UArgs{}, "lm_head"};
     UArgs& a = x.a;
     a.N = V; a.K = H; a.M = M; a.n_mats = 1; a.mat_rows[0] = V; a.lo = 1;
     a.ssq_in = f.ssq[2]; a.ssq_n = tiles_h; a.eps = g.rms_eps;
-    if (stats_pass) {
-      // S6 with more than 16 rows and the logits kept: the statistics in the tile epilogue are serial
-      // in the rows (20 rows of the 13B shape with sampling: 140 us), so the GEMM only stores the
-      // logits and a kernel of its own reads them back from L2 (83 us together)
-      a.out = logits_out; a.ldo = V;
-      x.name = nullptr;   // (timed together with the statistics pass below)
-    } else {  // S6 logits = W_lm rms(hdn), softmax statistics and top-n without a second pass over logits
-      a.logits_out = logits_out; a.parts = f.parts; a.ticket = f.ticket;
-      a.top_n = top_n; a.top_ids = top_ids; a.top_logit = top_logit; a.row_max = row_max; a.row_lse = row_lse;
-      a.R = R;
-      if (sa) { a.sample = 1; a.sa = *sa; }
-    }
+    a.logits_out = logits_out; a.parts = f.parts; a.ticket = f.ticket;
+    a.top_n = top_n; a.top_ids = top_ids; a.top_logit = top_logit; a.row_max = row_max; a.row_lse = row_lse;
+    a.R = R;
+    if (sa) { a.sample = 1; a.sa = *sa; }
   }
   if ((s = run_stages(c, d, n, chain, 1, f, st))) return s;
   if (chain) prof_mark(c, st, "chain_o_ffn_lm");
-  if (stats_pass) {
-    if ((s = launch_logit_stats(c, logits_out, M, V, R, top_n, top_ids, top_logit, row_max, row_lse, sa, st))) return s;
-    prof_mark(c, st, "lm_head");
-  }
   return PS_OK;
 }
 
@@ -2133,14 +2091,14 @@ static void ensure_maps(ps_ctx* c) {
                           (uintptr_t)w.w_o | (uintptr_t)w.w_gate | (uintptr_t)w.w_up | (uintptr_t)w.w_down |
                           (uintptr_t)w.w_lm | (uintptr_t)w.embed | (uintptr_t)w.mask_embed |
                           (uintptr_t)w.mask_feat) & 15u) == 0);
-  if (aligned && c->smem_optin >= umma::kSmemBytes)
+  if (aligned && c->smem_optin >= std::max(umma::kSmemBytes, pg::smem_bytes()))
     c->umma_maps = build_maps(c, carve_fused(g, (char*)c->fused_scratch));
 }
 
 bool fused_supported(ps_ctx* c, int M) {
   const ps_config& g = c->cfg;
   if (g.dtype != PS_DTYPE_BF16 || (g.flags & PS_FLAG_UNFUSED_KERNELS)) return false;
-  if (M > umma::kMaxRows || (g.head_dim != 64 && g.head_dim != 128)) return false;
+  if (M > std::max(draft_rows_cap(g), append_rows_cap(g)) || (g.head_dim != 64 && g.head_dim != 128)) return false;
   const int Hq = g.n_heads * g.head_dim;
   if (g.hidden % 8 || Hq % 8 || g.ffn % 8) return false;   // 16-byte operand rows
   if ((g.vocab + 127) / 128 > umma::kRingBytes / 32) return false;   // a row's tile summaries fit the ring (LM-head merge)
@@ -2157,19 +2115,27 @@ bool fused_supported(ps_ctx* c, int M) {
 }
 
 int fused_row_limit(ps_ctx* c) {
-  if (fused_supported(c, umma::kMaxRows)) return umma::kMaxRows;
+  const int most = draft_rows_cap(c->cfg);
+  if (fused_supported(c, most)) return most;
   return fused_supported(c, kMaxM) ? kMaxM : 0;
 }
 
 // Rows per pass ps_kv_append may hand to fused_kv_append (0: the plain kernels serve).
 int fused_kv_rows(ps_ctx* c) {
   if (c->cfg.flags & PS_FLAG_NO_FC) return 0;
-  return fused_supported(c, umma::kMaxRows) && c->umma_maps ? umma::kMaxRows : 0;
+  const int most = append_rows_cap(c->cfg);
+  return fused_supported(c, most) && c->umma_maps ? most : 0;
 }
 
 ps_status fused_kv_append(ps_ctx* c, const SeqMap& sm, int rows, const void* hidden, const int* tokens,
                           cudaStream_t st) {
-  return umma_kv_append(c, *static_cast<const UmmaMaps*>(c->umma_maps), sm, rows, hidden, tokens, st);
+  return umma_kv_append(c, *static_cast<UmmaMaps*>(c->umma_maps), sm, rows, hidden, tokens, st);
+}
+
+// Zeroes the counters that every launch leaves at zero.
+cudaError_t fused_init(ps_ctx* c, cudaStream_t st) {
+  const size_t n = carve_fused(c->cfg, nullptr).counter_bytes;
+  return n ? cudaMemsetAsync(c->fused_scratch, 0, n, st) : cudaSuccess;
 }
 
 size_t fused_scratch_bytes(const ps_config& g) { return carve_fused(g, nullptr).bytes; }
@@ -2188,12 +2154,25 @@ void fused_release(ps_ctx* c) {
 ps_status fused_debug_buffer(ps_ctx* c, const char* name, void** ptr, size_t* bytes) {
   const ps_config& g = c->cfg;
   FusedScratch f = carve_fused(g, (char*)c->fused_scratch);
+  const size_t rd = draft_rows_cap(g);
+  if (g.dtype != PS_DTYPE_BF16) return PS_ERR_INVALID_ARG;
   if (!std::strcmp(name, "qkv")) {
     *ptr = f.qkv;
-    *bytes = (size_t)umma::kMaxRows * (g.n_heads + 2 * g.n_kv_heads) * g.head_dim * 4;
+    *bytes = rd * (g.n_heads + 2 * g.n_kv_heads) * g.head_dim * 4;
     return PS_OK;
   }
-  if (!std::strcmp(name, "act")) { *ptr = f.act; *bytes = (size_t)umma::kMaxRows * g.ffn * 4; return PS_OK; }
+  if (!std::strcmp(name, "act")) {
+    if (c->act_rows > 0) {   // with more than 16 rows the step keeps only the planes of act
+      const size_t n = (size_t)c->act_rows * g.ffn;
+      cudaError_t e = cudaDeviceSynchronize();
+      k_join_planes<<<148, 256>>>(f.actp.hi, f.actp.lo, f.act, n);
+      if (e == cudaSuccess) e = cudaDeviceSynchronize();
+      if (e != cudaSuccess) return cuda_check(c, e, "act planes");
+    }
+    *ptr = f.act;
+    *bytes = rd * g.ffn * 4;
+    return PS_OK;
+  }
   return PS_ERR_INVALID_ARG;
 }
 
@@ -2210,14 +2189,14 @@ ps_status fused_draft_step(ps_ctx* c, const SeqMap& sm, int B, const void* hidde
   if (sa && !c->umma_maps && !logits_out)
     return fail(c, PS_ERR_UNSUPPORTED, "draft sampling on the mma.sync kernels needs logits_out");
   if (c->umma_maps && !(g.flags & PS_FLAG_MMA_SYNC_GEMM))
-    return umma_draft_step(c, *static_cast<const UmmaMaps*>(c->umma_maps), sm, B, hidden_last, token_last, top_n,
+    return umma_draft_step(c, *static_cast<UmmaMaps*>(c->umma_maps), sm, B, hidden_last, token_last, top_n,
                            top_ids, top_logit, row_max, row_lse, logits_out, feat_out, sa, st);
   ps_status s;
   prof_mark(c, st, "begin");
   const bool no_fc = (g.flags & PS_FLAG_NO_FC) != 0;
   if (no_fc) {   // embedding-only input: x0 and its planes come straight from the embedding rows
     k_embed_x0<<<M, 256, 0, st>>>((BP)w.embed, (BP)w.mask_embed, token_last, (BP)w.g_in, H, V, R, c->x0,
-                                  f.x0p.hi, f.x0p.lo, f.ssq[0]);
+                                  f.x0p.hi, f.x0p.lo, f.ssq[0], 0, g.rms_eps);
     c->launches++;
   } else {  // S1 fc: x0 = W_fc [e ; f] (+ b)
     GemmArgs a{};

@@ -1,0 +1,644 @@
+// GEMM of the draft step beyond 16 activation rows, and of the cache append: CTA pairs on the
+// 5th-generation tensor cores.
+//
+// Two CTAs (one cluster, the two SMs of a TPC) work on one tile of 256 weight rows (128 per CTA;
+// twice that with wt = 2) times Np <= 256 activation rows with tcgen05.mma.cta_group::2: each CTA
+// brings its own weight rows and HALF of the activation rows into shared memory, the tensor
+// cores read both halves.  What bounds these launches beside the weight stream is the traffic of
+// the activation planes from L2: a CTA that works alone needs 2 * Np * 128 bytes of planes (hi and
+// lo) beside every 16 KB weight box; in a pair it needs half of that, and with two weight
+// sub-tiles per CTA a quarter.
+// Activations are fp32 values split into bf16 hi + lo planes (x = hi + lo to about 2^-17); both
+// products go to the same fp32 accumulator in tensor memory.
+//
+// Warp roles per CTA: warp 0 issues the TMA loads of its own shared memory (completion counted
+// on the leader's barrier), warp 1 allocates tensor memory and, in the leader CTA, issues the
+// MMAs for both; warps 2..9 read the accumulators back and store them (two warps per lane
+// quadrant, alternating column chunks).  Accumulators are double buffered when two tiles' fit
+// tensor memory (wt * Np <= 256).
+//
+// A tile whose k range is shared by several pairs is left as partial sums in slots (see Plan) and
+// finished by a kernel of its own: no CTA waits for another cluster, the sums are added in k
+// order whoever finishes first, and for the stages whose output is normalised per row that
+// kernel sees whole rows, so it forms the norm on the spot.
+//
+// Measured (13B shape, whole calls) against one CTA per tile of 128 weight rows and at most 128
+// activation rows per pass over the weights: 80 rows 512 -> 454 us, 576 rows 2.97 -> 1.76 ms, 33B
+// shape 144 rows 1.39 -> 0.96 ms, 640 training rows 2.82 -> 1.50 ms, 4000 prompt rows appended
+// 5.69 -> 1.88 ms.  GEMM launches alone at 80 rows: gate|up 95 -> 59 us (4.8 TB/s of weights), at
+// 576 rows 475 -> 222 us (1.47 PFLOP/s of hi + lo products).
+#include <cfloat>
+
+#include "pair_gemm.cuh"
+#include "umma_gemm.cuh"
+
+namespace ps {
+namespace pg {
+namespace {
+
+using umma::fence_after_sync;
+using umma::fence_before_sync;
+using umma::kABytes;
+using umma::kBK;
+using umma::mbar_arrive_expect_tx;
+using umma::mbar_init;
+using umma::mbar_wait;
+using umma::smem_desc;
+using umma::smem_u32;
+
+constexpr int kEpiWarps = 8;
+constexpr int kThreads = 64 + 32 * kEpiWarps;
+constexpr int kRing = 222 * 1024;
+constexpr int kMaxStages = 12;
+constexpr uint32_t kPeerMask = 0xFEFFFFFFu;   // shared::cluster address of the same offset in the leader CTA
+
+struct Ctl {
+  uint64_t full[kMaxStages];    // leader: a stage's boxes of both CTAs have landed
+  uint64_t empty[kMaxStages];   // the MMAs that read a stage have completed (one per CTA)
+  uint64_t acc_full[2];         // an accumulator holds a finished segment (one per CTA)
+  uint64_t acc_empty[2];        // leader: the epilogue warps of both CTAs have read it back
+  uint32_t tmem_base;
+  int abort_flag;
+};
+constexpr int kSmem = kRing + 1024 + (int)sizeof(Ctl);
+
+__host__ __device__ constexpr int stage_bytes(int wt, int planes, int Np) {
+  return wt * kABytes + planes * (Np / 2) * kBK * 2;
+}
+__host__ __device__ constexpr int n_stages(int bytes) {
+  return kRing / bytes < kMaxStages ? kRing / bytes : kMaxStages;
+}
+
+// Instruction descriptor of kind::f16 for a CTA pair: fp32 accumulator, bf16 x bf16, both operands
+// K-major, N / 8 in bits [17,23), M / 16 = 16 in bits [24,29).
+__device__ __forceinline__ uint32_t pair_idesc(int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | (16u << 24);
+}
+__device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t leader_bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+          dst),
+      "l"(map), "r"(x), "r"(y), "r"(leader_bar)
+      : "memory");
+}
+__device__ __forceinline__ void mma_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+      "l"(a), "l"(b), "r"(id), "r"(acc)
+      : "memory");
+}
+// Arrives on the barrier of this offset in both CTAs once the MMAs issued so far have completed.
+__device__ __forceinline__ void commit_pair(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          smem_u32(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+__device__ __forceinline__ void arrive_leader(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(smem_u32(bar) & kPeerMask) : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// 16 accumulator columns of this thread's lane; the caller waits (tmem_ld_wait) before it uses them.
+__device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ void split1(float x, __nv_bfloat16& h, __nv_bfloat16& l) {
+  h = __float2bfloat16_rn(x);
+  l = __float2bfloat16_rn(x - __bfloat162float(h));
+}
+// hi/lo planes of four consecutive values as 8-byte stores.
+__device__ __forceinline__ void split4(const float4& v, __nv_bfloat16* hi, __nv_bfloat16* lo) {
+  __align__(8) __nv_bfloat16 h[4], l[4];
+  split1(v.x, h[0], l[0]); split1(v.y, h[1], l[1]); split1(v.z, h[2], l[2]); split1(v.w, h[3], l[3]);
+  *reinterpret_cast<uint2*>(hi) = *reinterpret_cast<uint2*>(h);
+  *reinterpret_cast<uint2*>(lo) = *reinterpret_cast<uint2*>(l);
+}
+// Four bf16 values (of a gain or bias vector, which the caller may have put on any 2-byte boundary).
+__device__ __forceinline__ float4 load_bf4(const __nv_bfloat16* x) {
+  return make_float4(__bfloat162float(x[0]), __bfloat162float(x[1]), __bfloat162float(x[2]), __bfloat162float(x[3]));
+}
+__device__ __forceinline__ float silu_mul(float g, float u) { return g / (1.f + __expf(-g)) * u; }
+
+// The segments (tile, k range) of a pair, in working order: its run of shared blocks first, then
+// its whole tiles.
+struct Seg { int t, kb0, kb1, j; bool whole; };
+struct SegWalk {
+  int x, x_end, d, P;
+  __device__ void start(const Plan& p, int pair, int n_pairs) {
+    P = n_pairs;
+    d = pair;
+    x = x_end = 0;
+    if (p.rem > 0 && pair < p.Pe) { x = run_begin(p, pair); x_end = run_begin(p, pair + 1); }
+  }
+  __device__ bool next(const Plan& p, int pair, Seg& s) {
+    if (x < x_end) {
+      const int tr = x / p.split, j0 = x - tr * p.split, x2 = min(x_end, (tr + 1) * p.split), j1 = x2 - tr * p.split;
+      s.t = p.n_dp + tr;
+      s.kb0 = j0 * p.KB / p.split;
+      s.kb1 = j1 * p.KB / p.split;
+      s.j = pair - run_owner(p, tr * p.split);
+      s.whole = j0 == 0 && j1 == p.split;
+      x = x2;
+      return true;
+    }
+    if (d < p.n_dp) {
+      s.t = d; s.kb0 = 0; s.kb1 = p.KB; s.j = 0; s.whole = true;
+      d += P;
+      return true;
+    }
+    return false;
+  }
+};
+// Walks a pair's units (segment, k-block) in working order.
+struct UnitWalk {
+  SegWalk sw;
+  Seg s;
+  int kb, mat, row0, yb;   // matrix and first weight row of the tile, first activation row
+  bool ok;
+  __device__ void enter(const Plan& p, int pair, bool zip) {
+    ok = sw.next(p, pair, s);
+    if (!ok) return;
+    kb = s.kb0;
+    int w = s.t / p.n_rt;
+    yb = (s.t - w * p.n_rt) * p.Np;
+    mat = 0;
+    if (!zip)
+      while (mat + 1 < p.n_mats && w >= p.mat_tiles[mat]) { w -= p.mat_tiles[mat]; ++mat; }
+    row0 = w * (zip ? 256 : 256 * p.wt);
+  }
+  __device__ void start(const Plan& p, int pair, int n_pairs, bool zip) {
+    sw.start(p, pair, n_pairs);
+    enter(p, pair, zip);
+  }
+  __device__ void next(const Plan& p, int pair, bool zip) {
+    if (++kb == s.kb1) enter(p, pair, zip);
+  }
+};
+
+template <int MODE, int WT>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+k_pair_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUtensorMap tA1,
+            const __grid_constant__ CUtensorMap tA2, const __grid_constant__ CUtensorMap tBh,
+            const __grid_constant__ CUtensorMap tBl, const __grid_constant__ Args a) {
+  constexpr bool kZip = MODE == MODE_SWIGLU;
+  static_assert(!kZip || WT == 2, "gate and up rows are the two sub-tiles");
+  extern __shared__ unsigned char smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  Ctl& ctl = *reinterpret_cast<Ctl*>(smem_raw + (base - raw) + kRing);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = cluster_rank();
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const Plan& p = a.p;
+  const int Np = p.Np, planes = a.planes;
+  const int sbytes = stage_bytes(WT, planes, Np), nst = n_stages(sbytes), plane_bytes = (Np / 2) * kBK * 2;
+  const bool two_buf = WT * Np <= 256;
+
+  if (tid == 0) {
+    for (int i = 0; i < kMaxStages; ++i) { mbar_init(&ctl.full[i], 1); mbar_init(&ctl.empty[i], 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&ctl.acc_full[i], 1); mbar_init(&ctl.acc_empty[i], 2 * kEpiWarps); }
+    ctl.abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    pdl_launch_dependents();
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl.tmem_base)), "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  __syncthreads();
+  fence_before_sync();
+  cluster_sync();   // both CTAs' barriers are initialised, both have their tensor memory
+  fence_after_sync();
+  const uint32_t tmem = *(volatile uint32_t*)&ctl.tmem_base;
+  volatile int* abort_flag = &ctl.abort_flag;
+
+  if (warp == 0) {
+    if (lane == 0) {   // ---- TMA producer
+      const uint32_t pair_bytes = 2u * (uint32_t)sbytes;
+      auto load_a = [&](const UnitWalk& u, int st) {
+        const uint32_t dst = base + st * sbytes, bar = smem_u32(&ctl.full[st]) & kPeerMask;
+        if (rank == 0) mbar_arrive_expect_tx(&ctl.full[st], pair_bytes);
+        const int x = u.kb * kBK, y = u.row0 + (int)rank * 128;
+        if (kZip) {
+          tma_load_pair(dst, &tA0, x, y, bar);
+          tma_load_pair(dst + kABytes, &tA1, x, y, bar);
+        } else {
+          const CUtensorMap* m = u.mat == 0 ? &tA0 : (u.mat == 1 ? &tA1 : &tA2);
+#pragma unroll
+          for (int s = 0; s < WT; ++s) tma_load_pair(dst + s * kABytes, m, x, y + 256 * s, bar);
+        }
+      };
+      auto load_b = [&](const UnitWalk& u, int st) {
+        const uint32_t dst = base + st * sbytes + WT * kABytes, bar = smem_u32(&ctl.full[st]) & kPeerMask;
+        const int x = u.kb * kBK, y = u.yb + (int)rank * (Np / 2);
+        tma_load_pair(dst, &tBh, x, y, bar);
+        if (planes == 2) tma_load_pair(dst + plane_bytes, &tBl, x, y, bar);
+      };
+      // the weights do not depend on the kernel before this one, the activations do
+      UnitWalk u;
+      u.start(p, pair, n_pairs, kZip);
+      int n_early = 0;
+      for (; n_early < nst && u.ok; ++n_early) { load_a(u, n_early); u.next(p, pair, kZip); }
+      pdl_wait();
+      UnitWalk v;
+      v.start(p, pair, n_pairs, kZip);
+      for (int i = 0; i < n_early; ++i) { load_b(v, i); v.next(p, pair, kZip); }
+      int st = 0;
+      uint32_t parity = 0;
+      while (u.ok) {
+        if (!mbar_wait(&ctl.empty[st], parity, abort_flag)) break;
+        load_a(u, st);
+        load_b(u, st);
+        u.next(p, pair, kZip);
+        if (++st == nst) { st = 0; parity ^= 1; }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0 && rank == 0) {   // ---- MMA issuer of the pair
+      SegWalk sw;
+      sw.start(p, pair, n_pairs);
+      Seg s;
+      const uint32_t id = pair_idesc(Np);
+      int st = 0, segc = 0;
+      uint32_t parity = 0;
+      bool alive = true;
+      for (; alive && sw.next(p, pair, s); ++segc) {
+        const int buf = two_buf ? (segc & 1) : 0;
+        const uint32_t use = two_buf ? (uint32_t)(segc >> 1) : (uint32_t)segc;
+        if (!mbar_wait(&ctl.acc_empty[buf], (use & 1) ^ 1, abort_flag)) break;
+        fence_after_sync();
+        const uint32_t d = tmem + buf * WT * Np;
+        uint32_t acc = 0;
+        for (int kb = s.kb0; kb < s.kb1; ++kb) {
+          if (!mbar_wait(&ctl.full[st], parity, abort_flag)) { alive = false; break; }
+          fence_after_sync();
+          const uint32_t sa = base + st * sbytes, sb = sa + WT * kABytes;
+#pragma unroll
+          for (int k = 0; k < kBK / 16; ++k) {
+#pragma unroll
+            for (int w = 0; w < WT; ++w)
+              mma_pair(d + w * Np, smem_desc(sa + w * kABytes + k * 32), smem_desc(sb + k * 32), id, acc | (k > 0));
+            if (planes == 2) {
+#pragma unroll
+              for (int w = 0; w < WT; ++w)
+                mma_pair(d + w * Np, smem_desc(sa + w * kABytes + k * 32), smem_desc(sb + plane_bytes + k * 32), id, 1u);
+            }
+          }
+          acc = 1;
+          commit_pair(&ctl.empty[st]);
+          if (++st == nst) { st = 0; parity ^= 1; }
+        }
+        if (alive) commit_pair(&ctl.acc_full[buf]);
+      }
+    }
+  } else {
+    // ---- epilogue warps: accumulator lane r = 32 q + lane, column chunks of 16 alternating
+    const int q = warp & 3, half = (warp - 2) >> 2, r = 32 * q + lane;
+    SegWalk sw;
+    sw.start(p, pair, n_pairs);
+    Seg s;
+    pdl_wait();   // the slots and outputs written below may still be read by the kernel before this one
+    for (int segc = 0; sw.next(p, pair, s); ++segc) {
+      const int buf = two_buf ? (segc & 1) : 0;
+      const uint32_t use = two_buf ? (uint32_t)(segc >> 1) : (uint32_t)segc;
+      const bool ok = mbar_wait(&ctl.acc_full[buf], use & 1, abort_flag);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      fence_after_sync();
+      int w = s.t / p.n_rt;
+      const int rt = s.t - w * p.n_rt, m0 = rt * Np, mrows = min(Np, p.M - m0);
+      const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + buf * WT * Np;
+      const bool slots = MODE == MODE_RAW || !s.whole;
+      if (slots || !kZip) {
+        float* dst0;
+        size_t ld;
+        bool valid[WT];
+        if (slots) {
+          dst0 = a.part + slot_row(p, s.j, s.t, 0) + rank * 128 + r;
+          ld = 256 * WT;
+#pragma unroll
+          for (int i = 0; i < WT; ++i) valid[i] = true;
+        } else {
+          int mat = 0;
+          while (mat + 1 < p.n_mats && w >= p.mat_tiles[mat]) { w -= p.mat_tiles[mat]; ++mat; }
+          const int n = w * 256 * WT + (int)rank * 128 + r;
+          dst0 = a.out + (size_t)m0 * a.ldo + p.mat_off[mat] + n;
+          ld = a.ldo;
+#pragma unroll
+          for (int i = 0; i < WT; ++i) valid[i] = n + 256 * i < p.mat_rows[mat];
+        }
+        for (int c0 = half * 16; c0 < mrows; c0 += 32) {
+          uint32_t x[WT][16];
+#pragma unroll
+          for (int i = 0; i < WT; ++i) tmem_ld16_async(ta + i * Np + c0, x[i]);
+          umma::tmem_ld_wait();
+          float* d = dst0 + (size_t)c0 * ld;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+#pragma unroll
+            for (int i = 0; i < WT; ++i)
+              if (c0 + j < mrows && valid[i]) d[256 * i] = __uint_as_float(x[i][j]);
+            d += ld;
+          }
+        }
+      } else {   // a whole gate / up tile
+        const int n = w * 256 + (int)rank * 128 + r;
+        const bool valid = n < p.mat_rows[0];
+        for (int c0 = half * 16; c0 < mrows; c0 += 32) {
+          uint32_t xg[16], xu[16];
+          tmem_ld16_async(ta + c0, xg);
+          tmem_ld16_async(ta + Np + c0, xu);
+          umma::tmem_ld_wait();
+          const size_t at = (size_t)(m0 + c0) * a.ld_plane + n;
+          __nv_bfloat16 *h = a.hi + at, *l = a.lo + at;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            if (valid && c0 + j < mrows) split1(silu_mul(__uint_as_float(xg[j]), __uint_as_float(xu[j])), *h, *l);
+            h += a.ld_plane;
+            l += a.ld_plane;
+          }
+        }
+      }
+      fence_before_sync();
+      __syncwarp();
+      if (lane == 0) arrive_leader(&ctl.acc_empty[buf]);   // read back: the MMA warp may reuse it
+    }
+    fence_before_sync();
+  }
+
+  __syncthreads();
+  if (ctl.abort_flag) {
+    // let copies and MMAs that are still in flight finish before shared and tensor memory go
+    for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+    if (tid == 0) atomicOr(a.status, kStatTimeout);
+    __syncthreads();
+  }
+  cluster_sync();   // neither CTA leaves while the other's copies, MMAs or arrivals may still touch it
+  if (warp == 1) {
+    fence_after_sync();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+  }
+}
+
+// Shared tiles of a MODE_STORE / MODE_SWIGLU stage: adds the contributors' slots in k order.
+// Block (tile, 8 rows); bound by the latency of its few loads, so a thread has all rows of a
+// contributor in flight together.
+constexpr int kFinRows = 8;
+template <bool ZIP>
+__global__ void __launch_bounds__(256) k_finish_shared(const __grid_constant__ Args a) {
+  pdl_launch_dependents();
+  const Plan& p = a.p;
+  const int t = p.n_dp + blockIdx.x, cnt = tile_contributors(p, t);
+  int w = t / p.n_rt;
+  const int rt = t - w * p.n_rt, mi0 = blockIdx.y * kFinRows, m0 = rt * p.Np + mi0;
+  const int rows = min(min(kFinRows, p.Np - mi0), p.M - m0);
+  pdl_wait();
+  if (cnt < 2 || rows <= 0) return;
+  const int TW = 256 * p.wt;
+  if (ZIP) {
+    const int n = w * 256 + threadIdx.x;
+    float g[kFinRows], u[kFinRows];
+#pragma unroll
+    for (int i = 0; i < kFinRows; ++i) g[i] = u[i] = 0.f;
+    for (int j = 0; j < cnt; ++j) {
+      const float* s = a.part + slot_row(p, j, t, mi0) + threadIdx.x;
+      float xg[kFinRows], xu[kFinRows];
+#pragma unroll
+      for (int i = 0; i < kFinRows; ++i) {
+        xg[i] = i < rows ? __ldcg(s + (size_t)i * TW) : 0.f;
+        xu[i] = i < rows ? __ldcg(s + (size_t)i * TW + 256) : 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < kFinRows; ++i) { g[i] += xg[i]; u[i] += xu[i]; }
+    }
+    if (n < p.mat_rows[0]) {
+#pragma unroll
+      for (int i = 0; i < kFinRows; ++i) {
+        const size_t at = (size_t)(m0 + i) * a.ld_plane + n;
+        if (i < rows) split1(silu_mul(g[i], u[i]), a.hi[at], a.lo[at]);
+      }
+    }
+  } else {
+    int mat = 0;
+    while (mat + 1 < p.n_mats && w >= p.mat_tiles[mat]) { w -= p.mat_tiles[mat]; ++mat; }
+    for (int c = threadIdx.x; c < TW; c += 256) {
+      const int n = w * TW + c;
+      float v[kFinRows];
+#pragma unroll
+      for (int i = 0; i < kFinRows; ++i) v[i] = 0.f;
+      for (int j = 0; j < cnt; ++j) {
+        const float* s = a.part + slot_row(p, j, t, mi0) + c;
+        float x[kFinRows];
+#pragma unroll
+        for (int i = 0; i < kFinRows; ++i) x[i] = i < rows ? __ldcg(s + (size_t)i * TW) : 0.f;
+#pragma unroll
+        for (int i = 0; i < kFinRows; ++i) v[i] += x[i];
+      }
+      if (n < p.mat_rows[mat]) {
+#pragma unroll
+        for (int i = 0; i < kFinRows; ++i)
+          if (i < rows) a.out[(size_t)(m0 + i) * a.ldo + p.mat_off[mat] + n] = v[i];
+      }
+    }
+  }
+}
+
+// Row m of a MODE_RAW stage: the row's slots added in k order, bias and residual, the row's sum
+// of squares, the planes of its RMS-normalised values.  One block per row; a thread holds NV
+// vectors of four features in registers from the loads to the stores.
+constexpr int kNormThreads = 256;
+template <int NV>
+__global__ void __launch_bounds__(kNormThreads) k_row_norm(const __grid_constant__ Args a, int H, float eps,
+                                                           const __nv_bfloat16* __restrict__ bias, const float* res,
+                                                           const __nv_bfloat16* __restrict__ gain, float* out,
+                                                           __nv_bfloat16* hi, __nv_bfloat16* lo) {
+  __shared__ float s_part[kNormThreads / 32];
+  pdl_launch_dependents();
+  const Plan& p = a.p;
+  const int m = blockIdx.x, rt = m / p.Np, mi = m - rt * p.Np, tid = threadIdx.x;
+  const int sh = p.wt == 2 ? 9 : 8, TW = 1 << sh;
+  const bool out_vec = ((uintptr_t)out & 15) == 0;     // (the caller's feature rows may sit anywhere)
+  const size_t layer = (size_t)p.slot_T * p.Np * TW;   // floats between contributors
+  float4 x[NV], g[NV];
+  int cnt[NV], cmax = 0;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int n = 4 * (tid + i * kNormThreads);
+    cnt[i] = 0;
+    x[i] = g[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (n < H) {
+      cnt[i] = tile_contributors(p, (n >> sh) * p.n_rt + rt);
+      cmax = max(cmax, cnt[i]);
+      g[i] = load_bf4(gain + n);
+      if (bias) x[i] = load_bf4(bias + n);
+    }
+  }
+  pdl_wait();
+  float4 rv[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int n = 4 * (tid + i * kNormThreads);
+    rv[i] = (res && n < H) ? __ldcg(reinterpret_cast<const float4*>(res + (size_t)m * H + n)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  for (int j = 0; j < cmax; ++j) {
+    float4 v[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int n = 4 * (tid + i * kNormThreads);
+      const float* s = a.part + (size_t)j * layer + ((size_t)((n >> sh) * p.n_rt + rt) * p.Np + mi) * TW + (n & (TW - 1));
+      v[i] = j < cnt[i] ? __ldcg(reinterpret_cast<const float4*>(s)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int i = 0; i < NV; ++i) { x[i].x += v[i].x; x[i].y += v[i].y; x[i].z += v[i].z; x[i].w += v[i].w; }
+  }
+  float ss = 0.f;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    x[i].x += rv[i].x; x[i].y += rv[i].y; x[i].z += rv[i].z; x[i].w += rv[i].w;
+    ss += (x[i].x * x[i].x + x[i].y * x[i].y) + (x[i].z * x[i].z + x[i].w * x[i].w);
+  }
+  ss = warp_sum(ss);
+  if ((tid & 31) == 0) s_part[tid >> 5] = ss;
+  __syncthreads();
+  float tot = 0.f;
+#pragma unroll
+  for (int w = 0; w < kNormThreads / 32; ++w) tot += s_part[w];
+  const float sc = rsqrtf(tot / (float)H + eps);
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int n = 4 * (tid + i * kNormThreads);
+    if (n < H) {
+      if (out) {
+        float* o = out + (size_t)m * H + n;
+        if (out_vec) *reinterpret_cast<float4*>(o) = x[i];
+        else { o[0] = x[i].x; o[1] = x[i].y; o[2] = x[i].z; o[3] = x[i].w; }
+      }
+      const float4 y = make_float4(x[i].x * sc * g[i].x, x[i].y * sc * g[i].y, x[i].z * sc * g[i].z, x[i].w * sc * g[i].w);
+      split4(y, hi + (size_t)m * H + n, lo + (size_t)m * H + n);
+    }
+  }
+}
+
+// Modelled time of a launch (microseconds), for the choice between plans only.  A unit of a pair
+// (wt weight boxes and the planes beside them in both CTAs) takes the longest of: its share of HBM,
+// its share of L2 -> SM traffic, its MMAs (58 cycles at least, Np / 2 above).  A contributor more
+// costs its slots' way through L2 twice.
+double plan_cost(const Plan& p, int planes, int units, int contributors, int n_pairs) {
+  const double t_hbm = p.wt * 32.768e3 / (6.4e6 / n_pairs) / p.n_rt;
+  const double t_l2 = (p.wt * 32.768e3 + planes * p.Np * 128.0) / (10.0e6 / n_pairs);
+  const double t_mma = p.wt * planes * 4 * std::max(58.0, p.Np / 2.0) / 1.85e3;
+  const double slots = (double)p.rem * contributors * p.Np * 256.0 * p.wt * 4.0;
+  return units * std::max(t_hbm, std::max(t_l2, t_mma)) + (contributors > 1 ? 1.0 : 0.0) + 2.0 * slots / 6.0e6 +
+         p.wt * p.Np * 0.012;
+}
+
+}  // namespace
+
+int smem_bytes() { return kSmem; }
+
+Plan make_plan(int M, const Weights& w, int K, int planes, Mode mode, size_t part_floats, int n_sm) {
+  const int P = n_sm / 2;
+  Plan best{};
+  double best_cost = 1e30;
+  for (int wt = mode == MODE_SWIGLU ? 2 : 1; wt <= 2; ++wt) {
+    Plan p{};
+    p.M = M;
+    p.n_rt = (M + kMaxNp - 1) / kMaxNp;
+    p.Np = ((M + p.n_rt - 1) / p.n_rt + kNpStep - 1) / kNpStep * kNpStep;
+    p.wt = wt;
+    p.KB = (K + kBK - 1) / kBK;
+    p.n_mats = w.zip ? 1 : w.n_mats;
+    const int tile_rows = w.zip ? 256 : 256 * wt;
+    int off = 0;
+    for (int i = 0; i < p.n_mats; ++i) {
+      p.mat_rows[i] = w.rows[i];
+      p.mat_tiles[i] = (w.rows[i] + tile_rows - 1) / tile_rows;
+      p.mat_off[i] = off;
+      off += w.rows[i];
+      p.tiles_w += p.mat_tiles[i];
+    }
+    p.T = p.tiles_w * p.n_rt;
+    p.n_dp = p.T / P * P;
+    p.rem = p.T - p.n_dp;
+    p.slot_t0 = mode == MODE_RAW ? 0 : p.n_dp;
+    p.slot_T = p.T - p.slot_t0;
+    const size_t layer = (size_t)p.slot_T * p.Np * 256 * wt;
+    for (int s = 1; s <= std::min(kMaxSplit, p.KB); ++s) {
+      if (p.rem == 0 && s > 1) break;
+      p.split = s;
+      p.S = p.rem * s;
+      p.Pe = std::max(1, std::min(P, p.S));
+      int units = p.n_dp / P * p.KB, jmax = 1;
+      if (p.rem > 0) {
+        units += (p.S + p.Pe - 1) / p.Pe * ((p.KB + s - 1) / s);
+        for (int t = p.n_dp; t < p.T; ++t) jmax = std::max(jmax, tile_contributors(p, t));
+      }
+      p.shared = jmax > 1;
+      if (layer * ((mode == MODE_RAW || jmax > 1) ? jmax : 0) > part_floats) continue;
+      const double cost = plan_cost(p, planes, units, jmax, P);
+      if (cost < best_cost) { best_cost = cost; best = p; }
+    }
+  }
+  return best;   // (T == 0: the slots hold not even one contributor)
+}
+
+ps_status launch_gemm(ps_ctx* c, const Weights& w, const PlaneMaps& hi, const PlaneMaps& lo, Args& a, Mode mode,
+                      cudaStream_t st) {
+  const Plan& p = a.p;
+  if (p.T == 0) return fail(c, PS_ERR_CAPACITY, "GEMM scratch too small for the rows of the call");
+  auto kern = mode == MODE_RAW     ? (p.wt == 2 ? k_pair_gemm<MODE_RAW, 2> : k_pair_gemm<MODE_RAW, 1>)
+              : mode == MODE_STORE ? (p.wt == 2 ? k_pair_gemm<MODE_STORE, 2> : k_pair_gemm<MODE_STORE, 1>)
+                                   : k_pair_gemm<MODE_SWIGLU, 2>;
+  a.status = c->dev_status;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  if (e != cudaSuccess) return cuda_check(c, e, "pair gemm smem attribute");
+  const CUtensorMap &m1 = *w.map[w.n_mats > 1 ? 1 : 0], &m2 = *w.map[w.n_mats > 2 ? 2 : 0];
+  e = launch_after(kern, dim3(c->n_sm & ~1), dim3(kThreads), kSmem, st, !c->prof, *w.map[0], m1, m2,
+                   hi.m[p.Np / kNpStep - 1], lo.m[p.Np / kNpStep - 1], a);
+  c->launches++;
+  return cuda_check(c, e, "k_pair_gemm");
+}
+
+ps_status launch_finish_shared(ps_ctx* c, const Args& a, Mode mode, cudaStream_t st) {
+  const Plan& p = a.p;
+  if (!p.shared) return PS_OK;
+  const dim3 grid(p.rem, (std::min(p.Np, p.M) + kFinRows - 1) / kFinRows);
+  const cudaError_t e = mode == MODE_SWIGLU ? launch_after(k_finish_shared<true>, grid, dim3(256), 0, st, !c->prof, a)
+                                            : launch_after(k_finish_shared<false>, grid, dim3(256), 0, st, !c->prof, a);
+  c->launches++;
+  return cuda_check(c, e, "k_finish_shared");
+}
+
+ps_status launch_row_norm(ps_ctx* c, const Args& a, int H, const __nv_bfloat16* bias, const float* res,
+                          const __nv_bfloat16* gain, float* out, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t st) {
+  const int nv = (H / 4 + kNormThreads - 1) / kNormThreads;
+  if (nv > 32) return fail(c, PS_ERR_UNSUPPORTED, "hidden size beyond 32768");
+  auto kern = nv <= 5 ? k_row_norm<5> : nv <= 8 ? k_row_norm<8> : nv <= 16 ? k_row_norm<16> : k_row_norm<32>;
+  const cudaError_t e = launch_after(kern, dim3(a.p.M), dim3(kNormThreads), 0, st, !c->prof, a, H, c->cfg.rms_eps, bias, res,
+                                     gain, out, hi, lo);
+  c->launches++;
+  return cuda_check(c, e, "k_row_norm");
+}
+
+}  // namespace pg
+}  // namespace ps

@@ -398,15 +398,15 @@ ps_status plain_draft_step(ps_ctx* c, const SeqMap& sm, int B, const void* hidde
                                          top_logit, row_max, row_lse, logits_out, feat_out, sa, st);
 }
 
-ps_status launch_rope_store_kv(ps_ctx* c, const SeqMap& sm, int rows, cudaStream_t st) {
+ps_status launch_rope_store_kv(ps_ctx* c, const SeqMap& sm, int rows, const float* kv, cudaStream_t st) {
   const ps_config& g = c->cfg;
   if (g.dtype == PS_DTYPE_F32)
     k_rope_store<float><<<rows, 128, g.head_dim * sizeof(float), st>>>(
-        sm, nullptr, c->kv_tmp, (float*)c->kcache, (float*)c->vcache, nullptr, g.n_heads, g.n_kv_heads,
+        sm, nullptr, kv, (float*)c->kcache, (float*)c->vcache, nullptr, g.n_heads, g.n_kv_heads,
         g.head_dim, g.max_ctx, g.rope_base);
   else
     k_rope_store<__nv_bfloat16><<<rows, 128, g.head_dim * sizeof(float), st>>>(
-        sm, nullptr, c->kv_tmp, (__nv_bfloat16*)c->kcache, (__nv_bfloat16*)c->vcache, nullptr, g.n_heads,
+        sm, nullptr, kv, (__nv_bfloat16*)c->kcache, (__nv_bfloat16*)c->vcache, nullptr, g.n_heads,
         g.n_kv_heads, g.head_dim, g.max_ctx, g.rope_base);
   c->launches++;
   return cuda_check(c, cudaGetLastError(), "k_rope_store");

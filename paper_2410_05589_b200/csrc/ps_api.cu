@@ -178,7 +178,7 @@ ps_status ps_init(ps_ctx** out, const ps_config* cfg, const ps_weights* w, void*
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + go, kGuardFill, kGuardBytes, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->dev_status, 0, 256, st);
   if (e == cudaSuccess)
-    e = cudaMemsetAsync(c->fused_scratch, 0, fused_scratch_bytes(*cfg), st);
+    e = fused_init(c, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->tickets, 0, sizeof(unsigned) * PS_MAX_BATCH, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->tree_tickets, 0, sizeof(unsigned) * PS_MAX_BATCH, st);
   if (e != cudaSuccess || launch_rope_table(c, st) != PS_OK) {
@@ -377,8 +377,7 @@ static ps_status run_draft_rows(ps_ctx* c, const SeqMap& sm, int B, const void* 
   if (per_max < 1)
     return plain_draft_step(c, sm, B, hidden, tokens, top_n, top_ids, top_logit, row_max, row_lse,
                             logits_out, feat_out, sa, st);
-  // full groups first: a launch costs by its padded row count (16, 32, 64 or 128), so the
-  // remainder is better off alone in a small launch than evened out over large ones
+  // (only the mma.sync kernels, which take 16 rows, need more than one group)
   const int per = per_max;
   const size_t eb = g.dtype == PS_DTYPE_F32 ? 4 : 2;
   for (int b0 = 0; b0 < B; b0 += per) {

@@ -141,6 +141,7 @@ struct ps_ctx {
   void* fused_scratch;      // buffers of the fused bf16 path (see fused_kernels.cu)
   void* umma_maps = nullptr;   // tensor maps of the tensor-core GEMMs, built on first use
   bool umma_tried = false;
+  int act_rows = 0;            // rows of the last draft step whose "act" exists as planes only
   double* rope_inv_freq;    // [head_dim/2] base^(-2i/d), filled once at ps_init
   int n_sm;                 // multiprocessors of the context's device
   int smem_optin;           // opt-in shared memory per block
@@ -186,10 +187,11 @@ bool fused_supported(ps_ctx* c, int M);
 int fused_kv_rows(ps_ctx* c);     // rows per pass of fused_kv_append (0: not available)
 ps_status fused_kv_append(ps_ctx* c, const SeqMap& sm, int rows, const void* hidden, const int* tokens,
                           cudaStream_t st);
-// RoPE on the k half of kv_tmp rows [0, rows) and the store of k and v into the cache rows.
-ps_status launch_rope_store_kv(ps_ctx* c, const SeqMap& sm, int rows, cudaStream_t st);
+// RoPE on the k half of kv rows [0, rows) and the store of k and v into the cache rows.
+ps_status launch_rope_store_kv(ps_ctx* c, const SeqMap& sm, int rows, const float* kv, cudaStream_t st);
 int fused_row_limit(ps_ctx* c);   // most rows fused_supported() takes for this context (0: none)
 size_t fused_scratch_bytes(const ps_config& g);
+cudaError_t fused_init(ps_ctx* c, cudaStream_t st);   // zeroes the fused path's counters
 void fused_release(ps_ctx* c);   // frees what the fused path holds on the host
 ps_status fused_debug_buffer(ps_ctx* c, const char* name, void** ptr, size_t* bytes);
 ps_status launch_rope_table(ps_ctx* c, cudaStream_t st);

@@ -1,0 +1,27 @@
+"""CTA-pair GEMM path (more than 16 rows): edges of its row padding and row tiles, whole and shared
+tiles, ragged matrix ends, grouped-query k / v, bias and the embedding-only input (needs a B200)."""
+import numpy as np
+import pytest
+
+import synth
+from harness import Pair, logits_close
+
+pytestmark = pytest.mark.gpu
+
+
+# rows B * (k + 1): 17 and 33 (one past a padding step), 32 (none), 255 (one row tile, almost full),
+# 258 (two row tiles), 1152 (five row tiles: more tiles than CTA pairs, so some go whole)
+@pytest.mark.parametrize("B,k,kv_heads,bias,flags", [(17, 0, 6, False, 0), (33, 0, 2, True, 0), (16, 1, 6, False, 8),
+                                                     (85, 2, 3, False, 0), (86, 2, 6, True, 0), (128, 8, 6, False, 0)])
+def test_pair_gemm_rows_match_oracle(B, k, kv_heads, bias, flags):
+    s = synth.CONFIGS["mini"].with_(k_masks=k, n_kv_heads=kv_heads)
+    seqs = sorted({0, B // 2, B - 1})
+    p = Pair(s, B, with_bias=bias, lens=[1 + (7 * b) % 41 for b in range(B)], flags=flags, oracle_seqs=seqs)
+    got = p.gpu_step(top_n=1)
+    for b in seqs:
+        want = p.oracle_step(b)
+        assert logits_close(got["logits"][b], want["logits"], s.dtype) <= 1.0, b     # the logits gate
+    assert np.isfinite(got["logits"]).all()
+    assert p.g.check_guards() == 0 and p.g.poll() == 0
+    again = p.gpu_step(top_n=1)
+    assert np.array_equal(got["logits"], again["logits"])     # sums are added in k order, whoever is first
