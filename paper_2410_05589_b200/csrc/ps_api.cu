@@ -74,6 +74,8 @@ size_t carve(const ps_config& g, ps_ctx* c, char* base) {
   void* status = take(256);
   void* tickets = take(sizeof(unsigned) * PS_MAX_BATCH);
   void* vrec = take(sizeof(VerifyRec) * PS_MAX_BATCH * (PS_MAX_MASKS + 2));
+  void* vrow = take(sizeof(VerifyRow) * PS_MAX_BATCH * (PS_MAX_MASKS + 2));
+  void* vdraw = take(sizeof(VerifyDraw) * PS_MAX_BATCH);
   void* trec = take(sizeof(TreeRec) * PS_MAX_BATCH * (PS_MAX_TREE_NODES + 1));
   void* ttick = take(sizeof(unsigned) * PS_MAX_BATCH);
   void* x_in = take(Mx * 2 * H * 4);
@@ -100,7 +102,7 @@ size_t carve(const ps_config& g, ps_ctx* c, char* base) {
   void* st_res = take((size_t)g.max_batch * (R + 3) * 4);
   if (c) {
     c->kcache = kc; c->vcache = vc; c->dev_status = (int*)status; c->tickets = (unsigned*)tickets;
-    c->vrec = (VerifyRec*)vrec;
+    c->vrec = (VerifyRec*)vrec; c->vrow = (VerifyRow*)vrow; c->vdraw = (VerifyDraw*)vdraw;
     c->trec = (TreeRec*)trec; c->tree_tickets = (unsigned*)ttick;
     c->x_in = (float*)x_in; c->x0 = (float*)x0; c->xn = (float*)xn; c->q = (float*)q;
     c->kv_tmp = (float*)kv_tmp; c->kv_side = kv_side; c->attn = (float*)attn; c->a = (float*)a; c->an = (float*)an;

@@ -113,6 +113,19 @@ struct TreeRec {    // one per (sequence, decision row) of the token-tree verifi
   int bad;          // a non-finite logit was met
 };
 
+struct VerifyRow {  // one per (sequence, position): verdict and statistics of a row pair (streaming kernel)
+  int flags;        // bit 0: accepted; bit 1: a non-finite logit was met
+  int targ;         // arg-max of the target row
+  float tmax, dmax;
+  double st, sd;    // sums of exponentials relative to the maxima
+};
+
+struct VerifyDraw { // one per sequence: where its chain stops
+  int pos, acc;     // position to draw at (-1: none), accepted drafts before it
+  float tmax, dmax; // statistics of the position's row pair
+  double st, sd;
+};
+
 struct VerifyRec {  // one per (sequence, position): result of the acceptance test
   int accept;       // bit 0: accepted; bit 1: a non-finite logit was met
   int token;        // token to emit if this position ends the chain
@@ -133,6 +146,8 @@ struct ps_ctx {
   int* dev_status;
   unsigned* tickets;        // [max_batch] arrival counters of the verify kernel (zero between calls)
   ps::VerifyRec* vrec;      // [max_batch][PS_MAX_MASKS+2]
+  ps::VerifyRow* vrow;      // [max_batch][PS_MAX_MASKS+2]
+  ps::VerifyDraw* vdraw;    // [max_batch]
   ps::TreeRec* trec;        // [max_batch][PS_MAX_TREE_NODES+1]
   unsigned* tree_tickets;   // [max_batch], zero between calls
   float *x_in, *x0, *xn, *q, *kv_tmp, *attn, *a, *an, *gate, *up, *hdn, *hn, *logits;

@@ -627,11 +627,435 @@ __global__ void __launch_bounds__(kCluThreads) k_verify_cluster16(VerifyArgs a) 
   verify_cluster_body<16, kCluV4>(a);
 }
 // Four blocks per row pair: for batches whose 8-block clusters would not be resident at once
-// (one block fills an SM), while a thread can still hold its share of a row (16 tokens).
+// (one block fills an SM) while these are, and a thread can still hold its share of a row (16 tokens).
 constexpr int kCluSmall = 4;
 constexpr int kCluSmallMaxVocab = kCluSmall * kCluThreads * 4 * kCluV4;
 __global__ void __cluster_dims__(kCluSmall, 1, 1) __launch_bounds__(kCluThreads) k_verify_cluster4(VerifyArgs a) {
   verify_cluster_body<kCluSmall, kCluV4>(a);
+}
+
+// ---- streaming variant: many row pairs --------------------------------------------------------
+// When a call has so many row pairs that the register-resident clusters above would run in
+// several waves, what counts is throughput: a row pair goes to a cluster of 1 to 8 blocks of few
+// registers, four of them resident per SM, that stream both rows once (so the HBM reads of one
+// hide the exponentials of another), and the draw, which needs the rows again, is done for ONE
+// position per sequence only: every row pair leaves its statistics and its verdict in a record, the
+// last cluster of a sequence to finish walks the verdicts and notes where the chain stops.
+// Exponentials are taken against a reference value of the block (the maximum of its first
+// batch) instead of the row's maximum, which is not known yet; their relative precision is the
+// same, and the sums are moved to the maximum once, in double.  Should the maximum lie far from the
+// reference, the sums are formed again.
+// The draws are a launch of their own (k_verify_draw) over all sequences, eight blocks each: done by
+// the last cluster of a sequence, a block or two would read a row pair while the rest of the chip
+// idles (576 pairs of 32000 tokens: 122 us in all, 43 us of it without the draws).
+// Measured (T = 1, rows from HBM) against the register-resident clusters in waves: 40 pairs of 32000
+// tokens 28.0 -> 20.6 us, 80 pairs 40.2 -> 23.7, 144 pairs 61.5 -> 32.9, 576 pairs 210 -> 50.9 us (2.9
+// TB/s; the exponentials and their double-precision sums bound it); 208 pairs of 128256 tokens 442 ->
+// 75.5 us.
+constexpr int kStrThreads = 256, kStrPerSm = 4, kStrWarps = kStrThreads / 32;
+struct StreamPart {    // one per block, read by its cluster
+  float tmax, dmax, tref, dref;
+  int targ, bad;
+  double st, sd;
+};
+struct StreamScratch {
+  float f[kStrWarps], f2[kStrWarps];
+  int i[kStrWarps];
+  double d[kStrWarps], d2[kStrWarps];
+};
+constexpr float kRefSlack = 60.f;   // exponent range left beside the reference before sums are formed again
+
+// exp argument (t - m) / T with one rounding: in single precision with the rounding errors of the
+// difference and of the product carried along (i_hi + i_lo = 1 / T).  UNIT: T = 1.
+template <bool UNIT>
+__device__ __forceinline__ float exp_arg(float t, float m, float i_hi, float i_lo) {
+  const float d = t - m;
+  if (UNIT) return d;
+  const float bv = t - d, av = d + bv;
+  const float e = (t - av) + (bv - m);
+  const float p = d * i_hi;
+  const float r = p + (fmaf(d, i_hi, -p) + fmaf(e, i_hi, d * i_lo));
+  return d == -INFINITY ? d : r;   // (a NaN stays one)
+}
+
+template <bool UNIT>
+__global__ void __launch_bounds__(kStrThreads, kStrPerSm) k_verify_stream(VerifyArgs a, VerifyRow* rows, VerifyDraw* draws) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ StreamPart part;
+  __shared__ StreamScratch s;
+  const int nclu = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int i = blockIdx.x / nclu, b = blockIdx.y, V = a.V;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool bonus = i >= a.n_draft, greedy = a.temperature == 0.f;
+  const float* trow = a.target_logits + ((size_t)b * a.n_target + i) * V;
+  const float* drow = (!bonus && !greedy && a.draft_logits) ? a.draft_logits + ((size_t)b * a.n_draft + i) * V : nullptr;
+  const int share = ((V + nclu - 1) / nclu + kSeg - 1) / kSeg * kSeg;
+  const int v_lo = min(V, rank * share), n_vec = (min(V, v_lo + share) - v_lo) / 4;   // V % 4 == 0
+  const double inv_t = greedy ? 1.0 : 1.0 / (double)a.temperature;
+  const float i_hi = (float)inv_t, i_lo = (float)(inv_t - (double)i_hi);
+  pdl_launch_dependents();
+
+  // ---- one pass over both rows
+  constexpr int U = 2;
+  const float4 none = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+  const float4 *t4 = reinterpret_cast<const float4*>(trow + v_lo), *d4 = reinterpret_cast<const float4*>(drow + (drow ? v_lo : 0));
+  float tm = -INFINITY, dm = -INFINITY;
+  int ti = 0x7fffffff;
+  double st = 0.0, sd = 0.0;
+  float tref = -INFINITY, dref = -INFINITY;
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    st = sd = 0.0;
+    const bool again = attempt > 0;
+    for (int v0 = tid; v0 - tid < n_vec; v0 += U * kStrThreads) {
+      float4 t[U], d[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int v = v0 + u * kStrThreads;
+        t[u] = v < n_vec ? __ldg(t4 + v) : none;
+        d[u] = (drow && v < n_vec) ? __ldg(d4 + v) : none;
+      }
+      if (!again) {
+        float bt = -INFINITY, bd = -INFINITY;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          bt = fmaxf(fmaxf(fmaxf(bt, t[u].x), fmaxf(t[u].y, t[u].z)), t[u].w);
+          bd = fmaxf(fmaxf(fmaxf(bd, d[u].x), fmaxf(d[u].y, d[u].z)), d[u].w);
+        }
+        if (bt > tm) {   // (rare after the first batch) the lowest id that holds the new maximum
+          tm = bt;
+#pragma unroll
+          for (int u = U - 1; u >= 0; --u) {
+            const int v = v_lo + 4 * (v0 + u * kStrThreads);
+            if (t[u].w == bt) ti = v + 3;
+            if (t[u].z == bt) ti = v + 2;
+            if (t[u].y == bt) ti = v + 1;
+            if (t[u].x == bt) ti = v;
+          }
+        }
+        dm = fmaxf(dm, bd);
+        if (!greedy && v0 == tid) {   // first batch: the block's reference
+          float rt = bt, rd = bd;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            rt = fmaxf(rt, __shfl_xor_sync(0xffffffffu, rt, o));
+            rd = fmaxf(rd, __shfl_xor_sync(0xffffffffu, rd, o));
+          }
+          if (lane == 0) { s.f[warp] = rt; s.f2[warp] = rd; }
+          __syncthreads();
+#pragma unroll
+          for (int w = 0; w < kStrWarps; ++w) { tref = fmaxf(tref, s.f[w]); dref = fmaxf(dref, s.f2[w]); }
+          if (tref == -INFINITY) tref = 0.f;   // (differences from a reference are NaN for NaN logits only)
+          if (dref == -INFINITY) dref = 0.f;
+        }
+      }
+      if (!greedy) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          st += (double)expf(exp_arg<UNIT>(t[u].x, tref, i_hi, i_lo)); st += (double)expf(exp_arg<UNIT>(t[u].y, tref, i_hi, i_lo));
+          st += (double)expf(exp_arg<UNIT>(t[u].z, tref, i_hi, i_lo)); st += (double)expf(exp_arg<UNIT>(t[u].w, tref, i_hi, i_lo));
+          if (drow) {
+            sd += (double)expf(exp_arg<UNIT>(d[u].x, dref, i_hi, i_lo)); sd += (double)expf(exp_arg<UNIT>(d[u].y, dref, i_hi, i_lo));
+            sd += (double)expf(exp_arg<UNIT>(d[u].z, dref, i_hi, i_lo)); sd += (double)expf(exp_arg<UNIT>(d[u].w, dref, i_hi, i_lo));
+          }
+        }
+      }
+    }
+    // ---- the block's values
+    if (!again) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, tm, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, ti, o);
+        if (ov > tm || (ov == tm && oi < ti)) { tm = ov; ti = oi; }
+        dm = fmaxf(dm, __shfl_xor_sync(0xffffffffu, dm, o));
+      }
+    }
+    st = warp_sum_d(st);
+    sd = warp_sum_d(sd);
+    __syncthreads();   // the references have been read
+    if (lane == 0) { s.f[warp] = tm; s.i[warp] = ti; s.f2[warp] = dm; s.d[warp] = st; s.d2[warp] = sd; }
+    __syncthreads();
+    st = sd = 0.0;
+#pragma unroll
+    for (int w = 0; w < kStrWarps; ++w) {
+      if (s.f[w] > tm || (s.f[w] == tm && s.i[w] < ti)) { tm = s.f[w]; ti = s.i[w]; }
+      dm = fmaxf(dm, s.f2[w]);
+      st += s.d[w];
+      sd += s.d2[w];
+    }
+    if (greedy) break;
+    const bool far_t = tm > -INFINITY && fabs((double)tm - (double)tref) * inv_t > kRefSlack;
+    const bool far_d = dm > -INFINITY && fabs((double)dm - (double)dref) * inv_t > kRefSlack;
+    if (!far_t && !far_d) break;
+    if (far_t) tref = tm;
+    if (far_d) dref = dm;
+    __syncthreads();
+  }
+  // (the maxima skip NaN, but a NaN logit leaves its row's sum NaN)
+  const int bad = tm == INFINITY || dm == INFINITY || st != st || sd != sd;
+  if (tid == 0) {
+    part.tmax = tm; part.targ = ti; part.dmax = dm; part.bad = bad; part.st = st; part.sd = sd;
+    part.tref = tref; part.dref = dref;
+  }
+  cl.sync();
+  // ---- first block: the row pair's verdict, its record, the ticket; as the last arriver of the
+  // sequence, the walk over the verdicts
+  if (rank == 0 && warp == 0) {
+    const StreamPart* pr = lane < nclu ? cl.map_shared_rank(&part, lane) : nullptr;
+    float m = pr ? pr->tmax : -INFINITY, q = pr ? pr->dmax : -INFINITY;
+    int mi = pr ? pr->targ : 0x7fffffff, bd = pr ? pr->bad : 0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, m, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
+      if (ov > m || (ov == m && oi < mi)) { m = ov; mi = oi; }
+      q = fmaxf(q, __shfl_xor_sync(0xffffffffu, q, o));
+      bd |= __shfl_xor_sync(0xffffffffu, bd, o);
+    }
+    m = __shfl_sync(0xffffffffu, m, 0); mi = __shfl_sync(0xffffffffu, mi, 0);
+    q = __shfl_sync(0xffffffffu, q, 0); bd = __shfl_sync(0xffffffffu, bd, 0);
+    if (m == -INFINITY || (drow && q == -INFINITY)) bd = 1;   // a row without a distribution
+    if (mi == 0x7fffffff) mi = 0;                             // (nothing above -inf: the lowest id)
+    double xt = 0.0, xd = 0.0;
+    if (!greedy && !bd && pr) {
+      if (pr->st > 0.0) xt = pr->st * exp(((double)pr->tref - (double)m) * inv_t);
+      if (drow && pr->sd > 0.0) xd = pr->sd * exp(((double)pr->dref - (double)q) * inv_t);
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      xt += __shfl_xor_sync(0xffffffffu, xt, o);
+      xd += __shfl_xor_sync(0xffffffffu, xd, o);
+    }
+    if (lane == 0) {
+      if (!drow) xd = 1.0;
+      const int x = bonus ? -1 : a.draft_tokens[(size_t)b * a.n_draft + i];
+      int accept = 0;
+      if (greedy) {
+        accept = (!bonus && x == mi) ? 1 : 0;
+        bd = 0;
+      } else if (!bd && !bonus) {
+        uint32_t c[4] = {(uint32_t)i, (uint32_t)b, a.off_lo, a.off_hi};
+        philox4x32_10(a.key0, a.key1, c);
+        const double r = (double)(c[0] >> 8) * (1.0 / 16777216.0);
+        const bool in_range = x >= 0 && x < V;
+        const double logp = in_range ? ((double)trow[x] - (double)m) * inv_t - log(xt) : -INFINITY;
+        const double logq = drow ? (in_range ? ((double)drow[x] - (double)q) * inv_t - log(xd) : -INFINITY) : 0.0;
+        const double diff = logp - logq;
+        const double ratio = (diff != diff) ? 0.0 : exp(fmin(diff, 0.0));
+        accept = r < ratio ? 1 : 0;
+      }
+      VerifyRow* recw = rows + (size_t)b * (PS_MAX_MASKS + 2);
+      VerifyRow rec;
+      rec.flags = accept | (bd << 1); rec.targ = mi; rec.tmax = m; rec.dmax = q; rec.st = xt; rec.sd = xd;
+      recw[i] = rec;
+      __threadfence();
+      if (atomicAdd(&a.tickets[b], 1u) == (unsigned)a.n_target - 1u) {
+        __threadfence();
+        a.tickets[b] = 0u;
+        int* out = a.out_tokens + (size_t)b * (a.n_draft + 1);
+        int acc = 0, any_bad = 0, stop = -1, flags = 0;
+        while (acc < a.n_draft) {
+          flags = __ldcg(&recw[acc].flags);
+          any_bad |= (flags >> 1) & 1;
+          if (!(flags & 1)) { stop = acc; break; }
+          out[acc] = a.draft_tokens[(size_t)b * a.n_draft + acc];
+          ++acc;
+        }
+        if (acc == a.n_draft && a.n_target == a.n_draft + 1) {
+          flags = __ldcg(&recw[acc].flags);
+          any_bad |= (flags >> 1) & 1;
+          stop = acc;
+        }
+        const int n = acc + (stop >= 0 ? 1 : 0);
+        for (int j = n; j <= a.n_draft; ++j) out[j] = -1;
+        a.accept_len[b] = acc;
+        a.n_out[b] = n;
+        if (any_bad) atomicOr(a.status, kStatNonfinite);
+        VerifyDraw dw;
+        dw.pos = -1;
+        if (stop >= 0) {
+          const VerifyRow* rr = recw + stop;
+          const int targ = __ldcg(&rr->targ);
+          out[acc] = targ;   // (a draw replaces it)
+          if (!greedy && !(flags & 2)) {
+            dw.pos = stop; dw.acc = acc;
+            dw.tmax = __ldcg(&rr->tmax); dw.dmax = __ldcg(&rr->dmax);
+            dw.st = __ldcg(&rr->st); dw.sd = __ldcg(&rr->sd);
+          }
+        }
+        draws[b] = dw;
+      }
+    }
+  }
+  cl.sync();   // no block leaves while another may still read its shared memory
+}
+
+// The token of each sequence whose chain stops at a position with a distribution: inverse-CDF draw
+// from max(0, p - q), or from p at the extra row and where the residual is empty.  A cluster of
+// kDrawClu blocks per sequence; a warp takes segments of kSeg tokens, four in flight.
+constexpr int kDrawClu = 8, kDrawBatch = 4;
+template <bool UNIT>
+__global__ void __cluster_dims__(kDrawClu, 1, 1) __launch_bounds__(kStrThreads)
+k_verify_draw(VerifyArgs a, const VerifyDraw* draws) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  extern __shared__ double seg_sum[];          // [segments of the block's share]
+  __shared__ double s_wsum;
+  __shared__ int s_done;
+  const int rank = (int)cl.block_rank(), b = blockIdx.y, V = a.V;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int share = ((V + kDrawClu - 1) / kDrawClu + kSeg - 1) / kSeg * kSeg;
+  const int v_lo = min(V, rank * share), n_vec = (min(V, v_lo + share) - v_lo) / 4;   // V % 4 == 0
+  const double inv_t = 1.0 / (double)a.temperature;
+  const float i_hi = (float)inv_t, i_lo = (float)(inv_t - (double)i_hi);
+  const float4 none = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+  pdl_launch_dependents();
+  pdl_wait();
+  const VerifyDraw dw = draws[b];
+  const int pos = dw.pos;
+  if (pos >= 0) {   // uniform over the cluster
+    const float tmax = dw.tmax, dmax = dw.dmax;
+    const float inv_st = (float)(1.0 / dw.st), inv_sd = (float)(1.0 / dw.sd);
+    const bool use_q0 = pos < a.n_draft;
+    const float* tr = a.target_logits + ((size_t)b * a.n_target + pos) * V;
+    const float* dr = (use_q0 && a.draft_logits) ? a.draft_logits + ((size_t)b * a.n_draft + pos) * V : nullptr;
+    const int x = use_q0 ? a.draft_tokens[(size_t)b * a.n_draft + pos] : -1;
+    uint32_t c[4] = {(uint32_t)pos, (uint32_t)b, a.off_lo, a.off_hi};
+    philox4x32_10(a.key0, a.key1, c);
+    const double u2 = (double)(c[1] >> 8) * (1.0 / 16777216.0);
+    const int n_seg = (4 * n_vec + kSeg - 1) / kSeg;
+    // this lane's four tokens of segment g, and their weights: max(0, p - q), or p
+    auto fetch = [&](int g, bool use_q, float4& tv, float4& dv) {
+      tv = dv = none;
+      if (g < 0 || g * (kSeg / 4) + lane >= n_vec) return;
+      const int v = v_lo + g * kSeg + 4 * lane;
+      tv = __ldg(reinterpret_cast<const float4*>(tr + v));
+      if (use_q && dr) dv = __ldg(reinterpret_cast<const float4*>(dr + v));
+    };
+    auto weights = [&](int g, bool use_q, const float4& tv, const float4& dv, float (&w)[4]) {
+      const int v = v_lo + g * kSeg + 4 * lane;
+      const float t[4] = {tv.x, tv.y, tv.z, tv.w}, d[4] = {dv.x, dv.y, dv.z, dv.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        w[e] = expf(exp_arg<UNIT>(t[e], tmax, i_hi, i_lo)) * inv_st;
+        if (use_q) {
+          const float qv = dr ? expf(exp_arg<UNIT>(d[e], dmax, i_hi, i_lo)) * inv_sd : (v + e == x ? 1.f : 0.f);
+          w[e] = fmaxf(w[e] - qv, 0.f);
+        }
+      }
+    };
+    bool done = false;
+    for (int attempt = use_q0 ? 0 : 1; attempt < 2 && !done; ++attempt) {
+      const bool use_q = attempt == 0;
+      for (int g0 = warp; g0 < n_seg; g0 += kDrawBatch * kStrWarps) {
+        float4 tv[kDrawBatch], dv[kDrawBatch];
+        double mine[kDrawBatch];
+#pragma unroll
+        for (int k = 0; k < kDrawBatch; ++k) fetch(g0 + k * kStrWarps, use_q, tv[k], dv[k]);   // (past the share: nothing)
+#pragma unroll
+        for (int k = 0; k < kDrawBatch; ++k) {
+          float w[4];
+          weights(g0 + k * kStrWarps, use_q, tv[k], dv[k], w);
+          mine[k] = ((double)w[0] + (double)w[1]) + ((double)w[2] + (double)w[3]);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int k = 0; k < kDrawBatch; ++k) mine[k] += __shfl_xor_sync(0xffffffffu, mine[k], o);
+#pragma unroll
+        for (int k = 0; k < kDrawBatch; ++k)
+          if (lane == 0 && g0 + k * kStrWarps < n_seg) seg_sum[g0 + k * kStrWarps] = mine[k];
+      }
+      __syncthreads();
+      // lane owns segments [lane * per, ...) of the block's share
+      double incl = 0.0, own = 0.0;
+      int g_lo = 0, g_hi = 0;
+      if (warp == 0) {
+        const int per = (n_seg + 31) / 32;
+        g_lo = min(n_seg, lane * per);
+        g_hi = min(n_seg, g_lo + per);
+        for (int g = g_lo; g < g_hi; ++g) own += seg_sum[g];
+        incl = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const double up = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += up;
+        }
+        if (lane == 31) s_wsum = incl;
+      }
+      cl.sync();
+      if (warp == 0) {
+        const double bw = lane < kDrawClu ? *cl.map_shared_rank(&s_wsum, lane) : 0.0;
+        double binc = bw;
+#pragma unroll
+        for (int o = 1; o < kDrawClu; o <<= 1) {
+          const double up = __shfl_up_sync(0xffffffffu, binc, o);
+          if (lane >= o) binc += up;
+        }
+        const double total = __shfl_sync(0xffffffffu, binc, kDrawClu - 1);
+        done = total > 0.0;
+        if (done) {
+          // At every level: the first holder of weight whose running sum exceeds the target; rounding
+          // may leave none, then the last holder of weight.
+          const double target = u2 * total;
+          const unsigned has_b = __ballot_sync(0xffffffffu, bw > 0.0);
+          const unsigned over_b = __ballot_sync(0xffffffffu, bw > 0.0 && binc > target);
+          const int sel = over_b ? __ffs(over_b) - 1 : 31 - __clz(has_b);
+          const double base = __shfl_sync(0xffffffffu, binc - bw, sel);
+          if (sel == rank) {
+            const unsigned has = __ballot_sync(0xffffffffu, own > 0.0);
+            const unsigned over = __ballot_sync(0xffffffffu, own > 0.0 && base + incl > target);
+            const int src = over ? __ffs(over) - 1 : 31 - __clz(has);
+            int gs = -1;
+            double gbase = 0.0;
+            if (lane == src) {
+              double run = base + incl - own;
+              for (int g = g_lo; g < g_hi; ++g) {
+                const double sg = seg_sum[g];
+                if (sg > 0.0) {
+                  gs = g;
+                  gbase = run;
+                  if (run + sg > target) break;
+                }
+                run += sg;
+              }
+            }
+            gs = __shfl_sync(0xffffffffu, gs, src);
+            gbase = __shfl_sync(0xffffffffu, gbase, src);
+            float4 tv, dv;
+            float w[4];
+            fetch(gs, use_q, tv, dv);
+            weights(gs, use_q, tv, dv, w);
+            const double mine = ((double)w[0] + (double)w[1]) + ((double)w[2] + (double)w[3]);
+            double linc = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const double up = __shfl_up_sync(0xffffffffu, linc, o);
+              if (lane >= o) linc += up;
+            }
+            const unsigned has2 = __ballot_sync(0xffffffffu, mine > 0.0);
+            const unsigned over2 = __ballot_sync(0xffffffffu, mine > 0.0 && gbase + linc > target);
+            const int src2 = over2 ? __ffs(over2) - 1 : 31 - __clz(has2);
+            if (lane == src2) {
+              double run = gbase + linc - mine;
+              int pick = -1;
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                if (w[e] > 0.f && (pick < 0 || !(run > target))) pick = e;
+                run += (double)w[e];
+              }
+              a.out_tokens[(size_t)b * (a.n_draft + 1) + dw.acc] = v_lo + gs * kSeg + 4 * lane + pick;
+            }
+          }
+        }
+        if (lane == 0) s_done = done;
+      }
+      __syncthreads();
+      done = s_done != 0;
+      cl.sync();   // the blocks' sums have been read
+    }
+  }
 }
 
 // ---- token-tree verification (Algorithm 1 in full) -------------------------------------------
@@ -1007,18 +1431,20 @@ ps_status launch_build_tree(ps_ctx* c, int B, int n_nodes, const int* parent, co
 }
 
 // Launch with a cluster of nclu blocks along x (a launch attribute, not a compile-time one).
-template <class Args>
-cudaError_t launch_cluster(void (*kern)(Args), dim3 grid, int nclu, cudaStream_t st, const Args& a) {
+template <class... KArgs, class... Args>
+cudaError_t launch_cluster(void (*kern)(KArgs...), dim3 grid, int nclu, int threads, size_t smem, cudaStream_t st,
+                           const Args&... a) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(kCluThreads);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = nclu; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, a);
+  return cudaLaunchKernelEx(&cfg, kern, a...);
 }
 
 // Whether the context's device can co-schedule nclu blocks of this kernel as one cluster (sizes
@@ -1059,7 +1485,30 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
   a.accept_len = accept_len; a.out_tokens = out_tokens; a.n_out = n_out;
   a.rec = c->vrec; a.tickets = c->tickets; a.status = c->dev_status;
   const bool aligned = (((uintptr_t)target_logits | (uintptr_t)draft_logits) & 15u) == 0;
-  const int nclu = a.V <= kCluMaxVocab ? kClu : 16;
+  const int nclu = a.V <= kCluMaxVocab ? kClu : 16, pairs = n_target * B;
+  // More row pairs than the register-resident clusters can take at once (each of their blocks fills
+  // an SM): the streaming kernel, with as many blocks per pair as are resident together.  Below that
+  // the register-resident ones win: one launch, and no second look at the rows.
+  const int reg_blocks = nclu == kClu && a.V <= kCluSmallMaxVocab ? kCluSmall : nclu;
+  if (a.V % 4 == 0 && aligned && pairs * reg_blocks > c->n_sm) {
+    int per = 1;
+    while (per < 8 && 2 * pairs * per <= kStrPerSm * c->n_sm) per *= 2;
+    const size_t bytes = (size_t)(((a.V + kDrawClu - 1) / kDrawClu + kSeg - 1) / kSeg) * sizeof(double);
+    if (bytes <= 40 * 1024) {
+      const bool unit = temperature == 1.f;
+      prof_mark(c, st, "begin");
+      cudaError_t e = launch_cluster(unit ? k_verify_stream<true> : k_verify_stream<false>, dim3(n_target * per, B), per,
+                                     kStrThreads, 0, st, a, c->vrow, c->vdraw);
+      c->launches++;
+      if (e == cudaSuccess && temperature > 0.f) {
+        e = launch_after(unit ? k_verify_draw<true> : k_verify_draw<false>, dim3(kDrawClu, B), dim3(kStrThreads), bytes, st,
+                         !c->prof, a, (const VerifyDraw*)c->vdraw);
+        c->launches++;
+      }
+      prof_mark(c, st, "verify");
+      return cuda_check(c, e, "k_verify_stream");
+    }
+  }
   if (a.V % 4 == 0 && a.V <= kCluMaxVocab16 && aligned && (nclu == kClu || cluster_size_ok(c->cluster_ok[0], k_verify_cluster16, 16))) {
     prof_mark(c, st, "begin");
     cudaError_t e;
@@ -1073,7 +1522,7 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
       e = launch_after(a.V <= kClu * kCluThreads * 4 * 2 ? k_verify_cluster_v2 : k_verify_cluster,
                        dim3(n_target * kClu, B), dim3(kCluThreads), 0, st, pdl, a);
     } else {
-      e = launch_cluster(k_verify_cluster16, dim3(n_target * 16, B), 16, st, a);
+      e = launch_cluster(k_verify_cluster16, dim3(n_target * 16, B), 16, kCluThreads, 0, st, a);
     }
     c->launches++;
     prof_mark(c, st, "verify");
@@ -1132,7 +1581,7 @@ ps_status launch_verify_tree(ps_ctx* c, int B, int n_nodes, const int* parent, c
     return fail(c, PS_ERR_UNSUPPORTED, "this device cannot run the 16-block clusters a vocabulary beyond 65536 needs");
   while (nclu > 1 && (long)(n_nodes + 1) * B * nclu > c->n_sm && a.V <= (nclu / 2) * kCluThreads * 4 * kCluV4)
     nclu /= 2;
-  cudaError_t e = launch_cluster(k_verify_tree, dim3((n_nodes + 1) * nclu, B), nclu, st, a);
+  cudaError_t e = launch_cluster(k_verify_tree, dim3((n_nodes + 1) * nclu, B), nclu, kCluThreads, 0, st, a);
   c->launches++;
   prof_mark(c, st, "verify_tree");
   return cuda_check(c, e, "k_verify_tree");
