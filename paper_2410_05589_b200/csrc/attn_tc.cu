@@ -1,0 +1,757 @@
+// Attention of a draft step on tcgen05, for batches whose keys and values are worth streaming at
+// full HBM rate (Sec. 4.1: the k+1 rows of a sequence see the cached real positions and the new
+// rows up to themselves).
+//
+// What bounds it: the K/V stream.  A persistent CTA per SM walks a contiguous range of (sequence,
+// kv head, 128-key tile) units; the K and V tiles come by tiled TMA into a ring of 32 KB slots
+// (five or six: 160-192 KB in flight per SM) that nothing but the tensor cores reads:
+//   S^T[key][row] = K[key][d] Q^T[d][row]     keys on the 128 lanes, the group's query rows (hi and
+//                                             lo planes side by side, N = 2 NR) on the columns
+//   O^T[d][row]  += V^T[d][key] P^T[key][row] channels on the lanes; V is read MN-major, as cached
+// Eight warps turn a tile's scores into probabilities, one key per thread: no reduction over the
+// keys is needed, because the exponentials are taken against a reference score per row (that of
+// the first key of the segment) instead of the running maximum; only when a score exceeds it by
+// 2^64 are the sums so far rescaled.  The probabilities are written to shared memory as bf16 hi + lo
+// planes.  Four more warps read a finished segment's O^T back while the next one runs.  All heads
+// that share a kv head are rows of one product, so its keys and values are read once.
+// Rows of a pair whose tiles are dealt to several CTAs: partial results, merged in CTA order by the
+// last of them to finish.
+// A small kernel ahead (k_attn_prep) rotates and splits the query rows and rounds the new k / v
+// rows as the cache would; the ring is filled with cached tiles while it runs.
+// Measured with it (event intervals) against mma.sync blocks that stage a tile, synchronise and
+// compute: 33B shape, 16 sequences of 1024-4096 keys, 9 rows: 343 -> 207 us (973 MB: 4.7 TB/s); 13B
+// shape, 64 x 256-2048 keys, 9 rows: 459 -> 360 us (1.5 GB: 4.2 TB/s); 16 sequences, 5 rows: 94 us
+// either way (whole call 437 -> 430 us: the small kernel ahead hides behind the ring's first fill).
+// What holds it now is the softmax warps' step (2200 cycles of a 2900-cycle tile at full HBM rate)
+// and the short steps of the new rows, one per pair.
+#include <cfloat>
+
+#include "attn_tc.cuh"
+#include "umma_gemm.cuh"
+
+namespace ps {
+namespace atc {
+namespace {
+
+using umma::fence_after_sync;
+using umma::fence_before_sync;
+using umma::mbar_arrive;
+using umma::mbar_arrive_expect_tx;
+using umma::mbar_init;
+using umma::mbar_wait;
+using umma::smem_desc;
+using umma::smem_u32;
+using umma::tma_load_2d;
+
+constexpr int kTile = 128;                 // keys of a unit
+constexpr int kSlotBytes = kTile * kD * 2; // a K or V tile
+constexpr int kBoxRows = 32;               // rows of a cache box: a ragged tile is fetched in steps of it
+constexpr int kSoftWarps = 8;              // two per lane quadrant, half of the rows each
+constexpr int kThreads = 96 + 32 * (kSoftWarps + 4);   // producer, two MMA issuers, softmax, 4 epilogue warps
+constexpr float kSlack = 64.f;             // a score this far above the reference (log2) forces a rescale
+
+__host__ __device__ constexpr int op_bytes(int NR) { return 2 * NR * kD * 2; }   // Q or P planes of one buffer
+__host__ __device__ constexpr int n_slots(int NR) { return NR <= 16 ? 6 : 5; }
+__host__ __device__ constexpr int tmem_cols(int NR) { return NR <= 8 ? 64 : (NR <= 16 ? 128 : 256); }
+
+template <int NR>
+struct Ctl {
+  uint64_t full[6], empty[6];              // ring slots
+  uint64_t q_full[2], q_empty[2];          // query planes, by segment
+  uint64_t s_full[2], s_empty[2];          // scores, by step
+  uint64_t p_full[2], p_empty[2];          // probabilities, by step
+  uint64_t o_full[2], o_empty[2];          // outputs, by segment
+  uint64_t l_full[2];                      // references and sums, by segment
+  uint32_t tmem_base;
+  int abort_flag, is_last;
+  float ref[2][NR];
+  float sum[2][4][NR];                     // per lane quadrant
+  float red[4][NR];
+};
+template <int NR>
+constexpr int smem_bytes() { return n_slots(NR) * kSlotBytes + 4 * op_bytes(NR) + (int)sizeof(Ctl<NR>) + 1024; }
+
+struct Work {
+  SeqMap sm;
+  int off[PS_MAX_BATCH + 1];   // units before sequence b (over all its kv heads)
+  int n_kv, group, R, max_ctx, n_heads;
+};
+__device__ __forceinline__ int units_of(int len) { return max(1, (len + kTile - 1) / kTile); }
+__device__ __forceinline__ int unit_begin(int c, int U, int G) { return (int)((unsigned)U * (unsigned)c / (unsigned)G); }
+__device__ __forceinline__ int unit_owner(int u, int U, int G) {
+  return (int)(((unsigned)(u + 1) * (unsigned)G - 1u) / (unsigned)U);
+}
+
+// Walks a CTA's steps: the cached tiles of a segment (one pair's share of the range), then, where
+// the segment holds the pair's last unit, the step of the new rows.
+struct Walk {
+  int u, u_end;                     // units left after the segment begin at u
+  int b, hk, len, nu, t, t_end;     // the segment: sequence, kv head, its cached tiles [t, t_end)
+  bool tail, in_tail, first, ok, whole;
+  int seg;
+  __device__ void enter() {         // the segment that begins at tile t of (b, hk)
+    ok = u < u_end;
+    if (!ok) return;
+    const int e = min(nu, t + u_end - u);
+    u += e - t;
+    tail = e == nu;
+    whole = tail && t == 0;
+    t_end = min(e, (len + kTile - 1) / kTile);
+    in_tail = t >= t_end;
+    first = true;
+  }
+  __device__ void sequence(const Work& w) {
+    len = w.sm.len[b];
+    nu = units_of(len);
+  }
+  __device__ void start(const Work& w, int u0, int u1) {
+    u = u0; u_end = u1; seg = 0;
+    int lo = 0, hi = w.sm.B - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (w.off[mid] <= u) lo = mid; else hi = mid - 1;
+    }
+    b = lo;
+    sequence(w);
+    const int r = u - w.off[b];
+    hk = r / nu;
+    t = r - hk * nu;
+    enter();
+  }
+  __device__ void next_segment(const Work& w) {
+    ++seg;
+    t = 0;
+    if (++hk == w.n_kv) {
+      hk = 0;
+      ++b;
+      if (b < w.sm.B) sequence(w);
+    }
+    enter();
+  }
+  __device__ bool last() const { return in_tail || (t + 1 == t_end && !tail); }
+  __device__ bool last_of_cta() const { return u >= u_end && last(); }
+  __device__ int keys(const Work& w) const { return in_tail ? w.R : min(kTile, len - t * kTile); }
+  __device__ void next(const Work& w) {
+    if (last()) { next_segment(w); return; }
+    first = false;
+    if (++t == t_end) in_tail = true;
+  }
+};
+
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ void split1(float x, __nv_bfloat16& h, __nv_bfloat16& l) {
+  h = __float2bfloat16_rn(x);
+  l = __float2bfloat16_rn(x - __bfloat162float(h));
+}
+__device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld4_async(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&r)[4]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]),
+               "r"(r[3])
+               : "memory");
+}
+// The sums hi + lo of the NR rows of an accumulator of 2 NR columns, for this thread's lane.
+template <int NR>
+__device__ __forceinline__ void tmem_rows(uint32_t taddr, float (&v)[NR]) {
+  uint32_t r[2 * NR / 16][16];
+#pragma unroll
+  for (int i = 0; i < 2 * NR / 16; ++i) tmem_ld16_async(taddr + 16 * i, r[i]);
+  umma::tmem_ld_wait();
+#pragma unroll
+  for (int i = 0; i < NR; ++i)
+    v[i] = __uint_as_float(r[i / 16][i % 16]) + __uint_as_float(r[(NR + i) / 16][(NR + i) % 16]);
+}
+// V^T as the MMA's M side: channels contiguous (MN-major), 128-byte swizzle; 64-channel blocks one
+// box (16 KB) apart, groups of 8 keys 1024 bytes apart.
+__device__ __forceinline__ uint64_t vt_desc(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)((kSlotBytes / 2) >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
+         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+// Barriers of 128 threads: the epilogue warps, and the four warps of either half of the rows.
+constexpr int kBarEpi = 1, kBarSoft = 2;
+__device__ __forceinline__ void bar_sync(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ bool bar_any(int id, bool pred) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 q, %1, 0;\n\t"
+      "bar.red.or.pred p, %2, 128, q;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)pred), "r"(id)
+      : "memory");
+  return r != 0;
+}
+
+// Query rows of a pair (rotated, scaled by log2(e) / sqrt(128), hi and lo planes, zero rows up to
+// NR) and its new k (rotated) and v rows rounded to the cache's type.  Block: kPrepHeads kv heads of
+// a sequence.  Bound by the read of q|k|v from L2; the rotation table is formed once per block.
+constexpr int kPrepHeads = 4;
+__global__ void __launch_bounds__(256) k_attn_prep(const __grid_constant__ Work w, const float* __restrict__ qkv, int ldq,
+                                                   int Hq, int Hkv, const double* __restrict__ inv_freq, int NR,
+                                                   __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ kv) {
+  __shared__ float cs[kMaxRowsPerSeq][kD / 2], sn[kMaxRowsPerSeq][kD / 2];
+  const int b = blockIdx.y, h0 = blockIdx.x * kPrepHeads, nh = min(kPrepHeads, w.n_kv - h0), R = w.R, G = w.group;
+  const int m0 = b * R, tid = threadIdx.x;
+  pdl_launch_dependents();
+  for (int i = tid; i < R * (kD / 2); i += blockDim.x) {
+    double ang = (double)(w.sm.len[b] + i / (kD / 2)) * inv_freq[i % (kD / 2)];
+    ang -= 6.283185307179586476925 * rint(ang * 0.15915494309189533577);
+    sincosf((float)ang, &sn[i / (kD / 2)][i % (kD / 2)], &cs[i / (kD / 2)][i % (kD / 2)]);
+  }
+  __syncthreads();
+  pdl_wait();
+  const float scale = rsqrtf((float)kD) * 1.4426950408889634f;
+  struct alignas(8) B4 { __nv_bfloat16 v[4]; };
+  // 16 threads per row: four channels i..i+3 of the lower half and their partners 64 above
+  const int n_q = nh * NR * 16;
+  for (int it = tid; it < n_q; it += blockDim.x) {
+    const int i = (it & 15) * 4, r = (it >> 4) % NR, hk = h0 + (it >> 4) / NR;
+    B4 h0v{}, l0v{}, h1v{}, l1v{};
+    if (r < G * R) {
+      const int g = r / R, j = r - g * R;
+      const float* src = qkv + (size_t)(m0 + j) * ldq + (hk * G + g) * kD + i;
+      const float4 x = __ldcg(reinterpret_cast<const float4*>(src)), y = __ldcg(reinterpret_cast<const float4*>(src + kD / 2));
+      const float xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float c = cs[j][i + e], s = sn[j][i + e];
+        split1((xa[e] * c - ya[e] * s) * scale, h0v.v[e], l0v.v[e]);
+        split1((ya[e] * c + xa[e] * s) * scale, h1v.v[e], l1v.v[e]);
+      }
+    }
+    __nv_bfloat16* d = q + ((size_t)(b * w.n_kv + hk) * 2 * NR + r) * kD + i;
+    *reinterpret_cast<B4*>(d) = h0v;
+    *reinterpret_cast<B4*>(d + kD / 2) = h1v;
+    *reinterpret_cast<B4*>(d + (size_t)NR * kD) = l0v;
+    *reinterpret_cast<B4*>(d + (size_t)NR * kD + kD / 2) = l1v;
+  }
+  const int n_kv_items = nh * kNewRows * 16;
+  for (int it = tid; it < n_kv_items; it += blockDim.x) {
+    const int i = (it & 15) * 4, j = (it >> 4) % kNewRows, hk = h0 + (it >> 4) / kNewRows;
+    B4 k0{}, k1{}, v0{}, v1{};
+    if (j < R) {
+      const float* src = qkv + (size_t)(m0 + j) * ldq + Hq + hk * kD + i;
+      const float4 x = __ldcg(reinterpret_cast<const float4*>(src)), y = __ldcg(reinterpret_cast<const float4*>(src + kD / 2));
+      const float4 a = __ldcg(reinterpret_cast<const float4*>(src + Hkv)),
+                   c4 = __ldcg(reinterpret_cast<const float4*>(src + Hkv + kD / 2));
+      const float xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w}, va[4] = {a.x, a.y, a.z, a.w},
+                  vb[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float c = cs[j][i + e], s = sn[j][i + e];
+        k0.v[e] = __float2bfloat16_rn(xa[e] * c - ya[e] * s);
+        k1.v[e] = __float2bfloat16_rn(ya[e] * c + xa[e] * s);
+        v0.v[e] = __float2bfloat16_rn(va[e]);
+        v1.v[e] = __float2bfloat16_rn(vb[e]);
+      }
+    }
+    __nv_bfloat16* d = kv + ((size_t)(b * w.n_kv + hk) * 2 * kNewRows + j) * kD + i;
+    *reinterpret_cast<B4*>(d) = k0;
+    *reinterpret_cast<B4*>(d + kD / 2) = k1;
+    *reinterpret_cast<B4*>(d + (size_t)kNewRows * kD) = v0;
+    *reinterpret_cast<B4*>(d + (size_t)kNewRows * kD + kD / 2) = v1;
+  }
+}
+
+template <int NR>
+__global__ void __launch_bounds__(kThreads, 1)
+k_attn_tc(const __grid_constant__ CUtensorMap t_k, const __grid_constant__ CUtensorMap t_v,
+          const __grid_constant__ CUtensorMap t_q, const __grid_constant__ CUtensorMap t_new, const __grid_constant__ Work w,
+          float* __restrict__ part_o, float2* __restrict__ part_ml, unsigned* tickets, __nv_bfloat16* __restrict__ out_hi,
+          __nv_bfloat16* __restrict__ out_lo, int* status) {
+  constexpr int N = 2 * NR, NS = n_slots(NR), kOp = op_bytes(NR);
+  extern __shared__ unsigned char smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  unsigned char* ring_g = smem_raw + (base - raw);
+  const uint32_t s_q = base + NS * kSlotBytes, s_p = s_q + 2 * kOp;
+  Ctl<NR>& ctl = *reinterpret_cast<Ctl<NR>*>(ring_g + NS * kSlotBytes + 4 * kOp);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int G = gridDim.x, U = w.off[w.sm.B];
+  const int u0 = unit_begin(blockIdx.x, U, G), u1 = unit_begin(blockIdx.x + 1, U, G);
+  volatile int* abort_flag = &ctl.abort_flag;
+
+  if (tid == 0) {
+    for (int i = 0; i < NS; ++i) { mbar_init(&ctl.full[i], 1); mbar_init(&ctl.empty[i], 1); }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&ctl.q_full[i], 1); mbar_init(&ctl.q_empty[i], 1);
+      mbar_init(&ctl.s_full[i], 1); mbar_init(&ctl.s_empty[i], kSoftWarps);
+      mbar_init(&ctl.p_full[i], kSoftWarps); mbar_init(&ctl.p_empty[i], 1);
+      mbar_init(&ctl.o_full[i], 1); mbar_init(&ctl.o_empty[i], 4);
+      mbar_init(&ctl.l_full[i], kSoftWarps);
+    }
+    ctl.abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    pdl_launch_dependents();
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl.tmem_base)),
+                 "r"(tmem_cols(NR))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  const uint32_t tmem = *(volatile uint32_t*)&ctl.tmem_base, tmem_o = tmem + 2 * N;
+
+  // Ring order of the loads, which is the order the MMAs use them in: K of step 0, then K of step
+  // i + 1 and V of step i for every i.
+  if (warp == 0) {
+    if (lane == 0) {   // ---- TMA producer
+      Walk wk, wv;
+      wk.start(w, u0, u1);
+      wv.start(w, u0, u1);
+      int slot = 0, n_issued = 0;
+      uint32_t use = 0;
+      bool dep = false, alive = true;          // dep: the kernel before this one (the query and new rows) is complete
+      auto load_q = [&](int b, int hk, int seg) {
+        uint64_t* bar = &ctl.q_full[seg & 1];
+        const uint32_t dst = s_q + (seg & 1) * kOp;
+        mbar_arrive_expect_tx(bar, kOp);
+        const int y = (b * w.n_kv + hk) * N;
+        tma_load_2d(dst, &t_q, 0, y, bar);
+        tma_load_2d(dst + kOp / 2, &t_q, 64, y, bar);
+      };
+      auto need_dep = [&]() {
+        if (dep) return;
+        pdl_wait();
+        dep = true;
+        Walk first;
+        first.start(w, u0, u1);
+        load_q(first.b, first.hk, 0);
+      };
+      auto load = [&](const Walk& x, const CUtensorMap* cache, int v) {
+        if (n_issued >= NS || x.in_tail) need_dep();
+        if (n_issued >= NS && !mbar_wait(&ctl.empty[slot], (use & 1) ^ 1, abort_flag)) { alive = false; return; }
+        const uint32_t dst = base + slot * kSlotBytes;
+        uint64_t* bar = &ctl.full[slot];
+        if (x.in_tail) {
+          mbar_arrive_expect_tx(bar, kNewRows * kD * 2);
+          const int y = ((x.b * w.n_kv + x.hk) * 2 + v) * kNewRows;
+          tma_load_2d(dst, &t_new, 0, y, bar);
+          tma_load_2d(dst + kSlotBytes / 2, &t_new, 64, y, bar);
+        } else {
+          const int nb = (min(kTile, x.len - x.t * kTile) + kBoxRows - 1) / kBoxRows;
+          mbar_arrive_expect_tx(bar, nb * kBoxRows * kD * 2);
+          const int y = (w.sm.slot[x.b] * w.n_kv + x.hk) * w.max_ctx + x.t * kTile;
+          for (int i = 0; i < nb; ++i) {
+            tma_load_2d(dst + i * kBoxRows * 128, cache, 0, y + i * kBoxRows, bar);
+            tma_load_2d(dst + kSlotBytes / 2 + i * kBoxRows * 128, cache, 64, y + i * kBoxRows, bar);
+          }
+        }
+        ++n_issued;
+        if (++slot == NS) { slot = 0; ++use; }
+      };
+      auto load_k = [&]() {
+        if (wk.first && wk.seg > 0) {
+          need_dep();
+          if (!mbar_wait(&ctl.q_empty[wk.seg & 1], ((wk.seg >> 1) & 1) ^ 1, abort_flag)) { alive = false; return; }
+          load_q(wk.b, wk.hk, wk.seg);
+        }
+        load(wk, &t_k, 0);
+        wk.next(w);
+      };
+      if (wk.ok) load_k();
+      while (alive && wv.ok) {
+        if (wk.ok) load_k();
+        if (alive) { load(wv, &t_v, 1); wv.next(w); }
+      }
+      if (alive && u0 < u1) need_dep();
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {   // ---- MMA issuer, scores (a thread issues about one MMA per 50-60 cycles: two of them keep up)
+      Walk x;
+      const uint32_t id = umma::idesc(N);
+      // (descriptors hold addresses in units of 16 bytes: offsets are added to them)
+      const uint64_t dk0 = smem_desc(base), dq0 = smem_desc(s_q);
+      x.start(w, u0, u1);
+      int slot = 0;            // of this step's K: ring position 0, then 2 i - 1
+      uint32_t use = 0;
+      for (int i = 0; x.ok; ++i) {
+        const int buf = i & 1, qb = x.seg & 1;
+        if ((x.first && !mbar_wait(&ctl.q_full[qb], (x.seg >> 1) & 1, abort_flag)) ||
+            !mbar_wait(&ctl.s_empty[buf], ((i >> 1) & 1) ^ 1, abort_flag) ||
+            !mbar_wait(&ctl.full[slot], use & 1, abort_flag)) break;
+        fence_after_sync();
+        const uint64_t da = dk0 + (uint64_t)(slot * (kSlotBytes / 16)), db = dq0 + (uint64_t)(qb * (kOp / 16));
+#pragma unroll
+        for (int ks = 0; ks < kD / 16; ++ks)
+          umma::mma_f16(tmem + buf * N, da + (ks >> 2) * (kSlotBytes / 32) + (ks & 3) * 2,
+                        db + (ks >> 2) * (kOp / 32) + (ks & 3) * 2, id, ks > 0);
+        umma::mma_commit(&ctl.s_full[buf]);
+        umma::mma_commit(&ctl.empty[slot]);
+        if (x.last()) umma::mma_commit(&ctl.q_empty[qb]);
+        slot += i == 0 ? 1 : 2;
+        if (slot >= NS) { slot -= NS; ++use; }
+        x.next(w);
+      }
+    }
+  } else if (warp == 2) {
+    if (lane == 0) {   // ---- MMA issuer, outputs
+      Walk x;
+      const uint32_t id = umma::idesc(N) | (1u << 15);
+      const uint64_t dv0 = vt_desc(base), dp0 = smem_desc(s_p);
+      x.start(w, u0, u1);
+      int slot = x.ok && x.last_of_cta() ? 1 : 2;   // of this step's V: ring position 2 i + 2, of the very last one 2 i + 1
+      uint32_t use = 0;
+      for (int i = 0; x.ok; ++i) {
+        const int buf = i & 1, ob = x.seg & 1;
+        if ((x.first && !mbar_wait(&ctl.o_empty[ob], ((x.seg >> 1) & 1) ^ 1, abort_flag)) ||
+            !mbar_wait(&ctl.full[slot], use & 1, abort_flag) ||
+            !mbar_wait(&ctl.p_full[buf], (i >> 1) & 1, abort_flag)) break;
+        fence_after_sync();
+        const uint64_t da = dv0 + (uint64_t)(slot * (kSlotBytes / 16)), db = dp0 + (uint64_t)(buf * (kOp / 16));
+        const int n_ks = (x.keys(w) + 15) >> 4;
+        const uint32_t d = tmem_o + ob * N, acc = x.first ? 0u : 1u;
+        if (n_ks == kTile / 16) {
+#pragma unroll
+          for (int ks = 0; ks < kTile / 16; ++ks)
+            umma::mma_f16(d, da + ks * (2048 / 16), db + (ks >> 2) * (kOp / 32) + (ks & 3) * 2, id, ks > 0 ? 1u : acc);
+        } else {
+#pragma unroll 1
+          for (int ks = 0; ks < n_ks; ++ks)
+            umma::mma_f16(d, da + ks * (2048 / 16), db + (ks >> 2) * (kOp / 32) + (ks & 3) * 2, id, ks > 0 ? 1u : acc);
+        }
+        umma::mma_commit(&ctl.p_empty[buf]);
+        umma::mma_commit(&ctl.empty[slot]);
+        if (x.last()) umma::mma_commit(&ctl.o_full[ob]);
+        x.next(w);
+        slot += x.ok && x.last_of_cta() ? 1 : 2;
+        if (slot >= NS) { slot -= NS; ++use; }
+      }
+    }
+  } else if (warp < 3 + kSoftWarps) {
+    // ---- softmax: thread = key of the tile, half of the rows
+    constexpr int NH = NR / 2, kSoft = 32 * kSoftWarps;
+    const int q = warp & 3, key = 32 * q + lane, half = (warp - 3) >> 2, r0 = half * NH, bar = kBarSoft + half;
+    const uint32_t lane_off = (uint32_t)(32 * q) << 16;
+    const int rows = w.group * w.R;
+    unsigned char* const p_base = ring_g + NS * kSlotBytes + 2 * kOp + (key >> 6) * (kOp / 2) + r0 * 128 + (key & 7) * 2;
+    const int chunk = (key & 63) >> 3;
+    Walk x;
+    x.start(w, u0, u1);
+    float ref[NH], l[NH];
+    for (int i = 0; x.ok; ++i) {
+      const int buf = i & 1, sb = x.seg & 1, n = x.keys(w);
+      const bool last = x.last();
+      bool ok = mbar_wait(&ctl.s_full[buf], (i >> 1) & 1, abort_flag);
+      if (x.first) ok = mbar_wait(&ctl.o_empty[sb], ((x.seg >> 1) & 1) ^ 1, abort_flag) && ok;
+      ok = __all_sync(0xffffffffu, ok);
+      fence_after_sync();
+      float s[NH];
+      if (ok) {
+        uint32_t h[NH / 4][4], lo[NH / 4][4];
+        const uint32_t at = tmem + lane_off + buf * N + r0;
+#pragma unroll
+        for (int c = 0; c < NH / 4; ++c) { tmem_ld4_async(at + 4 * c, h[c]); tmem_ld4_async(at + NR + 4 * c, lo[c]); }
+        umma::tmem_ld_wait();
+#pragma unroll
+        for (int r = 0; r < NH; ++r) s[r] = __uint_as_float(h[r / 4][r % 4]) + __uint_as_float(lo[r / 4][r % 4]);
+      }
+      fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&ctl.s_empty[buf]);   // read back: the next scores may be formed
+      if (x.first) {   // the references: the scores of the segment's first key
+        if (key == 0 && ok) {
+#pragma unroll
+          for (int r = 0; r < NH; ++r) ctl.ref[sb][r0 + r] = s[r];
+        }
+        bar_sync(bar);
+#pragma unroll
+        for (int r = 0; r < NH; ++r) { ref[r] = ctl.ref[sb][r0 + r]; l[r] = 0.f; }
+      }
+      if (n < kTile || x.in_tail) {   // keys past the end, new keys that a row does not see yet
+#pragma unroll
+        for (int r = 0; r < NH; ++r) {
+          const int rr = r0 + r;
+          if (key >= n || rr >= rows || (x.in_tail && key > rr % w.R)) s[r] = -INFINITY;
+        }
+      }
+      float top = -INFINITY;
+#pragma unroll
+      for (int r = 0; r < NH; ++r) top = fmaxf(top, s[r] - ref[r]);
+      if (bar_any(bar, !ok || top > kSlack)) {
+        if (bar_any(bar, *abort_flag != 0)) break;   // (one answer for all threads)
+        // Rare: some score lies far above its reference.  New references; the sums and the outputs
+        // so far are rescaled once the MMAs that form them have completed.
+        for (int r = 0; r < NH; ++r) {
+          float m = -INFINITY;
+#pragma unroll
+          for (int e = 0; e < NH; ++e) m = e == r ? s[e] : m;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+          if (lane == 0) ctl.red[q][r0 + r] = m;
+        }
+        bar_sync(bar);
+        float f[NH];
+#pragma unroll
+        for (int r = 0; r < NH; ++r) {
+          const int rr = r0 + r;
+          const float m = fmaxf(fmaxf(fmaxf(ctl.red[0][rr], ctl.red[1][rr]), fmaxf(ctl.red[2][rr], ctl.red[3][rr])), ref[r]);
+          f[r] = ex2(ref[r] - m);
+          l[r] *= f[r];
+          ref[r] = m;
+          if (key == 0) ctl.ref[sb][rr] = m;
+        }
+        bool rok = true;
+        if (!x.first) rok = mbar_wait(&ctl.p_empty[(i - 1) & 1], ((i - 1) >> 1) & 1, abort_flag);
+        if (bar_any(bar, !rok)) break;
+        if (!x.first) {
+          fence_after_sync();
+#pragma unroll
+          for (int c = 0; c < 2 * NH / 4; ++c) {   // this warp's columns: hi, then lo
+            uint32_t v[4];
+            const uint32_t at = tmem_o + lane_off + sb * N + (c < NH / 4 ? 0 : NR) + r0 + 4 * (c % (NH / 4));
+            tmem_ld4_async(at, v);
+            umma::tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * f[4 * (c % (NH / 4)) + e]);
+            tmem_st4(at, v);
+          }
+          asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+          fence_before_sync();
+        }
+      }
+      // ---- probabilities as hi/lo planes: row r of plane p at row p NR + r, keys along the row
+      float p[NH];
+#pragma unroll
+      for (int r = 0; r < NH; ++r) {
+        p[r] = ex2(s[r] - ref[r]);   // (0 for what is masked)
+        l[r] += p[r];
+      }
+      if (i >= 2) mbar_wait(&ctl.p_empty[buf], ((i >> 1) & 1) ^ 1, abort_flag);
+      const int n16 = (n + 15) & ~15;
+      if (key < n16) {
+        unsigned char* const pp = p_base + buf * kOp;
+#pragma unroll
+        for (int r = 0; r < NH; ++r) {
+          __nv_bfloat16 h, lo;
+          split1(p[r], h, lo);
+          const int at = r * 128 + ((chunk ^ ((r0 + r) & 7)) << 4);   // (NR is a multiple of 8: the same for both planes)
+          *reinterpret_cast<__nv_bfloat16*>(pp + at) = h;
+          *reinterpret_cast<__nv_bfloat16*>(pp + NR * 128 + at) = lo;
+        }
+      }
+      if (n16 > n && !x.in_tail) {
+        // rows of V between the tile's end and the next multiple of 16 meet probabilities of zero: they
+        // must be finite
+        const int pos = x.last_of_cta() ? 2 * i + 1 : 2 * i + 2, vs = pos % NS;   // ring position of this V
+        mbar_wait(&ctl.full[vs], (pos / NS) & 1, abort_flag);
+        for (int e = tid - 96; e < (n16 - n) * 16; e += kSoft) {
+          const int row = n + (e >> 4), c16 = e & 15;
+          *reinterpret_cast<uint4*>(ring_g + vs * kSlotBytes + (c16 >> 3) * (kSlotBytes / 2) + row * 128 + (c16 & 7) * 16) =
+              make_uint4(0u, 0u, 0u, 0u);
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&ctl.p_full[buf]);
+      if (last) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int r = 0; r < NH; ++r) l[r] += __shfl_xor_sync(0xffffffffu, l[r], o);
+        if (lane == 0) {
+#pragma unroll
+          for (int r = 0; r < NH; ++r) ctl.sum[sb][q][r0 + r] = l[r];
+          mbar_arrive(&ctl.l_full[sb]);
+        }
+      }
+      x.next(w);
+    }
+    fence_before_sync();
+  } else {
+    // ---- epilogue: thread = output channel
+    const int q = warp & 3, d = 32 * q + lane;
+    const uint32_t lane_off = (uint32_t)(32 * q) << 16;
+    const int rows = w.group * w.R;
+    Walk x;
+    for (x.start(w, u0, u1); x.ok;) {
+      const int sb = x.seg & 1;
+      const bool ok = mbar_wait(&ctl.o_full[sb], (x.seg >> 1) & 1, abort_flag) &&
+                      mbar_wait(&ctl.l_full[sb], (x.seg >> 1) & 1, abort_flag);
+      if (bar_any(kBarEpi, !ok)) break;
+      fence_after_sync();
+      float o[NR], l[NR];
+      tmem_rows<NR>(tmem_o + lane_off + sb * N, o);
+#pragma unroll
+      for (int r = 0; r < NR; ++r)
+        l[r] = (ctl.sum[sb][0][r] + ctl.sum[sb][1][r]) + (ctl.sum[sb][2][r] + ctl.sum[sb][3][r]);
+      const float my_ref = d < NR ? ctl.ref[sb][d] : 0.f;
+      float my_sum = 0.f;
+      if (d < NR) my_sum = (ctl.sum[sb][0][d] + ctl.sum[sb][1][d]) + (ctl.sum[sb][2][d] + ctl.sum[sb][3][d]);
+      fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&ctl.o_empty[sb]);
+      bool write = x.whole;
+      if (!x.whole) {
+        const int a = w.off[x.b] + x.hk * x.nu;                     // the pair's first unit
+        const int mine = blockIdx.x * 2 + (u0 >= a ? 0 : 1);        // its first segment, or its last
+        float* po = part_o + (size_t)mine * NR * kD + d;
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+          if (r < rows) po[r * kD] = o[r];
+        if (d < NR) part_ml[mine * NR + d] = make_float2(my_ref, my_sum);
+        bar_sync(kBarEpi);
+        const int c0 = unit_owner(a, U, G), c1 = unit_owner(a + x.nu - 1, U, G);
+        if (d == 0) {
+          __threadfence();
+          unsigned* tk = tickets + x.b * w.n_heads + x.hk;
+          const int is_last = atomicAdd(tk, 1u) == (unsigned)(c1 - c0);
+          if (is_last) { *tk = 0u; __threadfence(); }
+          ctl.is_last = is_last;
+        }
+        bar_sync(kBarEpi);
+        write = ctl.is_last != 0;
+        if (write) {   // all contributors in CTA order
+          float m[NR];
+#pragma unroll
+          for (int r = 0; r < NR; ++r) { m[r] = -FLT_MAX; l[r] = o[r] = 0.f; }
+          for (int c = c0; c <= c1; ++c) {
+            const int sl = c * 2 + (unit_begin(c, U, G) >= a ? 0 : 1);
+            float ov[NR];
+            float2 ml[NR];
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+              ov[r] = r < rows ? __ldcg(part_o + ((size_t)sl * NR + r) * kD + d) : 0.f;
+              ml[r] = r < rows ? __ldcg(part_ml + sl * NR + r) : make_float2(0.f, 0.f);
+            }
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+              const float mm = fmaxf(m[r], ml[r].x), f0 = ex2(m[r] - mm), f1 = ex2(ml[r].x - mm);
+              l[r] = l[r] * f0 + ml[r].y * f1;
+              o[r] = o[r] * f0 + ov[r] * f1;
+              m[r] = mm;
+            }
+          }
+        }
+        bar_sync(kBarEpi);   // everyone has read the flag
+      }
+      if (write) {
+        const int m0 = x.b * w.R;
+        int j = 0, g = 0;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          if (r < rows) {
+            const size_t at = (size_t)(m0 + j) * w.n_heads * kD + (size_t)(x.hk * w.group + g) * kD + d;
+            split1(o[r] / l[r], out_hi[at], out_lo[at]);
+          }
+          if (++j == w.R) { j = 0; ++g; }
+        }
+      }
+      x.next_segment(w);
+    }
+    fence_before_sync();
+  }
+
+  __syncthreads();
+  if (ctl.abort_flag) {
+    // let copies and MMAs that are still in flight finish before shared and tensor memory go
+    for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+    if (tid == 0) atomicOr(status, kStatTimeout);
+    __syncthreads();
+  }
+  if (warp == 1) {
+    fence_after_sync();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols(NR)) : "memory");
+  }
+}
+
+size_t take(size_t& off, size_t n) {
+  const size_t at = off;
+  off += (n + 255) & ~(size_t)255;
+  return at;
+}
+
+Buffers layout(const ps_config& g, char* base, size_t* total) {
+  Buffers b{};
+  const size_t nr = padded_rows(g), pairs = (size_t)g.max_batch * g.n_kv_heads;
+  size_t off = 0;
+  if (nr) {
+    const size_t q = take(off, pairs * 2 * nr * kD * 2), kv = take(off, pairs * 2 * kNewRows * kD * 2);
+    const size_t o = take(off, (size_t)kMaxSm * 2 * nr * kD * 4), ml = take(off, (size_t)kMaxSm * 2 * nr * sizeof(float2));
+    if (base) {
+      b.q = (__nv_bfloat16*)(base + q); b.kv_new = (__nv_bfloat16*)(base + kv);
+      b.part_o = (float*)(base + o); b.part_ml = (float2*)(base + ml);
+    }
+  }
+  *total = off;
+  return b;
+}
+
+template <int NR>
+cudaError_t launch_nr(ps_ctx* c, const Work& w, int grid, const Buffers& b, const Maps& m, unsigned* tickets,
+                      __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t st) {
+  auto kern = k_attn_tc<NR>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<NR>());
+  if (e != cudaSuccess) return e;
+  return launch_after(kern, dim3(grid), dim3(kThreads), smem_bytes<NR>(), st, !c->prof, m.kcache, m.vcache, m.q, m.kv_new, w,
+                      b.part_o, b.part_ml, tickets, hi, lo, c->dev_status);
+}
+
+}  // namespace
+
+size_t bytes(const ps_config& g) {
+  size_t n;
+  layout(g, nullptr, &n);
+  return n;
+}
+Buffers carve(const ps_config& g, char* base) {
+  size_t n;
+  return layout(g, base, &n);
+}
+
+bool build_maps(const ps_ctx* c, const Buffers& b, Maps* m) {
+  const ps_config& g = c->cfg;
+  const size_t nr = padded_rows(g), pairs = (size_t)g.max_batch * g.n_kv_heads, rows = pairs * g.max_ctx;
+  return nr && make_map(&m->kcache, c->kcache, rows, kD, kBoxRows) && make_map(&m->vcache, c->vcache, rows, kD, kBoxRows) &&
+         make_map(&m->q, b.q, pairs * 2 * nr, kD, (int)(2 * nr)) &&
+         make_map(&m->kv_new, b.kv_new, pairs * 2 * kNewRows, kD, kNewRows);
+}
+
+ps_status launch(ps_ctx* c, const SeqMap& sm, int B, const float* qkv, const Buffers& b, const Maps& m, unsigned* tickets,
+                 __nv_bfloat16* out_hi, __nv_bfloat16* out_lo, cudaStream_t st) {
+  const ps_config& g = c->cfg;
+  const int nr = padded_rows(g), Hq = g.n_heads * kD, Hkv = g.n_kv_heads * kD;
+  Work w;
+  std::memset(&w, 0, sizeof(w));
+  w.sm = sm;
+  w.n_kv = g.n_kv_heads; w.group = g.n_heads / g.n_kv_heads; w.R = g.k_masks + 1; w.max_ctx = g.max_ctx; w.n_heads = g.n_heads;
+  long long units = 0;
+  for (int i = 0; i < B; ++i) {
+    w.off[i] = (int)units;
+    units += (long long)std::max(1, (sm.len[i] + kTile - 1) / kTile) * g.n_kv_heads;
+  }
+  w.off[B] = (int)units;
+  if (units * (c->n_sm + 1) >= (1ll << 31)) return fail(c, PS_ERR_UNSUPPORTED, "too many key tiles in one call");
+  cudaError_t e = launch_after(k_attn_prep, dim3((g.n_kv_heads + kPrepHeads - 1) / kPrepHeads, B), dim3(256), 0, st, !c->prof, w,
+                               qkv, Hq + 2 * Hkv, Hq, Hkv, (const double*)c->rope_inv_freq, nr, b.q, b.kv_new);
+  c->launches++;
+  if (e != cudaSuccess) return cuda_check(c, e, "k_attn_prep");
+  const int grid = (int)std::min<long long>(c->n_sm, units);
+  e = nr == 8    ? launch_nr<8>(c, w, grid, b, m, tickets, out_hi, out_lo, st)
+      : nr == 16 ? launch_nr<16>(c, w, grid, b, m, tickets, out_hi, out_lo, st)
+      : nr == 24 ? launch_nr<24>(c, w, grid, b, m, tickets, out_hi, out_lo, st)
+                 : launch_nr<32>(c, w, grid, b, m, tickets, out_hi, out_lo, st);
+  c->launches++;
+  return cuda_check(c, e, "k_attn_tc");
+}
+
+}  // namespace atc
+}  // namespace ps

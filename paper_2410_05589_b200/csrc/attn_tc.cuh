@@ -1,0 +1,35 @@
+// Interface of the tensor-memory attention (attn_tc.cu).
+#pragma once
+#include "ps_internal.cuh"
+
+namespace ps {
+namespace atc {
+
+constexpr int kD = 128;          // head dimension
+constexpr int kNewRows = 16;     // rows kept per sequence and kv head for the step's new keys / values
+constexpr int kMaxRows = 32;     // query rows of a kv head's group (heads of the group x rows per sequence)
+
+// Query rows of a kv head's group padded to a multiple of 8 (0: the kernel does not take the shape).
+inline int padded_rows(const ps_config& g) {
+  const int rows = (g.n_heads / g.n_kv_heads) * (g.k_masks + 1);
+  return g.head_dim == kD && rows <= kMaxRows ? (rows + 7) / 8 * 8 : 0;
+}
+
+struct Buffers {
+  __nv_bfloat16* q;      // [pairs][hi, lo][NR][128] rotated, scaled query rows (pair = sequence x kv head)
+  __nv_bfloat16* kv_new; // [pairs][k, v][kNewRows][128] the step's new rows, rounded as a cache row is
+  float* part_o;         // [2 CTAs' segments][NR][128] partial outputs
+  float2* part_ml;       // [2 CTAs' segments][NR] their (reference, sum)
+};
+struct Maps { CUtensorMap kcache, vcache, q, kv_new; };
+
+size_t bytes(const ps_config& g);                 // of the buffers; 0 when padded_rows() is 0
+Buffers carve(const ps_config& g, char* base);
+bool build_maps(const ps_ctx* c, const Buffers& b, Maps* m);
+// qkv: float [B * R][Hq + 2 Hkv] before RoPE; merged output planes [B * R][n_heads * 128].
+// tickets: [B][n_heads], zero between calls.
+ps_status launch(ps_ctx* c, const SeqMap& sm, int B, const float* qkv, const Buffers& b, const Maps& m,
+                 unsigned* tickets, __nv_bfloat16* out_hi, __nv_bfloat16* out_lo, cudaStream_t st);
+
+}  // namespace atc
+}  // namespace ps

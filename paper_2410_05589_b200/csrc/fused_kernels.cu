@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cfloat>
 
+#include "attn_tc.cuh"
 #include "pair_gemm.cuh"
 #include "umma_gemm.cuh"
 #include "ws_gemm.cuh"
@@ -416,6 +417,7 @@ struct FusedScratch {
   __nv_bfloat16* xin;       // [rows][2H] gathered fc input (exact bf16: one plane)
   float* partials;          // [kMaxSm][2][16][128] partial tiles of CTAs that share a tile (up to 16 rows)
   float* slots; size_t slot_floats;   // partial tiles of the CTA-pair GEMM
+  atc::Buffers at;          // tensor-memory attention
   float* kv;                // [append rows][2 Hkv] k | v of appended positions before RoPE
   unsigned* tile_tickets;   // one per tile of the widest stage, zero between launches
   unsigned* chain_ctr;      // chained stages: finished-tile and passed-CTA counts, zero between launches
@@ -481,6 +483,7 @@ FusedScratch carve_fused(const ps_config& g, char* base) {
   s.slot_floats = std::max<size_t>((size_t)2 * (kMaxSm / 2) * 256 * pg::kMaxNp / 4 * 3, 2 * r_pad * h_pad);
   s.slots = (float*)take(s.slot_floats * 4);
   s.kv = (float*)take(ra * 2 * Hkv * 4);
+  s.at = atc::carve(g, take(atc::bytes(g)));
   s.x0p = planes(rx, g.hidden); s.ap = planes(rd, g.hidden); s.hdnp = planes(rd, g.hidden);
   s.attnp = planes(rd, Hq); s.actp = planes(rd, g.ffn);
   s.bytes = off;
@@ -1629,37 +1632,7 @@ __global__ void k_wait_expires(long long limit, int* status) {
   }
 }
 
-// ---- host side: tensor maps ---------------------------------------------------------------------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_tiled_fn() {
-  static EncodeTiledFn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      p = nullptr;
-    return (EncodeTiledFn)p;
-  }();
-  return fn;
-}
-
-// bf16 matrix [rows][cols] row-major; boxes of box_rows x 64 columns, 128-byte swizzle, zeros
-// outside the matrix.
-bool make_map(CUtensorMap* m, const void* base, size_t rows, size_t cols, int box_rows) {
-  EncodeTiledFn fn = encode_tiled_fn();
-  if (!fn) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-  cuuint32_t box[2] = {(cuuint32_t)umma::kBK, (cuuint32_t)box_rows};
-  cuuint32_t es[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
+// ---- host side: tensor maps of the operands -----------------------------------------------------
 struct PlaneMaps {   // one activation plane: boxes of 16 rows, and of every size the CTA-pair GEMM takes
   CUtensorMap m16;
   pg::PlaneMaps pair;
@@ -1669,6 +1642,8 @@ struct UmmaMaps {
   CUtensorMap w_fc, w_q, w_k, w_v, w_o, w_gate, w_up, w_down, w_lm;
   CUtensorMap w_gate128, w_up128;   // 128-row boxes (the others' gate / up boxes: 64 rows)
   PlaneMaps xin, x0_hi, x0_lo, attn_hi, attn_lo, a_hi, a_lo, act_hi, act_lo, hdn_hi, hdn_lo;
+  atc::Maps at;
+  bool at_ok = false;
   // how each stage was last dealt (a function of the shapes and the row count alone)
   pg::Plan plan[kPairStages] = {};
 };
@@ -1708,6 +1683,7 @@ UmmaMaps* build_maps(const ps_ctx* c, const FusedScratch& f) {
     delete u;
     return nullptr;
   }
+  u->at_ok = atc::build_maps(c, f.at, &u->at);
   return u;
 }
 
@@ -1894,7 +1870,9 @@ ps_status pair_draft_step(ps_ctx* c, UmmaMaps& u, const SeqMap& sm, int B, const
       return s;
   }
   prof_mark(c, st, "qkv_rope");
-  if ((s = launch_attn_split(c, sm, B, f.qkv, f.att_ml, f.att_o, f.attn_tickets, f.attnp.hi, f.attnp.lo, st))) return s;
+  s = u.at_ok ? atc::launch(c, sm, B, f.qkv, f.at, u.at, f.attn_tickets, f.attnp.hi, f.attnp.lo, st)
+              : launch_attn_split(c, sm, B, f.qkv, f.att_ml, f.att_o, f.attn_tickets, f.attnp.hi, f.attnp.lo, st);
+  if (s) return s;
   prof_mark(c, st, "attention");
   {  // S4 a = x0 + W_o attn, planes of rms(a) * g_post
     pg::Args a{};

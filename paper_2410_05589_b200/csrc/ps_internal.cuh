@@ -1,5 +1,6 @@
 // Internal declarations shared by the translation units of the library.
 #pragma once
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -197,6 +198,10 @@ ps_status plain_draft_step(ps_ctx* c, const SeqMap& sm, int B, const void* hidde
 // Gumbel-max token of every row (row_stats.cu).
 ps_status launch_logit_stats(ps_ctx* c, const float* logits, int M, int V, int R, int top_n, int* top_ids,
                              float* top_logit, float* row_max, float* row_lse, const SampleArgs* sa, cudaStream_t st);
+// bf16 matrix [rows][cols] row-major; boxes of box_rows x 64 columns, 128-byte swizzle, zeros
+// outside the matrix.  False when the driver cannot encode tensor maps (tensor_map.cu).
+constexpr int kMapCols = 64;
+bool make_map(CUtensorMap* m, const void* base, size_t rows, size_t cols, int box_rows);
 // ---- fused bf16 kernels for small M ---------------------------------------------------------
 bool fused_supported(ps_ctx* c, int M);
 int fused_kv_rows(ps_ctx* c);     // rows per pass of fused_kv_append (0: not available)

@@ -1,0 +1,55 @@
+"""Tensor-memory attention (draft steps of more than 16 rows, head_dim 128): edges of the key tiles
+and of the 16-key groups, empty contexts, pairs shared by several CTAs and many pairs per CTA,
+grouped query heads, scores that outgrow their reference (needs a B200)."""
+import numpy as np
+import pytest
+
+import synth
+from harness import Pair, as_f64, logits_close
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(p, s, seqs):
+    got = p.gpu_step(top_n=1)
+    for b in seqs:
+        want = p.oracle_step(b)
+        assert logits_close(got["logits"][b], want["logits"], s.dtype) <= 1.0, b     # the logits gate
+        assert logits_close(got["feat"][b], want["feat"], s.dtype) <= 1.0, b
+    assert np.isfinite(got["logits"]).all()
+    assert p.g.check_guards() == 0 and p.g.poll() == 0
+    again = p.gpu_step(top_n=1)
+    assert np.array_equal(got["logits"], again["logits"])
+
+
+# (heads, kv heads, k): rows of a kv head's group 3 -> 8, 9 -> 16, 6 x 3 = 18 -> 24, 2 x 16 = 32
+@pytest.mark.parametrize("heads,kv_heads,k", [(6, 6, 2), (6, 6, 8), (6, 1, 2), (6, 3, 15)])
+def test_key_tile_edges(heads, kv_heads, k):
+    s = synth.CONFIGS["mini"].with_(n_heads=heads, n_kv_heads=kv_heads, k_masks=k)
+    lens = [0, 1, 15, 16, 17, 31, 33, 127, 128, 129, 255, 257, 300]
+    p = Pair(s, len(lens), context="import", lens=lens)
+    _check(p, s, range(len(lens)))
+
+
+# 2 sequences x 1 kv head: 34 + 17 units, several CTAs per pair; 128 x 6 pairs: several pairs per CTA
+@pytest.mark.parametrize("kv_heads,lens", [(1, [4300, 2100]), (6, [130 + b for b in range(128)])])
+def test_units_dealt_to_ctas(kv_heads, lens):
+    s = synth.CONFIGS["mini"].with_(n_kv_heads=kv_heads, n_heads=3 * kv_heads if kv_heads == 1 else 6, k_masks=8)
+    seqs = [0, 1] if len(lens) == 2 else [0, 1, 63, 127]
+    p = Pair(s, len(lens), context="import", lens=lens, oracle_seqs=seqs)
+    _check(p, s, seqs)
+
+
+def test_scores_outgrow_their_reference():
+    """Keys whose scores exceed that of the first key by far more than 2^64, and keep growing from tile
+    to tile: the sums and outputs so far are rescaled."""
+    s = synth.CONFIGS["mini"].with_(k_masks=8)
+    lens = [700, 260]
+    p = Pair(s, 2, context="import", lens=lens)
+    for b, n in enumerate(lens):
+        K, V = synth.kv_rows(s, ("kv", b), n)
+        Kf = synth.bf16_bits_to_f32(K) * np.linspace(1, 250, n, dtype=np.float32)[:, None]
+        K = synth.f32_to_bf16_bits(Kf)
+        p.o.kv_import(b, as_f64(K, s.dtype), as_f64(V, s.dtype))
+        p.g.kv_import(b, p.to_device(K), p.to_device(V))
+    _check(p, s, range(2))
