@@ -67,7 +67,8 @@ def measured_peak():
 KERNEL_OF_STAGE = {
     "fc_norm": "k_gather_x + k_umma_gemm<STORE>", "qkv_rope": "k_umma_gemm<STORE>",
     "attention": "k_attn_mma", "o_proj": "k_umma_gemm<STORE>", "ffn_gate_up": "k_umma_gemm<SWIGLU>",
-    "ffn_down": "k_umma_gemm<STORE>", "lm_head": "k_umma_gemm<LMHEAD>", "verify": "k_verify_cluster",
+    "ffn_down": "k_umma_gemm<STORE>", "lm_head": "k_umma_gemm<STORE> + k_logit_stats", "verify": "k_verify_cluster",
+    "logit_stats": "k_logit_stats",
 }
 
 

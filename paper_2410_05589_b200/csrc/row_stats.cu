@@ -81,7 +81,6 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
   __shared__ Shared s;
   const int nclu = gridDim.x, rank = blockIdx.x, m = blockIdx.y;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  pdl_launch_dependents();
   if (tid == 0) s.n_list = 0;
   const float* row = logits + (size_t)m * V;
   const int share = ((V + nclu - 1) / nclu + 3) & ~3;          // tokens per block, whole vectors
@@ -96,6 +95,7 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
     row_id = ((uint32_t)b + sa.b_base) | ((uint32_t)(m - b * R) << 8);
   }
   pdl_wait();
+  pdl_launch_dependents();   // (not earlier: a dependent's blocks would wait beside the LM head's)
 
   // ---- the pass: per-thread running maximum and sum of exponentials, best perturbed logit
   float mx = -FLT_MAX, se = 0.f, gv = -FLT_MAX;
@@ -113,8 +113,11 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
     }
   };
   constexpr int U = 4;   // vectors in flight per thread
+  const bool held = n_vec <= U * kThreads;   // one batch: its logits stay in registers for the second look
+  float4 x[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) x[u] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
   for (int i0 = tid; i0 < n_vec; i0 += U * kThreads) {
-    float4 x[U];
 #pragma unroll
     for (int u = 0; u < U; ++u)
       x[u] = i0 + u * kThreads < n_vec ? __ldcg(row4 + i0 + u * kThreads) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
@@ -193,11 +196,19 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
           if (at < kListCap) { s.lv[at] = x; s.li[at] = v; }
         }
       };
+      if (held) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int i = tid + u * kThreads, v = v_lo + 4 * i;
+          if (i < n_vec) { offer(x[u].x, v); offer(x[u].y, v + 1); offer(x[u].z, v + 2); offer(x[u].w, v + 3); }
+        }
+      } else {
 #pragma unroll 4
-      for (int i = tid; i < n_vec; i += kThreads) {
-        const float4 x = __ldcg(row4 + i);
-        const int v = v_lo + 4 * i;
-        offer(x.x, v); offer(x.y, v + 1); offer(x.z, v + 2); offer(x.w, v + 3);
+        for (int i = tid; i < n_vec; i += kThreads) {
+          const float4 y = __ldcg(row4 + i);
+          const int v = v_lo + 4 * i;
+          offer(y.x, v); offer(y.y, v + 1); offer(y.z, v + 2); offer(y.w, v + 3);
+        }
       }
       for (int v = tail + tid; v < v_hi; v += kThreads) offer(__ldcg(row + v), v);
     }

@@ -1512,15 +1512,16 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
   if (a.V % 4 == 0 && a.V <= kCluMaxVocab16 && aligned && (nclu == kClu || cluster_size_ok(c->cluster_ok[0], k_verify_cluster16, 16))) {
     prof_mark(c, st, "begin");
     cudaError_t e;
-    // (plain launches: as dependents of the LM head these kernels start their loads earlier and
-    // run 3 us shorter alone, but the step gets 3 us longer -- measured twice: clusters of 8
-    // blocks that each fill an SM are slow to place while the LM head's CTAs drain)
-    const bool pdl = false;
+    // (The 8-block clusters are plain launches: as dependents they start their loads earlier and run
+    // 3 us shorter alone, but a step of one sequence gets 3-5 us longer -- clusters of 8 blocks that
+    // each fill an SM are slow to place while the LM head's CTAs drain.  The 4-block ones of a batch
+    // gain: four sequences 330 -> 326 us.)
+    const bool pdl = !c->prof;
     if (nclu == kClu && a.V <= kCluSmallMaxVocab && n_target * B * kClu > c->n_sm) {   // half the waves
       e = launch_after(k_verify_cluster4, dim3(n_target * kCluSmall, B), dim3(kCluThreads), 0, st, pdl, a);
     } else if (nclu == kClu) {
       e = launch_after(a.V <= kClu * kCluThreads * 4 * 2 ? k_verify_cluster_v2 : k_verify_cluster,
-                       dim3(n_target * kClu, B), dim3(kCluThreads), 0, st, pdl, a);
+                       dim3(n_target * kClu, B), dim3(kCluThreads), 0, st, false, a);
     } else {
       e = launch_cluster(k_verify_cluster16, dim3(n_target * 16, B), 16, kCluThreads, 0, st, a);
     }
