@@ -76,8 +76,7 @@ size_t carve(const ps_config& g, ps_ctx* c, char* base) {
   void* vrec = take(sizeof(VerifyRec) * PS_MAX_BATCH * (PS_MAX_MASKS + 2));
   void* vrow = take(sizeof(VerifyRow) * PS_MAX_BATCH * (PS_MAX_MASKS + 2));
   void* vdraw = take(sizeof(VerifyDraw) * PS_MAX_BATCH);
-  void* trec = take(sizeof(TreeRec) * PS_MAX_BATCH * (PS_MAX_TREE_NODES + 1));
-  void* ttick = take(sizeof(unsigned) * PS_MAX_BATCH);
+  void* tstat = take(sizeof(RowStat) * PS_MAX_BATCH * (2 * PS_MAX_TREE_NODES + 1));
   void* x_in = take(Mx * 2 * H * 4);
   void* x0 = take(Mx * H * 4);
   void* xn = take(Mx * H * 4);
@@ -103,7 +102,7 @@ size_t carve(const ps_config& g, ps_ctx* c, char* base) {
   if (c) {
     c->kcache = kc; c->vcache = vc; c->dev_status = (int*)status; c->tickets = (unsigned*)tickets;
     c->vrec = (VerifyRec*)vrec; c->vrow = (VerifyRow*)vrow; c->vdraw = (VerifyDraw*)vdraw;
-    c->trec = (TreeRec*)trec; c->tree_tickets = (unsigned*)ttick;
+    c->tree_stats = (RowStat*)tstat;
     c->x_in = (float*)x_in; c->x0 = (float*)x0; c->xn = (float*)xn; c->q = (float*)q;
     c->kv_tmp = (float*)kv_tmp; c->kv_side = kv_side; c->attn = (float*)attn; c->a = (float*)a; c->an = (float*)an;
     c->gate = (float*)gate; c->up = (float*)up; c->hdn = (float*)hdn; c->hn = (float*)hn;
@@ -182,7 +181,6 @@ ps_status ps_init(ps_ctx** out, const ps_config* cfg, const ps_weights* w, void*
   if (e == cudaSuccess)
     e = fused_init(c, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->tickets, 0, sizeof(unsigned) * PS_MAX_BATCH, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->tree_tickets, 0, sizeof(unsigned) * PS_MAX_BATCH, st);
   if (e != cudaSuccess || launch_rope_table(c, st) != PS_OK) {
     delete c;
     return PS_ERR_CUDA;

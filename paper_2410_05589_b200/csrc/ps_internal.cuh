@@ -108,10 +108,12 @@ __device__ __forceinline__ float gumbel_noise(const SampleArgs& sa, uint32_t v, 
 constexpr int kStatNonfinite = 1;
 constexpr int kStatTimeout = 2;
 
-struct TreeRec {    // one per (sequence, decision row) of the token-tree verification
-  int next;         // accepted child node, -1 if none
-  int token;        // token to emit if the walk stops here
-  int bad;          // a non-finite logit was met
+struct RowStat {    // softmax statistics of a row of logits (token-tree verification)
+  float max;
+  int arg;          // its lowest id
+  int bad;          // a non-finite logit was met, or nothing lies above -inf
+  int pad;
+  double sum;       // of exp((logit - max) / T)
 };
 
 struct VerifyRow {  // one per (sequence, position): verdict and statistics of a row pair (streaming kernel)
@@ -149,8 +151,7 @@ struct ps_ctx {
   ps::VerifyRec* vrec;      // [max_batch][PS_MAX_MASKS+2]
   ps::VerifyRow* vrow;      // [max_batch][PS_MAX_MASKS+2]
   ps::VerifyDraw* vdraw;    // [max_batch]
-  ps::TreeRec* trec;        // [max_batch][PS_MAX_TREE_NODES+1]
-  unsigned* tree_tickets;   // [max_batch], zero between calls
+  ps::RowStat* tree_stats;  // [max_batch][2 PS_MAX_TREE_NODES + 1]
   float *x_in, *x0, *xn, *q, *kv_tmp, *attn, *a, *an, *gate, *up, *hdn, *hn, *logits;
   void* kv_side;            // [max_rows][2 * Hkv] storage dtype: k / v of a draft step's new rows (plain kernels)
   // staging for ps_round_host

@@ -1059,14 +1059,17 @@ k_verify_draw(VerifyArgs a, const VerifyDraw* draws) {
 }
 
 // ---- token-tree verification (Algorithm 1 in full) -------------------------------------------
-// One cluster per (decision row, sequence): row u = 0 is the root, u = 1 + i the node i.  The
-// cluster holds the target row of u and the draft row of its children's depth in registers and
-// tries the children in turn.  After j rejections the target distribution of Algorithm 1 is
-// norm((p - c q)+) with c_0 = 0, c_{j+1} = c_j + Z(c_j), Z(c) = sum_v (p_v - c q_v)+ (the
-// repeated "subtract q, clip, renormalise" in closed form), so a rejection costs one reduction
-// over the cluster.  If no child is accepted (or u is a leaf) the cluster draws the token that
-// would be emitted at u.  The last cluster of a sequence to finish walks the tree from the root
-// along the accepted children.  Nothing spins.
+// Two launches.  (1) k_row_softmax streams the target rows that have children and the draft rows
+// once and leaves their maxima and sums (at temperature 0: the arg-max of every target row).  (2)
+// k_tree_walk: one cluster per sequence walks the tree from the root.  Whether the first child of a
+// node is accepted is a test of two scalars; only a rejection needs the rows again: the cluster then
+// holds them in registers.  After j rejections the target distribution of Algorithm 1 is
+// norm((p - c q)+) with c_0 = 0, c_{j+1} = c_j + Z(c_j), Z(c) = sum_v (p_v - c q_v)+ (the repeated
+// "subtract q, clip, renormalise" in closed form), so a rejection costs one reduction over the
+// cluster.  Where the walk stops the cluster draws the token.
+// Bound by the latency of the walk's cluster exchanges (1-2 us each).  A cluster per decision row
+// that tries its children speculatively was bound by its blocks' occupancy instead.  23 nodes, T = 1, before ->
+// after: 1 x 32000 tokens 31 -> 26 us, 4 x 62 -> 30, 16 x 207 -> 59; 1 x 128256 tokens 92 -> 35, 4 x 332 -> 46.
 struct TreeTopo {
   int n_nodes, max_depth;
   unsigned char depth[PS_MAX_TREE_NODES];
@@ -1083,10 +1086,134 @@ struct TreeArgs {
   float temperature;
   uint32_t key0, key1, off_lo, off_hi;
   int* accept_len; int* out_tokens; int* n_out; int* path;
-  TreeRec* rec;                // [B][PS_MAX_TREE_NODES+1]
-  unsigned* tickets;           // [B], zero on entry and on exit
+  RowStat* stats;              // [B][kTreeRows]: target rows by decision row, then draft rows by depth
   int* status;
 };
+constexpr int kTreeRows = 2 * PS_MAX_TREE_NODES + 1;
+// Rows whose statistics the walk needs: target rows with children (at temperature 0: all), draft rows.
+struct TreeRows { int n; unsigned char row[kTreeRows]; };
+
+// Statistics of row blockIdx.x / nclu of the list for sequence blockIdx.y; exponentials against a
+// reference of the block, as in k_verify_stream.
+template <bool UNIT>
+__global__ void __launch_bounds__(kStrThreads, kStrPerSm) k_row_softmax(const __grid_constant__ TreeArgs a,
+                                                                        const __grid_constant__ TreeRows list) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ StreamPart part;
+  __shared__ StreamScratch s;
+  const int nclu = (int)cl.num_blocks(), rank = (int)cl.block_rank(), b = blockIdx.y, V = a.V;
+  const int r = list.row[blockIdx.x / nclu], n_target = a.topo.n_nodes + 1;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool greedy = a.temperature == 0.f;
+  const float* row = r < n_target ? a.target_logits + ((size_t)b * n_target + r) * V
+                                  : a.draft_logits + ((size_t)b * a.topo.max_depth + (r - n_target)) * V;
+  const int share = ((V + nclu - 1) / nclu + kSeg - 1) / kSeg * kSeg;
+  const int v_lo = min(V, rank * share), n_vec = (min(V, v_lo + share) - v_lo) / 4;   // V % 4 == 0
+  const double inv_t = greedy ? 1.0 : 1.0 / (double)a.temperature;
+  const float i_hi = (float)inv_t, i_lo = (float)(inv_t - (double)i_hi);
+  pdl_launch_dependents();
+  pdl_wait();
+  constexpr int U = 4;
+  const float4* r4 = reinterpret_cast<const float4*>(row + v_lo);
+  float mx = -INFINITY, ref = -INFINITY;
+  int mi = 0x7fffffff;
+  double st = 0.0;
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    st = 0.0;
+    for (int v0 = tid; v0 - tid < n_vec; v0 += U * kStrThreads) {
+      float4 t[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int v = v0 + u * kStrThreads;
+        t[u] = v < n_vec ? __ldg(r4 + v) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      }
+      if (attempt == 0) {
+        float bt = -INFINITY;
+#pragma unroll
+        for (int u = 0; u < U; ++u) bt = fmaxf(fmaxf(fmaxf(bt, t[u].x), fmaxf(t[u].y, t[u].z)), t[u].w);
+        if (bt > mx) {   // (rare after the first batch) the lowest id that holds the new maximum
+          mx = bt;
+#pragma unroll
+          for (int u = U - 1; u >= 0; --u) {
+            const int v = v_lo + 4 * (v0 + u * kStrThreads);
+            if (t[u].w == bt) mi = v + 3;
+            if (t[u].z == bt) mi = v + 2;
+            if (t[u].y == bt) mi = v + 1;
+            if (t[u].x == bt) mi = v;
+          }
+        }
+        if (!greedy && v0 == tid) {   // first batch: the block's reference
+          float rt = bt;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) rt = fmaxf(rt, __shfl_xor_sync(0xffffffffu, rt, o));
+          if (lane == 0) s.f[warp] = rt;
+          __syncthreads();
+#pragma unroll
+          for (int w = 0; w < kStrWarps; ++w) ref = fmaxf(ref, s.f[w]);
+          if (ref == -INFINITY) ref = 0.f;   // (differences from the reference are NaN for NaN logits only)
+        }
+      }
+      if (!greedy) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          st += (double)expf(exp_arg<UNIT>(t[u].x, ref, i_hi, i_lo)); st += (double)expf(exp_arg<UNIT>(t[u].y, ref, i_hi, i_lo));
+          st += (double)expf(exp_arg<UNIT>(t[u].z, ref, i_hi, i_lo)); st += (double)expf(exp_arg<UNIT>(t[u].w, ref, i_hi, i_lo));
+        }
+      }
+    }
+    if (attempt == 0) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, mx, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
+        if (ov > mx || (ov == mx && oi < mi)) { mx = ov; mi = oi; }
+      }
+    }
+    st = warp_sum_d(st);
+    __syncthreads();   // the reference has been read
+    if (lane == 0) { s.f[warp] = mx; s.i[warp] = mi; s.d[warp] = st; }
+    __syncthreads();
+    st = 0.0;
+#pragma unroll
+    for (int w = 0; w < kStrWarps; ++w) {
+      if (s.f[w] > mx || (s.f[w] == mx && s.i[w] < mi)) { mx = s.f[w]; mi = s.i[w]; }
+      st += s.d[w];
+    }
+    if (greedy || !(mx > -INFINITY && fabs((double)mx - (double)ref) * inv_t > kRefSlack)) break;
+    ref = mx;
+    __syncthreads();
+  }
+  if (tid == 0) {   // (the maximum skips NaN, but a NaN logit leaves the sum NaN)
+    part.tmax = mx; part.targ = mi; part.tref = ref; part.st = st;
+    part.bad = mx == INFINITY || st != st;
+  }
+  cl.sync();
+  if (rank == 0 && warp == 0) {
+    const StreamPart* pr = lane < nclu ? cl.map_shared_rank(&part, lane) : nullptr;
+    float m = pr ? pr->tmax : -INFINITY;
+    int id = pr ? pr->targ : 0x7fffffff, bad = pr ? pr->bad : 0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, m, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, id, o);
+      if (ov > m || (ov == m && oi < id)) { m = ov; id = oi; }
+      bad |= __shfl_xor_sync(0xffffffffu, bad, o);
+    }
+    m = __shfl_sync(0xffffffffu, m, 0);
+    double x = 0.0;
+    if (!greedy && pr && pr->st > 0.0 && m > -INFINITY && m < INFINITY)
+      x = pr->st * exp(((double)pr->tref - (double)m) * inv_t);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (lane == 0) {
+      RowStat rs;
+      rs.max = m; rs.arg = id == 0x7fffffff ? 0 : id; rs.bad = bad | (m == -INFINITY ? 1 : 0); rs.pad = 0; rs.sum = x;
+      a.stats[(size_t)b * kTreeRows + r] = rs;
+    }
+  }
+  cl.sync();   // no block leaves while the first one reads its part
+}
 
 // Sum over the cluster of one double per thread; every thread of every block gets the value.
 __device__ double cluster_sum(cooperative_groups::cluster_group& cl, CluPart& part, CluScratch& s, double v,
@@ -1202,187 +1329,199 @@ __device__ int cluster_draw(cooperative_groups::cluster_group& cl, CluPart& part
   return token;
 }
 
-// (The cluster size is a launch attribute: 8 blocks per row, or fewer when a large tree would
-// otherwise need a second wave of blocks.)
-__global__ void __launch_bounds__(kCluThreads) k_verify_tree(TreeArgs a) {
+// (The cluster size is a launch attribute: 8 blocks, 16 for vocabularies beyond 65536.)
+__global__ void __launch_bounds__(kCluThreads) k_tree_walk(const __grid_constant__ TreeArgs a) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   __shared__ CluPart part;
   __shared__ CluScratch s;
-  const int rank = (int)cl.block_rank();
-  const int nclu = (int)cl.num_blocks();
-  const int u = blockIdx.x / nclu, b = blockIdx.y, V = a.V, n_nodes = a.topo.n_nodes;
+  const int rank = (int)cl.block_rank(), nclu = (int)cl.num_blocks();
+  const int b = blockIdx.y, V = a.V, n_nodes = a.topo.n_nodes;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int kid0 = a.topo.child_off[u], n_kids = a.topo.child_off[u + 1] - kid0;
-  const int dq = u == 0 ? 0 : a.topo.depth[u - 1] + 1;   // depth of the children of u
-  const bool greedy = a.temperature == 0.f;
-  const float* trow = a.target_logits + ((size_t)b * (n_nodes + 1) + u) * V;
-  const float* drow = (!greedy && n_kids > 0) ? a.draft_logits + ((size_t)b * a.topo.max_depth + dq) * V : nullptr;
+  const bool greedy = a.temperature == 0.f, writer = rank == 0 && tid == 0;
+  const double inv_t = greedy ? 1.0 : 1.0 / (double)a.temperature;
   const int* toks = a.tokens + (size_t)b * n_nodes;
   const int nv4 = ((V + nclu * kCluThreads - 1) / (nclu * kCluThreads) + 3) / 4;
   const int C = nv4 * 4, v0 = (rank * kCluThreads + tid) * C;
-
-  float t[kCluV4 * 4], d[kCluV4 * 4];
+  int* out = a.out_tokens + (size_t)b * (a.topo.max_depth + 1);
+  int* pth = a.path + (size_t)b * a.topo.max_depth;
+  pdl_launch_dependents();
+  pdl_wait();
+  const RowStat* stats = a.stats + (size_t)b * kTreeRows;
+  int u = 0, len = 0, any_bad = 0, token = -1;
+  // every block takes the same branches below: the values they depend on are identical
+  for (;;) {
+    const int kid0 = a.topo.child_off[u], n_kids = a.topo.child_off[u + 1] - kid0;
+    const float* trow = a.target_logits + ((size_t)b * (n_nodes + 1) + u) * V;
+    const int dq = len;   // depth of the children of u
+    const float* drow = (!greedy && n_kids > 0) ? a.draft_logits + ((size_t)b * a.topo.max_depth + dq) * V : nullptr;
+    RowStat ts, ds;
+    ts.max = 0.f; ts.arg = 0; ts.bad = 0; ts.sum = 1.0;
+    ds = ts;
+    if (greedy || n_kids > 0) ts = stats[u];
+    if (drow) ds = stats[n_nodes + 1 + dq];
+    int next = -1;
+    if (greedy) {
+      for (int j = 0; j < n_kids && next < 0; ++j)
+        if (toks[a.topo.child_idx[kid0 + j]] == ts.arg) next = a.topo.child_idx[kid0 + j];
+      if (next < 0) token = ts.arg;
+    } else if (ts.bad | ds.bad) {
+      any_bad = 1;
+      token = ts.arg;
+    } else {
+      float t[kCluV4 * 4], d[kCluV4 * 4];   // the rows' exponentials, once they are needed
+      bool loaded = false;
+      float tmax = ts.max;
+      auto load = [&]() {
+        loaded = true;
 #pragma unroll
-  for (int k = 0; k < kCluV4; ++k) {
-    const int v = v0 + 4 * k;   // V % 4 == 0: a vector lies inside the row or outside it
-    float4 tv = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY), dv = tv;
-    if (k < nv4 && v < V) {
-      tv = *reinterpret_cast<const float4*>(trow + v);
-      if (drow) dv = *reinterpret_cast<const float4*>(drow + v);
-    }
-    t[4 * k] = tv.x; t[4 * k + 1] = tv.y; t[4 * k + 2] = tv.z; t[4 * k + 3] = tv.w;
-    d[4 * k] = dv.x; d[4 * k + 1] = dv.y; d[4 * k + 2] = dv.z; d[4 * k + 3] = dv.w;
-  }
-  // ---- maxima (NaN counts as -inf, ties to the lower id) and non-finite flags
-  float tm = -INFINITY, dm = -INFINITY;
-  int ti = 0x7fffffff, bad = 0;
+        for (int k = 0; k < kCluV4; ++k) {
+          const int v = v0 + 4 * k;   // V % 4 == 0: a vector lies inside the row or outside it
+          float4 tv = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY), dv = tv;
+          if (k < nv4 && v < V) {
+            tv = *reinterpret_cast<const float4*>(trow + v);
+            if (drow) dv = *reinterpret_cast<const float4*>(drow + v);
+          }
+          t[4 * k] = tv.x; t[4 * k + 1] = tv.y; t[4 * k + 2] = tv.z; t[4 * k + 3] = tv.w;
+          d[4 * k] = dv.x; d[4 * k + 1] = dv.y; d[4 * k + 2] = dv.z; d[4 * k + 3] = dv.w;
+        }
+      };
+      auto exponentials = [&]() {
 #pragma unroll
-  for (int e = 0; e < kCluV4 * 4; ++e) {
-    const int v = v0 + e;
-    if (e < C && v < V) {
-      float xt = t[e];
-      if (xt != xt || xt == INFINITY) bad = 1;
-      if (xt != xt) xt = -INFINITY;
-      if (xt > tm || (xt == tm && v < ti)) { tm = xt; ti = v; }
-      if (drow) {
-        float xd = d[e];
-        if (xd != xd || xd == INFINITY) bad = 1;
-        if (xd != xd) xd = -INFINITY;
-        dm = fmaxf(dm, xd);
+        for (int e = 0; e < kCluV4 * 4; ++e) {
+          const bool in = e < C && v0 + e < V;
+          t[e] = in ? expf((float)(((double)t[e] - (double)tmax) * inv_t)) : 0.f;
+          d[e] = (in && drow) ? expf((float)(((double)d[e] - (double)ds.max) * inv_t)) : 0.f;
+        }
+      };
+      double st = ts.sum;
+      bool bad = false;
+      if (n_kids == 0) {   // a leaf: its statistics are formed here
+        load();
+        float tm = -INFINITY;
+        int ti = 0x7fffffff, bd = 0;
+#pragma unroll
+        for (int e = 0; e < kCluV4 * 4; ++e) {
+          const int v = v0 + e;
+          if (e < C && v < V) {
+            float xt = t[e];
+            if (xt != xt || xt == INFINITY) bd = 1;
+            if (xt != xt) xt = -INFINITY;
+            if (xt > tm || (xt == tm && v < ti)) { tm = xt; ti = v; }
+          }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const float ov = __shfl_xor_sync(0xffffffffu, tm, o);
+          const int oi = __shfl_xor_sync(0xffffffffu, ti, o);
+          if (ov > tm || (ov == tm && oi < ti)) { tm = ov; ti = oi; }
+          bd |= __shfl_xor_sync(0xffffffffu, bd, o);
+        }
+        __syncthreads();
+        if (lane == 0) { s.f[warp] = tm; s.i[warp] = ti; s.flag[warp] = bd; }
+        __syncthreads();
+        if (tid == 0) {
+          for (int w = 1; w < kCluWarps; ++w) {
+            if (s.f[w] > tm || (s.f[w] == tm && s.i[w] < ti)) { tm = s.f[w]; ti = s.i[w]; }
+            bd |= s.flag[w];
+          }
+          part.tmax = tm; part.targ = ti; part.bad = bd;
+        }
+        cl.sync();
+        tm = -INFINITY; ti = 0x7fffffff; bd = 0;
+        if (lane < nclu) {
+          const CluPart* pr = cl.map_shared_rank(&part, lane);
+          tm = pr->tmax; ti = pr->targ; bd = pr->bad;
+        }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+          const float ov = __shfl_xor_sync(0xffffffffu, tm, o);
+          const int oi = __shfl_xor_sync(0xffffffffu, ti, o);
+          if (ov > tm || (ov == tm && oi < ti)) { tm = ov; ti = oi; }
+          bd |= __shfl_xor_sync(0xffffffffu, bd, o);
+        }
+        tmax = __shfl_sync(0xffffffffu, tm, 0);
+        ts.arg = __shfl_sync(0xffffffffu, ti, 0);
+        bad = __shfl_sync(0xffffffffu, bd, 0) != 0 || tmax == -INFINITY;
+        if (ts.arg == 0x7fffffff) ts.arg = 0;
+        cl.sync();   // the partials are free again
+        if (!bad) {
+          exponentials();
+          double mine = 0.0;
+#pragma unroll
+          for (int e = 0; e < kCluV4 * 4; ++e) mine += (double)t[e];
+          st = cluster_sum(cl, part, s, mine, tid, warp, lane);
+        }
       }
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float ov = __shfl_xor_sync(0xffffffffu, tm, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, ti, o);
-    if (ov > tm || (ov == tm && oi < ti)) { tm = ov; ti = oi; }
-    dm = fmaxf(dm, __shfl_xor_sync(0xffffffffu, dm, o));
-    bad |= __shfl_xor_sync(0xffffffffu, bad, o);
-  }
-  if (lane == 0) { s.f[warp] = tm; s.i[warp] = ti; s.flag[warp] = bad; s.f2[warp] = dm; }
-  __syncthreads();
-  if (tid == 0) {
-    for (int w = 1; w < kCluWarps; ++w) {
-      if (s.f[w] > tm || (s.f[w] == tm && s.i[w] < ti)) { tm = s.f[w]; ti = s.i[w]; }
-      dm = fmaxf(dm, s.f2[w]);
-      bad |= s.flag[w];
-    }
-    part.tmax = tm; part.targ = ti; part.dmax = dm; part.bad = bad;
-    part.pick = -1; part.lastp = -1; part.wsum = 0.0; part.st = 0.0; part.sd = 0.0;
-  }
-  cl.sync();
-  tm = -INFINITY; dm = -INFINITY; ti = 0x7fffffff; bad = 0;
-  for (int r = 0; r < (int)cl.num_blocks(); ++r) {
-    const CluPart* pr = cl.map_shared_rank(&part, r);
-    const float ov = pr->tmax;
-    const int oi = pr->targ;
-    if (ov > tm || (ov == tm && oi < ti)) { tm = ov; ti = oi; }
-    dm = fmaxf(dm, pr->dmax);
-    bad |= pr->bad;
-  }
-  cl.sync();   // the partials are free again
-  if (tm == -INFINITY || (drow && dm == -INFINITY)) bad = 1;  // a row without a distribution
-  const float tmax = tm, dmax = dm;
-  const int targ = ti;
-
-  int next = -1, token = -1;
-  if (greedy) {
-    for (int j = 0; j < n_kids && next < 0; ++j)
-      if (toks[a.topo.child_idx[kid0 + j]] == targ) next = a.topo.child_idx[kid0 + j];
-    token = targ;
-    bad = 0;
-  } else if (bad) {
-    token = targ;
-  } else {
-    // every block takes the same branches below: the values they depend on are identical
-    const double inv_t = 1.0 / (double)a.temperature;
-    double st = 0.0, sd = 0.0;
-#pragma unroll
-    for (int e = 0; e < kCluV4 * 4; ++e) {
-      const bool in = e < C && v0 + e < V;
-      t[e] = in ? expf((float)(((double)t[e] - (double)tmax) * inv_t)) : 0.f;
-      st += (double)t[e];
-      d[e] = (in && drow) ? expf((float)(((double)d[e] - (double)dmax) * inv_t)) : 0.f;
-      sd += (double)d[e];
-    }
-    st = cluster_sum(cl, part, s, st, tid, warp, lane);
-    sd = drow ? cluster_sum(cl, part, s, sd, tid, warp, lane) : 1.0;
-    const float inv_st = (float)(1.0 / st), inv_sd = (float)(1.0 / sd);
-    double c = 0.0, Zc = 1.0;   // the target distribution at u is now (p - c q)+ / Zc
-    for (int j = 0; j < n_kids; ++j) {
-      const int kid = a.topo.child_idx[kid0 + j];
-      const int x = toks[kid];
-      uint32_t ctr[4] = {(uint32_t)u + ((uint32_t)j << 16), (uint32_t)b, a.off_lo, a.off_hi};
-      philox4x32_10(a.key0, a.key1, ctr);
-      const double r = (double)(ctr[0] >> 8) * (1.0 / 16777216.0);
-      const bool in_range = x >= 0 && x < V;
-      const double logp = in_range ? ((double)trow[x] - (double)tmax) * inv_t - log(st) : -INFINITY;
-      const double logq = in_range ? ((double)drow[x] - (double)dmax) * inv_t - log(sd) : -INFINITY;
-      double ratio;
-      if (c == 0.0) {
-        const double diff = logp - logq;
-        ratio = (diff != diff) ? 0.0 : exp(fmin(diff, 0.0));
+      if (bad) {
+        any_bad = 1;
+        token = ts.arg;
       } else {
-        const double px = exp(logp), qx = exp(logq);
-        const double wx = fmax(px - c * qx, 0.0) / Zc;
-        ratio = qx > 0.0 ? fmin(wx / qx, 1.0) : (wx > 0.0 ? 1.0 : 0.0);
+        const float inv_st = (float)(1.0 / st), inv_sd = (float)(1.0 / ds.sum);
+        const double log_st = log(st), log_sd = log(ds.sum);
+        double c = 0.0, Zc = 1.0;   // the target distribution at u is now (p - c q)+ / Zc
+        for (int j = 0; j < n_kids; ++j) {
+          const int kid = a.topo.child_idx[kid0 + j];
+          const int x = toks[kid];
+          uint32_t ctr[4] = {(uint32_t)u + ((uint32_t)j << 16), (uint32_t)b, a.off_lo, a.off_hi};
+          philox4x32_10(a.key0, a.key1, ctr);
+          const double r = (double)(ctr[0] >> 8) * (1.0 / 16777216.0);
+          const bool in_range = x >= 0 && x < V;
+          const double logp = in_range ? ((double)trow[x] - (double)tmax) * inv_t - log_st : -INFINITY;
+          const double logq = in_range ? ((double)drow[x] - (double)ds.max) * inv_t - log_sd : -INFINITY;
+          double ratio;
+          if (c == 0.0) {
+            const double diff = logp - logq;
+            ratio = (diff != diff) ? 0.0 : exp(fmin(diff, 0.0));
+          } else {
+            const double px = exp(logp), qx = exp(logq);
+            const double wx = fmax(px - c * qx, 0.0) / Zc;
+            ratio = qx > 0.0 ? fmin(wx / qx, 1.0) : (wx > 0.0 ? 1.0 : 0.0);
+          }
+          if (r < ratio) { next = kid; break; }
+          // rejected: the target distribution becomes norm((p - (c + Zc) q)+)
+          if (!loaded) { load(); exponentials(); }
+          const double c_new = c + Zc;
+          const float cf = (float)c_new;
+          double mine = 0.0;
+#pragma unroll
+          for (int e = 0; e < kCluV4 * 4; ++e) mine += (double)fmaxf(t[e] * inv_st - cf * (d[e] * inv_sd), 0.f);
+          const double Z = cluster_sum(cl, part, s, mine, tid, warp, lane);
+          if (Z > 0.0) { c = c_new; Zc = Z; } else { c = 0.0; Zc = 1.0; }   // nothing left: back to p
+        }
+        if (next < 0) {
+          uint32_t ctr[4] = {(uint32_t)u, (uint32_t)b, a.off_lo, a.off_hi};
+          philox4x32_10(a.key0, a.key1, ctr);
+          const double u2 = (double)(ctr[1] >> 8) * (1.0 / 16777216.0);
+          const float cf = (float)c;
+          float w[kCluV4 * 4];
+#pragma unroll
+          for (int e = 0; e < kCluV4 * 4; ++e) w[e] = fmaxf(t[e] * inv_st - cf * (d[e] * inv_sd), 0.f);
+          token = cluster_draw(cl, part, s, w, v0, u2, rank, tid, warp, lane);
+          if (token < 0 && c != 0.0) {   // the residual vanished in fp32: draw from p
+#pragma unroll
+            for (int e = 0; e < kCluV4 * 4; ++e) w[e] = t[e] * inv_st;
+            token = cluster_draw(cl, part, s, w, v0, u2, rank, tid, warp, lane);
+          }
+          if (token < 0) token = ts.arg;
+        }
       }
-      if (r < ratio) { next = kid; break; }
-      // rejected: the target distribution becomes norm((p - (c + Zc) q)+)
-      const double c_new = c + Zc;
-      const float cf = (float)c_new;
-      double mine = 0.0;
-#pragma unroll
-      for (int e = 0; e < kCluV4 * 4; ++e) mine += (double)fmaxf(t[e] * inv_st - cf * (d[e] * inv_sd), 0.f);
-      const double Z = cluster_sum(cl, part, s, mine, tid, warp, lane);
-      if (Z > 0.0) { c = c_new; Zc = Z; } else { c = 0.0; Zc = 1.0; }   // nothing left: back to p
     }
-    if (next < 0) {
-      uint32_t ctr[4] = {(uint32_t)u, (uint32_t)b, a.off_lo, a.off_hi};
-      philox4x32_10(a.key0, a.key1, ctr);
-      const double u2 = (double)(ctr[1] >> 8) * (1.0 / 16777216.0);
-      const float cf = (float)c;
-      float w[kCluV4 * 4];
-#pragma unroll
-      for (int e = 0; e < kCluV4 * 4; ++e) w[e] = fmaxf(t[e] * inv_st - cf * (d[e] * inv_sd), 0.f);
-      token = cluster_draw(cl, part, s, w, v0, u2, rank, tid, warp, lane);
-      if (token < 0 && c != 0.0) {   // the residual vanished in fp32: draw from p
-#pragma unroll
-        for (int e = 0; e < kCluV4 * 4; ++e) w[e] = t[e] * inv_st;
-        token = cluster_draw(cl, part, s, w, v0, u2, rank, tid, warp, lane);
-      }
-      if (token < 0) token = targ;
+    if (next < 0) break;
+    if (writer) {
+      out[len] = toks[next];
+      pth[len] = next;
     }
+    ++len;
+    u = next + 1;
   }
-  if (rank == 0 && tid == 0) {
-    TreeRec* rec = a.rec + (size_t)b * (PS_MAX_TREE_NODES + 1);
-    rec[u].next = next; rec[u].token = token; rec[u].bad = bad;
-    __threadfence();
-    const unsigned tk = atomicAdd(&a.tickets[b], 1u);
-    if (tk == (unsigned)n_nodes) {   // the last of the n_nodes + 1 decision rows
-      __threadfence();
-      volatile TreeRec* R = rec;
-      int* out = a.out_tokens + (size_t)b * (a.topo.max_depth + 1);
-      int* pth = a.path + (size_t)b * a.topo.max_depth;
-      int uu = 0, len = 0, any_bad = 0;
-      for (;;) {
-        any_bad |= R[uu].bad;
-        const int nx = R[uu].next;
-        if (nx < 0 || len >= a.topo.max_depth) { out[len] = R[uu].token; break; }
-        out[len] = toks[nx];
-        pth[len] = nx;
-        ++len;
-        uu = nx + 1;
-      }
-      for (int j = len + 1; j <= a.topo.max_depth; ++j) out[j] = -1;
-      for (int j = len; j < a.topo.max_depth; ++j) pth[j] = -1;
-      a.accept_len[b] = len;
-      a.n_out[b] = len + 1;
-      if (any_bad) atomicOr(a.status, kStatNonfinite);
-      a.tickets[b] = 0u;
-    }
+  if (writer) {
+    out[len] = token;
+    for (int j = len + 1; j <= a.topo.max_depth; ++j) out[j] = -1;
+    for (int j = len; j < a.topo.max_depth; ++j) pth[j] = -1;
+    a.accept_len[b] = len;
+    a.n_out[b] = len + 1;
+    if (any_bad) atomicOr(a.status, kStatNonfinite);
   }
   cl.sync();   // no block leaves while another may still read its shared memory
 }
@@ -1433,17 +1572,19 @@ ps_status launch_build_tree(ps_ctx* c, int B, int n_nodes, const int* parent, co
 // Launch with a cluster of nclu blocks along x (a launch attribute, not a compile-time one).
 template <class... KArgs, class... Args>
 cudaError_t launch_cluster(void (*kern)(KArgs...), dim3 grid, int nclu, int threads, size_t smem, cudaStream_t st,
-                           const Args&... a) {
+                           bool pdl, const Args&... a) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = nclu; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = pdl ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, a...);
 }
 
@@ -1498,7 +1639,7 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
       const bool unit = temperature == 1.f;
       prof_mark(c, st, "begin");
       cudaError_t e = launch_cluster(unit ? k_verify_stream<true> : k_verify_stream<false>, dim3(n_target * per, B), per,
-                                     kStrThreads, 0, st, a, c->vrow, c->vdraw);
+                                     kStrThreads, 0, st, false, a, c->vrow, c->vdraw);
       c->launches++;
       if (e == cudaSuccess && temperature > 0.f) {
         e = launch_after(unit ? k_verify_draw<true> : k_verify_draw<false>, dim3(kDrawClu, B), dim3(kStrThreads), bytes, st,
@@ -1523,7 +1664,7 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
       e = launch_after(a.V <= kClu * kCluThreads * 4 * 2 ? k_verify_cluster_v2 : k_verify_cluster,
                        dim3(n_target * kClu, B), dim3(kCluThreads), 0, st, false, a);
     } else {
-      e = launch_cluster(k_verify_cluster16, dim3(n_target * 16, B), 16, kCluThreads, 0, st, a);
+      e = launch_cluster(k_verify_cluster16, dim3(n_target * 16, B), 16, kCluThreads, 0, st, false, a);
     }
     c->launches++;
     prof_mark(c, st, "verify");
@@ -1573,19 +1714,28 @@ ps_status launch_verify_tree(ps_ctx* c, int B, int n_nodes, const int* parent, c
   a.key0 = (uint32_t)seed; a.key1 = (uint32_t)(seed >> 32);
   a.off_lo = (uint32_t)offset; a.off_hi = (uint32_t)(offset >> 32);
   a.accept_len = accept_len; a.out_tokens = out_tokens; a.n_out = n_out; a.path = path;
-  a.rec = c->trec; a.tickets = c->tree_tickets; a.status = c->dev_status;
-  prof_mark(c, st, "begin");
-  // blocks per decision row: 8 (16 for vocabularies beyond 65536), fewer when the tree would
-  // otherwise need a second wave of blocks and a thread can still hold its share of a row
-  int nclu = a.V <= kCluMaxVocab ? kClu : 16;
-  if (!cluster_size_ok(c->cluster_ok[1], k_verify_tree, nclu))
+  a.stats = c->tree_stats; a.status = c->dev_status;
+  const int nclu = a.V <= kCluMaxVocab ? kClu : 16;
+  if (!cluster_size_ok(c->cluster_ok[1], k_tree_walk, nclu))
     return fail(c, PS_ERR_UNSUPPORTED, "this device cannot run the 16-block clusters a vocabulary beyond 65536 needs");
-  while (nclu > 1 && (long)(n_nodes + 1) * B * nclu > c->n_sm && a.V <= (nclu / 2) * kCluThreads * 4 * kCluV4)
-    nclu /= 2;
-  cudaError_t e = launch_cluster(k_verify_tree, dim3((n_nodes + 1) * nclu, B), nclu, kCluThreads, 0, st, a);
+  TreeRows list;
+  list.n = 0;
+  for (int u = 0; u <= n_nodes; ++u)
+    if (temperature == 0.f || tp.child_off[u + 1] > tp.child_off[u]) list.row[list.n++] = (unsigned char)u;
+  if (temperature != 0.f)
+    for (int t = 0; t < tp.max_depth; ++t) list.row[list.n++] = (unsigned char)(n_nodes + 1 + t);
+  int per = 1;   // blocks per row: as many as are resident together
+  while (per < 8 && 2 * list.n * B * per <= kStrPerSm * c->n_sm) per *= 2;
+  prof_mark(c, st, "begin");
+  cudaError_t e = launch_cluster(temperature == 1.f ? k_row_softmax<true> : k_row_softmax<false>, dim3(list.n * per, B), per,
+                                 kStrThreads, 0, st, !c->prof, a, list);
   c->launches++;
+  if (e == cudaSuccess) {
+    e = launch_cluster(k_tree_walk, dim3(nclu, B), nclu, kCluThreads, 0, st, !c->prof, a);
+    c->launches++;
+  }
   prof_mark(c, st, "verify_tree");
-  return cuda_check(c, e, "k_verify_tree");
+  return cuda_check(c, e, "k_tree_walk");
 }
 
 }  // namespace ps
