@@ -1,9 +1,14 @@
-// Unfused kernels with fp32 activations.  They cover every dtype and shape the library
-// accepts and are the path for fp32 models; the fused bf16 kernels replace them stage by
-// stage where they apply.  One kernel per step of the layer:
-//   gather -> fc -> RMSNorm -> q,k,v -> RoPE + cache write -> attention -> o (+residual)
-//   -> RMSNorm -> gate, up -> silu*up -> down (+residual) -> RMSNorm -> LM head -> row stats
+// Kernels with fp32 activations.  They cover every dtype and shape the library accepts and are the
+// path for fp32 models (and for bf16 ones the tensor-core kernels do not take).  A draft step is seven
+// launches, each the dependent of the one before it:
+//   fc (rows gathered) -> q|k|v (RMSNorm) -> attention (RoPE) -> o (+ residual)
+//   -> silu(gate) * up (RMSNorm) -> down (+ residual) -> LM head (RMSNorm)   [-> row statistics]
 // (Sec. 4.1 "Inference", Sec. 4.3, Sec. 5.1 "Models".)
+// What bounds them at the sizes fp32 models are used at (a few MB of weights) is launches and the
+// latency of a handful of dependent loads: hence the neighbouring element-wise work inside the
+// products, the first weights in flight before the wait for the kernel ahead, and no predicates in
+// the inner loop.  Measured (hidden 256, 5 rows, 64 cached keys; draft + verify): 18 launches 114 us
+// -> 9 launches 49 us.
 #include <cfloat>
 
 #include "ps_internal.cuh"
@@ -15,8 +20,15 @@ __device__ __forceinline__ float to_f32(float x) { return x; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
 __device__ __forceinline__ void store_as(float* p, float v) { *p = v; }
 __device__ __forceinline__ void store_as(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
+// v as the cache holds it.
+template <typename WT>
+__device__ __forceinline__ float rounded(float v);
+template <>
+__device__ __forceinline__ float rounded<float>(float v) { return v; }
+template <>
+__device__ __forceinline__ float rounded<__nv_bfloat16>(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 
-// 8 consecutive weights as floats; p is 16-byte (bf16) / 32-byte (fp32) aligned.
+// 8 consecutive values as floats; p is 16-byte aligned.
 __device__ __forceinline__ void load8(const float* p, float (&w)[8]) {
   float4 a = __ldg(reinterpret_cast<const float4*>(p));
   float4 b = __ldg(reinterpret_cast<const float4*>(p) + 1);
@@ -31,243 +43,368 @@ __device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&w)[8]) {
     w[2 * i + 1] = __uint_as_float(u[i] & 0xffff0000u);
   }
 }
-
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-// S0: rows of the fc input.  Row j = 0 of a sequence: [embed[token] ; hidden]; rows j >= 1:
+// Source rows of the fc input.  Row j = 0 of a sequence: [embed[token] ; hidden]; rows j >= 1:
 // [mask_embed[j-1] ; mask_feat[j-1]].  With all_real every row is a real (token, hidden) pair.
 template <typename WT>
-__global__ void k_gather(SeqMap sm, int all_real, const WT* embed, const WT* mask_embed,
-                         const WT* mask_feat, const WT* hidden, const int* tokens, int H, int V,
-                         float* x_in) {
-  int m = blockIdx.x;
+struct GatherSrc {
+  const WT *embed, *mask_embed, *mask_feat, *hidden;
+  const int* tokens;
+  int all_real, H, V;
+};
+template <typename WT>
+__device__ __forceinline__ void gather_row(const GatherSrc<WT>& g, const SeqMap& sm, int m, const WT*& e, const WT*& f) {
   int b, j;
   seq_of_row(sm, m, b, j);
-  const WT *e, *f;
-  if (all_real || j == 0) {
-    int src = all_real ? (m + sm.row_base) : b;
-    int tok = tokens[src];
-    tok = min(max(tok, 0), V - 1);
-    e = embed + (size_t)tok * H;
-    f = hidden + (size_t)src * H;
+  if (g.all_real || j == 0) {
+    const int src = g.all_real ? (m + sm.row_base) : b;
+    const int tok = min(max(g.tokens[src], 0), g.V - 1);
+    e = g.embed + (size_t)tok * g.H;
+    f = g.hidden ? g.hidden + (size_t)src * g.H : nullptr;
   } else {
-    e = mask_embed + (size_t)(j - 1) * H;
-    f = mask_feat + (size_t)(j - 1) * H;
-  }
-  float* out = x_in + (size_t)m * 2 * H;
-  for (int i = threadIdx.x; i < H; i += blockDim.x) {
-    out[i] = to_f32(e[i]);
-    out[H + i] = hidden ? to_f32(f[i]) : 0.f;   // embedding-only input: no feature half
+    e = g.mask_embed + (size_t)(j - 1) * g.H;
+    f = g.mask_feat ? g.mask_feat + (size_t)(j - 1) * g.H : nullptr;
   }
 }
+// Embedding-only input (PS_FLAG_NO_FC): x0 is the embedding half.
+template <typename WT>
+__global__ void __launch_bounds__(256) k_gather_embed(const __grid_constant__ SeqMap sm, GatherSrc<WT> g, float* x0) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const WT *e, *f;
+  gather_row(g, sm, blockIdx.x, e, f);
+  for (int i = threadIdx.x; i < g.H; i += blockDim.x) x0[(size_t)blockIdx.x * g.H + i] = to_f32(e[i]);
+}
 
-// Y[m][n] = sum_k X[m][k] W[n][k] (+ bias[n]) (+ res[m][n]).  One warp per output feature n,
-// MC rows per pass.  K is a multiple of 8.
-template <typename WT, int MC>
-__global__ void __launch_bounds__(256) k_linear(const float* __restrict__ X, int ldx,
-                                                const WT* __restrict__ W,
-                                                const WT* __restrict__ bias,
-                                                const float* __restrict__ res, int ldr,
-                                                float* __restrict__ Y, int ldy, int M, int N,
-                                                int K) {
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int n = blockIdx.x * 8 + warp;
-  if (n >= N) return;
-  int m0 = blockIdx.y * MC;
-  float acc[MC];
+// Y[m][n] = sum_k x[m][k] W[n][k] over up to three concatenated matrices, one warp per output
+// feature, MC rows per block row.  K is a multiple of 8.  A block's warps share the activations: they
+// come through shared memory, kKC columns at a time (each warp reading them from L2 for itself was
+// bound by that: 64 KB per block and 256 columns), the weights of those columns in flight meanwhile.
+//   LIN_GATHER  x: the gathered fc input (K = 2 H); bias
+//   LIN_NORM    x = X * rsqrt(mean(X^2) + eps) * gain: the sums of squares are taken on the way into
+//               shared memory, the scale is applied to the result
+//   LIN_SWIGLU  LIN_NORM, and Y = silu(g) * u for matrices 0 (gate) and 1 (up)
+//   LIN_RES     x = X; Y += res
+enum { LIN_GATHER = 0, LIN_NORM = 1, LIN_SWIGLU = 2, LIN_RES = 3 };
+template <typename WT>
+struct LinArgs {
+  const float* X; int ldx;
+  const WT* W[3]; int n[3]; float* Y[3]; int ldy[3];
+  const WT* bias;
+  const WT* gain; float eps;
+  const float* res; int ldr;
+  int M, K, vec;      // vec: embedding, feature and gain rows are 16-byte aligned
+};
+// What only the gathering kind reads: the other kinds' parameters stay small (a kernel that runs for
+// 2 us feels the fetch of 2 KB of them).
+template <typename WT>
+struct GatherArgs { GatherSrc<WT> g; SeqMap sm; };
+struct NoGather {};
+// Sums of MC values over the warp, halving the values a lane carries at each step: lane l ends with
+// the sum of value l / (32 / MC).
+template <int MC>
+__device__ __forceinline__ float warp_sum_many(float (&v)[MC], int lane) {
 #pragma unroll
-  for (int i = 0; i < MC; ++i) acc[i] = 0.f;
-  const WT* wrow = W + (size_t)n * K;
-  for (int k = lane * 8; k < K; k += 256) {
-    float w[8];
-    load8(wrow + k, w);
+  for (int n = MC, o = 16; n > 1; n >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
 #pragma unroll
-    for (int i = 0; i < MC; ++i) {
-      if (m0 + i < M) {
-        const float4* xp = reinterpret_cast<const float4*>(X + (size_t)(m0 + i) * ldx + k);
-        float4 a = xp[0], c = xp[1];
-        acc[i] += w[0] * a.x + w[1] * a.y + w[2] * a.z + w[3] * a.w + w[4] * c.x + w[5] * c.y +
-                  w[6] * c.z + w[7] * c.w;
-      }
+    for (int i = 0; i < n / 2; ++i) {
+      const float keep = up ? v[i + n / 2] : v[i], give = up ? v[i] : v[i + n / 2];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
     }
   }
+  float t = v[0];
+#pragma unroll
+  for (int o = 16 / MC; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+// 4 consecutive values as floats; p is 8-byte (bf16) / 16-byte (fp32) aligned.
+__device__ __forceinline__ float4 load4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+  const uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
+  return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16),
+                     __uint_as_float(r.y & 0xffff0000u));
+}
+template <typename WT>
+__device__ __forceinline__ float4 load4_any(const WT* p, bool vec) {
+  return vec ? load4(p) : make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3]));
+}
+constexpr int kKC = 512;
+template <typename WT, int KIND, int MC, typename GA>
+__global__ void __launch_bounds__(256) k_linear(const __grid_constant__ LinArgs<WT> a, const __grid_constant__ GA ga) {
+  pdl_launch_dependents();
+  constexpr bool kNorm = KIND == LIN_NORM || KIND == LIN_SWIGLU, kTwo = KIND == LIN_SWIGLU;
+  constexpr int C = kKC / 128;                    // float4 groups of a warp per chunk
+  constexpr int NL = MC * (kKC / 4) / 256;        // vectors a thread brings in per chunk: rows 2 j + (tid >> 7)
+  static_assert(MC % 2 == 0 && kKC == 512, "a row of a chunk is half a block's vectors");
+  __shared__ __align__(16) float xs[MC][kKC];
+  __shared__ float s_sq[8][NL];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  int n = blockIdx.x * 8 + warp, mat = 0;
+  if (!kTwo) {
+    while (mat < 2 && n >= a.n[mat]) { n -= a.n[mat]; ++mat; }
+  }
+  const bool active = n < a.n[mat];
+  const int m0 = blockIdx.y * MC, K = a.K;
+  const bool vec = a.vec != 0;
+  const WT* w0 = active ? a.W[mat] + (size_t)n * K : a.W[0];   // (a warp without a feature follows feature 0)
+  const WT* w1 = kTwo ? (active ? a.W[1] + (size_t)n * K : a.W[1]) : nullptr;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  float acc[MC], acc2[kTwo ? MC : 1], sq[NL];
 #pragma unroll
   for (int i = 0; i < MC; ++i) {
-    float v = warp_sum(acc[i]);
-    if (lane == 0 && m0 + i < M) {
-      if (bias) v += to_f32(bias[n]);
-      if (res) v += res[(size_t)(m0 + i) * ldr + n];
-      Y[(size_t)(m0 + i) * ldy + n] = v;
-    }
+    acc[i] = 0.f;
+    if (kTwo) acc2[i] = 0.f;
   }
-}
-
-// y = x * g / sqrt(mean(x^2) + eps), one block per row.
-template <typename WT>
-__global__ void k_rmsnorm(const float* x, const WT* g, int H, float eps, float* y) {
-  __shared__ float red[32];
-  const float* xr = x + (size_t)blockIdx.x * H;
-  float ss = 0.f;
-  for (int i = threadIdx.x; i < H; i += blockDim.x) ss += xr[i] * xr[i];
-  ss = warp_sum(ss);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    float v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
-    v = warp_sum(v);
-    if (threadIdx.x == 0) red[0] = rsqrtf(v / (float)H + eps);
-  }
-  __syncthreads();
-  float inv = red[0];
-  float* yr = y + (size_t)blockIdx.x * H;
-  for (int i = threadIdx.x; i < H; i += blockDim.x) yr[i] = xr[i] * inv * to_f32(g[i]);
-}
-
-// RoPE on q (in place) and on k; k and v are written to the cache slab at the row's absolute
-// position.  One block per row.  kv_tmp row = [k (Hkv) ; v (Hkv)] fp32.  The pair
-// (i, i + d/2) of a head is rotated by pos * base^(-2i/d); angles are formed in double.
-// With `side` != nullptr the new k / v rows go to side[m][2 * Hkv] (k then v) instead of the
-// cache: a draft step leaves the cache untouched, and several groups may share one slot.
-template <typename WT>
-__global__ void k_rope_store(SeqMap sm, float* q, const float* kv_tmp, WT* kcache, WT* vcache, WT* side,
-                             int n_heads, int n_kv_heads, int d, int max_ctx, float rope_base) {
-  extern __shared__ float cs[];  // cos[d/2], sin[d/2]
-  int m = blockIdx.x;
-  int b, j;
-  seq_of_row(sm, m, b, j);
-  int pos = sm.len[b] + j;
-  int half = d >> 1;
-  for (int i = threadIdx.x; i < half; i += blockDim.x) {
-    double inv = exp2(-2.0 * (double)i / (double)d * log2((double)rope_base));
-    double s, c;
-    sincos((double)pos * inv, &s, &c);
-    cs[i] = (float)c;
-    cs[half + i] = (float)s;
-  }
-  __syncthreads();
-  int Hq = n_heads * d, Hkv = n_kv_heads * d;
-  if (q) {
-    float* qr = q + (size_t)m * Hq;
-    for (int t = threadIdx.x; t < n_heads * half; t += blockDim.x) {
-      int h = t / half, i = t - h * half;
-      float x = qr[h * d + i], y = qr[h * d + i + half];
-      qr[h * d + i] = x * cs[i] - y * cs[half + i];
-      qr[h * d + i + half] = y * cs[i] + x * cs[half + i];
-    }
-  }
-  const float* kr = kv_tmp + (size_t)m * 2 * Hkv;
-  const float* vr = kr + Hkv;
-  size_t slab = (size_t)sm.slot[b] * n_kv_heads;
-  for (int t = threadIdx.x; t < n_kv_heads * half; t += blockDim.x) {
-    int h = t / half, i = t - h * half;
-    float x = kr[h * d + i], y = kr[h * d + i + half];
-    WT *kd, *vd;
-    if (side) {
-      kd = side + (size_t)m * 2 * Hkv + h * d;
-      vd = kd + Hkv;
-    } else {
-      const size_t base = ((slab + h) * max_ctx + pos) * d;
-      kd = kcache + base;
-      vd = vcache + base;
-    }
-    store_as(kd + i, x * cs[i] - y * cs[half + i]);
-    store_as(kd + i + half, y * cs[i] + x * cs[half + i]);
-    store_as(vd + i, vr[h * d + i]);
-    store_as(vd + i + half, vr[h * d + i + half]);
-  }
-}
-
-// Attention under the parallel-draft mask: row j of a sequence sees cache rows [0, len) and
-// the new rows 0..j, which sit in side[m][2 * Hkv] (k then v).  One block (4 warps) per (head, b);
-// warps take keys round-robin, each lane owns D/32 channels; online softmax per (warp, row).
-template <typename WT, int D>
-__global__ void __launch_bounds__(128) k_attention(SeqMap sm, const float* q, const WT* kcache,
-                                                   const WT* vcache, const WT* side, int n_heads,
-                                                   int n_kv_heads, int max_ctx, float* attn) {
-  constexpr int C = D / 32;
-  constexpr int RMAX = kMaxRowsPerSeq;
-  __shared__ float s_m[4][RMAX], s_l[4][RMAX];
-  __shared__ float s_o[4][RMAX][D];
-  int h = blockIdx.x, b = blockIdx.y;
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int R = sm.row_off[b + 1] - sm.row_off[b];
-  int L = sm.len[b];
-  int m0 = sm.row_off[b] - sm.row_base;
-  int hk = h / (n_heads / n_kv_heads);
-  int Hq = n_heads * D;
-  const float scale = rsqrtf((float)D);
-  float qv[RMAX][C];
 #pragma unroll
-  for (int j = 0; j < RMAX; ++j)
-#pragma unroll
-    for (int c = 0; c < C; ++c)
-      qv[j][c] = (j < R) ? q[(size_t)(m0 + j) * Hq + h * D + lane + 32 * c] * scale : 0.f;
-  float mx[RMAX], l[RMAX], o[RMAX][C];
-#pragma unroll
-  for (int j = 0; j < RMAX; ++j) {
-    mx[j] = -FLT_MAX; l[j] = 0.f;
-#pragma unroll
-    for (int c = 0; c < C; ++c) o[j][c] = 0.f;
-  }
-  const WT* kb = kcache + ((size_t)sm.slot[b] * n_kv_heads + hk) * max_ctx * D;
-  const WT* vb = vcache + ((size_t)sm.slot[b] * n_kv_heads + hk) * max_ctx * D;
-  for (int t = warp; t < L + R; t += 4) {
-    float kx[C], vx[C];
-#pragma unroll
-    const WT* kr = t < L ? kb + (size_t)t * D : side + (size_t)(m0 + t - L) * 2 * n_kv_heads * D + hk * D;
-    const WT* vr = t < L ? vb + (size_t)t * D : kr + n_kv_heads * D;
+  for (int j = 0; j < NL; ++j) sq[j] = 0.f;
+  // the thread's place in the rows it brings in (rows past the end repeat the last one)
+  const int col = (tid & 127) * 4;
+  const float* xr[NL];
+  const WT *xe[NL], *xf[NL];
+  for (int k0 = 0; k0 < K; k0 += kKC) {
+    float4 wv[C], uv[kTwo ? C : 1];
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-      kx[c] = to_f32(kr[lane + 32 * c]);
-      vx[c] = to_f32(vr[lane + 32 * c]);
+      const int k = k0 + c * 128 + lane * 4;
+      wv[c] = k < K ? load4(w0 + k) : zero;
+      if (kTwo) uv[c] = k < K ? load4(w1 + k) : zero;
     }
-    int jmin = t < L ? 0 : t - L;  // rows that may see key t
+    float4 g = zero;
+    if (kNorm && k0 + col < K) g = load4_any(a.gain + k0 + col, vec);
+    if (k0 == 0) {
+      pdl_wait();
 #pragma unroll
-    for (int j = 0; j < RMAX; ++j) {
-      if (j >= jmin && j < R) {
-        float s = 0.f;
+      for (int j = 0; j < NL; ++j) {
+        const int m = min(m0 + 2 * j + (tid >> 7), a.M - 1);
+        if constexpr (KIND == LIN_GATHER) gather_row(ga.g, ga.sm, m, xe[j], xf[j]);
+        else xr[j] = a.X + (size_t)m * a.ldx;
+      }
+    } else {
+      __syncthreads();   // the chunk before has been consumed
+    }
+    float4 x[NL];
+    const int k = k0 + col;
 #pragma unroll
-        for (int c = 0; c < C; ++c) s += qv[j][c] * kx[c];
-        s = warp_sum(s);
-        float mnew = fmaxf(mx[j], s);
-        float corr = __expf(mx[j] - mnew), p = __expf(s - mnew);
-        l[j] = l[j] * corr + p;
+    for (int j = 0; j < NL; ++j) {
+      x[j] = zero;
+      if (k < K) {
+        if constexpr (KIND == LIN_GATHER) x[j] = load4_any(k < ga.g.H ? xe[j] + k : xf[j] + (k - ga.g.H), vec);   // (H is a multiple of 8)
+        else x[j] = __ldcg(reinterpret_cast<const float4*>(xr[j] + k));
+      }
+    }
 #pragma unroll
-        for (int c = 0; c < C; ++c) o[j][c] = o[j][c] * corr + p * vx[c];
-        mx[j] = mnew;
+    for (int j = 0; j < NL; ++j) {
+      if (kNorm) {
+        sq[j] += (x[j].x * x[j].x + x[j].y * x[j].y) + (x[j].z * x[j].z + x[j].w * x[j].w);
+        x[j].x *= g.x; x[j].y *= g.y; x[j].z *= g.z; x[j].w *= g.w;
+      }
+      *reinterpret_cast<float4*>(&xs[2 * j + (tid >> 7)][col]) = x[j];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+#pragma unroll
+      for (int i = 0; i < MC; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(&xs[i][c * 128 + lane * 4]);
+        acc[i] += (wv[c].x * v.x + wv[c].y * v.y) + (wv[c].z * v.z + wv[c].w * v.w);
+        if (kTwo) acc2[i] += (uv[c].x * v.x + uv[c].y * v.y) + (uv[c].z * v.z + uv[c].w * v.w);
       }
     }
   }
+  if (kNorm) {
 #pragma unroll
-  for (int j = 0; j < RMAX; ++j) {
-    if (lane == 0) { s_m[warp][j] = mx[j]; s_l[warp][j] = l[j]; }
-#pragma unroll
-    for (int c = 0; c < C; ++c) s_o[warp][j][lane + 32 * c] = o[j][c];
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < R * D; idx += blockDim.x) {
-    int j = idx / D, i = idx - j * D;
-    float M = fmaxf(fmaxf(s_m[0][j], s_m[1][j]), fmaxf(s_m[2][j], s_m[3][j]));
-    float num = 0.f, den = 0.f;
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      float f = __expf(s_m[w][j] - M);
-      num += f * s_o[w][j][i];
-      den += f * s_l[w][j];
+    for (int j = 0; j < NL; ++j) {
+      const float t = warp_sum(sq[j]);
+      if (lane == 0) s_sq[warp][j] = t;
     }
-    attn[(size_t)(m0 + j) * Hq + h * D + i] = num / den;
+    __syncthreads();
+  }
+  const float t = warp_sum_many<MC>(acc, lane);
+  float t2 = 0.f;
+  if constexpr (kTwo) t2 = warp_sum_many<MC>(acc2, lane);
+  const int i = lane / (32 / MC), m = m0 + i;
+  if (active && lane % (32 / MC) == 0 && m < a.M) {
+    float v = t;
+    if (KIND == LIN_GATHER && a.bias) v += to_f32(a.bias[n]);
+    if (kNorm) {
+      const int w = (i & 1) * 4, j = i >> 1;   // the four warps that brought row i in
+      const float sc = rsqrtf(((s_sq[w][j] + s_sq[w + 1][j]) + (s_sq[w + 2][j] + s_sq[w + 3][j])) / (float)K + a.eps);
+      v *= sc;
+      if (kTwo) v = v / (1.f + __expf(-v)) * (t2 * sc);
+    }
+    if (KIND == LIN_RES) v += __ldcg(a.res + (size_t)m * a.ldr + n);
+    a.Y[mat][(size_t)m * a.ldy[mat] + n] = v;
   }
 }
 
-__global__ void k_silu_mul(const float* gate, const float* up, float* out, size_t n) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) {
-    float g = gate[i];
-    out[i] = g / (1.f + __expf(-g)) * up[i];
+// RoPE on the k half of appended rows and the store of k and v into the cache slab at the row's
+// absolute position.  One block per row.  kv row = [k (Hkv) ; v (Hkv)] fp32.  The pair (i, i + d/2)
+// of a head is rotated by pos * base^(-2i/d); angles are formed in double.
+template <typename WT>
+__global__ void __launch_bounds__(128) k_rope_store(const __grid_constant__ SeqMap sm, const float* __restrict__ kv, WT* kcache,
+                                                    WT* vcache, int n_kv_heads, int d, int max_ctx,
+                                                    const double* __restrict__ inv_freq) {
+  __shared__ float cs[64], sn[64];
+  const int m = blockIdx.x, half = d >> 1;
+  int b, j;
+  seq_of_row(sm, m, b, j);
+  const int pos = sm.len[b] + j;
+  if ((int)threadIdx.x < half) {
+    double s, c;
+    sincos((double)pos * inv_freq[threadIdx.x], &s, &c);
+    cs[threadIdx.x] = (float)c;
+    sn[threadIdx.x] = (float)s;
+  }
+  __syncthreads();
+  pdl_wait();   // (and no early launch of dependents: see k_kv_store)
+  const int Hkv = n_kv_heads * d;
+  const float* kr = kv + (size_t)m * 2 * Hkv;
+  const float* vr = kr + Hkv;
+  const size_t slab = (size_t)sm.slot[b] * n_kv_heads;
+  for (int t = threadIdx.x; t < n_kv_heads * half; t += blockDim.x) {
+    const int h = t / half, i = t - h * half;
+    const float x = kr[h * d + i], y = kr[h * d + i + half];
+    const size_t at = ((slab + h) * max_ctx + pos) * d + i;
+    store_as(kcache + at, x * cs[i] - y * sn[i]);
+    store_as(kcache + at + half, y * cs[i] + x * sn[i]);
+    store_as(vcache + at, vr[h * d + i]);
+    store_as(vcache + at + half, vr[h * d + i + half]);
+  }
+}
+
+// Attention under the parallel-draft mask: row j of a sequence sees cache rows [0, len) and the new
+// rows 0..j, which come from q / kv before RoPE.  One block per (head, sequence).  A tile of 256 keys
+// at a time: a thread holds the scores of one key against all rows, then 256 / D groups of threads
+// walk the keys, a thread per channel; running maximum and sums between tiles.
+constexpr int kAttThreads = 256;
+template <typename WT, int D>
+__global__ void __launch_bounds__(kAttThreads) k_attention(const __grid_constant__ SeqMap sm, const float* __restrict__ q,
+                                                           const float* __restrict__ kv, const WT* __restrict__ kcache,
+                                                           const WT* __restrict__ vcache, int n_heads, int n_kv_heads,
+                                                           int max_ctx, const double* __restrict__ inv_freq, float* attn) {
+  constexpr int RMAX = kMaxRowsPerSeq, HALF = D / 2, GROUPS = kAttThreads / D, WARPS = kAttThreads / 32;
+  __shared__ __align__(16) float s_q[RMAX][D], s_k[RMAX][D], s_v[RMAX][D];   // rotated q (scaled), the new rows
+  __shared__ float s_p[RMAX][kAttThreads];
+  __shared__ float s_red[WARPS][RMAX];
+  const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int R = sm.row_off[b + 1] - sm.row_off[b], L = sm.len[b], m0 = sm.row_off[b] - sm.row_base;
+  const int hk = h / (n_heads / n_kv_heads), Hq = n_heads * D, Hkv = n_kv_heads * D;
+  const WT* kb = kcache + ((size_t)sm.slot[b] * n_kv_heads + hk) * max_ctx * D;
+  const WT* vb = vcache + ((size_t)sm.slot[b] * n_kv_heads + hk) * max_ctx * D;
+  pdl_launch_dependents();
+  // rotation table, parked in the score tile: cos then sin of (row, pair)
+  float* cs = &s_p[0][0];
+  float* sn = cs + RMAX * HALF;
+  static_assert(2 * RMAX * HALF <= RMAX * kAttThreads, "the table fits the score tile");
+  for (int i = tid; i < R * HALF; i += kAttThreads) {
+    double s, c;
+    sincos((double)(L + i / HALF) * inv_freq[i % HALF], &s, &c);
+    cs[i] = (float)c;
+    sn[i] = (float)s;
+  }
+  __syncthreads();
+  pdl_wait();
+  const float scale = rsqrtf((float)D);
+  for (int i = tid; i < R * HALF; i += kAttThreads) {
+    const int j = i / HALF, e = i - j * HALF;
+    const float* qr = q + (size_t)(m0 + j) * Hq + h * D + e;
+    const float* kr = kv + (size_t)(m0 + j) * 2 * Hkv + hk * D + e;
+    const float q0 = __ldcg(qr), q1 = __ldcg(qr + HALF), k0 = __ldcg(kr), k1 = __ldcg(kr + HALF), v0 = __ldcg(kr + Hkv),
+                v1 = __ldcg(kr + Hkv + HALF), c = cs[i], s = sn[i];
+    s_q[j][e] = (q0 * c - q1 * s) * scale;
+    s_q[j][e + HALF] = (q1 * c + q0 * s) * scale;
+    s_k[j][e] = rounded<WT>(k0 * c - k1 * s);
+    s_k[j][e + HALF] = rounded<WT>(k1 * c + k0 * s);
+    s_v[j][e] = rounded<WT>(v0);
+    s_v[j][e + HALF] = rounded<WT>(v1);
+  }
+  __syncthreads();
+  float m[RMAX], l[RMAX], o[RMAX];
+#pragma unroll
+  for (int j = 0; j < RMAX; ++j) { m[j] = -FLT_MAX; l[j] = 0.f; o[j] = 0.f; }
+  const int d = tid % D, grp = tid / D, total = L + R;
+  for (int t0 = 0; t0 < total; t0 += kAttThreads) {
+    const int t = t0 + tid, nk = min(kAttThreads, total - t0);
+    float s[RMAX];
+#pragma unroll
+    for (int j = 0; j < RMAX; ++j) s[j] = 0.f;
+    if (t < total) {
+      for (int c = 0; c < D; c += 8) {
+        float k8[8];
+        if (t < L) {
+          load8(kb + (size_t)t * D + c, k8);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) k8[e] = s_k[t - L][c + e];
+        }
+#pragma unroll
+        for (int j = 0; j < RMAX; ++j) {
+          if (j < R) {   // (uniform)
+            const float4 a = *reinterpret_cast<const float4*>(&s_q[j][c]), a2 = *reinterpret_cast<const float4*>(&s_q[j][c + 4]);
+            s[j] += (k8[0] * a.x + k8[1] * a.y + k8[2] * a.z + k8[3] * a.w) + (k8[4] * a2.x + k8[5] * a2.y + k8[6] * a2.z + k8[7] * a2.w);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < RMAX; ++j) {
+      if (j < R) {
+        if (t >= total || t - L > j) s[j] = -FLT_MAX;   // a new key is seen by its own row and the later ones
+        float mx = s[j];
+#pragma unroll
+        for (int x = 16; x > 0; x >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, x));
+        if (lane == 0) s_red[warp][j] = mx;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < RMAX; ++j) {
+      if (j < R) {
+        float mx = m[j];
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) mx = fmaxf(mx, s_red[w][j]);
+        const float f = __expf(m[j] - mx), p = s[j] > -FLT_MAX ? __expf(s[j] - mx) : 0.f;
+        l[j] = l[j] * f + p;      // (this thread's share of the row's sum)
+        o[j] *= f;
+        m[j] = mx;
+        s_p[j][tid] = p;
+      }
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int kk = grp; kk < nk; kk += GROUPS) {
+      const int tk = t0 + kk;
+      const float v = tk < L ? to_f32(vb[(size_t)tk * D + d]) : s_v[tk - L][d];
+#pragma unroll
+      for (int j = 0; j < RMAX; ++j)
+        if (j < R) o[j] += s_p[j][kk] * v;
+    }
+    __syncthreads();
+  }
+  // the rows' sums over all threads, the groups' partial outputs
+#pragma unroll
+  for (int j = 0; j < RMAX; ++j) {
+    if (j < R) {
+      const float t = warp_sum(l[j]);
+      if (lane == 0) s_red[warp][j] = t;
+      s_p[j][tid] = o[j];
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < R * D; i += kAttThreads) {
+    const int j = i / D, e = i - j * D;
+    float num = 0.f, den = 0.f;
+#pragma unroll
+    for (int g = 0; g < GROUPS; ++g) num += s_p[j][g * D + e];
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) den += s_red[w][j];
+    attn[(size_t)(m0 + j) * Hq + h * D + e] = num / den;
   }
 }
 
@@ -342,53 +479,71 @@ __global__ void __launch_bounds__(256) k_kv_copy(T* __restrict__ kcache, T* __re
   }
 }
 
-template <typename WT>
-ps_status linear(ps_ctx* c, const float* X, int ldx, const void* W, const void* bias,
-                 const float* res, int ldr, float* Y, int ldy, int M, int N, int K,
-                 cudaStream_t st) {
-  constexpr int MC = 8;
-  dim3 grid((N + 7) / 8, (M + MC - 1) / MC);
-  k_linear<WT, MC><<<grid, 256, 0, st>>>(X, ldx, (const WT*)W, (const WT*)bias, res, ldr, Y, ldy,
-                                         M, N, K);
+// One product: rows [0, a.M) of the stage's kind.
+template <typename WT, int KIND, typename GA = NoGather>
+ps_status linear(ps_ctx* c, const LinArgs<WT>& a, cudaStream_t st, const GA& ga = GA()) {
+  const int N = KIND == LIN_SWIGLU ? a.n[0] : a.n[0] + a.n[1] + a.n[2];
+  cudaError_t e;
+  if (a.M <= 4)
+    e = launch_after(k_linear<WT, KIND, 4, GA>, dim3((N + 7) / 8, 1), dim3(256), 0, st, !c->prof, a, ga);
+  else
+    e = launch_after(k_linear<WT, KIND, 8, GA>, dim3((N + 7) / 8, (a.M + 7) / 8), dim3(256), 0, st, !c->prof, a, ga);
   c->launches++;
-  return cuda_check(c, cudaGetLastError(), "k_linear");
+  return cuda_check(c, e, "k_linear");
 }
 
 template <typename WT>
-ps_status fc_norm_kv(ps_ctx* c, const SeqMap& sm, int rows, int all_real, const void* hidden,
-                     const int* tokens, bool with_q, cudaStream_t st) {
+bool rows_aligned(const ps_ctx* c, const void* hidden) {
+  const ps_weights& w = c->w;
+  return (((uintptr_t)w.embed | (uintptr_t)w.mask_embed | (uintptr_t)w.mask_feat | (uintptr_t)hidden | (uintptr_t)w.g_in |
+           (uintptr_t)w.g_post | (uintptr_t)w.g_final) & 15) == 0;
+}
+
+// x0 of `rows` rows, then their k | v (and q) projections of the normalised rows.
+template <typename WT>
+ps_status fc_qkv(ps_ctx* c, const SeqMap& sm, int rows, int all_real, const void* hidden, const int* tokens, bool with_q,
+                 cudaStream_t st) {
   const ps_config& g = c->cfg;
   const ps_weights& w = c->w;
-  int H = g.hidden, Hq = g.n_heads * g.head_dim, Hkv = g.n_kv_heads * g.head_dim;
-  prof_mark(c, st, "begin");
-  k_gather<WT><<<rows, 256, 0, st>>>(sm, all_real, (const WT*)w.embed, (const WT*)w.mask_embed,
-                                     (const WT*)w.mask_feat,
-                                     (g.flags & PS_FLAG_NO_FC) ? nullptr : (const WT*)hidden, tokens, H, g.vocab,
-                                     c->x_in);
-  c->launches++;
+  const int H = g.hidden, Hq = g.n_heads * g.head_dim, Hkv = g.n_kv_heads * g.head_dim;
+  const bool no_fc = (g.flags & PS_FLAG_NO_FC) != 0;
+  typedef const WT* P;
   ps_status s;
-  const void* bias = (g.flags & PS_FLAG_FC_BIAS) ? w.b_fc : nullptr;
-  if (g.flags & PS_FLAG_NO_FC) {   // x0 = the embedding half of x_in
-    cudaError_t e = cudaMemcpy2DAsync(c->x0, (size_t)H * 4, c->x_in, (size_t)2 * H * 4, (size_t)H * 4, rows,
-                                      cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return cuda_check(c, e, "x0 copy");
-  } else if ((s = linear<WT>(c, c->x_in, 2 * H, w.w_fc, bias, nullptr, 0, c->x0, H, rows, H, 2 * H, st))) {
-    return s;
+  prof_mark(c, st, "begin");
+  LinArgs<WT> a{};
+  a.M = rows; a.vec = rows_aligned<WT>(c, hidden); a.eps = g.rms_eps;
+  const GatherSrc<WT> src{(P)w.embed, (P)w.mask_embed, (P)w.mask_feat, no_fc ? nullptr : (P)hidden, tokens, all_real, H, g.vocab};
+  if (no_fc) {
+    const cudaError_t e = launch_after(k_gather_embed<WT>, dim3(rows), dim3(256), 0, st, !c->prof, sm, src, c->x0);
+    c->launches++;
+    if (e != cudaSuccess) return cuda_check(c, e, "k_gather_embed");
+  } else {
+    LinArgs<WT> f = a;
+    f.W[0] = (P)w.w_fc; f.n[0] = H; f.Y[0] = c->x0; f.ldy[0] = H; f.K = 2 * H;
+    f.bias = (g.flags & PS_FLAG_FC_BIAS) ? (P)w.b_fc : nullptr;
+    if ((s = linear<WT, LIN_GATHER>(c, f, st, GatherArgs<WT>{src, sm}))) return s;
   }
-  k_rmsnorm<WT><<<rows, 256, 0, st>>>(c->x0, (const WT*)w.g_in, H, g.rms_eps, c->xn);
-  c->launches++;
   prof_mark(c, st, "fc_norm");
-  if (with_q)
-    if ((s = linear<WT>(c, c->xn, H, w.w_q, nullptr, nullptr, 0, c->q, Hq, rows, Hq, H, st))) return s;
-  if ((s = linear<WT>(c, c->xn, H, w.w_k, nullptr, nullptr, 0, c->kv_tmp, 2 * Hkv, rows, Hkv, H, st))) return s;
-  if ((s = linear<WT>(c, c->xn, H, w.w_v, nullptr, nullptr, 0, c->kv_tmp + Hkv, 2 * Hkv, rows, Hkv, H, st))) return s;
-  k_rope_store<WT><<<rows, 128, g.head_dim * sizeof(float), st>>>(
-      sm, with_q ? c->q : nullptr, c->kv_tmp, (WT*)c->kcache, (WT*)c->vcache,
-      with_q ? (WT*)c->kv_side : nullptr,   // a draft step keeps its new rows out of the cache
-      g.n_heads, g.n_kv_heads, g.head_dim, g.max_ctx, g.rope_base);
+  a.X = c->x0; a.ldx = H; a.K = H; a.gain = (P)w.g_in;
+  int i = 0;
+  if (with_q) { a.W[i] = (P)w.w_q; a.n[i] = Hq; a.Y[i] = c->q; a.ldy[i++] = Hq; }
+  a.W[i] = (P)w.w_k; a.n[i] = Hkv; a.Y[i] = c->kv_tmp; a.ldy[i++] = 2 * Hkv;
+  a.W[i] = (P)w.w_v; a.n[i] = Hkv; a.Y[i] = c->kv_tmp + Hkv; a.ldy[i++] = 2 * Hkv;
+  if ((s = linear<WT, LIN_NORM>(c, a, st))) return s;
+  prof_mark(c, st, "qkv_rope");
+  return PS_OK;
+}
+
+template <typename WT>
+ps_status kv_append_impl(ps_ctx* c, const SeqMap& sm, int rows, const void* hidden, const int* tokens, cudaStream_t st) {
+  const ps_config& g = c->cfg;
+  const ps_status s = fc_qkv<WT>(c, sm, rows, 1, hidden, tokens, false, st);
+  if (s) return s;
+  const cudaError_t e = launch_after(k_rope_store<WT>, dim3(rows), dim3(128), 0, st, !c->prof, sm, c->kv_tmp, (WT*)c->kcache,
+                                     (WT*)c->vcache, g.n_kv_heads, g.head_dim, g.max_ctx, (const double*)c->rope_inv_freq);
   c->launches++;
   prof_mark(c, st, "qkv_rope");
-  return cuda_check(c, cudaGetLastError(), "fc_norm_kv");
+  return cuda_check(c, e, "k_rope_store");
 }
 
 template <typename WT>
@@ -398,48 +553,54 @@ ps_status draft_impl(ps_ctx* c, const SeqMap& sm, int B, const void* hidden_last
                      const SampleArgs* sa, cudaStream_t st) {
   const ps_config& g = c->cfg;
   const ps_weights& w = c->w;
-  int H = g.hidden, Hq = g.n_heads * g.head_dim, F = g.ffn, V = g.vocab;
-  int M = B * (g.k_masks + 1);
+  const int H = g.hidden, Hq = g.n_heads * g.head_dim, F = g.ffn, V = g.vocab, M = B * (g.k_masks + 1);
+  typedef const WT* P;
   ps_status s;
-  if ((s = fc_norm_kv<WT>(c, sm, M, 0, hidden_last, token_last, true, st))) return s;
-  dim3 ag(g.n_heads, B);
-  if (g.head_dim == 64)
-    k_attention<WT, 64><<<ag, 128, 0, st>>>(sm, c->q, (const WT*)c->kcache, (const WT*)c->vcache,
-                                            (const WT*)c->kv_side, g.n_heads, g.n_kv_heads, g.max_ctx, c->attn);
-  else
-    k_attention<WT, 128><<<ag, 128, 0, st>>>(sm, c->q, (const WT*)c->kcache, (const WT*)c->vcache,
-                                             (const WT*)c->kv_side, g.n_heads, g.n_kv_heads, g.max_ctx, c->attn);
+  if ((s = fc_qkv<WT>(c, sm, M, 0, hidden_last, token_last, true, st))) return s;
+  auto attn = g.head_dim == 64 ? k_attention<WT, 64> : k_attention<WT, 128>;
+  const cudaError_t e = launch_after(attn, dim3(g.n_heads, B), dim3(kAttThreads), 0, st, !c->prof, sm, c->q, c->kv_tmp,
+                                     (P)c->kcache, (P)c->vcache, g.n_heads, g.n_kv_heads, g.max_ctx,
+                                     (const double*)c->rope_inv_freq, c->attn);
   c->launches++;
+  if (e != cudaSuccess) return cuda_check(c, e, "k_attention");
   prof_mark(c, st, "attention");
-  if ((s = linear<WT>(c, c->attn, Hq, w.w_o, nullptr, c->x0, H, c->a, H, M, H, Hq, st))) return s;
+  LinArgs<WT> a{};
+  a.M = M; a.vec = rows_aligned<WT>(c, hidden_last); a.eps = g.rms_eps;
+  {
+    LinArgs<WT> x = a;
+    x.X = c->attn; x.ldx = Hq; x.K = Hq; x.W[0] = (P)w.w_o; x.n[0] = H; x.Y[0] = c->a; x.ldy[0] = H; x.res = c->x0; x.ldr = H;
+    if ((s = linear<WT, LIN_RES>(c, x, st))) return s;
+  }
   prof_mark(c, st, "o_proj");
-  k_rmsnorm<WT><<<M, 256, 0, st>>>(c->a, (const WT*)w.g_post, H, g.rms_eps, c->an);
-  c->launches++;
-  if ((s = linear<WT>(c, c->an, H, w.w_gate, nullptr, nullptr, 0, c->gate, F, M, F, H, st))) return s;
-  if ((s = linear<WT>(c, c->an, H, w.w_up, nullptr, nullptr, 0, c->up, F, M, F, H, st))) return s;
-  size_t n = (size_t)M * F;
-  k_silu_mul<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(c->gate, c->up, c->gate, n);
-  c->launches++;
   float* hdn = feat_out ? feat_out : c->hdn;
-  if ((s = linear<WT>(c, c->gate, F, w.w_down, nullptr, c->a, H, hdn, H, M, H, F, st))) return s;
+  {
+    LinArgs<WT> x = a;
+    x.X = c->a; x.ldx = H; x.K = H; x.gain = (P)w.g_post;
+    x.W[0] = (P)w.w_gate; x.W[1] = (P)w.w_up; x.n[0] = F; x.Y[0] = c->gate; x.ldy[0] = F;
+    if ((s = linear<WT, LIN_SWIGLU>(c, x, st))) return s;
+    x = a;
+    x.X = c->gate; x.ldx = F; x.K = F; x.W[0] = (P)w.w_down; x.n[0] = H; x.Y[0] = hdn; x.ldy[0] = H; x.res = c->a; x.ldr = H;
+    if ((s = linear<WT, LIN_RES>(c, x, st))) return s;
+  }
   prof_mark(c, st, "ffn");
-  k_rmsnorm<WT><<<M, 256, 0, st>>>(hdn, (const WT*)w.g_final, H, g.rms_eps, c->hn);
-  c->launches++;
   float* logits = logits_out ? logits_out : c->logits;
-  if ((s = linear<WT>(c, c->hn, H, w.w_lm, nullptr, nullptr, 0, logits, V, M, V, H, st))) return s;
+  {
+    LinArgs<WT> x = a;
+    x.X = hdn; x.ldx = H; x.K = H; x.gain = (P)w.g_final; x.W[0] = (P)w.w_lm; x.n[0] = V; x.Y[0] = logits; x.ldy[0] = V;
+    if ((s = linear<WT, LIN_NORM>(c, x, st))) return s;
+  }
   if ((s = launch_logit_stats(c, logits, M, V, g.k_masks + 1, top_n, top_ids, top_logit, row_max, row_lse, sa, st)))
     return s;
   prof_mark(c, st, "lm_head");
-  return cuda_check(c, cudaGetLastError(), "draft_step");
+  return PS_OK;
 }
 
 }  // namespace
 
 ps_status plain_kv_append(ps_ctx* c, const SeqMap& sm, int rows, const void* hidden,
                           const int* tokens, cudaStream_t st) {
-  return c->cfg.dtype == PS_DTYPE_F32
-             ? fc_norm_kv<float>(c, sm, rows, 1, hidden, tokens, false, st)
-             : fc_norm_kv<__nv_bfloat16>(c, sm, rows, 1, hidden, tokens, false, st);
+  return c->cfg.dtype == PS_DTYPE_F32 ? kv_append_impl<float>(c, sm, rows, hidden, tokens, st)
+                                      : kv_append_impl<__nv_bfloat16>(c, sm, rows, hidden, tokens, st);
 }
 
 ps_status plain_draft_step(ps_ctx* c, const SeqMap& sm, int B, const void* hidden_last,

@@ -77,19 +77,13 @@ size_t carve(const ps_config& g, ps_ctx* c, char* base) {
   void* vrow = take(sizeof(VerifyRow) * PS_MAX_BATCH * (PS_MAX_MASKS + 2));
   void* vdraw = take(sizeof(VerifyDraw) * PS_MAX_BATCH);
   void* tstat = take(sizeof(RowStat) * PS_MAX_BATCH * (2 * PS_MAX_TREE_NODES + 1));
-  void* x_in = take(Mx * 2 * H * 4);
   void* x0 = take(Mx * H * 4);
-  void* xn = take(Mx * H * 4);
   void* q = take(Md * Hq * 4);
   void* kv_tmp = take(Mx * 2 * Hkv * 4);
-  void* kv_side = take(Md * 2 * Hkv * elem_bytes(g));
   void* attn = take(Md * Hq * 4);
   void* a = take(Md * H * 4);
-  void* an = take(Md * H * 4);
   void* gate = take(Md * F * 4);
-  void* up = take(Md * F * 4);
   void* hdn = take(Md * H * 4);
-  void* hn = take(Md * H * 4);
   void* logits = take(Md * V * 4);
   void* fused = take(fused_scratch_bytes(g));
   void* inv_freq = take(sizeof(double) * 64);
@@ -103,9 +97,9 @@ size_t carve(const ps_config& g, ps_ctx* c, char* base) {
     c->kcache = kc; c->vcache = vc; c->dev_status = (int*)status; c->tickets = (unsigned*)tickets;
     c->vrec = (VerifyRec*)vrec; c->vrow = (VerifyRow*)vrow; c->vdraw = (VerifyDraw*)vdraw;
     c->tree_stats = (RowStat*)tstat;
-    c->x_in = (float*)x_in; c->x0 = (float*)x0; c->xn = (float*)xn; c->q = (float*)q;
-    c->kv_tmp = (float*)kv_tmp; c->kv_side = kv_side; c->attn = (float*)attn; c->a = (float*)a; c->an = (float*)an;
-    c->gate = (float*)gate; c->up = (float*)up; c->hdn = (float*)hdn; c->hn = (float*)hn;
+    c->x0 = (float*)x0; c->q = (float*)q;
+    c->kv_tmp = (float*)kv_tmp; c->attn = (float*)attn; c->a = (float*)a;
+    c->gate = (float*)gate; c->hdn = (float*)hdn;
     c->logits = (float*)logits;
     c->fused_scratch = fused;
     c->rope_inv_freq = (double*)inv_freq;

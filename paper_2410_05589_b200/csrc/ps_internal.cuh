@@ -152,8 +152,7 @@ struct ps_ctx {
   ps::VerifyRow* vrow;      // [max_batch][PS_MAX_MASKS+2]
   ps::VerifyDraw* vdraw;    // [max_batch]
   ps::RowStat* tree_stats;  // [max_batch][2 PS_MAX_TREE_NODES + 1]
-  float *x_in, *x0, *xn, *q, *kv_tmp, *attn, *a, *an, *gate, *up, *hdn, *hn, *logits;
-  void* kv_side;            // [max_rows][2 * Hkv] storage dtype: k / v of a draft step's new rows (plain kernels)
+  float *x0, *q, *kv_tmp, *attn, *a, *gate, *hdn, *logits;
   // staging for ps_round_host
   void* fused_scratch;      // buffers of the fused bf16 path (see fused_kernels.cu)
   void* umma_maps = nullptr;   // tensor maps of the tensor-core GEMMs, built on first use
