@@ -270,9 +270,8 @@ __global__ void __launch_bounds__(256) k_attn_prep(const __grid_constant__ Work 
 
 template <int NR>
 __global__ void __launch_bounds__(kThreads, 1)
-k_attn_tc(const __grid_constant__ CUtensorMap t_k, const __grid_constant__ CUtensorMap t_v,
-          const __grid_constant__ CUtensorMap t_q, const __grid_constant__ CUtensorMap t_new, const __grid_constant__ Work w,
-          float* __restrict__ part_o, float2* __restrict__ part_ml, unsigned* tickets, __nv_bfloat16* __restrict__ out_hi,
+k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtensorMap t_q, const __grid_constant__ CUtensorMap t_new,
+          const __grid_constant__ Work w, float* __restrict__ part_o, float2* __restrict__ part_ml, unsigned* tickets, __nv_bfloat16* __restrict__ out_hi,
           __nv_bfloat16* __restrict__ out_lo, int* status) {
   constexpr int N = 2 * NR, NS = n_slots(NR), kOp = op_bytes(NR);
   extern __shared__ unsigned char smem_raw[];
@@ -336,7 +335,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap t_k, const __grid_constant__ CUten
         first.start(w, u0, u1);
         load_q(first.b, first.hk, 0);
       };
-      auto load = [&](const Walk& x, const CUtensorMap* cache, int v) {
+      auto load = [&](const Walk& x, int v) {
         if (n_issued >= NS || x.in_tail) need_dep();
         if (n_issued >= NS && !mbar_wait(&ctl.empty[slot], (use & 1) ^ 1, abort_flag)) { alive = false; return; }
         const uint32_t dst = base + slot * kSlotBytes;
@@ -347,12 +346,17 @@ k_attn_tc(const __grid_constant__ CUtensorMap t_k, const __grid_constant__ CUten
           tma_load_2d(dst, &t_new, 0, y, bar);
           tma_load_2d(dst + kSlotBytes / 2, &t_new, 64, y, bar);
         } else {
-          const int nb = (min(kTile, x.len - x.t * kTile) + kBoxRows - 1) / kBoxRows;
+          const int n = min(kTile, x.len - x.t * kTile), nb = (n + kBoxRows - 1) / kBoxRows;
           mbar_arrive_expect_tx(bar, nb * kBoxRows * kD * 2);
           const int y = (w.sm.slot[x.b] * w.n_kv + x.hk) * w.max_ctx + x.t * kTile;
-          for (int i = 0; i < nb; ++i) {
-            tma_load_2d(dst + i * kBoxRows * 128, cache, 0, y + i * kBoxRows, bar);
-            tma_load_2d(dst + kSlotBytes / 2 + i * kBoxRows * 128, cache, 64, y + i * kBoxRows, bar);
+          if (nb == kTile / kBoxRows) {   // a (nearly) full tile: one box per 64 channels
+            tma_load_2d(dst, &t_c.full[v], 0, y, bar);
+            tma_load_2d(dst + kSlotBytes / 2, &t_c.full[v], 64, y, bar);
+          } else {
+            for (int i = 0; i < nb; ++i) {
+              tma_load_2d(dst + i * kBoxRows * 128, &t_c.part[v], 0, y + i * kBoxRows, bar);
+              tma_load_2d(dst + kSlotBytes / 2 + i * kBoxRows * 128, &t_c.part[v], 64, y + i * kBoxRows, bar);
+            }
           }
         }
         ++n_issued;
@@ -364,13 +368,13 @@ k_attn_tc(const __grid_constant__ CUtensorMap t_k, const __grid_constant__ CUten
           if (!mbar_wait(&ctl.q_empty[wk.seg & 1], ((wk.seg >> 1) & 1) ^ 1, abort_flag)) { alive = false; return; }
           load_q(wk.b, wk.hk, wk.seg);
         }
-        load(wk, &t_k, 0);
+        load(wk, 0);
         wk.next(w);
       };
       if (wk.ok) load_k();
       while (alive && wv.ok) {
         if (wk.ok) load_k();
-        if (alive) { load(wv, &t_v, 1); wv.next(w); }
+        if (alive) { load(wv, 1); wv.next(w); }
       }
       if (alive && u0 < u1) need_dep();
     }
@@ -701,7 +705,7 @@ cudaError_t launch_nr(ps_ctx* c, const Work& w, int grid, const Buffers& b, cons
   auto kern = k_attn_tc<NR>;
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<NR>());
   if (e != cudaSuccess) return e;
-  return launch_after(kern, dim3(grid), dim3(kThreads), smem_bytes<NR>(), st, !c->prof, m.kcache, m.vcache, m.q, m.kv_new, w,
+  return launch_after(kern, dim3(grid), dim3(kThreads), smem_bytes<NR>(), st, !c->prof, m.cache, m.q, m.kv_new, w,
                       b.part_o, b.part_ml, tickets, hi, lo, c->dev_status);
 }
 
@@ -720,7 +724,11 @@ Buffers carve(const ps_config& g, char* base) {
 bool build_maps(const ps_ctx* c, const Buffers& b, Maps* m) {
   const ps_config& g = c->cfg;
   const size_t nr = padded_rows(g), pairs = (size_t)g.max_batch * g.n_kv_heads, rows = pairs * g.max_ctx;
-  return nr && make_map(&m->kcache, c->kcache, rows, kD, kBoxRows) && make_map(&m->vcache, c->vcache, rows, kD, kBoxRows) &&
+  const void* slab[2] = {c->kcache, c->vcache};
+  for (int v = 0; v < 2; ++v)
+    if (!make_map(&m->cache.full[v], slab[v], rows, kD, kTile) || !make_map(&m->cache.part[v], slab[v], rows, kD, kBoxRows))
+      return false;
+  return nr &&
          make_map(&m->q, b.q, pairs * 2 * nr, kD, (int)(2 * nr)) &&
          make_map(&m->kv_new, b.kv_new, pairs * 2 * kNewRows, kD, kNewRows);
 }
