@@ -18,12 +18,13 @@
 // last of them to finish.
 // A small kernel ahead (k_attn_prep) rotates and splits the query rows and rounds the new k / v
 // rows as the cache would; the ring is filled with cached tiles while it runs.
-// Measured with it (event intervals) against mma.sync blocks that stage a tile, synchronise and
-// compute: 33B shape, 16 sequences of 1024-4096 keys, 9 rows: 343 -> 207 us (973 MB: 4.7 TB/s); 13B
-// shape, 64 x 256-2048 keys, 9 rows: 459 -> 360 us (1.5 GB: 4.2 TB/s); 16 sequences, 5 rows: 94 us
-// either way (whole call 437 -> 430 us: the small kernel ahead hides behind the ring's first fill).
-// What holds it now is the softmax warps' step (2200 cycles of a 2900-cycle tile at full HBM rate)
-// and the short steps of the new rows, one per pair.
+// Measured (attention alone, with the small kernel) against mma.sync blocks that stage a tile,
+// synchronise and compute: 33B shape, 16 sequences of 1024-4096 keys, 9 rows: 343 -> 210 us (973 MB:
+// 4.8 TB/s of K/V in the main kernel); 13B shape, 64 x 256-2048 keys, 9 rows: 459 -> 332 us (1.5 GB); 16
+// sequences, 5 rows: 94 -> 82 us; 128 training groups of 300-428 keys: 273 -> 198 us.  What was worth
+// most after the first version: one TMA instruction per tile (the producer thread issued sixteen:
+// 351 -> 318 us on the 64-sequence case, 282 -> 179 on the groups), two MMA issuers, eight softmax
+// warps.  Putting the new rows into the last cached tile was slower (more, smaller boxes).
 #include <cfloat>
 
 #include "attn_tc.cuh"
@@ -41,11 +42,10 @@ using umma::mbar_init;
 using umma::mbar_wait;
 using umma::smem_desc;
 using umma::smem_u32;
-using umma::tma_load_2d;
 
 constexpr int kTile = 128;                 // keys of a unit
 constexpr int kSlotBytes = kTile * kD * 2; // a K or V tile
-constexpr int kBoxRows = 32;               // rows of a cache box: a ragged tile is fetched in steps of it
+constexpr int kBoxRows = 32;               // a ragged tile is fetched up to a multiple of it
 constexpr int kSoftWarps = 8;              // two per lane quadrant, half of the rows each
 constexpr int kThreads = 96 + 32 * (kSoftWarps + 4);   // producer, two MMA issuers, softmax, 4 epilogue warps
 constexpr float kSlack = 64.f;             // a score this far above the reference (log2) forces a rescale
@@ -131,6 +131,8 @@ struct Walk {
   __device__ bool last() const { return in_tail || (t + 1 == t_end && !tail); }
   __device__ bool last_of_cta() const { return u >= u_end && last(); }
   __device__ int keys(const Work& w) const { return in_tail ? w.R : min(kTile, len - t * kTile); }
+  // rows of the step's box: the halves of its tile lie that many rows apart
+  __device__ int box(const Work& w) const { return in_tail ? kNewRows : (keys(w) + kBoxRows - 1) & ~(kBoxRows - 1); }
   __device__ void next(const Work& w) {
     if (last()) { next_segment(w); return; }
     first = false;
@@ -138,6 +140,14 @@ struct Walk {
   }
 };
 
+// One box of rows y.. of a [rows][128] matrix seen as [2][rows][64]: both 64-channel halves, one behind
+// the other (the producer thread is bound by the instructions it issues, not by their size).
+__device__ __forceinline__ void tma_load_rows(uint32_t dst, const CUtensorMap* map, int y, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+      "l"(map), "r"(0), "r"(y), "r"(0), "r"(smem_u32(bar))
+      : "memory");
+}
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -175,10 +185,10 @@ __device__ __forceinline__ void tmem_rows(uint32_t taddr, float (&v)[NR]) {
   for (int i = 0; i < NR; ++i)
     v[i] = __uint_as_float(r[i / 16][i % 16]) + __uint_as_float(r[(NR + i) / 16][(NR + i) % 16]);
 }
-// V^T as the MMA's M side: channels contiguous (MN-major), 128-byte swizzle; 64-channel blocks one
-// box (16 KB) apart, groups of 8 keys 1024 bytes apart.
-__device__ __forceinline__ uint64_t vt_desc(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)((kSlotBytes / 2) >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
+// V^T as the MMA's M side: channels contiguous (MN-major), 128-byte swizzle; 64-channel halves
+// half_bytes apart, groups of 8 keys 1024 bytes apart.
+__device__ __forceinline__ uint64_t vt_desc(uint32_t saddr, uint32_t half_bytes) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(half_bytes >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
          ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 // Barriers of 128 threads: the epilogue warps, and the four warps of either half of the rows.
@@ -324,8 +334,7 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
         const uint32_t dst = s_q + (seg & 1) * kOp;
         mbar_arrive_expect_tx(bar, kOp);
         const int y = (b * w.n_kv + hk) * N;
-        tma_load_2d(dst, &t_q, 0, y, bar);
-        tma_load_2d(dst + kOp / 2, &t_q, 64, y, bar);
+        tma_load_rows(dst, &t_q, y, bar);
       };
       auto need_dep = [&]() {
         if (dep) return;
@@ -340,25 +349,10 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
         if (n_issued >= NS && !mbar_wait(&ctl.empty[slot], (use & 1) ^ 1, abort_flag)) { alive = false; return; }
         const uint32_t dst = base + slot * kSlotBytes;
         uint64_t* bar = &ctl.full[slot];
-        if (x.in_tail) {
-          mbar_arrive_expect_tx(bar, kNewRows * kD * 2);
-          const int y = ((x.b * w.n_kv + x.hk) * 2 + v) * kNewRows;
-          tma_load_2d(dst, &t_new, 0, y, bar);
-          tma_load_2d(dst + kSlotBytes / 2, &t_new, 64, y, bar);
-        } else {
-          const int n = min(kTile, x.len - x.t * kTile), nb = (n + kBoxRows - 1) / kBoxRows;
-          mbar_arrive_expect_tx(bar, nb * kBoxRows * kD * 2);
-          const int y = (w.sm.slot[x.b] * w.n_kv + x.hk) * w.max_ctx + x.t * kTile;
-          if (nb == kTile / kBoxRows) {   // a (nearly) full tile: one box per 64 channels
-            tma_load_2d(dst, &t_c.full[v], 0, y, bar);
-            tma_load_2d(dst + kSlotBytes / 2, &t_c.full[v], 64, y, bar);
-          } else {
-            for (int i = 0; i < nb; ++i) {
-              tma_load_2d(dst + i * kBoxRows * 128, &t_c.part[v], 0, y + i * kBoxRows, bar);
-              tma_load_2d(dst + kSlotBytes / 2 + i * kBoxRows * 128, &t_c.part[v], 64, y + i * kBoxRows, bar);
-            }
-          }
-        }
+        const int rows = x.box(w);
+        mbar_arrive_expect_tx(bar, rows * kD * 2);
+        if (x.in_tail) tma_load_rows(dst, &t_new, ((x.b * w.n_kv + x.hk) * 2 + v) * kNewRows, bar);
+        else tma_load_rows(dst, &t_c.m[v][rows / kBoxRows - 1], (w.sm.slot[x.b] * w.n_kv + x.hk) * w.max_ctx + x.t * kTile, bar);
         ++n_issued;
         if (++slot == NS) { slot = 0; ++use; }
       };
@@ -394,9 +388,10 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
             !mbar_wait(&ctl.full[slot], use & 1, abort_flag)) break;
         fence_after_sync();
         const uint64_t da = dk0 + (uint64_t)(slot * (kSlotBytes / 16)), db = dq0 + (uint64_t)(qb * (kOp / 16));
+        const uint64_t half = (uint64_t)(x.box(w) * 128 / 16);
 #pragma unroll
         for (int ks = 0; ks < kD / 16; ++ks)
-          umma::mma_f16(tmem + buf * N, da + (ks >> 2) * (kSlotBytes / 32) + (ks & 3) * 2,
+          umma::mma_f16(tmem + buf * N, da + (ks >> 2) * half + (ks & 3) * 2,
                         db + (ks >> 2) * (kOp / 32) + (ks & 3) * 2, id, ks > 0);
         umma::mma_commit(&ctl.s_full[buf]);
         umma::mma_commit(&ctl.empty[slot]);
@@ -410,7 +405,7 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
     if (lane == 0) {   // ---- MMA issuer, outputs
       Walk x;
       const uint32_t id = umma::idesc(N) | (1u << 15);
-      const uint64_t dv0 = vt_desc(base), dp0 = smem_desc(s_p);
+      const uint64_t dv0 = vt_desc(base, 0), dp0 = smem_desc(s_p);
       x.start(w, u0, u1);
       int slot = x.ok && x.last_of_cta() ? 1 : 2;   // of this step's V: ring position 2 i + 2, of the very last one 2 i + 1
       uint32_t use = 0;
@@ -420,7 +415,8 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
             !mbar_wait(&ctl.full[slot], use & 1, abort_flag) ||
             !mbar_wait(&ctl.p_full[buf], (i >> 1) & 1, abort_flag)) break;
         fence_after_sync();
-        const uint64_t da = dv0 + (uint64_t)(slot * (kSlotBytes / 16)), db = dp0 + (uint64_t)(buf * (kOp / 16));
+        const uint64_t da = dv0 + (uint64_t)(slot * (kSlotBytes / 16)) + ((uint64_t)(x.box(w) * 128 / 16) << 16),
+                       db = dp0 + (uint64_t)(buf * (kOp / 16));
         const int n_ks = (x.keys(w) + 15) >> 4;
         const uint32_t d = tmem_o + ob * N, acc = x.first ? 0u : 1u;
         if (n_ks == kTile / 16) {
@@ -555,11 +551,12 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
       if (n16 > n && !x.in_tail) {
         // rows of V between the tile's end and the next multiple of 16 meet probabilities of zero: they
         // must be finite
+        const int half_bytes = x.box(w) * 128;
         const int pos = x.last_of_cta() ? 2 * i + 1 : 2 * i + 2, vs = pos % NS;   // ring position of this V
         mbar_wait(&ctl.full[vs], (pos / NS) & 1, abort_flag);
         for (int e = tid - 96; e < (n16 - n) * 16; e += kSoft) {
           const int row = n + (e >> 4), c16 = e & 15;
-          *reinterpret_cast<uint4*>(ring_g + vs * kSlotBytes + (c16 >> 3) * (kSlotBytes / 2) + row * 128 + (c16 & 7) * 16) =
+          *reinterpret_cast<uint4*>(ring_g + vs * kSlotBytes + (c16 >> 3) * half_bytes + row * 128 + (c16 & 7) * 16) =
               make_uint4(0u, 0u, 0u, 0u);
         }
       }
@@ -725,12 +722,12 @@ bool build_maps(const ps_ctx* c, const Buffers& b, Maps* m) {
   const ps_config& g = c->cfg;
   const size_t nr = padded_rows(g), pairs = (size_t)g.max_batch * g.n_kv_heads, rows = pairs * g.max_ctx;
   const void* slab[2] = {c->kcache, c->vcache};
+  if (!nr) return false;
   for (int v = 0; v < 2; ++v)
-    if (!make_map(&m->cache.full[v], slab[v], rows, kD, kTile) || !make_map(&m->cache.part[v], slab[v], rows, kD, kBoxRows))
-      return false;
-  return nr &&
-         make_map(&m->q, b.q, pairs * 2 * nr, kD, (int)(2 * nr)) &&
-         make_map(&m->kv_new, b.kv_new, pairs * 2 * kNewRows, kD, kNewRows);
+    for (int i = 0; i < kTile / kBoxRows; ++i)
+      if (!make_halves_map(&m->cache.m[v][i], slab[v], rows, (i + 1) * kBoxRows)) return false;
+  return make_halves_map(&m->q, b.q, pairs * 2 * nr, (int)(2 * nr)) &&
+         make_halves_map(&m->kv_new, b.kv_new, pairs * 2 * kNewRows, kNewRows);
 }
 
 ps_status launch(ps_ctx* c, const SeqMap& sm, int B, const float* qkv, const Buffers& b, const Maps& m, unsigned* tickets,

@@ -21,7 +21,7 @@ struct Buffers {
   float* part_o;         // [2 CTAs' segments][NR][128] partial outputs
   float2* part_ml;       // [2 CTAs' segments][NR] their (reference, sum)
 };
-struct CacheMaps { CUtensorMap full[2], part[2]; };   // K and V slabs: boxes of a whole tile, of a part of one
+struct CacheMaps { CUtensorMap m[2][4]; };   // K and V slabs: boxes of 32, 64, 96 and 128 rows
 struct Maps { CacheMaps cache; CUtensorMap q, kv_new; };
 
 size_t bytes(const ps_config& g);                 // of the buffers; 0 when padded_rows() is 0

@@ -202,6 +202,8 @@ ps_status launch_logit_stats(ps_ctx* c, const float* logits, int M, int V, int R
 // outside the matrix.  False when the driver cannot encode tensor maps (tensor_map.cu).
 constexpr int kMapCols = 64;
 bool make_map(CUtensorMap* m, const void* base, size_t rows, size_t cols, int box_rows);
+// bf16 matrix [rows][128] seen as [2][rows][64]; boxes of both halves of box_rows rows.
+bool make_halves_map(CUtensorMap* m, const void* base, size_t rows, int box_rows);
 // ---- fused bf16 kernels for small M ---------------------------------------------------------
 bool fused_supported(ps_ctx* c, int M);
 int fused_kv_rows(ps_ctx* c);     // rows per pass of fused_kv_append (0: not available)
