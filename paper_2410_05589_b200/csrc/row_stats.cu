@@ -6,9 +6,11 @@
 // block's shared memory.  What bounds it: the arithmetic of the sampler (a Philox evaluation per
 // logit, about 30 multiplies), not the read, which comes from L2 right behind the LM head.  Two
 // things keep the rest small:
-//  - the noise G = -ln(-ln u) <= -ln(1 - u), so a logit can only beat the thread's best y when
+//  - the noise G = -ln(-ln u) <= -ln(1 - u), so a logit can only beat the best y so far when
 //    1 - u <= exp(x / T - y): one exponential decides, and the two logarithms are taken for the
-//    few that pass;
+//    few that pass.  The best y is the block's (a warp's after every vector, shared through memory
+//    after every batch): against each thread's own, some lane of a warp passed nearly every time
+//    (576 rows of 32000: 89 -> 75 us);
 //  - top-n: the n-th largest of the threads' maxima bounds the n-th largest logit from below, so
 //    only threads whose own maximum reaches it (n of them, ties aside) look at their logits
 //    again and put what reaches the bound on a list that one warp ranks.
@@ -40,6 +42,7 @@ struct Shared {
   int i[kWarps];
   unsigned keys[kWarps][kTop];
   float bound;
+  unsigned thr;      // key of the block's best perturbed logit so far
   int n_list;
   float lv[kListCap];
   int li[kListCap];
@@ -81,7 +84,8 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
   __shared__ Shared s;
   const int nclu = gridDim.x, rank = blockIdx.x, m = blockIdx.y;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (tid == 0) s.n_list = 0;
+  if (tid == 0) { s.n_list = 0; s.thr = 0u; }
+  __syncthreads();
   const float* row = logits + (size_t)m * V;
   const int share = ((V + nclu - 1) / nclu + 3) & ~3;          // tokens per block, whole vectors
   const int v_lo = min(V, rank * share), v_hi = min(V, v_lo + share);
@@ -98,7 +102,7 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
   pdl_launch_dependents();   // (not earlier: a dependent's blocks would wait beside the LM head's)
 
   // ---- the pass: per-thread running maximum and sum of exponentials, best perturbed logit
-  float mx = -FLT_MAX, se = 0.f, gv = -FLT_MAX;
+  float mx = -FLT_MAX, se = 0.f, gv = -FLT_MAX, thr = -FLT_MAX;
   int gi = 0x7fffffff;
   auto sample_one = [&](float x, int v) {
     uint32_t c[4] = {(uint32_t)v, row_id, sa.off_lo, sa.off_hi};
@@ -107,7 +111,7 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
     const float y0 = x * sa.inv_temp;
     // 1 - u up to its last bit; the margins cover the rounding of the test and of y = y0 + G
     const float rest = ((float)(16777216u - w) - 0.5f) * (1.0f / 16777216.0f);
-    if (!(rest > 1.01f * __expf(y0 - gv + fabsf(y0) * 2.4e-7f))) {
+    if (!(rest > 1.01f * __expf(y0 - thr + fabsf(y0) * 2.4e-7f))) {
       const float y = y0 + gumbel_of_word(w);
       if (ranks_before(y, v, gv, gi)) { gv = y; gi = v; }
     }
@@ -117,7 +121,7 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
   float4 x[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) x[u] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-  for (int i0 = tid; i0 < n_vec; i0 += U * kThreads) {
+  for (int i0 = tid; i0 - tid < n_vec; i0 += U * kThreads) {
 #pragma unroll
     for (int u = 0; u < U; ++u)
       x[u] = i0 + u * kThreads < n_vec ? __ldcg(row4 + i0 + u * kThreads) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
@@ -136,7 +140,12 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
           const int v = v_lo + 4 * (i0 + u * kThreads);
           sample_one(x[u].x, v); sample_one(x[u].y, v + 1); sample_one(x[u].z, v + 2); sample_one(x[u].w, v + 3);
         }
+        const unsigned k = __reduce_max_sync(0xffffffffu, key_of(gv));
+        thr = fmaxf(thr, key_value(k));
       }
+      if (lane == 0) atomicMax(&s.thr, key_of(thr));
+      const unsigned k = *(volatile unsigned*)&s.thr;   // (any value seen is one that some lane has reached)
+      if (k) thr = fmaxf(thr, key_value(k));
     }
   }
   for (int v = tail + tid; v < v_hi; v += kThreads) {
@@ -293,10 +302,17 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
 ps_status launch_logit_stats(ps_ctx* c, const float* logits, int M, int V, int R, int top_n, int* top_ids,
                              float* top_logit, float* row_max, float* row_lse, const SampleArgs* sa, cudaStream_t st) {
   if (top_n <= 0 && !row_max && !row_lse && !sa) return PS_OK;
-  // Blocks per row: enough that the rows cover the SMs twice over, at least 2048 tokens each (below
-  // that a block's fixed cost, about 2 us of reductions, outweighs what it takes off the pass).
+  // Blocks per row (two are resident per SM): the count whose waves of 1 / nclu rows each are over first,
+  // with at least 2048 tokens a block (below that its fixed cost, about 2 us of reductions, outweighs
+  // what it takes off the pass).  144 rows of 32000 tokens: 2 blocks in one wave, 50 -> 30 us against 4
+  // in two; a single full wave is worth more than its share says (80 rows: 7 blocks in two waves 31 us).
   int nclu = 1;
-  while (nclu < 8 && M * nclu < 2 * c->n_sm && V / (2 * nclu) >= 2048) nclu *= 2;
+  double best = 1e30;
+  for (int n = 1; n <= 8 && (n == 1 || V / n >= 2048); ++n) {
+    const long waves = ((long)M * n + 2 * c->n_sm - 1) / (2 * c->n_sm);
+    const double cost = (waves > 1 ? 1.15 : 1.0) * waves / n + 0.005 * n;
+    if (cost < best) { best = cost; nclu = n; }
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nclu, M);
   cfg.blockDim = dim3(kThreads);
