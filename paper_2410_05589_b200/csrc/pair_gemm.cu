@@ -464,32 +464,35 @@ __global__ void __launch_bounds__(256) k_finish_shared(const __grid_constant__ A
 }
 
 // Row m of a MODE_RAW stage: the row's slots added in k order, bias and residual, the row's sum
-// of squares, the planes of its RMS-normalised values.  One block per row; a thread holds NV
-// vectors of four features in registers from the loads to the stores.
-constexpr int kNormThreads = 256;
-template <int NV>
-__global__ void __launch_bounds__(kNormThreads) k_row_norm(const __grid_constant__ Args a, int H, float eps,
+// of squares, the planes of its RMS-normalised values.  One block per row, a thread for every two
+// vectors of four features (beyond 8192 features more vectors), held in registers from the loads to the stores.
+// Bound by the latency of its loads from L2, so the slots of JB contributors are in flight together.
+template <int NV, int JB, int NT>
+__global__ void __launch_bounds__(NT) k_row_norm(const __grid_constant__ Args a, int H, float eps,
                                                            const __nv_bfloat16* __restrict__ bias, const float* res,
                                                            const __nv_bfloat16* __restrict__ gain, float* out,
                                                            __nv_bfloat16* hi, __nv_bfloat16* lo) {
-  __shared__ float s_part[kNormThreads / 32];
+  __shared__ float s_part[32];
   pdl_launch_dependents();
   const Plan& p = a.p;
-  const int m = blockIdx.x, rt = m / p.Np, mi = m - rt * p.Np, tid = threadIdx.x;
+  const int m = blockIdx.x, rt = m / p.Np, mi = m - rt * p.Np, tid = threadIdx.x, nthr = blockDim.x;
   const int sh = p.wt == 2 ? 9 : 8, TW = 1 << sh;
   const bool out_vec = ((uintptr_t)out & 15) == 0;     // (the caller's feature rows may sit anywhere)
   const size_t layer = (size_t)p.slot_T * p.Np * TW;   // floats between contributors
-  float4 x[NV], g[NV];
+  float4 x[NV];
+  const float* slot[NV];
   int cnt[NV], cmax = 0;
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
-    const int n = 4 * (tid + i * kNormThreads);
+    const int n = 4 * (tid + i * nthr);
     cnt[i] = 0;
-    x[i] = g[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    slot[i] = a.part;
+    x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (n < H) {
-      cnt[i] = tile_contributors(p, (n >> sh) * p.n_rt + rt);
+      const int t = (n >> sh) * p.n_rt + rt;
+      cnt[i] = tile_contributors(p, t);
       cmax = max(cmax, cnt[i]);
-      g[i] = load_bf4(gain + n);
+      slot[i] += ((size_t)t * p.Np + mi) * TW + (n & (TW - 1));
       if (bias) x[i] = load_bf4(bias + n);
     }
   }
@@ -497,19 +500,21 @@ __global__ void __launch_bounds__(kNormThreads) k_row_norm(const __grid_constant
   float4 rv[NV];
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
-    const int n = 4 * (tid + i * kNormThreads);
+    const int n = 4 * (tid + i * nthr);
     rv[i] = (res && n < H) ? __ldcg(reinterpret_cast<const float4*>(res + (size_t)m * H + n)) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  for (int j = 0; j < cmax; ++j) {
-    float4 v[NV];
+  for (int j = 0; j < cmax; j += JB) {
+    float4 v[JB][NV];
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      const int n = 4 * (tid + i * kNormThreads);
-      const float* s = a.part + (size_t)j * layer + ((size_t)((n >> sh) * p.n_rt + rt) * p.Np + mi) * TW + (n & (TW - 1));
-      v[i] = j < cnt[i] ? __ldcg(reinterpret_cast<const float4*>(s)) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    for (int b = 0; b < JB; ++b)
 #pragma unroll
-    for (int i = 0; i < NV; ++i) { x[i].x += v[i].x; x[i].y += v[i].y; x[i].z += v[i].z; x[i].w += v[i].w; }
+      for (int i = 0; i < NV; ++i)
+        v[b][i] = j + b < cnt[i] ? __ldcg(reinterpret_cast<const float4*>(slot[i] + (size_t)(j + b) * layer))
+                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int b = 0; b < JB; ++b)
+#pragma unroll
+      for (int i = 0; i < NV; ++i) { x[i].x += v[b][i].x; x[i].y += v[b][i].y; x[i].z += v[b][i].z; x[i].w += v[b][i].w; }
   }
   float ss = 0.f;
 #pragma unroll
@@ -520,20 +525,19 @@ __global__ void __launch_bounds__(kNormThreads) k_row_norm(const __grid_constant
   ss = warp_sum(ss);
   if ((tid & 31) == 0) s_part[tid >> 5] = ss;
   __syncthreads();
-  float tot = 0.f;
-#pragma unroll
-  for (int w = 0; w < kNormThreads / 32; ++w) tot += s_part[w];
+  const float tot = warp_sum((tid & 31) < (nthr >> 5) ? s_part[tid & 31] : 0.f);
   const float sc = rsqrtf(tot / (float)H + eps);
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
-    const int n = 4 * (tid + i * kNormThreads);
+    const int n = 4 * (tid + i * nthr);
     if (n < H) {
       if (out) {
         float* o = out + (size_t)m * H + n;
         if (out_vec) *reinterpret_cast<float4*>(o) = x[i];
         else { o[0] = x[i].x; o[1] = x[i].y; o[2] = x[i].z; o[3] = x[i].w; }
       }
-      const float4 y = make_float4(x[i].x * sc * g[i].x, x[i].y * sc * g[i].y, x[i].z * sc * g[i].z, x[i].w * sc * g[i].w);
+      const float4 g = load_bf4(gain + n);
+      const float4 y = make_float4(x[i].x * sc * g.x, x[i].y * sc * g.y, x[i].z * sc * g.z, x[i].w * sc * g.w);
       split4(y, hi + (size_t)m * H + n, lo + (size_t)m * H + n);
     }
   }
@@ -631,11 +635,11 @@ ps_status launch_finish_shared(ps_ctx* c, const Args& a, Mode mode, cudaStream_t
 
 ps_status launch_row_norm(ps_ctx* c, const Args& a, int H, const __nv_bfloat16* bias, const float* res,
                           const __nv_bfloat16* gain, float* out, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t st) {
-  const int nv = (H / 4 + kNormThreads - 1) / kNormThreads;
-  if (nv > 32) return fail(c, PS_ERR_UNSUPPORTED, "hidden size beyond 32768");
-  auto kern = nv <= 5 ? k_row_norm<5> : nv <= 8 ? k_row_norm<8> : nv <= 16 ? k_row_norm<16> : k_row_norm<32>;
-  const cudaError_t e = launch_after(kern, dim3(a.p.M), dim3(kNormThreads), 0, st, !c->prof, a, H, c->cfg.rms_eps, bias, res,
-                                     gain, out, hi, lo);
+  if (H > 32768) return fail(c, PS_ERR_UNSUPPORTED, "hidden size beyond 32768");
+  const int threads = H <= 8192 ? (H / 4 + 63) / 64 * 32 : 512;
+  auto kern = H <= 8192 ? k_row_norm<2, 4, 1024> : H <= 16384 ? k_row_norm<8, 1, 512> : k_row_norm<16, 1, 512>;
+  const cudaError_t e = launch_after(kern, dim3(a.p.M), dim3(threads), 0, st, !c->prof, a, H, c->cfg.rms_eps, bias, res, gain,
+                                     out, hi, lo);
   c->launches++;
   return cuda_check(c, e, "k_row_norm");
 }
