@@ -436,7 +436,7 @@ class Workload:
         stages = {}
         for name, (tot, cnt) in prof.items():
             if cnt and name in sb:
-                us = tot / n * 1e3   # per step: a batch beyond 128 rows runs a stage several times a step
+                us = tot / n * 1e3   # per step
                 gbs = sb[name] / (us * 1e-6) / 1e9
                 stages[name] = {"us": round(us, 2), "gbs": round(gbs, 1), "frac_of_peak": round(gbs / peak, 4),
                                 "launches_per_step": round(cnt / n, 2)}
@@ -720,7 +720,7 @@ def main():
         h1.record()
         torch.cuda.synchronize()
         group = {"ms_per_call": h0.elapsed_time(h1) / 5, "groups": n_g, "rows": n_g * R,
-                 "note": "ps_group_forward; the groups run as draft steps of up to 128 rows per launch"}
+                 "note": "ps_group_forward; the groups run as one draft step over all their rows"}
 
     # ---- token-tree verification (Algorithm 1 in full) and the whole tree round -----------------
     tree, tree_round = (None, None)

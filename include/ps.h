@@ -134,9 +134,9 @@ ps_status ps_kv_append(ps_ctx* ctx, int B, const int* seq_slot, const int* n_new
  * to rows 0..j, and its logits are the drafter's distribution for the token j places after
  * the next one.  Neither the committed cache length nor the cache rows change (the new rows'
  * k / v live in a side buffer of the workspace).  Calling it twice gives identical outputs.
- * A batch of more than 128 rows B*(k+1) runs as several launches per stage, each over a group
- * of whole sequences; a sequence's outputs do not depend on which other sequences are in the
- * call beyond fp32 rounding (the GEMMs' summation order follows the rows of a launch).
+ * A batch of any size runs as one launch per stage; a sequence's outputs do not depend on which
+ * other sequences are in the call beyond fp32 rounding (the GEMMs' summation order follows the
+ * rows of a launch).
  *   B            sequences (1..max_batch);  seq_slot host [B], distinct
  *   hidden_last  device [B][H], config dtype;  token_last device [B] int32
  *   top_n        0..PS_MAX_TOP_N entries per row (0: top_ids/top_logit unused)
