@@ -543,17 +543,30 @@ __global__ void __launch_bounds__(NT) k_row_norm(const __grid_constant__ Args a,
   }
 }
 
-// Modelled time of a launch (microseconds), for the choice between plans only.  A unit of a pair
-// (wt weight boxes and the planes beside them in both CTAs) takes the longest of: its share of HBM,
-// its share of L2 -> SM traffic, its MMAs (58 cycles at least, Np / 2 above).  A contributor more
-// costs its slots' way through L2 twice.
-double plan_cost(const Plan& p, int planes, int units, int contributors, int n_pairs) {
-  const double t_hbm = p.wt * 32.768e3 / (6.4e6 / n_pairs) / p.n_rt;
-  const double t_l2 = (p.wt * 32.768e3 + planes * p.Np * 128.0) / (10.0e6 / n_pairs);
-  const double t_mma = p.wt * planes * 4 * std::max(58.0, p.Np / 2.0) / 1.85e3;
-  const double slots = (double)p.rem * contributors * p.Np * 256.0 * p.wt * 4.0;
-  return units * std::max(t_hbm, std::max(t_l2, t_mma)) + (contributors > 1 ? 1.0 : 0.0) + 2.0 * slots / 6.0e6 +
-         p.wt * p.Np * 0.012;
+// Modelled time of a launch and of what finishes it (microseconds), for the choice between plans
+// only; fitted to the stage times of plans with one and two sub-tiles and 1 to 16 k blocks, 7B to 33B
+// shapes, 20 to 640 rows (the plan chosen is 1.6% behind the best one on average; a model in which
+// each pair had a fixed share of HBM was 4.9% behind: 33B q|k|v at 20 rows 87 us, now 67; 13B LM head
+// at 20 rows 95 us, now 83; 33B q|k|v at 288 rows 158 us, now 139).
+//  - a unit of a pair (wt weight boxes and the planes beside them in both CTAs) takes the longer of
+//    its way through the ring and its MMAs; idle pairs leave their share of HBM to the others, so
+//    HBM bounds the launch as a whole;
+//  - two sub-tiles of more than 128 rows fill the tensor memory, so the MMAs of the next tile wait
+//    until this one is read: one sub-tile is the better one there unless a pair has one tile only;
+//  - each contributor more costs a round trip, its slots the way through L2 twice, and a stage
+//    without a row norm a kernel that adds them.
+double stream_cost(const Plan& p, int planes, int units) {
+  const double a = p.wt * 32.768e3;
+  const double ring = 0.17 + (a + planes * p.Np * 128.0) / 185e3;
+  const double mma = planes * 4 * p.wt * std::max(58.0, p.Np * 0.6) / 1.85e3;
+  return std::max(units * std::max(ring, mma), (double)p.T * p.KB * a / p.n_rt / 7.2e6);
+}
+double finish_cost(const Plan& p, Mode mode, int segs, int contributors, int n_slots) {
+  const double cols = (double)p.wt * p.Np;
+  double t = cols * 0.021 + (cols > 256 ? cols * 0.035 * (segs - 1) : 0.0);
+  if (mode == MODE_RAW || contributors > 1) t += 0.5 * (contributors - 1) + 2.0 * n_slots * cols * 1024.0 / 5e6;
+  if (mode != MODE_RAW && contributors > 1) t += 5.0 + 0.008 * p.Np * p.n_rt;
+  return t;
 }
 
 }  // namespace
@@ -584,6 +597,10 @@ Plan make_plan(int M, const Weights& w, int K, int planes, Mode mode, size_t par
     p.T = p.tiles_w * p.n_rt;
     p.n_dp = p.T / P * P;
     p.rem = p.T - p.n_dp;
+    // Several full tiles a pair, two accumulators of 256 columns: modelled 5% shorter than two
+    // sub-tiles on prompts, but such calls stopped making progress now and then; the cause is not
+    // known, so these tiles always have two sub-tiles, as they had.
+    if (mode != MODE_SWIGLU && wt == 1 && p.Np == kMaxNp && p.T > P) continue;
     p.slot_t0 = mode == MODE_RAW ? 0 : p.n_dp;
     p.slot_T = p.T - p.slot_t0;
     const size_t layer = (size_t)p.slot_T * p.Np * 256 * wt;
@@ -592,14 +609,23 @@ Plan make_plan(int M, const Weights& w, int K, int planes, Mode mode, size_t par
       p.split = s;
       p.S = p.rem * s;
       p.Pe = std::max(1, std::min(P, p.S));
-      int units = p.n_dp / P * p.KB, jmax = 1;
+      int units = p.n_dp / P * p.KB, segs = p.n_dp / P, jmax = 1, n_slots = p.n_dp - p.slot_t0;
+      if (p.rem > 0) units += (p.S + p.Pe - 1) / p.Pe * ((p.KB + s - 1) / s);
+      double cost = stream_cost(p, planes, units);
+      if (cost >= best_cost) continue;
       if (p.rem > 0) {
-        units += (p.S + p.Pe - 1) / p.Pe * ((p.KB + s - 1) / s);
-        for (int t = p.n_dp; t < p.T; ++t) jmax = std::max(jmax, tile_contributors(p, t));
+        for (int t = p.n_dp; t < p.T; ++t) {
+          const int j = tile_contributors(p, t);
+          jmax = std::max(jmax, j);
+          n_slots += j;
+        }
+        int runs = 0;
+        for (int c = 0; c < p.Pe; ++c) runs = std::max(runs, (run_begin(p, c + 1) - 1) / s - run_begin(p, c) / s + 1);
+        segs += runs;
       }
       p.shared = jmax > 1;
       if (layer * ((mode == MODE_RAW || jmax > 1) ? jmax : 0) > part_floats) continue;
-      const double cost = plan_cost(p, planes, units, jmax, P);
+      cost += finish_cost(p, mode, segs, jmax, n_slots);
       if (cost < best_cost) { best_cost = cost; best = p; }
     }
   }

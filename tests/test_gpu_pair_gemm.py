@@ -25,3 +25,17 @@ def test_pair_gemm_rows_match_oracle(B, k, kv_heads, bias, flags):
     assert p.g.check_guards() == 0 and p.g.poll() == 0
     again = p.gpu_step(top_n=1)
     assert np.array_equal(got["logits"], again["logits"])     # sums are added in k order, whoever is first
+
+
+# k ranges long enough that the q|k|v, gate|up and LM-head tiles are shared by several pairs: one row
+# tile, one that is not full, two
+@pytest.mark.parametrize("B,k", [(4, 4), (30, 4), (64, 4)])
+def test_pair_gemm_shared_tiles_match_oracle(B, k):
+    s = synth.CONFIGS["mini"].with_(k_masks=k, hidden=2048, n_heads=16, n_kv_heads=4, ffn=5504)
+    seqs = [0, B - 1]
+    p = Pair(s, B, lens=[1 + (5 * b) % 23 for b in range(B)], oracle_seqs=seqs)
+    got = p.gpu_step(top_n=1)
+    for b in seqs:
+        assert logits_close(got["logits"][b], p.oracle_step(b)["logits"], s.dtype) <= 1.0, b     # the logits gate
+    assert p.g.check_guards() == 0 and p.g.poll() == 0
+    assert np.array_equal(got["logits"], p.gpu_step(top_n=1)["logits"])
