@@ -383,8 +383,14 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
       uint32_t use = 0;
       for (int i = 0; x.ok; ++i) {
         const int buf = i & 1, qb = x.seg & 1;
+        // In a ring of odd length the slot's use before this one was a V tile, whose arrival the other
+        // issuer waits for.  A wait by parity cannot tell a use from the one two before it, so it must not
+        // begin until the V tile has been consumed (which the arrival of this K implies: nothing is
+        // lost).  In a ring of even length a slot's uses are all waited for by one issuer, but for the
+        // first (K of step 0) and the last (V of the last step), whose neighbours have long landed.
         if ((x.first && !mbar_wait(&ctl.q_full[qb], (x.seg >> 1) & 1, abort_flag)) ||
             !mbar_wait(&ctl.s_empty[buf], ((i >> 1) & 1) ^ 1, abort_flag) ||
+            ((NS & 1) && use > 0 && !mbar_wait(&ctl.empty[slot], (use - 1) & 1, abort_flag)) ||
             !mbar_wait(&ctl.full[slot], use & 1, abort_flag)) break;
         fence_after_sync();
         const uint64_t da = dk0 + (uint64_t)(slot * (kSlotBytes / 16)), db = dq0 + (uint64_t)(qb * (kOp / 16));

@@ -54,3 +54,30 @@ def test_scores_outgrow_their_reference():
         p.o.kv_import(b, as_f64(K, s.dtype), as_f64(V, s.dtype))
         p.g.kv_import(b, p.to_device(K), p.to_device(V))
     _check(p, s, range(2))
+
+
+# groups of 20 and 32 query rows run on a ring of five slots, whose slots alternate between the two MMA
+# issuers; more K / V than the L2 holds, so that tiles come late and out of order
+@pytest.mark.parametrize("kv_heads,k", [(8, 4), (16, 15)])
+def test_odd_ring_with_late_tiles(kv_heads, k):
+    import torch
+    import paper_2410_05589_b200 as ps
+    from harness import oracle_for
+    B, L = 12, 4000
+    s = synth.CONFIGS["mini"].with_(hidden=256, n_heads=32, n_kv_heads=kv_heads, ffn=256, vocab=1000, k_masks=k)
+    W = synth.weights(s)
+    g = ps.drafter_from_shape(s, W, max_batch=B, max_ctx=L + k + 1)
+    o = oracle_for(s, W, 1, L + k + 1)
+    K, V = synth.kv_rows(s, "kv", L)
+    o.kv_import(0, as_f64(K, s.dtype), as_f64(V, s.dtype))
+    for b in range(B):
+        g.kv_import(b, ps.to_device(K), ps.to_device(V))
+    h, t = synth.hidden_states(s, "last", 1), synth.token_ids(s, "last", 1)
+    want = o.draft_step(0, h, int(t[0]))["logits"]
+    hl, tl = ps.to_device(np.repeat(h, B, 0)), ps.to_device(np.repeat(t, B))
+    outs = [g.draft_step(list(range(B)), hl, tl, top_n=1)["logits"] for _ in range(8)]
+    torch.cuda.synchronize()
+    got = outs[0].cpu().numpy()
+    for b in range(B):
+        assert logits_close(got[b], want, s.dtype) <= 1.0, b     # the logits gate
+    assert all(torch.equal(outs[0], x) for x in outs[1:]) and g.poll() == 0
