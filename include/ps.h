@@ -308,6 +308,12 @@ ps_status ps_debug_check_guards(ps_ctx* ctx, void* stream, int* n_bad);
  * (at most 4e9), on a barrier nothing completes; ps_poll then returns PS_ERR_TIMEOUT. */
 ps_status ps_debug_wait_expires(ps_ctx* ctx, long long limit_cycles, void* stream);
 
+/* Test helper for the order of the stream: enqueues a kernel that lets the launches behind it start
+ * at once (programmatic dependent launch), waits `delay_us` microseconds (at most 1000) and only then
+ * copies `bytes` (a multiple of 4) from src to dst, both device memory and 4-byte aligned.  A call
+ * enqueued right behind it must find dst written. */
+ps_status ps_debug_late_copy(ps_ctx* ctx, void* dst, const void* src, size_t bytes, int delay_us, void* stream);
+
 /* Number of kernel launches the context has enqueued so far (host counter). */
 long long ps_launch_count(ps_ctx* ctx);
 

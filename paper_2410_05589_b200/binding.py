@@ -31,7 +31,7 @@ EXPORTS = (
     "ps_kv_len", "ps_kv_reset", "ps_kv_export", "ps_kv_import", "ps_poll", "ps_launch_count",
     "ps_last_error", "ps_destroy", "ps_philox_fill", "ps_profile", "ps_profile_read",
     "ps_verify_static", "ps_debug_buffer", "ps_verify_tree", "ps_draft_step_sampled", "ps_group_forward",
-    "ps_build_tree", "ps_debug_wait_expires", "ps_debug_check_guards",
+    "ps_build_tree", "ps_debug_wait_expires", "ps_debug_check_guards", "ps_debug_late_copy",
 )
 
 
@@ -84,6 +84,7 @@ def load_library(path: str | None = None) -> C.CDLL:
     lib.ps_build_tree.argtypes = [vp, C.c_int, C.c_int, ip, ip, vp, C.c_int, vp, vp, vp]
     lib.ps_debug_wait_expires.argtypes = [vp, C.c_longlong, vp]
     lib.ps_debug_check_guards.argtypes = [vp, vp, ip]
+    lib.ps_debug_late_copy.argtypes = [vp, vp, vp, C.c_size_t, C.c_int, vp]
     lib.ps_kv_len.argtypes = [vp, C.c_int, ip]
     lib.ps_kv_reset.argtypes = [vp, C.c_int]
     lib.ps_kv_export.argtypes = [vp, C.c_int, vp, vp, vp]
@@ -381,6 +382,12 @@ class Drafter:
     def debug_wait_expires(self, limit_cycles: int, stream=None) -> None:
         """ps_debug_wait_expires: a bounded device wait that runs out (sets the status word)."""
         self._check(self.lib.ps_debug_wait_expires(self.h, int(limit_cycles), _stream(stream)))
+
+    def debug_late_copy(self, dst: torch.Tensor, src: torch.Tensor, delay_us: int, stream=None) -> None:
+        """ps_debug_late_copy: dst <- src by a kernel that lets the launches behind it start early."""
+        assert dst.dtype == src.dtype and dst.numel() == src.numel()
+        self._check(self.lib.ps_debug_late_copy(self.h, _dptr(dst), _dptr(src), dst.numel() * dst.element_size(),
+                                                int(delay_us), _stream(stream)))
 
     def poll(self) -> int:
         """Waits for the stream and returns the device status (PS_OK, PS_ERR_NONFINITE, ...)."""

@@ -1617,6 +1617,12 @@ __global__ void k_join_planes(const __nv_bfloat16* hi, const __nv_bfloat16* lo, 
     out[i] = __bfloat162float(hi[i]) + __bfloat162float(lo[i]);
 }
 
+__device__ __forceinline__ long long globaltimer_ns() {
+  long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
 // The bounded wait of the GEMM kernels on a barrier that nothing ever completes: what a lost
 // copy would look like to them.  The wait gives up after `limit` cycles, the kernel raises the
 // status word as they do and returns normally.
@@ -1629,6 +1635,16 @@ __global__ void k_wait_expires(long long limit, int* status) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (!mbar_wait(&bar, 0, &abort_flag, limit)) atomicOr(status, kStatTimeout);
   }
+}
+
+// A kernel that lets its dependents start at once and writes its output late, as a producer of a
+// call's inputs may (test helper).
+__global__ void k_late_copy(uint32_t* dst, const uint32_t* src, size_t n, long long delay_ns) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const long long t0 = globaltimer_ns();
+  for (int i = 0; i < 100000 && globaltimer_ns() - t0 < delay_ns; ++i) __nanosleep(100);
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) dst[i] = src[i];
 }
 
 // ---- host side: tensor maps of the operands -----------------------------------------------------
@@ -2138,6 +2154,13 @@ ps_status launch_wait_expires(ps_ctx* c, long long limit_cycles, cudaStream_t st
   k_wait_expires<<<1, 32, 0, st>>>(limit_cycles, c->dev_status);
   c->launches++;
   return cuda_check(c, cudaGetLastError(), "k_wait_expires");
+}
+
+ps_status launch_late_copy(ps_ctx* c, uint32_t* dst, const uint32_t* src, size_t n, long long delay_ns, cudaStream_t st) {
+  // (few blocks: the dependents find room beside them)
+  k_late_copy<<<16, 256, 0, st>>>(dst, src, n, delay_ns);
+  c->launches++;
+  return cuda_check(c, cudaGetLastError(), "k_late_copy");
 }
 
 void fused_release(ps_ctx* c) {

@@ -269,6 +269,11 @@ ps_status ps_debug_wait_expires(ps_ctx* c, long long limit_cycles, void* stream)
   return launch_wait_expires(c, limit_cycles, (cudaStream_t)stream);
 }
 
+ps_status ps_debug_late_copy(ps_ctx* c, void* dst, const void* src, size_t bytes, int delay_us, void* stream) {
+  if (!c || !dst || !src || bytes % 4 || delay_us < 0 || delay_us > 1000) return PS_ERR_INVALID_ARG;
+  return launch_late_copy(c, (uint32_t*)dst, (const uint32_t*)src, bytes / 4, 1000LL * delay_us, (cudaStream_t)stream);
+}
+
 ps_status ps_kv_len(ps_ctx* c, int slot, int* len) {
   if (!c || !len || slot < 0 || slot >= c->cfg.max_batch) return PS_ERR_INVALID_ARG;
   *len = c->len[slot];

@@ -219,6 +219,7 @@ ps_status fused_debug_buffer(ps_ctx* c, const char* name, void** ptr, size_t* by
 ps_status launch_rope_table(ps_ctx* c, cudaStream_t st);
 // Test kernel: a bounded barrier wait that runs out after `limit_cycles` and raises the status word.
 ps_status launch_wait_expires(ps_ctx* c, long long limit_cycles, cudaStream_t st);
+ps_status launch_late_copy(ps_ctx* c, uint32_t* dst, const uint32_t* src, size_t n, long long delay_ns, cudaStream_t st);
 ps_status launch_attn_split(ps_ctx* c, const SeqMap& sm, int B, const float* qkv, float* att_ml,
                             float* att_o, unsigned* tickets, __nv_bfloat16* out_hi,
                             __nv_bfloat16* out_lo, cudaStream_t st);

@@ -359,10 +359,11 @@ __device__ __forceinline__ void verify_cluster_body(const VerifyArgs& a) {
   const int nv4 = ((V + nclu * kCluThreads - 1) / (nclu * kCluThreads) + 3) / 4;
   const int C = nv4 * 4, v0 = (rank * kCluThreads + tid) * C;
 
-  // The target rows are an input of the call; the draft rows and the draft tokens may be what the
-  // kernel before this one in the stream (the draft step) wrote last.  Were this kernel launched
-  // as its dependent, it would ask for the target row first and wait for that kernel only then.
+  // All rows may be what the kernel before this one in the stream wrote last (the target model's LM
+  // head, the draft step), and that kernel may let its dependents start before it writes: nothing of
+  // them is read before the wait.
   pdl_launch_dependents();
+  pdl_wait();
   float t[V4 * 4], d[V4 * 4];
 #pragma unroll
   for (int k = 0; k < V4; ++k) {
@@ -371,7 +372,6 @@ __device__ __forceinline__ void verify_cluster_body(const VerifyArgs& a) {
     if (k < nv4 && v < V) tv = __ldcs(reinterpret_cast<const float4*>(trow + v));
     t[4 * k] = tv.x; t[4 * k + 1] = tv.y; t[4 * k + 2] = tv.z; t[4 * k + 3] = tv.w;
   }
-  pdl_wait();
   const int x = bonus ? -1 : a.draft_tokens[(size_t)b * a.n_draft + i];
 #pragma unroll
   for (int k = 0; k < V4; ++k) {
