@@ -314,6 +314,16 @@ ps_status ps_debug_wait_expires(ps_ctx* ctx, long long limit_cycles, void* strea
  * enqueued right behind it must find dst written. */
 ps_status ps_debug_late_copy(ps_ctx* ctx, void* dst, const void* src, size_t bytes, int delay_us, void* stream);
 
+/* Test helper: how a GEMM of more than 16 rows is dealt to the CTA pairs of a device with n_sm
+ * multiprocessors (host only, no device access).  mat_rows: host [n_mats], n_mats <= 3; zip: the first two are
+ * gate and up; planes: 1 or 2 operand planes; raw: every tile's sums go through partial-sum slots;
+ * slot_floats: capacity of the slots.  out: host [12] = sub-tiles, rows of a row tile, row tiles, k-blocks,
+ * tiles, whole tiles, shared tiles, k blocks of a shared tile, pairs that share them, most
+ * contributors of a tile, contributors of all shared tiles together, slots used (in tiles).
+ * PS_ERR_CAPACITY: no way of dealing fits the slots. */
+ps_status ps_debug_gemm_plan(int rows, int k, int n_mats, const int* mat_rows, int zip, int planes, int raw,
+                             size_t slot_floats, int n_sm, int* out);
+
 /* Number of kernel launches the context has enqueued so far (host counter). */
 long long ps_launch_count(ps_ctx* ctx);
 

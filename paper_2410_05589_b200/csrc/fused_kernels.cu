@@ -1652,6 +1652,7 @@ struct PlaneMaps {   // one activation plane: boxes of 16 rows, and of every siz
   CUtensorMap m16;
   pg::PlaneMaps pair;
 };
+constexpr int kPlanSlots = 128;
 constexpr int kPairStages = 8;   // fc, q|k|v, o, gate|up, down, LM head of a draft step; fc, k|v of an append
 struct UmmaMaps {
   CUtensorMap w_fc, w_q, w_k, w_v, w_o, w_gate, w_up, w_down, w_lm;
@@ -1659,8 +1660,9 @@ struct UmmaMaps {
   PlaneMaps xin, x0_hi, x0_lo, attn_hi, attn_lo, a_hi, a_lo, act_hi, act_lo, hdn_hi, hdn_lo;
   atc::Maps at;
   bool at_ok = false;
-  // how each stage was last dealt (a function of the shapes and the row count alone)
-  pg::Plan plan[kPairStages] = {};
+  // how each stage is dealt, by row count (a function of the shapes and the count alone): a server's
+  // count changes from step to step, and finding the plans of one takes the host 10 to 16 us
+  pg::Plan plan[kPairStages][kPlanSlots] = {};
 };
 
 bool make_plane_maps(PlaneMaps* pm, const void* base, size_t rows, size_t cols) {
@@ -1805,7 +1807,7 @@ ps_status run_stages(ps_ctx* c, StageDesc* d, int n, bool chain, int chain_id, c
 // `id` names the stage's place in the plan cache.
 ps_status pair_stage(ps_ctx* c, UmmaMaps& u, int id, pg::Mode mode, int M, int K, int planes, const pg::Weights& w,
                      const PlaneMaps& hi, const PlaneMaps& lo, const FusedScratch& f, pg::Args& a, cudaStream_t st) {
-  pg::Plan& plan = u.plan[id];
+  pg::Plan& plan = u.plan[id][(uint32_t)M * 2654435761u >> 25];   // (the counts of one context spread over the slots)
   if (plan.T == 0 || plan.M != M) plan = pg::make_plan(M, w, K, planes, mode, f.slot_floats, c->n_sm);
   a.p = plan;
   a.planes = planes;

@@ -614,13 +614,26 @@ Plan make_plan(int M, const Weights& w, int K, int planes, Mode mode, size_t par
       double cost = stream_cost(p, planes, units);
       if (cost >= best_cost) continue;
       if (p.rem > 0) {
-        for (int t = p.n_dp; t < p.T; ++t) {
-          const int j = tile_contributors(p, t);
-          jmax = std::max(jmax, j);
-          n_slots += j;
+        // at least so many contributors to a tile and in all: most candidates need not be walked
+        if (cost + finish_cost(p, mode, segs + 1, (p.Pe + p.rem - 1) / p.rem, n_slots + std::max(p.rem, p.Pe)) >= best_cost)
+          continue;
+        // one walk over the runs (run_begin without its divisions): contributors of each tile, tiles of a run
+        const int q = p.S / p.Pe, r = p.S % p.Pe;
+        int runs = 0, err = 0, pos = 0, j = 0;
+        for (int c = 0; c < p.Pe; ++c) {
+          int len = q, tiles = 0;
+          if ((err += r) >= p.Pe) { err -= p.Pe; ++len; }
+          while (len > 0) {
+            j = pos == 0 ? 1 : j + 1;
+            jmax = std::max(jmax, j);
+            ++tiles;
+            const int take = std::min(len, s - pos);
+            len -= take;
+            if ((pos += take) == s) pos = 0;
+          }
+          n_slots += tiles;
+          runs = std::max(runs, tiles);
         }
-        int runs = 0;
-        for (int c = 0; c < p.Pe; ++c) runs = std::max(runs, (run_begin(p, c + 1) - 1) / s - run_begin(p, c) / s + 1);
         segs += runs;
       }
       p.shared = jmax > 1;

@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cstring>
 
+#include "pair_gemm.cuh"
 #include "ps_internal.cuh"
 
 namespace ps {
@@ -272,6 +273,30 @@ ps_status ps_debug_wait_expires(ps_ctx* c, long long limit_cycles, void* stream)
 ps_status ps_debug_late_copy(ps_ctx* c, void* dst, const void* src, size_t bytes, int delay_us, void* stream) {
   if (!c || !dst || !src || bytes % 4 || delay_us < 0 || delay_us > 1000) return PS_ERR_INVALID_ARG;
   return launch_late_copy(c, (uint32_t*)dst, (const uint32_t*)src, bytes / 4, 1000LL * delay_us, (cudaStream_t)stream);
+}
+
+ps_status ps_debug_gemm_plan(int rows, int k, int n_mats, const int* mat_rows, int zip, int planes, int raw,
+                             size_t slot_floats, int n_sm, int* out) {
+  if (rows < 1 || k < 1 || n_mats < 1 || n_mats > 3 || (zip && n_mats != 2) || !mat_rows || n_sm < 2 || !out)
+    return PS_ERR_INVALID_ARG;
+  pg::Weights w{};
+  w.n_mats = n_mats;
+  w.zip = zip != 0;
+  for (int i = 0; i < n_mats; ++i) w.rows[i] = mat_rows[i];
+  const pg::Mode mode = zip ? pg::MODE_SWIGLU : raw ? pg::MODE_RAW : pg::MODE_STORE;
+  const pg::Plan p = pg::make_plan(rows, w, k, planes, mode, slot_floats, n_sm);
+  if (p.T == 0) return PS_ERR_CAPACITY;
+  int most = 1, all = 0;
+  size_t end = 0;
+  for (int t = p.slot_t0; t < p.T; ++t) {
+    const int j = pg::tile_contributors(p, t);
+    if (t >= p.n_dp) { most = std::max(most, j); all += j; }
+    if (raw || j > 1) end = std::max(end, pg::slot_row(p, j - 1, t, p.Np));
+  }
+  const int v[12] = {p.wt, p.Np, p.n_rt, p.KB, p.T, p.n_dp, p.rem, p.split, p.Pe, most, all,
+                     (int)(end / ((size_t)p.Np * 256 * p.wt))};
+  std::copy(v, v + 12, out);
+  return PS_OK;
 }
 
 ps_status ps_kv_len(ps_ctx* c, int slot, int* len) {

@@ -1,0 +1,58 @@
+"""How GEMMs of more than 16 rows are dealt to the CTA pairs: host code, no GPU."""
+import ctypes as C
+import time
+
+import pytest
+
+from paper_2410_05589_b200.binding import load_library
+
+SLOTS = 24 << 20
+P = 148 // 2
+
+
+def plan(rows, k, mats, zip_=0, planes=2, raw=0, slots=SLOTS, n_sm=148):
+    out = (C.c_int * 12)()
+    rc = load_library().ps_debug_gemm_plan(rows, k, len(mats), (C.c_int * len(mats))(*mats), zip_, planes, raw, slots, n_sm, out)
+    assert rc == 0, (rows, k, mats, rc)
+    keys = "wt Np row_tiles KB T whole shared split pairs most contributors slots"
+    return dict(zip(keys.split(), out))
+
+
+def stages(H, nq, nkv, F, V):
+    return [dict(k=2 * H, mats=[H], planes=1, raw=1), dict(k=H, mats=[nq * 128, nkv * 128, nkv * 128]),
+            dict(k=nq * 128, mats=[H], raw=1), dict(k=H, mats=[F, F], zip_=1), dict(k=F, mats=[H], raw=1),
+            dict(k=H, mats=[V])]
+
+
+MODELS = {"7b": stages(4096, 32, 32, 11008, 32000), "13b": stages(5120, 40, 40, 13824, 32000),
+          "llama3_8b": stages(4096, 32, 8, 14336, 128256), "mini": stages(768, 6, 6, 2072, 5000)}
+
+
+@pytest.mark.parametrize("model", sorted(MODELS))
+def test_every_row_count_has_a_plan_that_covers_its_tiles(model):
+    for rows in list(range(17, 130, 7)) + [160, 255, 256, 257, 288, 576, 640, 903, 1152, 2048]:
+        for st in MODELS[model]:
+            p = plan(rows, **st)
+            assert p["Np"] * p["row_tiles"] >= rows and p["Np"] % 32 == 0 and p["Np"] <= 256
+            assert p["whole"] % P == 0 and p["whole"] + p["shared"] == p["T"]
+            if not p["shared"]:
+                continue
+            # the runs of blocks, by their definition
+            S = p["shared"] * p["split"]
+            edges = [S * c // p["pairs"] for c in range(p["pairs"] + 1)]
+            tiles = [set(x // p["split"] for x in range(a, b)) for a, b in zip(edges, edges[1:])]
+            per_tile = [sum(t in r for r in tiles) for t in range(p["shared"])]
+            assert all(tiles) and max(per_tile) == p["most"] and sum(per_tile) == p["contributors"]
+            assert p["slots"] * p["Np"] * 256 * p["wt"] <= SLOTS
+
+
+def test_planning_a_step_is_quick():
+    """A server whose row count changes plans anew: 110 us a step when contributors were counted tile by tile."""
+    best = 1e9
+    for _ in range(5):
+        t0 = time.perf_counter()
+        for rows in range(20, 660, 20):
+            for st in MODELS["13b"]:
+                plan(rows, **st)
+        best = min(best, (time.perf_counter() - t0) / 32)
+    assert best < 80e-6, best

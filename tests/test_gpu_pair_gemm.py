@@ -39,3 +39,17 @@ def test_pair_gemm_shared_tiles_match_oracle(B, k):
         assert logits_close(got["logits"][b], p.oracle_step(b)["logits"], s.dtype) <= 1.0, b     # the logits gate
     assert p.g.check_guards() == 0 and p.g.poll() == 0
     assert np.array_equal(got["logits"], p.gpu_step(top_n=1)["logits"])
+
+
+def test_row_counts_change_on_one_context():
+    s = synth.CONFIGS["mini"].with_(k_masks=4)
+    B = 60
+    p = Pair(s, B, lens=[1 + (7 * b) % 41 for b in range(B)], oracle_seqs=[0])
+    want = p.oracle_step(0)["logits"]
+    first = {}
+    for n in (4, 60, 17, 4, 9, 33, 60, 17, 2, 9):     # rows 20, 300, 85, ..., and 10 on the kernels of up to 16
+        out = p.g.draft_step(list(range(n)), p.to_device(p.hidden_last[:n]), p.to_device(p.token_last[:n]), top_n=1)
+        got = out["logits"].cpu().numpy()
+        assert logits_close(got[0], want, s.dtype) <= 1.0, n     # the logits gate
+        assert np.array_equal(got, first.setdefault(n, got)), n
+    assert p.g.poll() == 0
