@@ -100,8 +100,11 @@ __device__ __forceinline__ void commit_pair(uint64_t* bar) {
 __device__ __forceinline__ void arrive_leader(uint64_t* bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(smem_u32(bar) & kPeerMask) : "memory");
 }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -221,16 +224,24 @@ k_pair_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     pdl_launch_dependents();
   }
+  __syncwarp();
+  // Tensor memory is allocated by the pair together: not before both CTAs run (an allocation that one of
+  // them asked for while the other was still to start left the other waiting for good), and the right
+  // to allocate is given up once both have it.
+  cluster_sync();   // both run, both CTAs' barriers are initialised
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl.tmem_base)), "r"(512)
                  : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    fence_before_sync();
   }
-  __syncthreads();
-  fence_before_sync();
-  cluster_sync();   // both CTAs' barriers are initialised, both have their tensor memory
-  fence_after_sync();
-  const uint32_t tmem = *(volatile uint32_t*)&ctl.tmem_base;
+  // (the producer needs no tensor memory: it waits for this barrier's phase only when it is done)
+  cluster_arrive();
+  if (warp != 0) {
+    cluster_wait();   // both have their tensor memory
+    fence_after_sync();
+  }
+  if (warp == 1) asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  const uint32_t tmem = warp == 0 ? 0u : *(volatile uint32_t*)&ctl.tmem_base;
   volatile int* abort_flag = &ctl.abort_flag;
 
   if (warp == 0) {
@@ -274,6 +285,8 @@ k_pair_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
         if (++st == nst) { st = 0; parity ^= 1; }
       }
     }
+    __syncwarp();
+    cluster_wait();
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {   // ---- MMA issuer of the pair
       SegWalk sw;

@@ -53,3 +53,17 @@ def test_row_counts_change_on_one_context():
         assert logits_close(got[0], want, s.dtype) <= 1.0, n     # the logits gate
         assert np.array_equal(got, first.setdefault(n, got)), n
     assert p.g.poll() == 0
+
+
+def test_many_steps_in_a_row():
+    """30 000 GEMM launches of CTA pairs behind one another, each behind kernels whose blocks may hold one SM of
+    a pair longer than the other (the pair's allocation of tensor memory must not mind)."""
+    s = synth.CONFIGS["mini"].with_(k_masks=4)
+    p = Pair(s, 6, lens=[1 + 5 * b for b in range(6)], oracle_seqs=[0])
+    hl, tl = p.to_device(p.hidden_last), p.to_device(p.token_last)
+    out = {}
+    first = p.g.draft_step(list(range(6)), hl, tl, out=out)["logits"].cpu().numpy()
+    for _ in range(5000):
+        p.g.draft_step(list(range(6)), hl, tl, out=out)
+    assert p.g.poll() == 0 and np.array_equal(first, out["logits"].cpu().numpy())
+    assert logits_close(first[0], p.oracle_step(0)["logits"], s.dtype) <= 1.0     # the logits gate
