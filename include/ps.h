@@ -98,7 +98,11 @@ typedef struct ps_weights {
 } ps_weights;
 
 /* Bytes of device workspace ps_init needs for this configuration (KV slabs for max_batch
- * slots, activation buffers, verify scratch).  Returns 0 if the configuration is invalid. */
+ * slots, activation buffers, verify scratch).  Returns 0 if the configuration is invalid.
+ * Beside the slabs: what a step of max_batch * (k_masks + 1) rows and, on the tensor-core kernels, one
+ * pass of ps_kv_append need (2048 rows, or half of all cache rows if that is less, 128 at least).
+ * 13B shape: 112 MB for one sequence of 1024 positions, 230 MB for 4 of 2100, 682 MB for 64 of 2100
+ * with 8 masks (slabs 21, 172 and 2753 MB). */
 size_t ps_workspace_bytes(const ps_config* cfg);
 
 /* Creates a context.  `workspace` is device memory of at least ps_workspace_bytes(cfg) bytes,

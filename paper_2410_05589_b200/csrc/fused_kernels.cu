@@ -417,8 +417,9 @@ struct FusedScratch {
   __nv_bfloat16* xin;       // [rows][2H] gathered fc input (exact bf16: one plane)
   float* partials;          // [kMaxSm][2][16][128] partial tiles of CTAs that share a tile (up to 16 rows)
   float* slots; size_t slot_floats;   // partial tiles of the CTA-pair GEMM
+  float* kv_slots; size_t kv_slot_floats;   // those of an append's k | v projection
   atc::Buffers at;          // tensor-memory attention
-  float* kv;                // [append rows][2 Hkv] k | v of appended positions before RoPE
+  float* kv;                // [append rows][2 Hkv] k | v of appended positions before RoPE (on top of xin, slots)
   unsigned* tile_tickets;   // one per tile of the widest stage, zero between launches
   unsigned* chain_ctr;      // chained stages: finished-tile and passed-CTA counts, zero between launches
   int n_part_rows;          // rows of `parts` and of each ssq array
@@ -470,19 +471,28 @@ FusedScratch carve_fused(const ps_config& g, char* base) {
   const size_t att = std::max<size_t>((size_t)kMaxM * kAttnMaxSplit, rd) * g.n_heads;
   s.att_ml = (float*)take(att * 2 * 4);
   s.att_o = (float*)take(att * g.head_dim * 4);
-  s.act = (float*)take(rd * g.ffn * 4);
+  s.act = (float*)take((size_t)kMaxM * g.ffn * 4);
   // per-CTA (mma.sync path) or per-tile (tensor-core path) summaries
   s.n_part_rows = std::max(kMaxSm, std::max(tiles_v, tiles_h));
   s.parts = (LmPart*)take((size_t)s.n_part_rows * kMaxM * sizeof(LmPart));
   for (int i = 0; i < 3; ++i) s.ssq[i] = (float*)take((size_t)s.n_part_rows * kMaxM * 4);
-  s.xin = (__nv_bfloat16*)take(rx * 2 * g.hidden * 2);
   s.partials = (float*)take((size_t)kMaxSm * 2 * kMaxM * 128 * 4);
-  // room for one contributor of every pair of a 148-SM chip at the largest tile twice over, and for
-  // two contributors of every row of a hidden-wide stage
+  // The gathered fc input, then the slots: every row of a hidden-wide stage once (any plan's least), and
+  // for contributors beyond the first a tile of 512 features for every pair, of 320 up to 1024 rows (with
+  // that the plans are those that unbounded slots give, 7B to 33B shapes).  An append's k | v rows lie on
+  // top of the fc input and of the slots that the norm before them has read, and their own GEMM's slots
+  // behind both.
+  const size_t np_max = std::min<size_t>(pg::kMaxNp, (rx + pg::kNpStep - 1) / pg::kNpStep * pg::kNpStep);
   const size_t h_pad = ((size_t)g.hidden + 511) / 512 * 512, r_pad = (rx + 511) / 256 * 256;
-  s.slot_floats = std::max<size_t>((size_t)2 * (kMaxSm / 2) * 256 * pg::kMaxNp / 4 * 3, 2 * r_pad * h_pad);
-  s.slots = (float*)take(s.slot_floats * 4);
-  s.kv = (float*)take(ra * 2 * Hkv * 4);
+  const size_t more = (size_t)(kMaxSm / 2) * (rx > 1024 ? 512 : 320) * np_max * 4, xin = (rx * 2 * g.hidden * 2 + 255) & ~(size_t)255;
+  const size_t kv = (ra * 2 * Hkv * 4 + 255) & ~(size_t)255, kv_end = std::max(xin, kv);
+  const size_t region = std::max(xin + r_pad * h_pad * 4, kv_end) + more;
+  s.xin = (__nv_bfloat16*)take(region);
+  s.kv = (float*)s.xin;
+  s.slots = base ? (float*)((char*)s.xin + xin) : nullptr;
+  s.slot_floats = (region - xin) / 4;
+  s.kv_slots = base ? (float*)((char*)s.xin + kv_end) : nullptr;
+  s.kv_slot_floats = (region - kv_end) / 4;
   s.at = atc::carve(g, take(atc::bytes(g)));
   s.x0p = planes(rx, g.hidden); s.ap = planes(rd, g.hidden); s.hdnp = planes(rd, g.hidden);
   s.attnp = planes(rd, Hq); s.actp = planes(rd, g.ffn);
@@ -1654,6 +1664,7 @@ struct PlaneMaps {   // one activation plane: boxes of 16 rows, and of every siz
 };
 constexpr int kPlanSlots = 128;
 constexpr int kPairStages = 8;   // fc, q|k|v, o, gate|up, down, LM head of a draft step; fc, k|v of an append
+constexpr int kAppendKv = 7;
 struct UmmaMaps {
   CUtensorMap w_fc, w_q, w_k, w_v, w_o, w_gate, w_up, w_down, w_lm;
   CUtensorMap w_gate128, w_up128;   // 128-row boxes (the others' gate / up boxes: 64 rows)
@@ -1807,11 +1818,12 @@ ps_status run_stages(ps_ctx* c, StageDesc* d, int n, bool chain, int chain_id, c
 // `id` names the stage's place in the plan cache.
 ps_status pair_stage(ps_ctx* c, UmmaMaps& u, int id, pg::Mode mode, int M, int K, int planes, const pg::Weights& w,
                      const PlaneMaps& hi, const PlaneMaps& lo, const FusedScratch& f, pg::Args& a, cudaStream_t st) {
+  const bool kv = id == kAppendKv;
   pg::Plan& plan = u.plan[id][(uint32_t)M * 2654435761u >> 25];   // (the counts of one context spread over the slots)
-  if (plan.T == 0 || plan.M != M) plan = pg::make_plan(M, w, K, planes, mode, f.slot_floats, c->n_sm);
+  if (plan.T == 0 || plan.M != M) plan = pg::make_plan(M, w, K, planes, mode, kv ? f.kv_slot_floats : f.slot_floats, c->n_sm);
   a.p = plan;
   a.planes = planes;
-  a.part = f.slots;
+  a.part = kv ? f.kv_slots : f.slots;
   ps_status s = pg::launch_gemm(c, w, hi.pair, lo.pair, a, mode, st);
   if (s == PS_OK && mode != pg::MODE_RAW) s = pg::launch_finish_shared(c, a, mode, st);
   return s;
@@ -1840,7 +1852,7 @@ ps_status pair_kv_append(ps_ctx* c, UmmaMaps& u, const SeqMap& sm, int rows, con
   prof_mark(c, st, "fc_norm");
   pg::Args b{};
   b.out = f.kv; b.ldo = 2 * Hkv;
-  if ((s = pair_stage(c, u, 7, pg::MODE_STORE, rows, H, 2, pg::Weights{{&u.w_k, &u.w_v}, {Hkv, Hkv}, 2, false}, u.x0_hi,
+  if ((s = pair_stage(c, u, kAppendKv, pg::MODE_STORE, rows, H, 2, pg::Weights{{&u.w_k, &u.w_v}, {Hkv, Hkv}, 2, false}, u.x0_hi,
                       u.x0_lo, f, b, st)))
     return s;
   if ((s = launch_rope_store_kv(c, sm, rows, f.kv, st))) return s;
@@ -2184,12 +2196,15 @@ ps_status fused_debug_buffer(ps_ctx* c, const char* name, void** ptr, size_t* by
     if (c->act_rows > 0) {   // with more than 16 rows the step keeps only the planes of act
       const size_t n = (size_t)c->act_rows * g.ffn;
       cudaError_t e = cudaDeviceSynchronize();
-      k_join_planes<<<148, 256>>>(f.actp.hi, f.actp.lo, f.act, n);
+      k_join_planes<<<148, 256>>>(f.actp.hi, f.actp.lo, c->gate, n);   // (a buffer of the plain kernels)
       if (e == cudaSuccess) e = cudaDeviceSynchronize();
       if (e != cudaSuccess) return cuda_check(c, e, "act planes");
+      *ptr = c->gate;
+      *bytes = n * 4;
+      return PS_OK;
     }
     *ptr = f.act;
-    *bytes = rd * g.ffn * 4;
+    *bytes = (size_t)kMaxM * g.ffn * 4;
     return PS_OK;
   }
   return PS_ERR_INVALID_ARG;

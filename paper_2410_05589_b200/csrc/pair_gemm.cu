@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(NT) k_row_norm(const __grid_constant__ Args a,
   const int m = blockIdx.x, rt = m / p.Np, mi = m - rt * p.Np, tid = threadIdx.x, nthr = blockDim.x;
   const int sh = p.wt == 2 ? 9 : 8, TW = 1 << sh;
   const bool out_vec = ((uintptr_t)out & 15) == 0;     // (the caller's feature rows may sit anywhere)
-  const size_t layer = (size_t)p.slot_T * p.Np * TW;   // floats between contributors
+  const size_t layer = (size_t)p.Np * TW;              // floats between a tile's contributors
   float4 x[NV];
   const float* slot[NV];
   int cnt[NV], cmax = 0;
@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(NT) k_row_norm(const __grid_constant__ Args a,
       const int t = (n >> sh) * p.n_rt + rt;
       cnt[i] = tile_contributors(p, t);
       cmax = max(cmax, cnt[i]);
-      slot[i] += ((size_t)t * p.Np + mi) * TW + (n & (TW - 1));
+      slot[i] += slot_row(p, 0, t, mi) + (n & (TW - 1));
       if (bias) x[i] = load_bf4(bias + n);
     }
   }
@@ -615,8 +615,7 @@ Plan make_plan(int M, const Weights& w, int K, int planes, Mode mode, size_t par
     // known, so these tiles always have two sub-tiles, as they had.
     if (mode != MODE_SWIGLU && wt == 1 && p.Np == kMaxNp && p.T > P) continue;
     p.slot_t0 = mode == MODE_RAW ? 0 : p.n_dp;
-    p.slot_T = p.T - p.slot_t0;
-    const size_t layer = (size_t)p.slot_T * p.Np * 256 * wt;
+    const size_t slot = (size_t)p.Np * 256 * wt;
     for (int s = 1; s <= std::min(kMaxSplit, p.KB); ++s) {
       if (p.rem == 0 && s > 1) break;
       p.split = s;
@@ -650,7 +649,7 @@ Plan make_plan(int M, const Weights& w, int K, int planes, Mode mode, size_t par
         segs += runs;
       }
       p.shared = jmax > 1;
-      if (layer * ((mode == MODE_RAW || jmax > 1) ? jmax : 0) > part_floats) continue;
+      if ((mode == MODE_RAW || jmax > 1) && slot_tiles(p) * slot > part_floats) continue;
       cost += finish_cost(p, mode, segs, jmax, n_slots);
       if (cost < best_cost) { best_cost = cost; best = p; }
     }

@@ -19,13 +19,16 @@ constexpr int kMaxSplit = 16;     // k blocks a shared tile is dealt in
 // each of the `rem` tiles behind them is cut into `split` blocks and the S = rem * split blocks
 // are dealt to the first Pe pairs as contiguous runs, so that the last wave keeps every pair busy.
 // A pair that holds part of a tile's k range is its contributor number j (in k order) and
-// leaves its sums in slot (j, tile).
+// leaves its sums in a slot.  Slots are as large as a tile: one for every whole tile that goes
+// through them, then one for every (shared tile, contributor), in the order of the runs, at
+// shared tile + pair (from one to the next the tile, the pair or both go up by one, so these
+// numbers are distinct and below rem + Pe).  A tile's contributors lie one behind the other.
 struct Plan {
   int M, Np, n_rt;          // activation rows, rows per row tile, row tiles
   int wt, tiles_w;          // 128-row sub-tiles per CTA; weight tiles over all matrices
   int KB;                   // k-blocks of 64 columns
   int T, n_dp, rem, split, S, Pe;
-  int slot_t0, slot_T;      // first tile that has slots, tiles per contributor layer
+  int slot_t0;              // first tile that has slots
   int shared;               // some tile has more than one contributor
   int n_mats, mat_tiles[3], mat_rows[3], mat_off[3];
 };
@@ -38,10 +41,14 @@ __host__ __device__ inline int tile_contributors(const Plan& p, int t) {
   const int x = (t - p.n_dp) * p.split;
   return run_owner(p, x + p.split - 1) - run_owner(p, x) + 1;
 }
-// Element offset of row mi of slot (j, t): rows of TW floats.
+// Element offset of row mi of contributor j's slot of tile t: rows of TW floats.
 __host__ __device__ inline size_t slot_row(const Plan& p, int j, int t, int mi) {
-  return (((size_t)j * p.slot_T + (t - p.slot_t0)) * p.Np + mi) * (size_t)(256 * p.wt);
+  int s = t - p.slot_t0 + j;
+  if (t >= p.n_dp && p.split > 1) s += run_owner(p, (t - p.n_dp) * p.split);   // (else one pair a tile: its number)
+  return ((size_t)s * p.Np + mi) * (size_t)(256 * p.wt);
 }
+// Tiles the slots must hold.
+__host__ __device__ inline int slot_tiles(const Plan& p) { return p.T - p.slot_t0 + (p.split > 1 ? p.Pe - 1 : 0); }
 
 enum Mode {
   MODE_RAW = 0,      // every tile's sums go to slots; a row kernel finishes them

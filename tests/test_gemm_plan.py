@@ -46,6 +46,29 @@ def test_every_row_count_has_a_plan_that_covers_its_tiles(model):
             assert p["slots"] * p["Np"] * 256 * p["wt"] <= SLOTS
 
 
+def test_last_wave_of_a_long_append_keeps_the_pairs_busy():
+    """fc of 2048 rows, 13B shape: 80 tiles on 74 pairs.  With slots for two contributors of every tile the six
+    tiles of the last wave could be cut in two only, and 62 pairs waited for them: 72% of the pairs' time."""
+    cap = (2048 + 256) * 5120 + 96 * 512 * 256
+    p = plan(2048, 10240, [5120], planes=1, raw=1, slots=cap)
+    whole = p["whole"] // P * p["KB"]
+    blocks = -(-p["shared"] * p["split"] // p["pairs"])
+    most = whole + blocks * -(-p["KB"] // p["split"])
+    assert p["T"] * p["KB"] / (P * most) > 0.9, p
+
+
+def test_workspace_beside_the_caches():
+    """Scratch of a context, in MB beside its K/V slabs (13B: 311 and 794 with the earlier slots)."""
+    from paper_2410_05589_b200.binding import ps_config
+    lib = load_library()
+    for shape, B, ctx, k, most in (((5120, 40, 40, 13824, 32000), 1, 1029, 4, 115), ((5120, 40, 40, 13824, 32000), 4, 2100, 4, 235),
+                                   ((5120, 40, 40, 13824, 32000), 64, 2100, 8, 690), ((4096, 32, 8, 14336, 128256), 1, 1100, 4, 105)):
+        H, nh, nkv, F, V = shape
+        cfg = ps_config(1, H, nh, nkv, 128, F, V, k, B, ctx, 1e4, 1e-5, 0)
+        n = lib.ps_workspace_bytes(C.byref(cfg)) - 2 * B * nkv * ctx * 128 * 2
+        assert 0 < n <= most * 1e6, (shape, B, n)
+
+
 def test_planning_a_step_is_quick():
     """A server whose row count changes plans anew: 110 us a step when contributors were counted tile by tile."""
     best = 1e9

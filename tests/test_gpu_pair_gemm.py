@@ -67,3 +67,30 @@ def test_many_steps_in_a_row():
         p.g.draft_step(list(range(6)), hl, tl, out=out)
     assert p.g.poll() == 0 and np.array_equal(first, out["logits"].cpu().numpy())
     assert logits_close(first[0], p.oracle_step(0)["logits"], s.dtype) <= 1.0     # the logits gate
+
+
+def test_long_append_with_whole_and_shared_tiles():
+    """2048 new rows, hidden 5120: the fc's 80 tiles are one wave of whole ones and six shared ones, all
+    through slots; k | v of the same pass lie on top of the fc's input and slots.  Twice, so that a pass
+    follows one of another length."""
+    import paper_2410_05589_b200 as ps
+    import torch
+    from harness import oracle_for
+    B, n, n2 = 128, 16, 3
+    s = synth.CONFIGS["mini"].with_(hidden=5120, n_heads=2, n_kv_heads=2, ffn=64, vocab=1000, k_masks=1)
+    W = synth.weights(s)
+    g = ps.drafter_from_shape(s, W, max_batch=B, max_ctx=40)
+    seqs = [0, 77, B - 1]
+    o = oracle_for(s, W, B, 40)
+    for part, m in ((0, n), (1, n2), (2, n)):
+        h, t = synth.hidden_states(s, ("new", part), B * m), synth.token_ids(s, ("new", part), B * m)
+        g.kv_append(list(range(B)), [m] * B, ps.to_device(h), ps.to_device(t))
+        for b in seqs:
+            assert o.kv_append(b, h[b * m:(b + 1) * m], t[b * m:(b + 1) * m]) == 0
+    torch.cuda.synchronize()
+    for b in seqs:
+        got = [x.float().cpu().numpy() for x in g.kv_export(b)]
+        for a, w in zip(got, o.kv_export(b)):
+            # values that agree to fp32 sums of 5120 and 10240 terms, rounded to bf16: one unit in the last place
+            assert (np.abs(a - w) <= 2.0 ** -7 * np.abs(w) + 1e-4).all(), b
+    assert g.poll() == 0 and g.check_guards() == 0
