@@ -478,13 +478,13 @@ FusedScratch carve_fused(const ps_config& g, char* base) {
   for (int i = 0; i < 3; ++i) s.ssq[i] = (float*)take((size_t)s.n_part_rows * kMaxM * 4);
   s.partials = (float*)take((size_t)kMaxSm * 2 * kMaxM * 128 * 4);
   // The gathered fc input, then the slots: every row of a hidden-wide stage once (any plan's least), and
-  // for contributors beyond the first a tile of 512 features for every pair, of 320 up to 1024 rows (with
+  // for contributors beyond the first a tile of 512 features for every pair, of 352 up to 768 rows (with
   // that the plans are those that unbounded slots give, 7B to 33B shapes).  An append's k | v rows lie on
   // top of the fc input and of the slots that the norm before them has read, and their own GEMM's slots
   // behind both.
   const size_t np_max = std::min<size_t>(pg::kMaxNp, (rx + pg::kNpStep - 1) / pg::kNpStep * pg::kNpStep);
   const size_t h_pad = ((size_t)g.hidden + 511) / 512 * 512, r_pad = (rx + 511) / 256 * 256;
-  const size_t more = (size_t)(kMaxSm / 2) * (rx > 1024 ? 512 : 320) * np_max * 4, xin = (rx * 2 * g.hidden * 2 + 255) & ~(size_t)255;
+  const size_t more = (size_t)(kMaxSm / 2) * (rx > 768 ? 512 : 352) * np_max * 4, xin = (rx * 2 * g.hidden * 2 + 255) & ~(size_t)255;
   const size_t kv = (ra * 2 * Hkv * 4 + 255) & ~(size_t)255, kv_end = std::max(xin, kv);
   const size_t region = std::max(xin + r_pad * h_pad * 4, kv_end) + more;
   s.xin = (__nv_bfloat16*)take(region);

@@ -610,9 +610,9 @@ Plan make_plan(int M, const Weights& w, int K, int planes, Mode mode, size_t par
     p.T = p.tiles_w * p.n_rt;
     p.n_dp = p.T / P * P;
     p.rem = p.T - p.n_dp;
-    // Several full tiles a pair, two accumulators of 256 columns: modelled 5% shorter than two
-    // sub-tiles on prompts, but such calls stopped making progress now and then; the cause is not
-    // known, so these tiles always have two sub-tiles, as they had.
+    // Several full tiles a pair, two accumulators of 256 columns: the model has them 4% shorter than two
+    // sub-tiles on prompts.  They are on 7B shapes (4096 rows 676 -> 639 us), but 13B ones are 3% and 33B
+    // ones 16% longer (1527 -> 1778), so these tiles always have two sub-tiles.
     if (mode != MODE_SWIGLU && wt == 1 && p.Np == kMaxNp && p.T > P) continue;
     p.slot_t0 = mode == MODE_RAW ? 0 : p.n_dp;
     const size_t slot = (size_t)p.Np * 256 * wt;
