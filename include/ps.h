@@ -101,7 +101,7 @@ typedef struct ps_weights {
  * slots, activation buffers, verify scratch).  Returns 0 if the configuration is invalid.
  * Beside the slabs: what a step of max_batch * (k_masks + 1) rows and, on the tensor-core kernels, one
  * pass of ps_kv_append need (2048 rows, or half of all cache rows if that is less, 128 at least).
- * 13B shape: 112 MB for one sequence of 1024 positions, 230 MB for 4 of 2100, 682 MB for 64 of 2100
+ * 13B shape: 116 MB for one sequence of 1024 positions, 230 MB for 4 of 2100, 682 MB for 64 of 2100
  * with 8 masks (slabs 21, 172 and 2753 MB). */
 size_t ps_workspace_bytes(const ps_config* cfg);
 
