@@ -572,7 +572,9 @@ ps_status draft_impl(ps_ctx* c, const SeqMap& sm, int B, const void* hidden_last
     if ((s = linear<WT, LIN_RES>(c, x, st))) return s;
   }
   prof_mark(c, st, "o_proj");
-  float* hdn = feat_out ? feat_out : c->hdn;
+  // (the LM head reads these rows in 16-byte vectors; the caller's feature rows may sit anywhere)
+  const bool in_place = feat_out && ((uintptr_t)feat_out & 15) == 0;
+  float* hdn = in_place ? feat_out : c->hdn;
   {
     LinArgs<WT> x = a;
     x.X = c->a; x.ldx = H; x.K = H; x.gain = (P)w.g_post;
@@ -588,6 +590,10 @@ ps_status draft_impl(ps_ctx* c, const SeqMap& sm, int B, const void* hidden_last
     LinArgs<WT> x = a;
     x.X = hdn; x.ldx = H; x.K = H; x.gain = (P)w.g_final; x.W[0] = (P)w.w_lm; x.n[0] = V; x.Y[0] = logits; x.ldy[0] = V;
     if ((s = linear<WT, LIN_NORM>(c, x, st))) return s;
+  }
+  if (feat_out && !in_place) {
+    const cudaError_t ce = cudaMemcpyAsync(feat_out, hdn, (size_t)M * H * 4, cudaMemcpyDeviceToDevice, st);
+    if (ce != cudaSuccess) return cuda_check(c, ce, "feature rows");
   }
   if ((s = launch_logit_stats(c, logits, M, V, g.k_masks + 1, top_n, top_ids, top_logit, row_max, row_lse, sa, st)))
     return s;

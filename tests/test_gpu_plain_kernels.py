@@ -28,3 +28,22 @@ def test_plain_draft_step_matches_oracle(name, over, B, k, lens, bias):
         assert logits_close(got["logits"][b], want["logits"], s.dtype) <= 1.0, b     # the logits gate
         assert logits_close(got["feat"][b], want["feat"], s.dtype) <= 1.0, b
     assert np.isfinite(got["logits"]).all() and p.g.check_guards() == 0
+
+
+# feature and logit rows one float off a 16-byte boundary: fp32, bf16 on these kernels, the chained
+# launches, CTA pairs (H and vocab multiples of 4, so that every row is off)
+@pytest.mark.parametrize("name,B,flags", [("mini32", 2, 0), ("mini", 2, 2), ("mini", 2, 0), ("mini", 6, 0), ("mini", 2, 4)])
+def test_outputs_at_any_address(name, B, flags):
+    import torch
+    s = synth.CONFIGS[name]
+    p = Pair(s, B, lens=[9 + 7 * b for b in range(B)], flags=flags)
+    want = p.gpu_step(top_n=2)
+    R, V, H = s.rows, s.vocab, s.hidden
+    out = {"top_ids": torch.empty((B, R, 2), dtype=torch.int32, device="cuda"), "top_logit": torch.empty((B, R, 2), device="cuda"),
+           "row_max": torch.empty((B, R), device="cuda"), "row_lse": torch.empty((B, R), device="cuda"),
+           "logits": torch.empty(B * R * V + 1, device="cuda")[1:].view(B, R, V),
+           "feat": torch.empty(B * R * H + 1, device="cuda")[1:].view(B, R, H)}
+    p.g.draft_step(list(range(B)), p.to_device(p.hidden_last), p.to_device(p.token_last), top_n=2, out=out)
+    assert p.g.poll() == 0
+    for k in ("logits", "feat", "top_ids"):
+        assert np.array_equal(out[k].cpu().numpy(), want[k]), k
