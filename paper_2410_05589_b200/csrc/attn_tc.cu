@@ -344,6 +344,8 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
         first.start(w, u0, u1);
         load_q(first.b, first.hk, 0);
       };
+      // (Cached tiles are asked for before the wait: what stored them belongs to a call before this one or to
+      // its append, and the first kernel of a step lets the others start only when that is complete.)
       auto load = [&](const Walk& x, int v) {
         if (n_issued >= NS || x.in_tail) need_dep();
         if (n_issued >= NS && !mbar_wait(&ctl.empty[slot], (use & 1) ^ 1, abort_flag)) { alive = false; return; }

@@ -1569,8 +1569,11 @@ __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_c
 __global__ void k_gather_x(const __nv_bfloat16* __restrict__ embed, const __nv_bfloat16* __restrict__ mask_embed,
                            const __nv_bfloat16* __restrict__ mask_feat, const __nv_bfloat16* __restrict__ hidden,
                            const int* __restrict__ tokens, int H, int V, int R, __nv_bfloat16* __restrict__ xin) {
-  pdl_launch_dependents();
+  // The first kernel of a call waits before it lets the next ones start: those ask for weights and cached
+  // keys ahead of their own waits, and whatever was enqueued before the call may have written them.
+  // (Letting them start first is worth 0.2-0.7% of a step: 13B, one sequence 243.8 -> 245.6 us.)
   pdl_wait();
+  pdl_launch_dependents();
   const int m = blockIdx.x, b = m / R, j = m - b * R;
   const __nv_bfloat16 *e, *f;
   if (j == 0) {
@@ -1600,8 +1603,8 @@ __global__ void __launch_bounds__(256) k_embed_x0(const __nv_bfloat16* __restric
                                                   __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
                                                   float* __restrict__ ssq, int normalise, float eps) {
   __shared__ float s_part[8];
+  pdl_wait();   // (first: see k_gather_x)
   pdl_launch_dependents();
-  pdl_wait();
   const int m = blockIdx.x, b = m / R, j = m - b * R;
   const __nv_bfloat16* e = j == 0 ? embed + (size_t)min(max(tokens[b], 0), V - 1) * H : mask_embed + (size_t)(j - 1) * H;
   float ss = 0.f;

@@ -74,8 +74,8 @@ __device__ __forceinline__ void gather_row(const GatherSrc<WT>& g, const SeqMap&
 // Embedding-only input (PS_FLAG_NO_FC): x0 is the embedding half.
 template <typename WT>
 __global__ void __launch_bounds__(256) k_gather_embed(const __grid_constant__ SeqMap sm, GatherSrc<WT> g, float* x0) {
+  pdl_wait();   // (first: see k_linear)
   pdl_launch_dependents();
-  pdl_wait();
   const WT *e, *f;
   gather_row(g, sm, blockIdx.x, e, f);
   for (int i = threadIdx.x; i < g.H; i += blockDim.x) x0[(size_t)blockIdx.x * g.H + i] = to_f32(e[i]);
@@ -137,6 +137,10 @@ __device__ __forceinline__ float4 load4_any(const WT* p, bool vec) {
 constexpr int kKC = 512;
 template <typename WT, int KIND, int MC, typename GA>
 __global__ void __launch_bounds__(256) k_linear(const __grid_constant__ LinArgs<WT> a, const __grid_constant__ GA ga) {
+  // The first kernel of a call: whatever the caller enqueued before it, an update of the weights for
+  // one, is complete before it reads and before any kernel behind it, which asks for weights
+  // ahead of its own wait, can start.
+  if (KIND == LIN_GATHER) pdl_wait();
   pdl_launch_dependents();
   constexpr bool kNorm = KIND == LIN_NORM || KIND == LIN_SWIGLU, kTwo = KIND == LIN_SWIGLU;
   constexpr int C = kKC / 128;                    // float4 groups of a warp per chunk

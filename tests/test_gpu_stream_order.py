@@ -68,3 +68,27 @@ def test_draft_step_and_append_find_late_inputs(name, B):
 
     for a, b in zip(run(False), run(True)):
         assert np.array_equal(a, b)
+
+
+# weights written by the kernel just ahead (an optimiser's step): fp32 activations (2: these kernels), chained
+# launches, CTA pairs; 8: no fc
+@pytest.mark.parametrize("name,B,flags", [("tiny", 1, 0), ("mini", 1, 2), ("mini", 1, 10), ("mini", 1, 0), ("mini", 6, 0),
+                                          ("mini", 1, 8), ("mini", 6, 8)])
+def test_draft_step_finds_late_weights(name, B, flags):
+    import paper_2410_05589_b200 as ps
+    s = synth.CONFIGS[name].with_(batch=B)
+    g = ps.drafter_from_shape(s, synth.weights(s), max_batch=B, max_ctx=32, flags=flags)
+    hl, tl = ps.to_device(synth.hidden_states(s, "last", B)), ps.to_device(synth.token_ids(s, "last", B))
+    slots = list(range(B))
+    want = g.draft_step(slots, hl, tl)["logits"].clone()
+    for n in ("w_fc", "w_q", "w_o", "w_up", "w_down", "w_lm"):
+        if flags & 8 and n == "w_fc":
+            continue
+        w = g.weights[n]
+        true = w.clone()
+        w.zero_()
+        torch.cuda.synchronize()
+        g.debug_late_copy(w, true, 30)
+        got = g.draft_step(slots, hl, tl)["logits"]
+        torch.cuda.synchronize()
+        assert torch.equal(got, want), n
