@@ -89,10 +89,11 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
   const float* row = logits + (size_t)m * V;
   const int share = ((V + nclu - 1) / nclu + 3) & ~3;          // tokens per block, whole vectors
   const int v_lo = min(V, rank * share), v_hi = min(V, v_lo + share);
-  const bool vec = ((uintptr_t)(row + v_lo) & 15) == 0;
-  const int n_vec = vec ? (v_hi - v_lo) / 4 : 0;
-  const float4* row4 = reinterpret_cast<const float4*>(row + v_lo);
-  const int tail = v_lo + 4 * n_vec;                            // tokens from here on one by one
+  // vectors from the first 16-byte boundary on; the up to three tokens before it and after them one by one
+  const int v_al = min(v_hi, v_lo + (int)((16u - ((unsigned)(uintptr_t)(row + v_lo) & 15u)) & 15u) / 4);
+  const int n_vec = (v_hi - v_al) / 4, n_head = v_al - v_lo, n_one = v_hi - v_lo - 4 * n_vec;
+  const float4* row4 = reinterpret_cast<const float4*>(row + v_al);
+  auto one_at = [&](int i) { return i < n_head ? v_lo + i : v_al + 4 * n_vec + (i - n_head); };
   uint32_t row_id = 0;
   if (SAMPLE) {
     const int b = m / R;
@@ -137,7 +138,7 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (i0 + u * kThreads < n_vec) {
-          const int v = v_lo + 4 * (i0 + u * kThreads);
+          const int v = v_al + 4 * (i0 + u * kThreads);
           sample_one(x[u].x, v); sample_one(x[u].y, v + 1); sample_one(x[u].z, v + 2); sample_one(x[u].w, v + 3);
         }
         const unsigned k = __reduce_max_sync(0xffffffffu, key_of(gv));
@@ -148,7 +149,8 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
       if (k) thr = fmaxf(thr, key_value(k));
     }
   }
-  for (int v = tail + tid; v < v_hi; v += kThreads) {
+  if (tid < n_one) {
+    const int v = one_at(tid);
     const float x = __ldcg(row + v), bm = fmaxf(mx, x);
     se = se * __expf(mx - bm) + __expf(x - bm);
     mx = bm;
@@ -208,18 +210,18 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
       if (held) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int i = tid + u * kThreads, v = v_lo + 4 * i;
+          const int i = tid + u * kThreads, v = v_al + 4 * i;
           if (i < n_vec) { offer(x[u].x, v); offer(x[u].y, v + 1); offer(x[u].z, v + 2); offer(x[u].w, v + 3); }
         }
       } else {
 #pragma unroll 4
         for (int i = tid; i < n_vec; i += kThreads) {
           const float4 y = __ldcg(row4 + i);
-          const int v = v_lo + 4 * i;
+          const int v = v_al + 4 * i;
           offer(y.x, v); offer(y.y, v + 1); offer(y.z, v + 2); offer(y.w, v + 3);
         }
       }
-      for (int v = tail + tid; v < v_hi; v += kThreads) offer(__ldcg(row + v), v);
+      if (tid < n_one) offer(__ldcg(row + one_at(tid)), one_at(tid));
     }
     __syncthreads();
     const int n_list = s.n_list;
