@@ -669,10 +669,11 @@ __device__ __forceinline__ void tile_epilogue(const UArgs& a, umma::Ctl& ctl, in
       }
     }
     epi_sync();
-  } else {  // EPI_LMHEAD (the logits stay out of memory): the tile's softmax / top-n summary per row
+  } else {  // EPI_LMHEAD: the logits if they are kept, and the tile's softmax / top-n summary per row
 #pragma unroll 1
     for (int m = 0; m < mc; ++m) {
       const float x = acc[m * 128] * ctl.scale[m0 + m];
+      if (valid && a.out && !dry) a.out[(size_t)(m0 + m) * a.ldo + n] = x;
       float mx = valid ? x : -FLT_MAX;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -1986,6 +1987,9 @@ ps_status umma_kv_append(ps_ctx* c, UmmaMaps& u, const SeqMap& sm, int rows, con
   return PS_OK;
 }
 
+// Most rows whose kept logits get their statistics in the LM head's epilogue (see below).
+constexpr int kEpiRows = 5, kEpiRowsSampled = 6;
+
 ps_status umma_draft_step(ps_ctx* c, UmmaMaps& u, const SeqMap& sm, int B, const void* hidden_last,
                           const int* token_last, int top_n, int* top_ids, float* top_logit, float* row_max,
                           float* row_lse, float* logits_out, float* feat_out, const SampleArgs* sa,
@@ -2072,11 +2076,14 @@ ps_status umma_draft_step(ps_ctx* c, UmmaMaps& u, const SeqMap& sm, int B, const
     a.ssq_out = f.ssq[2];
     a.out_hi = f.hdnp.hi; a.out_lo = f.hdnp.lo; a.ld_plane = H; a.gain_next = (BP)w.g_final;
   }
-  // With the logits kept, the last stage only stores them and the statistics are a pass of their own
-  // over L2: the tile epilogue's reductions are serial in rows, picks and tiles (128256 tokens, 5
-  // rows, top-4: chained launch 362 -> 245 us and 14 us for the pass; 32000 tokens, sampled: 167 ->
-  // 155 and 14, the same in all).
-  const bool stats_pass = logits_out != nullptr;
+  // With the logits kept, the last stage of many rows or picks only stores them and the statistics are a
+  // pass of their own over L2: the tile epilogue's reductions are serial in rows, picks and tiles
+  // (128256 tokens, 5 rows, top-4: chained launch 362 -> 245 us and 14 us for the pass).  With one pick
+  // and few rows the epilogue is the shorter one (7B shape, sampled: 1 row 176 -> 170 us, 5 rows even, 9
+  // rows 190 -> 198; 128256 tokens 1 row 299 -> 285, 5 rows 305 -> 301; arg-max: 1 row 169 -> 167.5, 9 rows 185
+  // -> 191).
+  const bool wanted = top_n > 0 || row_max || row_lse || sa;
+  const bool stats_pass = logits_out && !(wanted && top_n <= 1 && M <= (sa ? kEpiRowsSampled : kEpiRows));
   {  // S6 logits = W_lm rms(hdn), softmax statistics and top-n without a second pass over logits
     StageDesc& x = d[n++];
     x = StageDesc{EPI_LMHEAD, &u.w_lm, &u.w_lm, &u.w_lm, &u.hdn_hi, &u.hdn_lo, UArgs{}, "lm_head"};
@@ -2088,6 +2095,7 @@ ps_status umma_draft_step(ps_ctx* c, UmmaMaps& u, const SeqMap& sm, int B, const
       a.out = logits_out; a.ldo = V;
       x.name = nullptr;   // (timed together with the statistics below)
     } else {
+      a.out = logits_out; a.ldo = V;
       a.parts = f.parts; a.ticket = f.ticket;
       a.top_n = top_n; a.top_ids = top_ids; a.top_logit = top_logit; a.row_max = row_max; a.row_lse = row_lse;
       a.R = R;

@@ -191,3 +191,30 @@ def test_round_host_is_lossless(name):
     for k in ("accept_len", "out_tokens", "n_out"):
         assert np.array_equal(r_out[k].numpy(), want[k]), k
     assert p.g.poll() == 0
+
+
+@pytest.mark.parametrize("k", [0, 4, 5, 6])
+@pytest.mark.parametrize("top_n", [0, 1, 2])
+def test_kept_logits_on_both_sides_of_the_epilogue_rule(k, top_n):
+    """Up to 5 rows (6 with a draw) and one pick take their statistics in the LM head's epilogue, the rest in a
+    pass over the stored logits: the same values, ranks and draws from the logits that come back."""
+    import oracle
+    import paper_2410_05589_b200 as ps
+    import synth
+    s = synth.CONFIGS["mini"].with_(k_masks=k)
+    g = ps.drafter_from_shape(s, synth.weights(s), max_batch=1, max_ctx=32)
+    hl, tl = ps.to_device(synth.hidden_states(s, "last", 1)), ps.to_device(synth.token_ids(s, "last", 1))
+    for o in (g.draft_step([0], hl, tl, top_n=top_n), g.draft_step_sampled([0], hl, tl, 0.9, 3, 4, top_n=top_n)):
+        torch.cuda.synchronize()
+        lg = o["logits"][0].double().cpu().numpy()
+        assert np.array_equal(o["row_max"][0].cpu().numpy(), lg.max(-1).astype(np.float32))
+        # exponentials to 2^-20 each, fp32 sums over a tree of depth < 20, the stored value's rounding
+        lse = lg.max(-1) + np.log(np.exp(lg - lg.max(-1, keepdims=True)).sum(-1))
+        assert np.abs(o["row_lse"][0].cpu().numpy() - lse).max() < 2.0 ** -18 + 2.0 ** -23 * np.abs(lse).max()
+        if top_n:
+            assert np.array_equal(o["top_ids"][0].cpu().numpy(), np.argsort(-lg, axis=-1, kind="stable")[:, :top_n])
+        if "sampled" in o:
+            ids = np.arange(k + 1, dtype=np.int32) << 8
+            tok, margin = oracle.gumbel_sample(lg, 0.9, 3, 4, ids)
+            # single-precision noise: 2^-21 of values up to 17
+            assert all(a == b or m < 2e-5 for a, b, m in zip(o["sampled"][0].cpu().numpy(), tok, margin))
