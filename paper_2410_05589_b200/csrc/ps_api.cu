@@ -605,14 +605,14 @@ ps_status ps_round_host(ps_ctx* c, int B, const int* seq_slot, const void* hidde
                               nullptr, nullptr, nullptr, nullptr, c->st_dlogits, nullptr, st);
   else
     s = ps_draft_step(c, B, seq_slot, c->st_hidden, c->st_tok, 1, c->st_top, (float*)(c->st_top + (size_t)c->max_rows),
-                      nullptr, nullptr, c->st_dlogits, nullptr, st);
+                      nullptr, nullptr, nullptr, nullptr, st);   // (a greedy verify reads no draft logits)
   if (s != PS_OK) return s;
   int* r_acc = c->st_res;
   int* r_n = c->st_res + B;
   int* r_out = c->st_res + 2 * B;
   e = cudaStreamWaitEvent(st, c->copy_done, 0);
   if (e != cudaSuccess) return cuda_check(c, e, "ps_round_host wait");
-  s = ps_verify(c, B, R, R, c->st_top, c->st_dlogits, c->st_tlogits, temperature, seed, offset,
+  s = ps_verify(c, B, R, R, c->st_top, temperature > 0.f ? c->st_dlogits : nullptr, c->st_tlogits, temperature, seed, offset,
                 r_acc, r_out, r_n, st);
   if (s != PS_OK) return s;
   // one copy back for the three results (they are adjacent in the staging slice), into pinned
