@@ -1635,9 +1635,12 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
   const int nclu = a.V <= kCluMaxVocab ? kClu : 16, pairs = n_target * B;
   // More row pairs than the register-resident clusters can take at once (each of their blocks fills
   // an SM): the streaming kernel, with as many blocks per pair as are resident together.  Below that
-  // the register-resident ones win: one launch, and no second look at the rows.
+  // the register-resident ones win: one launch, and no second look at the rows.  Arg-max alone of many rows
+  // beyond 131072 tokens is one pass of k_verify's blocks (64 x 5 rows of 131076: 48 us, streamed 54; 16 x 6
+  // rows: 20, streamed 13).
+  const bool greedy_long = temperature == 0.f && a.V > kCluMaxVocab16 && 4 * pairs > 3 * c->n_sm;
   const int reg_blocks = a.V <= kOneMaxVocab ? 1 : nclu == kClu && a.V <= kCluSmallMaxVocab ? kCluSmall : nclu;
-  if (a.V % 4 == 0 && aligned && pairs * reg_blocks > c->n_sm) {
+  if (a.V % 4 == 0 && aligned && !greedy_long && pairs * reg_blocks > c->n_sm) {
     int per = 1;
     while (per < 8 && 2 * pairs * per <= kStrPerSm * c->n_sm) per *= 2;
     const size_t bytes = (size_t)(((a.V + kDrawClu - 1) / kDrawClu + kSeg - 1) / kSeg) * sizeof(double);
@@ -1664,7 +1667,13 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
     // each fill an SM are slow to place while the LM head's CTAs drain.  The 4-block ones of a batch
     // gain: four sequences 330 -> 326 us.)
     const bool pdl = !c->prof;
-    if (a.V <= kOneMaxVocab) {
+    // One block holds rows of up to 8192 tokens; from 6144 on, clusters that are resident together share a
+    // row's exponentials to more gain than their barriers cost (8192 tokens, 5 pairs 11.2 -> 9.9 us, 30 pairs
+    // 11.4 -> 10.2; 5000 tokens 9.9 against 10.0), unless an extra row's draw is among many (24: 12.6, 12.9).
+    // (Clusters of 8 that need most of the chip's SMs don't all find room at once: 16 pairs 15.1, one block 10.2.)
+    const bool share = a.V > 6144 && (4 * pairs * kClu <= 3 * c->n_sm ||
+                                      (n_target == n_draft && pairs * kClu > c->n_sm && pairs * kCluSmall <= c->n_sm));
+    if (a.V <= kOneMaxVocab && !share) {
       e = launch_after(k_verify_block, dim3(n_target, B), dim3(kCluThreads), 0, st, pdl, a);
     } else if (nclu == kClu && a.V <= kCluSmallMaxVocab && n_target * B * kClu > c->n_sm) {   // half the waves
       e = launch_after(k_verify_cluster4, dim3(n_target * kCluSmall, B), dim3(kCluThreads), 0, st, pdl, a);

@@ -198,9 +198,7 @@ def test_round_host_is_lossless(name):
 def test_kept_logits_on_both_sides_of_the_epilogue_rule(k, top_n):
     """Up to 5 rows (6 with a draw) and one pick take their statistics in the LM head's epilogue, the rest in a
     pass over the stored logits: the same values, ranks and draws from the logits that come back."""
-    import oracle
     import paper_2410_05589_b200 as ps
-    import synth
     s = synth.CONFIGS["mini"].with_(k_masks=k)
     g = ps.drafter_from_shape(s, synth.weights(s), max_batch=1, max_ctx=32)
     hl, tl = ps.to_device(synth.hidden_states(s, "last", 1)), ps.to_device(synth.token_ids(s, "last", 1))

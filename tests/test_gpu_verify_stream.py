@@ -43,3 +43,20 @@ def test_stream_verify_matches_oracle(vocab, B, n_draft, bonus, T, odd):
         assert_verify_same({k: v.cpu().numpy() for k, v in out.items()}, want)
         status = g.poll()
         assert T == 0.0 or status == (-6 if want["nonfinite"].any() else 0)
+
+
+# both sides of the dispatch's lines: one block and clusters of 8 and 4 from 6144 tokens on, arg-max of many
+# rows beyond 131072
+@pytest.mark.parametrize("vocab,B,n_draft,bonus", [(6144, 2, 5, 0), (6148, 2, 5, 0), (8192, 1, 13, 0), (8192, 1, 14, 0),
+                                                   (8192, 4, 5, 0), (8192, 4, 5, 1), (8192, 7, 5, 1), (131076, 11, 10, 0),
+                                                   (131076, 12, 10, 0)])
+@pytest.mark.parametrize("T", [0.0, 0.7])
+def test_verify_dispatch_lines(vocab, B, n_draft, bonus, T):
+    ps, g = _drafter(vocab, n_draft - 1, B)
+    tl = synth.zipf_logits(9, (vocab, B), B, n_draft + bonus, vocab)
+    dl = synth.noisy_draft_logits(9, (vocab, B), tl[:, :n_draft], 0.4)
+    tok = synth.sample_from_logits(9, (vocab, B), dl, 0.7)
+    want = oracle.verify(tok, dl, tl, T, 3, 8)
+    out = g.verify(ps.to_device(tok), ps.to_device(dl), ps.to_device(tl), T, 3, 8)
+    torch.cuda.synchronize()
+    assert_verify_same({k: v.cpu().numpy() for k, v in out.items()}, want)
