@@ -1075,12 +1075,14 @@ k_verify_draw(VerifyArgs a, const VerifyDraw* draws) {
 // cluster.  Where the walk stops the cluster draws the token.
 // Bound by the latency of the walk's cluster exchanges (1-2 us each).  A cluster per decision row
 // that tries its children speculatively was bound by its blocks' occupancy instead.  23 nodes, T = 1, before ->
-// after: 1 x 32000 tokens 31 -> 26 us, 4 x 62 -> 30, 16 x 207 -> 59; 1 x 128256 tokens 92 -> 35, 4 x 332 -> 46.
+// after: 1 x 32000 tokens 23.5 -> 18.0 us, 4 x 57 -> 24.7, 16 x 201 -> 34.8; 1 x 128256 tokens 83 -> 25, 4 x 318 -> 40.
 struct TreeTopo {
   int n_nodes, max_depth;
   unsigned char depth[PS_MAX_TREE_NODES];
   unsigned char child_off[PS_MAX_TREE_NODES + 2];   // children of decision row u: child_idx[off[u] .. off[u+1])
   unsigned char child_idx[PS_MAX_TREE_NODES];
+  signed char parent[PS_MAX_TREE_NODES];
+  unsigned char nth[PS_MAX_TREE_NODES];             // node i is the nth child of its parent
 };
 
 struct TreeArgs {
@@ -1093,10 +1095,12 @@ struct TreeArgs {
   uint32_t key0, key1, off_lo, off_hi;
   int* accept_len; int* out_tokens; int* n_out; int* path;
   RowStat* stats;              // [B][kTreeRows]: target rows by decision row, then draft rows by depth
+  int leaf_stats;              // the rows of leaves are among them
   int* status;
 };
 constexpr int kTreeRows = 2 * PS_MAX_TREE_NODES + 1;
-// Rows whose statistics the walk needs: target rows with children (at temperature 0: all), draft rows.
+// Rows whose statistics the walk needs: target rows with children (all at temperature 0, and where few rows
+// leave the chip idle: the leaf where a walk ends then needs no exchanges of its own), draft rows.
 struct TreeRows { int n; unsigned char row[kTreeRows]; };
 
 // Statistics of row blockIdx.x / nclu of the list for sequence blockIdx.y; exponentials against a
@@ -1335,12 +1339,23 @@ __device__ int cluster_draw(cooperative_groups::cluster_group& cl, CluPart& part
   return token;
 }
 
-// (The cluster size is a launch attribute: 8 blocks, 16 for vocabularies beyond 65536.)
+// What the walk reads of a node before it knows whether it gets there, formed for all nodes at once: level
+// by level the chain of loads, logarithms and exponentials was 2.5 us a level (a chain of four nodes, one
+// sequence of 32000 tokens: 22.0 -> 13.9 us in all).
+struct TreeNodes {
+  double logp[PS_MAX_TREE_NODES], logq[PS_MAX_TREE_NODES];   // of the node's token at its parent's row
+  double ratio[PS_MAX_TREE_NODES], r[PS_MAX_TREE_NODES];     // p / q (1 at most), the uniform it is tried with
+  int tok[PS_MAX_TREE_NODES];
+  RowStat stat[kTreeRows];
+};
+
+// (The cluster size is a launch attribute: see launch_verify_tree.)
 __global__ void __launch_bounds__(kCluThreads) k_tree_walk(const __grid_constant__ TreeArgs a) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   __shared__ CluPart part;
   __shared__ CluScratch s;
+  __shared__ TreeNodes nd;
   const int rank = (int)cl.block_rank(), nclu = (int)cl.num_blocks();
   const int b = blockIdx.y, V = a.V, n_nodes = a.topo.n_nodes;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1354,6 +1369,27 @@ __global__ void __launch_bounds__(kCluThreads) k_tree_walk(const __grid_constant
   pdl_launch_dependents();
   pdl_wait();
   const RowStat* stats = a.stats + (size_t)b * kTreeRows;
+  const int n_rows = n_nodes + 1 + (greedy ? 0 : a.topo.max_depth);
+  for (int i = tid; i < n_rows; i += kCluThreads) nd.stat[i] = stats[i];   // (rows nobody formed are not used)
+  if (tid < n_nodes) nd.tok[tid] = toks[tid];
+  __syncthreads();
+  if (!greedy && tid < n_nodes) {
+    const int up = a.topo.parent[tid] + 1, dep = a.topo.depth[tid], x = nd.tok[tid], j = a.topo.nth[tid];
+    const RowStat ts = nd.stat[up], ds = nd.stat[n_nodes + 1 + dep];
+    uint32_t ctr[4] = {(uint32_t)up + ((uint32_t)j << 16), (uint32_t)b, a.off_lo, a.off_hi};
+    philox4x32_10(a.key0, a.key1, ctr);
+    const bool in_range = x >= 0 && x < V;
+    const double logp = in_range ? ((double)a.target_logits[((size_t)b * (n_nodes + 1) + up) * V + x] - (double)ts.max) * inv_t -
+                                       log(ts.sum) : -INFINITY;
+    const double logq = in_range ? ((double)a.draft_logits[((size_t)b * a.topo.max_depth + dep) * V + x] - (double)ds.max) * inv_t -
+                                       log(ds.sum) : -INFINITY;
+    const double diff = logp - logq;
+    nd.logp[tid] = logp;
+    nd.logq[tid] = logq;
+    nd.ratio[tid] = (diff != diff) ? 0.0 : exp(fmin(diff, 0.0));
+    nd.r[tid] = (double)(ctr[0] >> 8) * (1.0 / 16777216.0);
+  }
+  __syncthreads();
   int u = 0, len = 0, any_bad = 0, token = -1;
   // every block takes the same branches below: the values they depend on are identical
   for (;;) {
@@ -1364,12 +1400,12 @@ __global__ void __launch_bounds__(kCluThreads) k_tree_walk(const __grid_constant
     RowStat ts, ds;
     ts.max = 0.f; ts.arg = 0; ts.bad = 0; ts.sum = 1.0;
     ds = ts;
-    if (greedy || n_kids > 0) ts = stats[u];
-    if (drow) ds = stats[n_nodes + 1 + dq];
+    if (greedy || n_kids > 0 || a.leaf_stats) ts = nd.stat[u];
+    if (drow) ds = nd.stat[n_nodes + 1 + dq];
     int next = -1;
     if (greedy) {
       for (int j = 0; j < n_kids && next < 0; ++j)
-        if (toks[a.topo.child_idx[kid0 + j]] == ts.arg) next = a.topo.child_idx[kid0 + j];
+        if (nd.tok[a.topo.child_idx[kid0 + j]] == ts.arg) next = a.topo.child_idx[kid0 + j];
       if (next < 0) token = ts.arg;
     } else if (ts.bad | ds.bad) {
       any_bad = 1;
@@ -1402,7 +1438,10 @@ __global__ void __launch_bounds__(kCluThreads) k_tree_walk(const __grid_constant
       };
       double st = ts.sum;
       bool bad = false;
-      if (n_kids == 0) {   // a leaf: its statistics are formed here
+      if (n_kids == 0 && a.leaf_stats) {
+        load();
+        exponentials();
+      } else if (n_kids == 0) {   // a leaf: its statistics are formed here
         load();
         float tm = -INFINITY;
         int ti = 0x7fffffff, bd = 0;
@@ -1464,27 +1503,18 @@ __global__ void __launch_bounds__(kCluThreads) k_tree_walk(const __grid_constant
         token = ts.arg;
       } else {
         const float inv_st = (float)(1.0 / st), inv_sd = (float)(1.0 / ds.sum);
-        const double log_st = log(st), log_sd = log(ds.sum);
         double c = 0.0, Zc = 1.0;   // the target distribution at u is now (p - c q)+ / Zc
         for (int j = 0; j < n_kids; ++j) {
           const int kid = a.topo.child_idx[kid0 + j];
-          const int x = toks[kid];
-          uint32_t ctr[4] = {(uint32_t)u + ((uint32_t)j << 16), (uint32_t)b, a.off_lo, a.off_hi};
-          philox4x32_10(a.key0, a.key1, ctr);
-          const double r = (double)(ctr[0] >> 8) * (1.0 / 16777216.0);
-          const bool in_range = x >= 0 && x < V;
-          const double logp = in_range ? ((double)trow[x] - (double)tmax) * inv_t - log_st : -INFINITY;
-          const double logq = in_range ? ((double)drow[x] - (double)ds.max) * inv_t - log_sd : -INFINITY;
           double ratio;
           if (c == 0.0) {
-            const double diff = logp - logq;
-            ratio = (diff != diff) ? 0.0 : exp(fmin(diff, 0.0));
+            ratio = nd.ratio[kid];
           } else {
-            const double px = exp(logp), qx = exp(logq);
+            const double px = exp(nd.logp[kid]), qx = exp(nd.logq[kid]);
             const double wx = fmax(px - c * qx, 0.0) / Zc;
             ratio = qx > 0.0 ? fmin(wx / qx, 1.0) : (wx > 0.0 ? 1.0 : 0.0);
           }
-          if (r < ratio) { next = kid; break; }
+          if (nd.r[kid] < ratio) { next = kid; break; }
           // rejected: the target distribution becomes norm((p - (c + Zc) q)+)
           if (!loaded) { load(); exponentials(); }
           const double c_new = c + Zc;
@@ -1515,7 +1545,7 @@ __global__ void __launch_bounds__(kCluThreads) k_tree_walk(const __grid_constant
     }
     if (next < 0) break;
     if (writer) {
-      out[len] = toks[next];
+      out[len] = nd.tok[next];
       pth[len] = next;
     }
     ++len;
@@ -1718,7 +1748,11 @@ ps_status launch_verify_tree(ps_ctx* c, int B, int n_nodes, const int* parent, c
   for (int u = 0; u <= n_nodes; ++u) {   // children of decision row u in increasing node id
     tp.child_off[u] = (unsigned char)off;
     for (int i = 0; i < n_nodes; ++i)
-      if (parent[i] == u - 1) tp.child_idx[off++] = (unsigned char)i;
+      if (parent[i] == u - 1) {
+        tp.parent[i] = (signed char)parent[i];
+        tp.nth[i] = (unsigned char)(off - tp.child_off[u]);
+        tp.child_idx[off++] = (unsigned char)i;
+      }
   }
   tp.child_off[n_nodes + 1] = (unsigned char)off;
   if (max_depth_out) *max_depth_out = tp.max_depth;
@@ -1732,17 +1766,25 @@ ps_status launch_verify_tree(ps_ctx* c, int B, int n_nodes, const int* parent, c
   a.off_lo = (uint32_t)offset; a.off_hi = (uint32_t)(offset >> 32);
   a.accept_len = accept_len; a.out_tokens = out_tokens; a.n_out = n_out; a.path = path;
   a.stats = c->tree_stats; a.status = c->dev_status;
-  const int nclu = a.V <= kCluMaxVocab ? kClu : 16;
+  const int least = a.V <= kOneMaxVocab ? 1 : a.V <= 2 * kOneMaxVocab ? 2 : a.V <= kCluSmallMaxVocab ? kCluSmall
+                  : a.V <= kCluMaxVocab ? kClu : 16;   // blocks that hold a row
+  // One block for short rows (16 trees of 9 nodes, 1000 tokens: 37.7 us with clusters of 8, 17.1 with one block;
+  // 8192 tokens, one tree: one block 18.4, four 16.6); no more than hold a row where larger clusters would
+  // not find room at once (16 trees of 23 nodes, 32000 tokens: 47.0 with clusters of 8, 34.8 with 4).
+  const int want = a.V <= kOneMaxVocab / 2 ? 1 : a.V <= kOneMaxVocab ? kCluSmall : a.V <= kCluMaxVocab ? kClu : 16;
+  const int nclu = 4 * B * want > 3 * c->n_sm ? least : want;
   if (!cluster_size_ok(c->cluster_ok[1], k_tree_walk, nclu))
     return fail(c, PS_ERR_UNSUPPORTED, "this device cannot run the 16-block clusters a vocabulary beyond 65536 needs");
   TreeRows list;
   list.n = 0;
+  // (the leaves' rows too where all rows' blocks fit the chip twice over)
+  a.leaf_stats = temperature != 0.f && 2 * (n_nodes + 1 + tp.max_depth) * B <= kStrPerSm * c->n_sm;
   for (int u = 0; u <= n_nodes; ++u)
-    if (temperature == 0.f || tp.child_off[u + 1] > tp.child_off[u]) list.row[list.n++] = (unsigned char)u;
+    if (temperature == 0.f || a.leaf_stats || tp.child_off[u + 1] > tp.child_off[u]) list.row[list.n++] = (unsigned char)u;
   if (temperature != 0.f)
     for (int t = 0; t < tp.max_depth; ++t) list.row[list.n++] = (unsigned char)(n_nodes + 1 + t);
-  int per = 1;   // blocks per row: as many as are resident together
-  while (per < 8 && 2 * list.n * B * per <= kStrPerSm * c->n_sm) per *= 2;
+  int per = 1;   // blocks per row: as many as are resident together, with a vector for each of their threads
+  while (per < 8 && 2 * list.n * B * per <= kStrPerSm * c->n_sm && a.V >= 2 * per * 4 * kStrThreads) per *= 2;
   prof_mark(c, st, "begin");
   cudaError_t e = launch_cluster(temperature == 1.f ? k_row_softmax<true> : k_row_softmax<false>, dim3(list.n * per, B), per,
                                  kStrThreads, 0, st, !c->prof, a, list);

@@ -26,3 +26,18 @@ def test_tree_walk_edges(V, B, T, odd):
         got, want = _run_both(g, TREE26, toks, dl, tl, T, 9, offset)
         _assert_same(got, want)
     assert g.poll() in (0, -6) and g.check_guards() == 0
+
+
+# the walk's clusters of 1, 2, 4 and 8 blocks (few trees and 14 or more: the fewest that hold a row), leaves
+# with statistics of their own and without (B = 1 and 30)
+@pytest.mark.parametrize("V", [4096, 4100, 8196, 16388])
+@pytest.mark.parametrize("B", [1, 14, 30])
+@pytest.mark.parametrize("tree", ["26", "chain"])
+def test_tree_walk_cluster_sizes(V, B, tree):
+    parent = TREE26 if tree == "26" else [-1, 0, 1, 2]
+    g = _ctx(V)
+    toks, dl, tl = _case(parent, B, V, seed=7, T=0.8)
+    for offset in (1, 2, 3):
+        got, want = _run_both(g, parent, toks, dl, tl, 0.8, 4, offset)
+        _assert_same(got, want)
+    assert g.poll() == 0
