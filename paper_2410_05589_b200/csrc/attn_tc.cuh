@@ -15,6 +15,18 @@ inline int padded_rows(const ps_config& g) {
   return g.head_dim == kD && rows <= kMaxRows ? (rows + 7) / 8 * 8 : 0;
 }
 
+// Whether a batch has enough keys for this kernel: it reads a kv head's keys once for all query heads
+// and hides everything behind the stream, but costs a launch more and the way through its warps'
+// barriers, where k_attn_mma's blocks, one per query head and key split, are through at once.  What
+// separates the two is the key tiles of all query heads for every SM (884 whole steps, 1 to 64 heads, 1 to
+// 16 rows, contexts of 16 to 4000): with up to 16 query rows a kv head 6 of them, with more (a ring of five
+// slots, scores of 24 or 32 rows a tile) 16.  Llama-3-8B shape, 4 x 512 keys, 5 rows: 40 -> 24 us.
+inline bool worth_it(const ps_config& g, const SeqMap& sm, int B, int n_sm) {
+  long long tiles = 0;
+  for (int b = 0; b < B; ++b) tiles += std::max(1, (sm.len[b] + 127) / 128);
+  return tiles * g.n_heads >= (long long)(padded_rows(g) <= 16 ? 6 : 16) * n_sm;
+}
+
 struct Buffers {
   __nv_bfloat16* q;      // [pairs][hi, lo][NR][128] rotated, scaled query rows (pair = sequence x kv head)
   __nv_bfloat16* kv_new; // [pairs][k, v][kNewRows][128] the step's new rows, rounded as a cache row is

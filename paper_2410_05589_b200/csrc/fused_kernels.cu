@@ -1903,7 +1903,7 @@ ps_status pair_draft_step(ps_ctx* c, UmmaMaps& u, const SeqMap& sm, int B, const
       return s;
   }
   prof_mark(c, st, "qkv_rope");
-  s = u.at_ok ? atc::launch(c, sm, B, f.qkv, f.at, u.at, f.attn_tickets, f.attnp.hi, f.attnp.lo, st)
+  s = u.at_ok && atc::worth_it(g, sm, B, c->n_sm) ? atc::launch(c, sm, B, f.qkv, f.at, u.at, f.attn_tickets, f.attnp.hi, f.attnp.lo, st)
               : launch_attn_split(c, sm, B, f.qkv, f.att_ml, f.att_o, f.attn_tickets, f.attnp.hi, f.attnp.lo, st);
   if (s) return s;
   prof_mark(c, st, "attention");

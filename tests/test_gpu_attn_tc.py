@@ -81,3 +81,40 @@ def test_odd_ring_with_late_tiles(kv_heads, k):
     for b in range(B):
         assert logits_close(got[b], want, s.dtype) <= 1.0, b     # the logits gate
     assert all(torch.equal(outs[0], x) for x in outs[1:]) and g.poll() == 0
+
+
+# The rule of the dispatch: 6 key tiles of a query head for every SM (16 with more than 16 query rows a kv
+# head).  The edges once more in batches beyond it, 8 times the same lengths.
+@pytest.mark.parametrize("heads,kv_heads,k", [(6, 6, 2), (6, 6, 8), (18, 3, 2), (16, 8, 15)])
+def test_key_tile_edges_in_full_batches(heads, kv_heads, k):
+    s = synth.CONFIGS["mini"].with_(n_heads=heads, n_kv_heads=kv_heads, k_masks=k)
+    lens = [0, 1, 8, 15, 16, 17, 31, 33, 112, 113, 127, 128, 129, 255, 257, 300] * 8
+    p = Pair(s, len(lens), context="import", lens=lens, oracle_seqs=range(16))
+    _check(p, s, range(16))
+
+
+def test_long_sequences_dealt_to_several_ctas():
+    s = synth.CONFIGS["mini"].with_(n_heads=24, n_kv_heads=8, k_masks=4)
+    p = Pair(s, 4, context="import", lens=[4300, 2100, 900, 3000], oracle_seqs=[0, 2])
+    _check(p, s, [0, 2])
+
+
+def test_scores_outgrow_their_reference_in_a_full_batch():
+    s = synth.CONFIGS["mini"].with_(k_masks=8)
+    lens = [700, 260] + [700] * 24
+    p = Pair(s, len(lens), context="import", lens=lens, oracle_seqs=[0, 1])
+    for b in (0, 1):
+        K, V = synth.kv_rows(s, ("kv", b), lens[b])
+        Kf = synth.bf16_bits_to_f32(K) * np.linspace(1, 250, lens[b], dtype=np.float32)[:, None]
+        K = synth.f32_to_bf16_bits(Kf)
+        p.o.kv_import(b, as_f64(K, s.dtype), as_f64(V, s.dtype))
+        p.g.kv_import(b, p.to_device(K), p.to_device(V))
+    _check(p, s, range(2))
+
+
+@pytest.mark.parametrize("heads,kv_heads,B,L", [(6, 6, 37, 500), (6, 6, 36, 500), (16, 4, 37, 500), (16, 4, 36, 500)])
+def test_both_sides_of_the_line(heads, kv_heads, B, L):
+    """6 heads x 37 sequences x 4 tiles are 888 = 6 x 148; 16 heads 2368 = 16 x 148."""
+    s = synth.CONFIGS["mini"].with_(n_heads=heads, n_kv_heads=kv_heads, k_masks=4)
+    p = Pair(s, B, context="import", lens=[L] * B, oracle_seqs=[0, B - 1])
+    _check(p, s, [0, B - 1])
