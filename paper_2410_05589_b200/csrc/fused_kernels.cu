@@ -2136,6 +2136,7 @@ bool fused_supported(ps_ctx* c, int M) {
   if (M > std::max(draft_rows_cap(g), append_rows_cap(g)) || (g.head_dim != 64 && g.head_dim != 128)) return false;
   const int Hq = g.n_heads * g.head_dim;
   if (g.hidden % 8 || Hq % 8 || g.ffn % 8) return false;   // 16-byte operand rows
+  if (M > kMaxM && g.hidden > pg::kMaxNormWidth) return false;   // (groups of up to 16 rows then)
   if ((g.vocab + 127) / 128 > umma::kRingBytes / 32) return false;   // a row's tile summaries fit the ring (LM-head merge)
   ensure_maps(c);
   if (c->umma_maps) return true;

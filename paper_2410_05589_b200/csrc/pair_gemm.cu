@@ -686,7 +686,7 @@ ps_status launch_finish_shared(ps_ctx* c, const Args& a, Mode mode, cudaStream_t
 
 ps_status launch_row_norm(ps_ctx* c, const Args& a, int H, const __nv_bfloat16* bias, const float* res,
                           const __nv_bfloat16* gain, float* out, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t st) {
-  if (H > 32768) return fail(c, PS_ERR_UNSUPPORTED, "hidden size beyond 32768");
+  if (H > kMaxNormWidth) return fail(c, PS_ERR_UNSUPPORTED, "hidden size beyond 32768");
   const int threads = H <= 8192 ? (H / 4 + 63) / 64 * 32 : 512;
   auto kern = H <= 8192 ? k_row_norm<2, 4, 1024> : H <= 16384 ? k_row_norm<8, 1, 512> : k_row_norm<16, 1, 512>;
   const cudaError_t e = launch_after(kern, dim3(a.p.M), dim3(threads), 0, st, !c->prof, a, H, c->cfg.rms_eps, bias, res, gain,

@@ -10,6 +10,7 @@ namespace pg {
 
 constexpr int kMaxNp = 256;       // activation rows of a tile (the widest N a tcgen05.mma takes)
 constexpr int kNpStep = 32;       // rows are padded to a multiple of this (16 rows per CTA of the pair)
+constexpr int kMaxNormWidth = 32768;   // features of a row that launch_row_norm takes
 constexpr int kMaxSplit = 16;     // k blocks a shared tile is dealt in
 
 // How a stage's tiles are dealt to the CTA pairs; computed on the host, read by the GEMM and by

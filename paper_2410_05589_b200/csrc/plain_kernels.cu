@@ -639,24 +639,29 @@ ps_status launch_rope_store_kv(ps_ctx* c, const SeqMap& sm, int rows, const floa
 
 ps_status launch_kv_copy(ps_ctx* c, int slot, int len, void* K, void* V, bool to_cache, cudaStream_t st) {
   const ps_config& g = c->cfg;
-  if (len == 0) return PS_OK;
   const size_t eb = g.dtype == PS_DTYPE_F32 ? 4 : 2, row = (size_t)g.n_kv_heads * g.head_dim * eb;
   const bool vec = (((uintptr_t)K | (uintptr_t)V) & 15) == 0;
-  const size_t tb = vec ? 16 : eb, n = (size_t)len * row / tb;
-  if (n >= (1ull << 31)) return fail(c, PS_ERR_UNSUPPORTED, "too many cache rows in one copy");
+  const size_t tb = vec ? 16 : eb, per_row = row / tb;   // (tb divides a row: 64 or 128 channels a head)
   const unsigned vpr = (unsigned)(g.head_dim * eb / tb);
-  const int blocks = (int)std::min<size_t>((n + 255) / 256, (size_t)c->n_sm * 16), to = to_cache ? 1 : 0;
-  if (vec)
-    k_kv_copy<uint4><<<blocks, 256, 0, st>>>((uint4*)c->kcache, (uint4*)c->vcache, (uint4*)K, (uint4*)V, slot, (unsigned)n,
-                                             g.n_kv_heads, vpr, g.max_ctx, to);
-  else if (eb == 4)
-    k_kv_copy<float><<<blocks, 256, 0, st>>>((float*)c->kcache, (float*)c->vcache, (float*)K, (float*)V, slot, (unsigned)n,
-                                             g.n_kv_heads, vpr, g.max_ctx, to);
-  else
-    k_kv_copy<uint16_t><<<blocks, 256, 0, st>>>((uint16_t*)c->kcache, (uint16_t*)c->vcache, (uint16_t*)K, (uint16_t*)V, slot,
-                                                (unsigned)n, g.n_kv_heads, vpr, g.max_ctx, to);
-  c->launches++;
-  return cuda_check(c, cudaGetLastError(), "k_kv_copy");
+  const int most = (int)std::min<size_t>(len, ((size_t)1 << 30) / per_row), to = to_cache ? 1 : 0;   // rows of a launch (32-bit indices)
+  if (len > 0 && most < 1) return fail(c, PS_ERR_UNSUPPORTED, "cache row too long");
+  for (int t0 = 0; t0 < len; t0 += most) {
+    const unsigned n = (unsigned)(std::min(most, len - t0) * per_row);
+    const int blocks = (int)std::min<size_t>((n + 255) / 256, (size_t)c->n_sm * 16);
+    const size_t at = (size_t)t0 * g.head_dim * eb;      // of the first row, within each head's slab
+    char *kc = (char*)c->kcache + at, *vc = (char*)c->vcache + at, *k = (char*)K + t0 * row, *v = (char*)V + t0 * row;
+    if (vec)
+      k_kv_copy<uint4><<<blocks, 256, 0, st>>>((uint4*)kc, (uint4*)vc, (uint4*)k, (uint4*)v, slot, n, g.n_kv_heads, vpr, g.max_ctx, to);
+    else if (eb == 4)
+      k_kv_copy<float><<<blocks, 256, 0, st>>>((float*)kc, (float*)vc, (float*)k, (float*)v, slot, n, g.n_kv_heads, vpr, g.max_ctx, to);
+    else
+      k_kv_copy<uint16_t><<<blocks, 256, 0, st>>>((uint16_t*)kc, (uint16_t*)vc, (uint16_t*)k, (uint16_t*)v, slot, n, g.n_kv_heads,
+                                                  vpr, g.max_ctx, to);
+    c->launches++;
+    const ps_status s = cuda_check(c, cudaGetLastError(), "k_kv_copy");
+    if (s) return s;
+  }
+  return PS_OK;
 }
 
 }  // namespace ps

@@ -27,3 +27,16 @@ def test_import_export_round_trip(name, kv_heads, aligned):
         rc = d.lib.ps_kv_export(d.h, slot, Ko.data_ptr(), Vo.data_ptr(), torch.cuda.current_stream().cuda_stream)
         assert rc == 0 and torch.equal(Ko, K) and torch.equal(Vo, V)
     assert d.check_guards() == 0
+
+
+def test_copy_of_more_rows_than_one_launch_indexes():
+    import paper_2410_05589_b200 as ps
+    s = synth.CONFIGS["mini"].with_(vocab=64, ffn=64)
+    width = s.n_kv_heads * s.head_dim
+    n = (1 << 30) // width + 5                        # single elements: 2^30 of them to a launch
+    d = ps.drafter_from_shape(s, synth.weights(s), max_batch=1, max_ctx=n + s.rows)
+    flat = torch.empty(n * width + 1, dtype=torch.bfloat16, device="cuda").uniform_(-1, 1)
+    K = flat[1:].view(n, width)
+    d.kv_import(0, K, K)
+    Ko, Vo = d.kv_export(0)                           # aligned: vectors, one launch
+    assert torch.equal(Ko, K) and torch.equal(Vo, K)

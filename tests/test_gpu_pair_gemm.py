@@ -94,3 +94,20 @@ def test_long_append_with_whole_and_shared_tiles():
             # values that agree to fp32 sums of 5120 and 10240 terms, rounded to bf16: one unit in the last place
             assert (np.abs(a - w) <= 2.0 ** -7 * np.abs(w) + 1e-4).all(), b
     assert g.poll() == 0 and g.check_guards() == 0
+
+
+def test_hidden_sizes_beyond_the_row_norm():
+    """Rows of more than 32768 features run in groups of up to 16 rows, as before the CTA-pair GEMM."""
+    s = synth.CONFIGS["mini"].with_(hidden=32776, n_heads=1, n_kv_heads=1, ffn=64, vocab=200, k_masks=4)
+    W = synth.weights(s.with_(hidden=64))            # (8: no fc, whose 4 GB are not drawn)
+    H, d = s.hidden, s.head_dim
+    rnd = np.random.default_rng(1)
+    for n, shape in dict(embed=(200, H), mask_embed=(4, H), mask_feat=(4, H), w_q=(d, H), w_k=(d, H), w_v=(d, H), w_o=(H, d),
+                         w_gate=(64, H), w_up=(64, H), w_down=(H, 64), w_lm=(200, H), g_in=(H,), g_post=(H,), g_final=(H,)).items():
+        x = rnd.standard_normal(shape, np.float32) * 0.02 + (1.0 if n[0] == "g" else 0.0)
+        W[n] = synth.f32_to_bf16_bits(x.astype(np.float32))
+    p = Pair(s, 5, lens=[3, 0, 9, 1, 2], flags=8, context="import", oracle_seqs=[0, 4], weights=W)
+    got = p.gpu_step(top_n=1)
+    for b in (0, 4):
+        assert logits_close(got["logits"][b], p.oracle_step(b)["logits"], s.dtype) <= 1.0, b     # the logits gate
+    assert p.g.poll() == 0
