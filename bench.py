@@ -67,7 +67,7 @@ def measured_peak():
 KERNEL_OF_STAGE = {
     "fc_norm": "k_gather_x + k_umma_gemm<STORE>", "qkv_rope": "k_umma_gemm<STORE>",
     "attention": "k_attn_mma", "o_proj": "k_umma_gemm<STORE>", "ffn_gate_up": "k_umma_gemm<SWIGLU>",
-    "ffn_down": "k_umma_gemm<STORE>", "lm_head": "k_umma_gemm<STORE> + k_logit_stats", "verify": "k_verify_cluster",
+    "ffn_down": "k_umma_gemm<STORE>", "lm_head": "k_umma_gemm<LMHEAD>", "verify": "k_verify_cluster",
     "logit_stats": "k_logit_stats",
 }
 
@@ -83,10 +83,15 @@ KERNEL_OF_STAGE_PAIR = {   # more than 16 rows
     "fc_norm": "k_gather_x + k_pair_gemm + k_row_norm", "qkv_rope": "k_pair_gemm + k_finish_shared",
     "o_proj": "k_pair_gemm + k_row_norm", "ffn_gate_up": "k_pair_gemm + k_finish_shared",
     "ffn_down": "k_pair_gemm + k_row_norm", "lm_head": "k_pair_gemm + k_finish_shared + k_logit_stats",
+    "attention": "k_attn_prep + k_attn_tc (k_attn_mma where an SM gets fewer than 6 key tiles of a head)",
 }
 
 
 def kernel_of_stage(stage, rows):
+    if stage == "verify" and rows > 18:
+        return "k_verify_cluster4" if rows <= 37 else "k_verify_stream + k_verify_draw"
+    if stage == "lm_head" and 6 < rows <= 16:
+        return "k_umma_gemm<STORE> + k_logit_stats"
     if rows > 16 and stage in KERNEL_OF_STAGE_PAIR:
         return KERNEL_OF_STAGE_PAIR[stage]
     return KERNEL_OF_STAGE.get(stage, stage)
