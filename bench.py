@@ -725,7 +725,7 @@ def main():
         h1.record()
         torch.cuda.synchronize()
         group = {"ms_per_call": h0.elapsed_time(h1) / 5, "groups": n_g, "rows": n_g * R,
-                 "note": "ps_group_forward; the groups run as one draft step over all their rows"}
+                 "note": "ps_group_forward; the groups run as draft steps of as many groups as the context has slots"}
 
     # ---- token-tree verification (Algorithm 1 in full) and the whole tree round -----------------
     tree, tree_round = (None, None)
