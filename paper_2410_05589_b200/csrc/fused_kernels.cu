@@ -1683,7 +1683,7 @@ struct UmmaMaps {
 bool make_plane_maps(PlaneMaps* pm, const void* base, size_t rows, size_t cols) {
   if (!make_map(&pm->m16, base, rows, cols, 16)) return false;
   for (int i = 0; i < pg::kMaxNp / pg::kNpStep; ++i) {
-    if (i > 0 && (size_t)i * pg::kNpStep >= rows) { pm->pair.m[i] = pm->pair.m[i - 1]; continue; }   // never that many rows
+    if (i > 1 && (size_t)(i / 2) * pg::kNpStep >= rows) { pm->pair.m[i] = pm->pair.m[i - 1]; continue; }   // never that many rows
     if (!make_map(&pm->pair.m[i], base, rows, cols, (i + 1) * pg::kNpStep / 2)) return false;
   }
   return true;

@@ -8,8 +8,13 @@
 // the activation planes from L2: a CTA that works alone needs 2 * Np * 128 bytes of planes (hi and
 // lo) beside every 16 KB weight box; in a pair it needs half of that, and with two weight
 // sub-tiles per CTA a quarter.
-// Activations are fp32 values split into bf16 hi + lo planes (x = hi + lo to about 2^-17); both
-// products go to the same fp32 accumulator in tensor memory.
+// Activations are fp32 values split into bf16 hi + lo planes (x = hi + lo to about 2^-17).  Beyond 128
+// rows both products go to the same fp32 accumulator in tensor memory, one MMA each.  Up to 128 rows
+// the planes are one operand of 2 Np columns (the leader's half of it is the hi plane, the other CTA's the
+// lo plane) and the epilogue adds the two halves of the accumulator: an MMA of a pair costs about 95
+// cycles however narrow it is, so that two of Np <= 96 columns took 0.85 us a unit where the weights
+// arrive in 0.6.  Steps of the 13B shape: 20 rows 314 -> 290 us, 80 rows 393 -> 375, 125 rows 389 -> 381;
+// 33B shape, 60 rows 432 -> 413.
 //
 // Warp roles per CTA: warp 0 issues the TMA loads of its own shared memory (completion counted
 // on the leader's barrier), warp 1 allocates tensor memory and, in the leader CTA, issues the
@@ -50,6 +55,7 @@ constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kRing = 222 * 1024;
 constexpr int kMaxStages = 12;
+constexpr int kMaxComb = 128;     // rows of a tile up to which hi and lo planes are one operand (2 Np <= 256)
 constexpr uint32_t kPeerMask = 0xFEFFFFFFu;   // shared::cluster address of the same offset in the leader CTA
 
 struct Ctl {
@@ -118,6 +124,11 @@ __device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t (&r)[16
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
+}
+// x += y, as floats.
+__device__ __forceinline__ void add16(uint32_t (&x)[16], const uint32_t (&y)[16]) {
+#pragma unroll
+  for (int j = 0; j < 16; ++j) x[j] = __float_as_uint(__uint_as_float(x[j]) + __uint_as_float(y[j]));
 }
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -215,7 +226,9 @@ k_pair_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
   const Plan& p = a.p;
   const int Np = p.Np, planes = a.planes;
   const int sbytes = stage_bytes(WT, planes, Np), nst = n_stages(sbytes), plane_bytes = (Np / 2) * kBK * 2;
-  const bool two_buf = WT * Np <= 256;
+  const bool comb = p.comb != 0;
+  const int nc = comb ? 2 * Np : Np;   // accumulator columns of a sub-tile
+  const bool two_buf = WT * nc <= 256;
 
   if (tid == 0) {
     for (int i = 0; i < kMaxStages; ++i) { mbar_init(&ctl.full[i], 1); mbar_init(&ctl.empty[i], 1); }
@@ -262,7 +275,12 @@ k_pair_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
       };
       auto load_b = [&](const UnitWalk& u, int st) {
         const uint32_t dst = base + st * sbytes + WT * kABytes, bar = smem_u32(&ctl.full[st]) & kPeerMask;
-        const int x = u.kb * kBK, y = u.yb + (int)rank * (Np / 2);
+        const int x = u.kb * kBK;
+        if (comb) {   // all rows of one plane
+          tma_load_pair(dst, rank == 0 ? &tBh : &tBl, x, u.yb, bar);
+          return;
+        }
+        const int y = u.yb + (int)rank * (Np / 2);
         tma_load_pair(dst, &tBh, x, y, bar);
         if (planes == 2) tma_load_pair(dst + plane_bytes, &tBl, x, y, bar);
       };
@@ -292,7 +310,7 @@ k_pair_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
       SegWalk sw;
       sw.start(p, pair, n_pairs);
       Seg s;
-      const uint32_t id = pair_idesc(Np);
+      const uint32_t id = pair_idesc(nc);
       int st = 0, segc = 0;
       uint32_t parity = 0;
       bool alive = true;
@@ -301,7 +319,7 @@ k_pair_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
         const uint32_t use = two_buf ? (uint32_t)(segc >> 1) : (uint32_t)segc;
         if (!mbar_wait(&ctl.acc_empty[buf], (use & 1) ^ 1, abort_flag)) break;
         fence_after_sync();
-        const uint32_t d = tmem + buf * WT * Np;
+        const uint32_t d = tmem + buf * WT * nc;
         uint32_t acc = 0;
         for (int kb = s.kb0; kb < s.kb1; ++kb) {
           if (!mbar_wait(&ctl.full[st], parity, abort_flag)) { alive = false; break; }
@@ -311,11 +329,11 @@ k_pair_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
           for (int k = 0; k < kBK / 16; ++k) {
 #pragma unroll
             for (int w = 0; w < WT; ++w)
-              mma_pair(d + w * Np, smem_desc(sa + w * kABytes + k * 32), smem_desc(sb + k * 32), id, acc | (k > 0));
-            if (planes == 2) {
+              mma_pair(d + w * nc, smem_desc(sa + w * kABytes + k * 32), smem_desc(sb + k * 32), id, acc | (k > 0));
+            if (planes == 2 && !comb) {
 #pragma unroll
               for (int w = 0; w < WT; ++w)
-                mma_pair(d + w * Np, smem_desc(sa + w * kABytes + k * 32), smem_desc(sb + plane_bytes + k * 32), id, 1u);
+                mma_pair(d + w * nc, smem_desc(sa + w * kABytes + k * 32), smem_desc(sb + plane_bytes + k * 32), id, 1u);
             }
           }
           acc = 1;
@@ -340,7 +358,7 @@ k_pair_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
       fence_after_sync();
       int w = s.t / p.n_rt;
       const int rt = s.t - w * p.n_rt, m0 = rt * Np, mrows = min(Np, p.M - m0);
-      const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + buf * WT * Np;
+      const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + buf * WT * nc;
       const bool slots = MODE == MODE_RAW || !s.whole;
       if (slots || !kZip) {
         float* dst0;
@@ -363,8 +381,17 @@ k_pair_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
         for (int c0 = half * 16; c0 < mrows; c0 += 32) {
           uint32_t x[WT][16];
 #pragma unroll
-          for (int i = 0; i < WT; ++i) tmem_ld16_async(ta + i * Np + c0, x[i]);
-          umma::tmem_ld_wait();
+          for (int i = 0; i < WT; ++i) tmem_ld16_async(ta + i * nc + c0, x[i]);
+          if (comb) {
+            uint32_t y[WT][16];
+#pragma unroll
+            for (int i = 0; i < WT; ++i) tmem_ld16_async(ta + i * nc + Np + c0, y[i]);
+            umma::tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < WT; ++i) add16(x[i], y[i]);
+          } else {
+            umma::tmem_ld_wait();
+          }
           float* d = dst0 + (size_t)c0 * ld;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
@@ -380,8 +407,17 @@ k_pair_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
         for (int c0 = half * 16; c0 < mrows; c0 += 32) {
           uint32_t xg[16], xu[16];
           tmem_ld16_async(ta + c0, xg);
-          tmem_ld16_async(ta + Np + c0, xu);
-          umma::tmem_ld_wait();
+          tmem_ld16_async(ta + nc + c0, xu);
+          if (comb) {
+            uint32_t yg[16], yu[16];
+            tmem_ld16_async(ta + Np + c0, yg);
+            tmem_ld16_async(ta + nc + Np + c0, yu);
+            umma::tmem_ld_wait();
+            add16(xg, yg);
+            add16(xu, yu);
+          } else {
+            umma::tmem_ld_wait();
+          }
           const size_t at = (size_t)(m0 + c0) * a.ld_plane + n;
           __nv_bfloat16 *h = a.hi + at, *l = a.lo + at;
 #pragma unroll
@@ -571,7 +607,7 @@ __global__ void __launch_bounds__(NT) k_row_norm(const __grid_constant__ Args a,
 double stream_cost(const Plan& p, int planes, int units) {
   const double a = p.wt * 32.768e3;
   const double ring = 0.17 + (a + planes * p.Np * 128.0) / 185e3;
-  const double mma = planes * 4 * p.wt * std::max(58.0, p.Np * 0.6) / 1.85e3;
+  const double mma = (p.comb ? std::max(58.0, p.Np * 1.2) : planes * std::max(58.0, p.Np * 0.6)) * 4 * p.wt / 1.85e3;
   return std::max(units * std::max(ring, mma), (double)p.T * p.KB * a / p.n_rt / 7.2e6);
 }
 double finish_cost(const Plan& p, Mode mode, int segs, int contributors, int n_slots) {
@@ -596,6 +632,7 @@ Plan make_plan(int M, const Weights& w, int K, int planes, Mode mode, size_t par
     p.n_rt = (M + kMaxNp - 1) / kMaxNp;
     p.Np = ((M + p.n_rt - 1) / p.n_rt + kNpStep - 1) / kNpStep * kNpStep;
     p.wt = wt;
+    p.comb = planes == 2 && p.Np <= kMaxComb;
     p.KB = (K + kBK - 1) / kBK;
     p.n_mats = w.zip ? 1 : w.n_mats;
     const int tile_rows = w.zip ? 256 : 256 * wt;
@@ -668,8 +705,9 @@ ps_status launch_gemm(ps_ctx* c, const Weights& w, const PlaneMaps& hi, const Pl
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   if (e != cudaSuccess) return cuda_check(c, e, "pair gemm smem attribute");
   const CUtensorMap &m1 = *w.map[w.n_mats > 1 ? 1 : 0], &m2 = *w.map[w.n_mats > 2 ? 2 : 0];
+  const int box = (p.comb ? 2 : 1) * p.Np / kNpStep - 1;
   e = launch_after(kern, dim3(c->n_sm & ~1), dim3(kThreads), kSmem, st, !c->prof, *w.map[0], m1, m2,
-                   hi.m[p.Np / kNpStep - 1], lo.m[p.Np / kNpStep - 1], a);
+                   hi.m[box], lo.m[box], a);
   c->launches++;
   return cuda_check(c, e, "k_pair_gemm");
 }

@@ -27,6 +27,7 @@ constexpr int kMaxSplit = 16;     // k blocks a shared tile is dealt in
 struct Plan {
   int M, Np, n_rt;          // activation rows, rows per row tile, row tiles
   int wt, tiles_w;          // 128-row sub-tiles per CTA; weight tiles over all matrices
+  int comb;                 // hi and lo planes are one MMA operand of 2 Np columns
   int KB;                   // k-blocks of 64 columns
   int T, n_dp, rem, split, S, Pe;
   int slot_t0;              // first tile that has slots
@@ -66,7 +67,7 @@ struct Args {
   int* status;
 };
 
-// Tensor maps of a plane with boxes of Np / 2 rows, one per padded row count.
+// Tensor maps of a plane with boxes of 16, 32, ... rows: Np / 2 of them, or Np where the planes are one operand.
 struct PlaneMaps { CUtensorMap m[kMaxNp / kNpStep]; };
 
 struct Weights { const CUtensorMap* map[3]; int rows[3]; int n_mats; bool zip; };

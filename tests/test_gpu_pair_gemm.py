@@ -41,6 +41,19 @@ def test_pair_gemm_shared_tiles_match_oracle(B, k):
     assert np.array_equal(got["logits"], p.gpu_step(top_n=1)["logits"])
 
 
+# up to 128 rows hi and lo planes are one operand: full and one past a padding step, the last count that is, the
+# first that is not; whole and shared tiles
+@pytest.mark.parametrize("B,k", [(32, 1), (97, 0), (64, 1), (43, 2)])
+def test_planes_as_one_operand_match_oracle(B, k):
+    s = synth.CONFIGS["mini"].with_(k_masks=k, hidden=2048, n_heads=16, n_kv_heads=4, ffn=5504)
+    seqs = [0, B - 1]
+    p = Pair(s, B, lens=[1 + (5 * b) % 23 for b in range(B)], oracle_seqs=seqs)
+    got = p.gpu_step(top_n=1)
+    for b in seqs:
+        assert logits_close(got["logits"][b], p.oracle_step(b)["logits"], s.dtype) <= 1.0, b     # the logits gate
+    assert p.g.check_guards() == 0 and p.g.poll() == 0
+
+
 def test_row_counts_change_on_one_context():
     s = synth.CONFIGS["mini"].with_(k_masks=4)
     B = 60
