@@ -140,12 +140,20 @@ __device__ __forceinline__ void split1(float x, __nv_bfloat16& h, __nv_bfloat16&
   h = __float2bfloat16_rn(x);
   l = __float2bfloat16_rn(x - __bfloat162float(h));
 }
+// Two values' hi and lo parts, packed (the conversion takes two values an instruction).
+__device__ __forceinline__ void split2(float x, float y, uint32_t& h, uint32_t& l) {
+  const __nv_bfloat162 hv = __floats2bfloat162_rn(x, y);
+  h = *reinterpret_cast<const uint32_t*>(&hv);
+  const __nv_bfloat162 lv = __floats2bfloat162_rn(x - __uint_as_float(h << 16), y - __uint_as_float(h & 0xFFFF0000u));
+  l = *reinterpret_cast<const uint32_t*>(&lv);
+}
 // hi/lo planes of four consecutive values as 8-byte stores.
 __device__ __forceinline__ void split4(const float4& v, __nv_bfloat16* hi, __nv_bfloat16* lo) {
-  __align__(8) __nv_bfloat16 h[4], l[4];
-  split1(v.x, h[0], l[0]); split1(v.y, h[1], l[1]); split1(v.z, h[2], l[2]); split1(v.w, h[3], l[3]);
-  *reinterpret_cast<uint2*>(hi) = *reinterpret_cast<uint2*>(h);
-  *reinterpret_cast<uint2*>(lo) = *reinterpret_cast<uint2*>(l);
+  uint2 h, l;
+  split2(v.x, v.y, h.x, l.x);
+  split2(v.z, v.w, h.y, l.y);
+  *reinterpret_cast<uint2*>(hi) = h;
+  *reinterpret_cast<uint2*>(lo) = l;
 }
 // Four bf16 values (of a gain or bias vector, which the caller may have put on any 2-byte boundary).
 __device__ __forceinline__ float4 load_bf4(const __nv_bfloat16* x) {
@@ -513,44 +521,65 @@ __global__ void __launch_bounds__(256) k_finish_shared(const __grid_constant__ A
 }
 
 // Row m of a MODE_RAW stage: the row's slots added in k order, bias and residual, the row's sum
-// of squares, the planes of its RMS-normalised values.  One block per row, a thread for every two
-// vectors of four features (beyond 8192 features more vectors), held in registers from the loads to the stores.
-// Bound by the latency of its loads from L2, so the slots of JB contributors are in flight together.
-template <int NV, int JB, int NT>
-__global__ void __launch_bounds__(NT) k_row_norm(const __grid_constant__ Args a, int H, float eps,
+// of squares, the planes of its RMS-normalised values.  One block per row, NV vectors of four features a
+// thread, held in registers from the loads to the stores.
+// Bound by the latency of its loads from L2, which are hidden in two ways: few rows (a block an SM) have two
+// vectors a thread and the slots of JB = 4 contributors in flight together; many rows one contributor, in
+// so few registers that several blocks share an SM.  The divisions that find a tile's slots are made once
+// per tile and block.
+template <int NV, int JB, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_row_norm(const __grid_constant__ Args a, int H, float eps,
                                                            const __nv_bfloat16* __restrict__ bias, const float* res,
                                                            const __nv_bfloat16* __restrict__ gain, float* out,
                                                            __nv_bfloat16* hi, __nv_bfloat16* lo) {
   __shared__ float s_part[32];
+  __shared__ unsigned s_slot[kMaxNormWidth / 256];   // by weight tile: where the row's first slot lies (in vectors)
+  __shared__ int s_cnt[kMaxNormWidth / 256];         // and how many contributors it has
   pdl_launch_dependents();
   const Plan& p = a.p;
-  const int m = blockIdx.x, rt = m / p.Np, mi = m - rt * p.Np, tid = threadIdx.x, nthr = blockDim.x;
-  const int sh = p.wt == 2 ? 9 : 8, TW = 1 << sh;
+  const int m = blockIdx.x, tid = threadIdx.x, nthr = blockDim.x;
+  const int sh = p.wt == 2 ? 7 : 6;                    // vectors of a tile's row: 128 or 64
   const bool out_vec = ((uintptr_t)out & 15) == 0;     // (the caller's feature rows may sit anywhere)
-  const size_t layer = (size_t)p.Np * TW;              // floats between a tile's contributors
+  const bool gain_vec = ((uintptr_t)gain & 7) == 0;    // (and so may the gains)
+  const unsigned layer = (unsigned)p.Np << sh;         // vectors between a tile's contributors
+  for (int w = tid; w < p.tiles_w; w += nthr) {
+    const int rt = m / p.Np, mi = m - rt * p.Np, t = w * p.n_rt + rt;
+    s_cnt[w] = tile_contributors(p, t);
+    s_slot[w] = (unsigned)(slot_row(p, 0, t, mi) / 4);
+  }
+  __syncthreads();
+  const float4* part = reinterpret_cast<const float4*>(a.part);
+  const int nv = H >> 2;                               // H % 8 == 0
   float4 x[NV];
-  const float* slot[NV];
+  uint2 gr[NV];                                        // the gains' bits
+  unsigned slot[NV];
   int cnt[NV], cmax = 0;
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
-    const int n = 4 * (tid + i * nthr);
+    const int n = tid + i * nthr;
     cnt[i] = 0;
-    slot[i] = a.part;
+    slot[i] = 0;
     x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (n < H) {
-      const int t = (n >> sh) * p.n_rt + rt;
-      cnt[i] = tile_contributors(p, t);
+    if (n < nv) {
+      cnt[i] = s_cnt[n >> sh];
       cmax = max(cmax, cnt[i]);
-      slot[i] += slot_row(p, 0, t, mi) + (n & (TW - 1));
-      if (bias) x[i] = load_bf4(bias + n);
+      slot[i] = s_slot[n >> sh] + (n & ((1 << sh) - 1));
+      if (bias) x[i] = load_bf4(bias + 4 * n);
     }
   }
   pdl_wait();
   float4 rv[NV];
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
-    const int n = 4 * (tid + i * nthr);
-    rv[i] = (res && n < H) ? __ldcg(reinterpret_cast<const float4*>(res + (size_t)m * H + n)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const int n = tid + i * nthr;
+    gr[i] = make_uint2(0u, 0u);
+    if (n < nv && gain_vec) {
+      gr[i] = __ldg(reinterpret_cast<const uint2*>(gain) + n);
+    } else if (n < nv) {
+      const unsigned short* gp = reinterpret_cast<const unsigned short*>(gain) + 4 * n;
+      gr[i] = make_uint2(gp[0] | (unsigned)gp[1] << 16, gp[2] | (unsigned)gp[3] << 16);
+    }
+    rv[i] = (res && n < nv) ? __ldcg(reinterpret_cast<const float4*>(res + (size_t)m * H) + n) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   for (int j = 0; j < cmax; j += JB) {
     float4 v[JB][NV];
@@ -558,8 +587,7 @@ __global__ void __launch_bounds__(NT) k_row_norm(const __grid_constant__ Args a,
     for (int b = 0; b < JB; ++b)
 #pragma unroll
       for (int i = 0; i < NV; ++i)
-        v[b][i] = j + b < cnt[i] ? __ldcg(reinterpret_cast<const float4*>(slot[i] + (size_t)(j + b) * layer))
-                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[b][i] = j + b < cnt[i] ? __ldcg(part + (slot[i] + (j + b) * layer)) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int b = 0; b < JB; ++b)
 #pragma unroll
@@ -585,8 +613,8 @@ __global__ void __launch_bounds__(NT) k_row_norm(const __grid_constant__ Args a,
         if (out_vec) *reinterpret_cast<float4*>(o) = x[i];
         else { o[0] = x[i].x; o[1] = x[i].y; o[2] = x[i].z; o[3] = x[i].w; }
       }
-      const float4 g = load_bf4(gain + n);
-      const float4 y = make_float4(x[i].x * sc * g.x, x[i].y * sc * g.y, x[i].z * sc * g.z, x[i].w * sc * g.w);
+      const float4 y = make_float4(x[i].x * sc * __uint_as_float(gr[i].x << 16), x[i].y * sc * __uint_as_float(gr[i].x & 0xFFFF0000u),
+                                   x[i].z * sc * __uint_as_float(gr[i].y << 16), x[i].w * sc * __uint_as_float(gr[i].y & 0xFFFF0000u));
       split4(y, hi + (size_t)m * H + n, lo + (size_t)m * H + n);
     }
   }
@@ -725,8 +753,12 @@ ps_status launch_finish_shared(ps_ctx* c, const Args& a, Mode mode, cudaStream_t
 ps_status launch_row_norm(ps_ctx* c, const Args& a, int H, const __nv_bfloat16* bias, const float* res,
                           const __nv_bfloat16* gain, float* out, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t st) {
   if (H > kMaxNormWidth) return fail(c, PS_ERR_UNSUPPORTED, "hidden size beyond 32768");
-  const int threads = H <= 8192 ? (H / 4 + 63) / 64 * 32 : 512;
-  auto kern = H <= 8192 ? k_row_norm<2, 4, 1024> : H <= 16384 ? k_row_norm<8, 1, 512> : k_row_norm<16, 1, 512>;
+  // more rows than SMs: blocks that share an SM (see k_row_norm)
+  const bool many = H <= 8192 && a.p.M > c->n_sm;
+  const int per_thread = H > 8192 ? 0 : many && H > 5120 ? 16 : 8;   // features
+  const int threads = per_thread ? ((H + per_thread - 1) / per_thread + 31) / 32 * 32 : 512;
+  auto kern = many ? (H <= 5120 ? k_row_norm<2, 1, 640, 2> : k_row_norm<4, 1, 512, 2>)
+              : H <= 8192 ? k_row_norm<2, 4, 1024, 1> : H <= 16384 ? k_row_norm<8, 1, 512, 1> : k_row_norm<16, 1, 512, 1>;
   const cudaError_t e = launch_after(kern, dim3(a.p.M), dim3(threads), 0, st, !c->prof, a, H, c->cfg.rms_eps, bias, res, gain,
                                      out, hi, lo);
   c->launches++;
