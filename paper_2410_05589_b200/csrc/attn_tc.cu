@@ -62,11 +62,13 @@ struct Ctl {
   uint64_t p_full[2], p_empty[2];          // probabilities, by step
   uint64_t o_full[2], o_empty[2];          // outputs, by segment
   uint64_t l_full[2];                      // references and sums, by segment
+  uint64_t checked[2][2];                  // by half of the rows and step: its four warps have looked for outgrown scores
+  uint64_t soft[2];                        // by half: its four warps have come this far
   uint32_t tmem_base;
   int abort_flag, is_last;
+  int outgrown[2][2];                      // by half and step: some score has outgrown its reference
   float ref[2][NR];
-  float sum[2][4][NR];                     // per lane quadrant
-  float red[4][NR];
+  float sum[2][4][NR];                     // per lane quadrant; new maxima while a segment is under way
 };
 template <int NR>
 constexpr int smem_bytes() { return n_slots(NR) * kSlotBytes + 4 * op_bytes(NR) + (int)sizeof(Ctl<NR>) + 1024; }
@@ -191,8 +193,23 @@ __device__ __forceinline__ uint64_t vt_desc(uint32_t saddr, uint32_t half_bytes)
   return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(half_bytes >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
          ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
-// Barriers of 128 threads: the epilogue warps, and the four warps of either half of the rows.
-constexpr int kBarEpi = 1, kBarSoft = 2;
+// Probabilities as the MMA's N side: a key's 2 NR values (rows of the hi plane, then of the lo plane) contiguous
+// (MN-major), 32-byte swizzle; 16 values at a time, the next 16 kAtomStride bytes on; groups of 8 keys 256 bytes
+// apart.
+constexpr int kAtomStride = kTile * 32;
+__device__ __forceinline__ uint64_t p_desc(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(kAtomStride >> 4) << 16) | ((uint64_t)(256 >> 4) << 32) |
+         ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
+}
+// Two values' hi and lo parts, packed.
+__device__ __forceinline__ void split2(float x, float y, uint32_t& h, uint32_t& l) {
+  const __nv_bfloat162 hv = __floats2bfloat162_rn(x, y);
+  h = *reinterpret_cast<const uint32_t*>(&hv);
+  const __nv_bfloat162 lv = __floats2bfloat162_rn(x - __uint_as_float(h << 16), y - __uint_as_float(h & 0xFFFF0000u));
+  l = *reinterpret_cast<const uint32_t*>(&lv);
+}
+// Barrier of the 128 epilogue threads.
+constexpr int kBarEpi = 1;
 __device__ __forceinline__ void bar_sync(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
 __device__ __forceinline__ bool bar_any(int id, bool pred) {
   uint32_t r;
@@ -303,6 +320,8 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
       mbar_init(&ctl.p_full[i], kSoftWarps); mbar_init(&ctl.p_empty[i], 1);
       mbar_init(&ctl.o_full[i], 1); mbar_init(&ctl.o_empty[i], 4);
       mbar_init(&ctl.l_full[i], kSoftWarps);
+      for (int h = 0; h < 2; ++h) { mbar_init(&ctl.checked[h][i], kSoftWarps / 2); ctl.outgrown[h][i] = 0; }
+      mbar_init(&ctl.soft[i], kSoftWarps / 2);
     }
     ctl.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -412,8 +431,8 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
   } else if (warp == 2) {
     if (lane == 0) {   // ---- MMA issuer, outputs
       Walk x;
-      const uint32_t id = umma::idesc(N) | (1u << 15);
-      const uint64_t dv0 = vt_desc(base, 0), dp0 = smem_desc(s_p);
+      const uint32_t id = umma::idesc(N) | (1u << 15) | (1u << 16);   // (both operands MN-major)
+      const uint64_t dv0 = vt_desc(base, 0), dp0 = p_desc(s_p);
       x.start(w, u0, u1);
       int slot = x.ok && x.last_of_cta() ? 1 : 2;   // of this step's V: ring position 2 i + 2, of the very last one 2 i + 1
       uint32_t use = 0;
@@ -430,11 +449,11 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
         if (n_ks == kTile / 16) {
 #pragma unroll
           for (int ks = 0; ks < kTile / 16; ++ks)
-            umma::mma_f16(d, da + ks * (2048 / 16), db + (ks >> 2) * (kOp / 32) + (ks & 3) * 2, id, ks > 0 ? 1u : acc);
+            umma::mma_f16(d, da + ks * (2048 / 16), db + ks * (512 / 16), id, ks > 0 ? 1u : acc);
         } else {
 #pragma unroll 1
           for (int ks = 0; ks < n_ks; ++ks)
-            umma::mma_f16(d, da + ks * (2048 / 16), db + (ks >> 2) * (kOp / 32) + (ks & 3) * 2, id, ks > 0 ? 1u : acc);
+            umma::mma_f16(d, da + ks * (2048 / 16), db + ks * (512 / 16), id, ks > 0 ? 1u : acc);
         }
         umma::mma_commit(&ctl.p_empty[buf]);
         umma::mma_commit(&ctl.empty[slot]);
@@ -445,13 +464,29 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
       }
     }
   } else if (warp < 3 + kSoftWarps) {
-    // ---- softmax: thread = key of the tile, half of the rows
-    constexpr int NH = NR / 2, kSoft = 32 * kSoftWarps;
-    const int q = warp & 3, key = 32 * q + lane, half = (warp - 3) >> 2, r0 = half * NH, bar = kBarSoft + half;
+    // ---- softmax: thread = key of the tile, half of the rows.  The four warps of a half share their rows'
+    // references, so they meet in every step; they do so a few hundred cycles after each has said
+    // whether one of its scores has outgrown its reference, and find the others' words there.  (A barrier at that
+    // point cost 500-800 cycles a step, more than the arithmetic: below the clock that the power limit
+    // leaves, a step's cycles are what bounds the kernel.)  All these waits are bounded.
+    constexpr int NH = NR / 2, kSoft = 32 * kSoftWarps, kPiece = NH % 8 == 0 ? 8 : 4;
+    const int q = warp & 3, key = 32 * q + lane, half = (warp - 3) >> 2, r0 = half * NH;
     const uint32_t lane_off = (uint32_t)(32 * q) << 16;
     const int rows = w.group * w.R;
-    unsigned char* const p_base = ring_g + NS * kSlotBytes + 2 * kOp + (key >> 6) * (kOp / 2) + r0 * 128 + (key & 7) * 2;
-    const int chunk = (key & 63) >> 3;
+    // this thread's key in the probabilities; the 16-byte halves of its 32 change places every four keys
+    unsigned char* const p_base = ring_g + NS * kSlotBytes + 2 * kOp + key * 32;
+    const int flip = ((key >> 2) & 1) << 4;
+    uint32_t soft_phase = 0;
+    auto meet = [&]() {   // the half's warps; what each wrote to shared memory is visible to the others
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&ctl.soft[half]);
+      const bool ok = mbar_wait(&ctl.soft[half], soft_phase, abort_flag);
+      soft_phase ^= 1;
+      return (bool)__all_sync(0xffffffffu, ok);
+    };
+    int jr[NH];   // a row's place in its sequence: it sees the new keys up to there (-1: no such row)
+#pragma unroll
+    for (int r = 0; r < NH; ++r) jr[r] = r0 + r < rows ? (r0 + r) % w.R : -1;
     Walk x;
     x.start(w, u0, u1);
     float ref[NH], l[NH];
@@ -460,10 +495,10 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
       const bool last = x.last();
       bool ok = mbar_wait(&ctl.s_full[buf], (i >> 1) & 1, abort_flag);
       if (x.first) ok = mbar_wait(&ctl.o_empty[sb], ((x.seg >> 1) & 1) ^ 1, abort_flag) && ok;
-      ok = __all_sync(0xffffffffu, ok);
+      if (!__all_sync(0xffffffffu, ok)) break;
       fence_after_sync();
       float s[NH];
-      if (ok) {
+      {
         uint32_t h[NH / 4][4], lo[NH / 4][4];
         const uint32_t at = tmem + lane_off + buf * N + r0;
 #pragma unroll
@@ -476,26 +511,32 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctl.s_empty[buf]);   // read back: the next scores may be formed
       if (x.first) {   // the references: the scores of the segment's first key
-        if (key == 0 && ok) {
+        if (key == 0) {
 #pragma unroll
           for (int r = 0; r < NH; ++r) ctl.ref[sb][r0 + r] = s[r];
         }
-        bar_sync(bar);
+        if (!meet()) break;
 #pragma unroll
         for (int r = 0; r < NH; ++r) { ref[r] = ctl.ref[sb][r0 + r]; l[r] = 0.f; }
       }
-      if (n < kTile || x.in_tail) {   // keys past the end, new keys that a row does not see yet
+      if (n < kTile) {   // keys past the end, new keys that a row does not see yet
 #pragma unroll
-        for (int r = 0; r < NH; ++r) {
-          const int rr = r0 + r;
-          if (key >= n || rr >= rows || (x.in_tail && key > rr % w.R)) s[r] = -INFINITY;
-        }
+        for (int r = 0; r < NH; ++r)
+          if (key >= n || jr[r] < 0 || (x.in_tail && key > jr[r])) s[r] = -INFINITY;
       }
       float top = -INFINITY;
 #pragma unroll
       for (int r = 0; r < NH; ++r) top = fmaxf(top, s[r] - ref[r]);
-      if (bar_any(bar, !ok || top > kSlack)) {
-        if (bar_any(bar, *abort_flag != 0)) break;   // (one answer for all threads)
+      const bool mine = __any_sync(0xffffffffu, top > kSlack);
+      if (lane == 0) {
+        if (mine) *(volatile int*)&ctl.outgrown[half][buf] = 1;
+        mbar_arrive(&ctl.checked[half][buf]);
+      }
+      float p[NH];
+#pragma unroll
+      for (int r = 0; r < NH; ++r) p[r] = ex2(s[r] - ref[r]);   // (0 for what is masked)
+      if (!__all_sync(0xffffffffu, mbar_wait(&ctl.checked[half][buf], (i >> 1) & 1, abort_flag))) break;
+      if (*(volatile int*)&ctl.outgrown[half][buf]) {
         // Rare: some score lies far above its reference.  New references; the sums and the outputs
         // so far are rescaled once the MMAs that form them have completed.
         for (int r = 0; r < NH; ++r) {
@@ -504,23 +545,25 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
           for (int e = 0; e < NH; ++e) m = e == r ? s[e] : m;
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-          if (lane == 0) ctl.red[q][r0 + r] = m;
+          if (lane == 0) ctl.sum[sb][q][r0 + r] = m;
         }
-        bar_sync(bar);
+        if (!meet()) break;
+        if (key == 0) *(volatile int*)&ctl.outgrown[half][buf] = 0;   // (everyone has read it)
+        const auto& mx = ctl.sum[sb];
         float f[NH];
 #pragma unroll
         for (int r = 0; r < NH; ++r) {
           const int rr = r0 + r;
-          const float m = fmaxf(fmaxf(fmaxf(ctl.red[0][rr], ctl.red[1][rr]), fmaxf(ctl.red[2][rr], ctl.red[3][rr])), ref[r]);
+          const float m = fmaxf(fmaxf(fmaxf(mx[0][rr], mx[1][rr]), fmaxf(mx[2][rr], mx[3][rr])), ref[r]);
           f[r] = ex2(ref[r] - m);
           l[r] *= f[r];
           ref[r] = m;
+          p[r] = ex2(s[r] - m);
           if (key == 0) ctl.ref[sb][rr] = m;
         }
-        bool rok = true;
-        if (!x.first) rok = mbar_wait(&ctl.p_empty[(i - 1) & 1], ((i - 1) >> 1) & 1, abort_flag);
-        if (bar_any(bar, !rok)) break;
+        if (last && !meet()) break;   // (the sums are written below)
         if (!x.first) {
+          if (!__all_sync(0xffffffffu, mbar_wait(&ctl.p_empty[(i - 1) & 1], ((i - 1) >> 1) & 1, abort_flag))) break;
           fence_after_sync();
 #pragma unroll
           for (int c = 0; c < 2 * NH / 4; ++c) {   // this warp's columns: hi, then lo
@@ -536,24 +579,29 @@ k_attn_tc(const __grid_constant__ CacheMaps t_c, const __grid_constant__ CUtenso
           fence_before_sync();
         }
       }
-      // ---- probabilities as hi/lo planes: row r of plane p at row p NR + r, keys along the row
-      float p[NH];
+      // ---- probabilities as hi/lo planes, the key's values side by side
 #pragma unroll
-      for (int r = 0; r < NH; ++r) {
-        p[r] = ex2(s[r] - ref[r]);   // (0 for what is masked)
-        l[r] += p[r];
-      }
+      for (int r = 0; r < NH; ++r) l[r] += p[r];
       if (i >= 2) mbar_wait(&ctl.p_empty[buf], ((i >> 1) & 1) ^ 1, abort_flag);
       const int n16 = (n + 15) & ~15;
       if (key < n16) {
         unsigned char* const pp = p_base + buf * kOp;
 #pragma unroll
-        for (int r = 0; r < NH; ++r) {
-          __nv_bfloat16 h, lo;
-          split1(p[r], h, lo);
-          const int at = r * 128 + ((chunk ^ ((r0 + r) & 7)) << 4);   // (NR is a multiple of 8: the same for both planes)
-          *reinterpret_cast<__nv_bfloat16*>(pp + at) = h;
-          *reinterpret_cast<__nv_bfloat16*>(pp + NR * 128 + at) = lo;
+        for (int c = 0; c < NH; c += kPiece) {
+          uint32_t h[kPiece / 2], lo[kPiece / 2];
+#pragma unroll
+          for (int e = 0; e < kPiece / 2; ++e) split2(p[c + 2 * e], p[c + 2 * e + 1], h[e], lo[e]);
+          // value v of the key: 16 values to an atom, 8 to a 16-byte half of its 32 bytes
+          const int vh = r0 + c, vl = NR + vh;
+          unsigned char* const ph = pp + (vh >> 4) * kAtomStride + ((((vh >> 3) & 1) << 4) ^ flip) + (vh & 7) * 2;
+          unsigned char* const pl = pp + (vl >> 4) * kAtomStride + ((((vl >> 3) & 1) << 4) ^ flip) + (vl & 7) * 2;
+          if constexpr (kPiece == 8) {
+            *reinterpret_cast<uint4*>(ph) = make_uint4(h[0], h[1], h[2], h[3]);
+            *reinterpret_cast<uint4*>(pl) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+          } else {
+            *reinterpret_cast<uint2*>(ph) = make_uint2(h[0], h[1]);
+            *reinterpret_cast<uint2*>(pl) = make_uint2(lo[0], lo[1]);
+          }
         }
       }
       if (n16 > n && !x.in_tail) {
