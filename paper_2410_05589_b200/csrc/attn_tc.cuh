@@ -6,7 +6,7 @@ namespace ps {
 namespace atc {
 
 constexpr int kD = 128;          // head dimension
-constexpr int kNewRows = 16;     // rows kept per sequence and kv head for the step's new keys / values
+constexpr int kNewRows = 16;     // rows kept per sequence (or bundle of them) and kv head for the step's new keys / values
 constexpr int kMaxRows = 32;     // query rows of a kv head's group (heads of the group x rows per sequence)
 
 // Query rows of a kv head's group padded to a multiple of 8 (0: the kernel does not take the shape).
@@ -28,13 +28,13 @@ inline bool worth_it(const ps_config& g, const SeqMap& sm, int B, int n_sm) {
 }
 
 struct Buffers {
-  __nv_bfloat16* q;      // [pairs][hi, lo][NR][128] rotated, scaled query rows (pair = sequence x kv head)
+  __nv_bfloat16* q;      // [pairs][hi, lo][NR][128] rotated, scaled query rows (pair = sequence or bundle x kv head)
   __nv_bfloat16* kv_new; // [pairs][k, v][kNewRows][128] the step's new rows, rounded as a cache row is
   float* part_o;         // [2 CTAs' segments][NR][128] partial outputs
   float2* part_ml;       // [2 CTAs' segments][NR] their (reference, sum)
 };
 struct CacheMaps { CUtensorMap m[2][4]; };   // K and V slabs: boxes of 32, 64, 96 and 128 rows
-struct Maps { CacheMaps cache; CUtensorMap q, kv_new; };
+struct Maps { CacheMaps cache; CUtensorMap q, kv_new, q_bundle; };
 
 size_t bytes(const ps_config& g);                 // of the buffers; 0 when padded_rows() is 0
 Buffers carve(const ps_config& g, char* base);
