@@ -8,7 +8,7 @@
 // latency of a handful of dependent loads: hence the neighbouring element-wise work inside the
 // products, the first weights in flight before the wait for the kernel ahead, and no predicates in
 // the inner loop.  Measured (hidden 256, 5 rows, 64 cached keys; draft + verify): 18 launches 114 us
-// -> 9 launches 49 us.
+// -> 9 launches 49 us -> 39 (attention, verify).
 #include <cfloat>
 
 #include "ps_internal.cuh"
@@ -282,130 +282,179 @@ __global__ void __launch_bounds__(128) k_rope_store(const __grid_constant__ SeqM
   }
 }
 
+// 8 consecutive cached values in shared memory as floats; p is 16-byte aligned.
+__device__ __forceinline__ void shared8(const float* p, float (&w)[8]) {
+  const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+  w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+}
+__device__ __forceinline__ void shared8(const __nv_bfloat16* p, float (&w)[8]) {
+  const uint4 r = *reinterpret_cast<const uint4*>(p);
+  const uint32_t u[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    w[2 * i] = __uint_as_float(u[i] << 16);
+    w[2 * i + 1] = __uint_as_float(u[i] & 0xffff0000u);
+  }
+}
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
 // Attention under the parallel-draft mask: row j of a sequence sees cache rows [0, len) and the new
-// rows 0..j, which come from q / kv before RoPE.  One block per (head, sequence).  A tile of 256 keys
-// at a time: a thread holds the scores of one key against all rows, then 256 / D groups of threads
+// rows 0..j, which come from q / kv before RoPE.  One block per (head, sequence).  A tile of keys at a
+// time: one or two threads hold the scores of a key against all rows, then 256 / D groups of threads
 // walk the keys, a thread per channel; running maximum and sums between tiles.
+// What bounds it at the lengths fp32 models are used at is a chain of latencies, so the first tile's cached rows
+// are asked for before the wait for the kernel ahead, all at once, and RC rows (4, 8 or 16) are computed
+// without a branch per row, each of which waited for a shared-memory load of its own (5 rows, 64 keys:
+// 11.5 -> 6.9 us; draft + verify, 5 rows 47.9 -> 41.8 us; what the rows past R hold is not kept).
 constexpr int kAttThreads = 256;
 template <typename WT, int D>
+constexpr int att_pitch() { return D + 16 / (int)sizeof(WT); }
+template <int D>
+constexpr int att_tile() { return 16384 / D; }
+template <typename WT, int D>
+constexpr int att_smem() { return 2 * att_tile<D>() * att_pitch<WT, D>() * (int)sizeof(WT); }
+template <typename WT, int D, int RC>
 __global__ void __launch_bounds__(kAttThreads) k_attention(const __grid_constant__ SeqMap sm, const float* __restrict__ q,
                                                            const float* __restrict__ kv, const WT* __restrict__ kcache,
                                                            const WT* __restrict__ vcache, int n_heads, int n_kv_heads,
                                                            int max_ctx, const double* __restrict__ inv_freq, float* attn) {
-  constexpr int RMAX = kMaxRowsPerSeq, HALF = D / 2, GROUPS = kAttThreads / D, WARPS = kAttThreads / 32;
-  __shared__ __align__(16) float s_q[RMAX][D], s_k[RMAX][D], s_v[RMAX][D];   // rotated q (scaled), the new rows
-  __shared__ float s_p[RMAX][kAttThreads];
-  __shared__ float s_red[WARPS][RMAX];
+  constexpr int HALF = D / 2, GROUPS = kAttThreads / D, WARPS = kAttThreads / 32, TK = att_tile<D>(), P = att_pitch<WT, D>();
+  constexpr int PARTS = kAttThreads / TK, VEC = 16 / (int)sizeof(WT), VPR = D / VEC;
+  extern __shared__ __align__(16) unsigned char att_smem_raw[];
+  WT* const s_kt = reinterpret_cast<WT*>(att_smem_raw);   // [TK][P]
+  WT* const s_vt = s_kt + TK * P;
+  __shared__ __align__(16) float s_q[RC][D];               // rotated q (scaled)
+  __shared__ __align__(16) WT s_kn[RC][D], s_vn[RC][D];    // the new rows, as the cache holds them
+  __shared__ float s_p[RC][TK];
+  __shared__ float s_cs[RC][HALF], s_sn[RC][HALF];
+  __shared__ float s_red[WARPS][RC];
   const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int R = sm.row_off[b + 1] - sm.row_off[b], L = sm.len[b], m0 = sm.row_off[b] - sm.row_base;
-  const int hk = h / (n_heads / n_kv_heads), Hq = n_heads * D, Hkv = n_kv_heads * D;
+  const int hk = h / (n_heads / n_kv_heads), Hq = n_heads * D, Hkv = n_kv_heads * D, total = L + R;
   const WT* kb = kcache + ((size_t)sm.slot[b] * n_kv_heads + hk) * max_ctx * D;
   const WT* vb = vcache + ((size_t)sm.slot[b] * n_kv_heads + hk) * max_ctx * D;
   pdl_launch_dependents();
-  // rotation table, parked in the score tile: cos then sin of (row, pair)
-  float* cs = &s_p[0][0];
-  float* sn = cs + RMAX * HALF;
-  static_assert(2 * RMAX * HALF <= RMAX * kAttThreads, "the table fits the score tile");
-  for (int i = tid; i < R * HALF; i += kAttThreads) {
+  auto stage = [&](int t0) {   // cached rows of the tile, asynchronously
+    const int n = min(TK, L - t0);
+    for (int i = tid; i < n * VPR; i += kAttThreads) {
+      const int r = i / VPR, c = (i % VPR) * VEC;
+      cp_async16(s_kt + r * P + c, kb + (size_t)(t0 + r) * D + c);
+      cp_async16(s_vt + r * P + c, vb + (size_t)(t0 + r) * D + c);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  stage(0);   // (the cache is older than the launch before)
+  for (int i = tid; i < R * HALF; i += kAttThreads) {   // rotations of the new positions
     double s, c;
     sincos((double)(L + i / HALF) * inv_freq[i % HALF], &s, &c);
-    cs[i] = (float)c;
-    sn[i] = (float)s;
+    s_cs[i / HALF][i % HALF] = (float)c;
+    s_sn[i / HALF][i % HALF] = (float)s;
   }
-  __syncthreads();
   pdl_wait();
   const float scale = rsqrtf((float)D);
+  __syncthreads();
   for (int i = tid; i < R * HALF; i += kAttThreads) {
     const int j = i / HALF, e = i - j * HALF;
     const float* qr = q + (size_t)(m0 + j) * Hq + h * D + e;
     const float* kr = kv + (size_t)(m0 + j) * 2 * Hkv + hk * D + e;
     const float q0 = __ldcg(qr), q1 = __ldcg(qr + HALF), k0 = __ldcg(kr), k1 = __ldcg(kr + HALF), v0 = __ldcg(kr + Hkv),
-                v1 = __ldcg(kr + Hkv + HALF), c = cs[i], s = sn[i];
+                v1 = __ldcg(kr + Hkv + HALF), c = s_cs[j][e], s = s_sn[j][e];
     s_q[j][e] = (q0 * c - q1 * s) * scale;
     s_q[j][e + HALF] = (q1 * c + q0 * s) * scale;
-    s_k[j][e] = rounded<WT>(k0 * c - k1 * s);
-    s_k[j][e + HALF] = rounded<WT>(k1 * c + k0 * s);
-    s_v[j][e] = rounded<WT>(v0);
-    s_v[j][e + HALF] = rounded<WT>(v1);
+    store_as(&s_kn[j][e], k0 * c - k1 * s);
+    store_as(&s_kn[j][e + HALF], k1 * c + k0 * s);
+    store_as(&s_vn[j][e], v0);
+    store_as(&s_vn[j][e + HALF], v1);
   }
-  __syncthreads();
-  float m[RMAX], l[RMAX], o[RMAX];
+  float m[RC], l[RC], o[RC];
 #pragma unroll
-  for (int j = 0; j < RMAX; ++j) { m[j] = -FLT_MAX; l[j] = 0.f; o[j] = 0.f; }
-  const int d = tid % D, grp = tid / D, total = L + R;
-  for (int t0 = 0; t0 < total; t0 += kAttThreads) {
-    const int t = t0 + tid, nk = min(kAttThreads, total - t0);
-    float s[RMAX];
+  for (int j = 0; j < RC; ++j) { m[j] = -FLT_MAX; l[j] = 0.f; o[j] = 0.f; }
+  const int d = tid % D, grp = tid / D, key = tid / PARTS, part = tid % PARTS;
+  for (int t0 = 0; t0 < total; t0 += TK) {
+    const int nk = min(TK, total - t0), r_new = max(0, L - t0);
+    if (t0 > 0) stage(t0);
+    __syncthreads();   // the new rows are formed
+    for (int i = tid; i < (nk - r_new) * D; i += kAttThreads) {   // those of them in the tile
+      const int r = r_new + i / D, c = i % D, j = t0 + r - L;
+      s_kt[r * P + c] = s_kn[j][c];
+      s_vt[r * P + c] = s_vn[j][c];
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    float s[RC];
 #pragma unroll
-    for (int j = 0; j < RMAX; ++j) s[j] = 0.f;
-    if (t < total) {
-      for (int c = 0; c < D; c += 8) {
+    for (int j = 0; j < RC; ++j) s[j] = 0.f;
+    if (key < nk) {
+#pragma unroll 2
+      for (int c0 = 0; c0 < D / PARTS; c0 += 8) {
+        const int c = c0 + part * (D / PARTS);
         float k8[8];
-        if (t < L) {
-          load8(kb + (size_t)t * D + c, k8);
-        } else {
+        shared8(s_kt + key * P + c, k8);
 #pragma unroll
-          for (int e = 0; e < 8; ++e) k8[e] = s_k[t - L][c + e];
-        }
-#pragma unroll
-        for (int j = 0; j < RMAX; ++j) {
-          if (j < R) {   // (uniform)
-            const float4 a = *reinterpret_cast<const float4*>(&s_q[j][c]), a2 = *reinterpret_cast<const float4*>(&s_q[j][c + 4]);
-            s[j] += (k8[0] * a.x + k8[1] * a.y + k8[2] * a.z + k8[3] * a.w) + (k8[4] * a2.x + k8[5] * a2.y + k8[6] * a2.z + k8[7] * a2.w);
-          }
+        for (int j = 0; j < RC; ++j) {
+          const float4 a = *reinterpret_cast<const float4*>(&s_q[j][c]), a2 = *reinterpret_cast<const float4*>(&s_q[j][c + 4]);
+          s[j] += (k8[0] * a.x + k8[1] * a.y + k8[2] * a.z + k8[3] * a.w) + (k8[4] * a2.x + k8[5] * a2.y + k8[6] * a2.z + k8[7] * a2.w);
         }
       }
     }
+    __syncwarp();
+    float mx[RC];
 #pragma unroll
-    for (int j = 0; j < RMAX; ++j) {
-      if (j < R) {
-        if (t >= total || t - L > j) s[j] = -FLT_MAX;   // a new key is seen by its own row and the later ones
-        float mx = s[j];
+    for (int j = 0; j < RC; ++j) {
 #pragma unroll
-        for (int x = 16; x > 0; x >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, x));
-        if (lane == 0) s_red[warp][j] = mx;
-      }
+      for (int x = 1; x < PARTS; x <<= 1) s[j] += __shfl_xor_sync(0xffffffffu, s[j], x);
+      if (key >= nk || t0 + key - L > j || j >= R) s[j] = -FLT_MAX;   // a new key is seen by its own row and the later ones
+      mx[j] = s[j];
+    }
+#pragma unroll
+    for (int x = 16; x > 0; x >>= 1)
+#pragma unroll
+      for (int j = 0; j < RC; ++j) mx[j] = fmaxf(mx[j], __shfl_xor_sync(0xffffffffu, mx[j], x));
+    if (lane == 0) {
+#pragma unroll
+      for (int j = 0; j < RC; ++j) s_red[warp][j] = mx[j];
     }
     __syncthreads();
 #pragma unroll
-    for (int j = 0; j < RMAX; ++j) {
-      if (j < R) {
-        float mx = m[j];
+    for (int j = 0; j < RC; ++j) {
+      float t = m[j];
 #pragma unroll
-        for (int w = 0; w < WARPS; ++w) mx = fmaxf(mx, s_red[w][j]);
-        const float f = __expf(m[j] - mx), p = s[j] > -FLT_MAX ? __expf(s[j] - mx) : 0.f;
-        l[j] = l[j] * f + p;      // (this thread's share of the row's sum)
-        o[j] *= f;
-        m[j] = mx;
-        s_p[j][tid] = p;
-      }
+      for (int w = 0; w < WARPS; ++w) t = fmaxf(t, s_red[w][j]);
+      const float f = __expf(m[j] - t), p = s[j] > -FLT_MAX ? __expf(s[j] - t) : 0.f;
+      l[j] = l[j] * f + (part == 0 ? p : 0.f);      // (this thread's share of the row's sum)
+      o[j] *= f;
+      m[j] = t;
+      if (part == 0) s_p[j][key] = p;
     }
     __syncthreads();
 #pragma unroll 4
     for (int kk = grp; kk < nk; kk += GROUPS) {
-      const int tk = t0 + kk;
-      const float v = tk < L ? to_f32(vb[(size_t)tk * D + d]) : s_v[tk - L][d];
+      const float v = to_f32(s_vt[kk * P + d]);
 #pragma unroll
-      for (int j = 0; j < RMAX; ++j)
-        if (j < R) o[j] += s_p[j][kk] * v;
+      for (int j = 0; j < RC; ++j) o[j] += s_p[j][kk] * v;
     }
     __syncthreads();
   }
-  // the rows' sums over all threads, the groups' partial outputs
+  // the rows' sums over all threads, the groups' partial outputs (in the keys' place)
+  float (*const s_o)[kAttThreads] = reinterpret_cast<float (*)[kAttThreads]>(att_smem_raw);
+  static_assert(RC * kAttThreads * 4 <= att_smem<WT, D>(), "they fit it");
 #pragma unroll
-  for (int j = 0; j < RMAX; ++j) {
-    if (j < R) {
-      const float t = warp_sum(l[j]);
-      if (lane == 0) s_red[warp][j] = t;
-      s_p[j][tid] = o[j];
-    }
+  for (int x = 16; x > 0; x >>= 1)
+#pragma unroll
+    for (int j = 0; j < RC; ++j) l[j] += __shfl_xor_sync(0xffffffffu, l[j], x);
+#pragma unroll
+  for (int j = 0; j < RC; ++j) {
+    if (lane == 0) s_red[warp][j] = l[j];
+    s_o[j][tid] = o[j];
   }
   __syncthreads();
   for (int i = tid; i < R * D; i += kAttThreads) {
     const int j = i / D, e = i - j * D;
     float num = 0.f, den = 0.f;
 #pragma unroll
-    for (int g = 0; g < GROUPS; ++g) num += s_p[j][g * D + e];
+    for (int g = 0; g < GROUPS; ++g) num += s_o[j][g * D + e];
 #pragma unroll
     for (int w = 0; w < WARPS; ++w) den += s_red[w][j];
     attn[(size_t)(m0 + j) * Hq + h * D + e] = num / den;
@@ -564,6 +613,18 @@ ps_status kv_append_impl(ps_ctx* c, const SeqMap& sm, int rows, const void* hidd
   return cuda_check(c, e, "k_rope_store");
 }
 
+template <typename WT, int D>
+cudaError_t attention(ps_ctx* c, const SeqMap& sm, int B, cudaStream_t st) {
+  const ps_config& g = c->cfg;
+  const int R = g.k_masks + 1;
+  auto kern = R <= 4 ? k_attention<WT, D, 4> : R <= 8 ? k_attention<WT, D, 8> : k_attention<WT, D, 16>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, att_smem<WT, D>());
+  if (e != cudaSuccess) return e;
+  return launch_after(kern, dim3(g.n_heads, B), dim3(kAttThreads), att_smem<WT, D>(), st, !c->prof, sm, c->q, c->kv_tmp,
+                      (const WT*)c->kcache, (const WT*)c->vcache, g.n_heads, g.n_kv_heads, g.max_ctx,
+                      (const double*)c->rope_inv_freq, c->attn);
+}
+
 template <typename WT>
 ps_status draft_impl(ps_ctx* c, const SeqMap& sm, int B, const void* hidden_last,
                      const int* token_last, int top_n, int* top_ids, float* top_logit,
@@ -575,10 +636,9 @@ ps_status draft_impl(ps_ctx* c, const SeqMap& sm, int B, const void* hidden_last
   typedef const WT* P;
   ps_status s;
   if ((s = fc_qkv<WT>(c, sm, M, 0, hidden_last, token_last, true, st))) return s;
-  auto attn = g.head_dim == 64 ? k_attention<WT, 64> : k_attention<WT, 128>;
-  const cudaError_t e = launch_after(attn, dim3(g.n_heads, B), dim3(kAttThreads), 0, st, !c->prof, sm, c->q, c->kv_tmp,
-                                     (P)c->kcache, (P)c->vcache, g.n_heads, g.n_kv_heads, g.max_ctx,
-                                     (const double*)c->rope_inv_freq, c->attn);
+  cudaError_t e;
+  if (g.head_dim == 64) e = attention<WT, 64>(c, sm, B, st);
+  else e = attention<WT, 128>(c, sm, B, st);
   c->launches++;
   if (e != cudaSuccess) return cuda_check(c, e, "k_attention");
   prof_mark(c, st, "attention");
