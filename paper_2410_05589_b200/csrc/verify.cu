@@ -624,10 +624,12 @@ __global__ void __cluster_dims__(kClu, 1, 1) __launch_bounds__(kCluThreads) k_ve
   verify_cluster_body<kClu, 2>(a);
 }
 // (Rows of up to 8192 tokens: one block, whose barriers cost less than a cluster's; 1000 tokens, 5 row
-// pairs: 13.3 -> 11.1 us.)
+// pairs: 13.3 -> 11.1 us.  Rows of up to 2048 and 4096 tokens: a quarter and a half of the tokens a thread, for
+// the unrolled loops of a kernel that runs its code once: 1000 tokens, draft + verify 41.8 -> 39.0 us.)
 constexpr int kOneMaxVocab = kCluThreads * 4 * kCluV4;
+template <int V4>
 __global__ void __launch_bounds__(kCluThreads) k_verify_block(VerifyArgs a) {
-  verify_cluster_body<1, kCluV4>(a);
+  verify_cluster_body<1, V4>(a);
 }
 __global__ void __launch_bounds__(kCluThreads) k_verify_cluster16(VerifyArgs a) {
   verify_cluster_body<16, kCluV4>(a);
@@ -1704,7 +1706,10 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
     const bool share = a.V > 6144 && (4 * pairs * kClu <= 3 * c->n_sm ||
                                       (n_target == n_draft && pairs * kClu > c->n_sm && pairs * kCluSmall <= c->n_sm));
     if (a.V <= kOneMaxVocab && !share) {
-      e = launch_after(k_verify_block, dim3(n_target, B), dim3(kCluThreads), 0, st, pdl, a);
+      // (as few tokens a thread as hold the row: see verify_cluster_body)
+      constexpr int kPer = kCluThreads * 4;
+      e = launch_after(a.V <= kPer ? k_verify_block<1> : a.V <= 2 * kPer ? k_verify_block<2> : k_verify_block<kCluV4>,
+                       dim3(n_target, B), dim3(kCluThreads), 0, st, pdl, a);
     } else if (nclu == kClu && a.V <= kCluSmallMaxVocab && n_target * B * kClu > c->n_sm) {   // half the waves
       e = launch_after(k_verify_cluster4, dim3(n_target * kCluSmall, B), dim3(kCluThreads), 0, st, pdl, a);
     } else if (nclu == kClu) {

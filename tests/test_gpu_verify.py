@@ -151,3 +151,17 @@ def test_monte_carlo_losslessness_on_device():
         out = g.verify(ps.to_device(toks), dl, tl, 1.0, seed=3, offset=r)
         counts += np.bincount(out["out_tokens"][:, 0].cpu().numpy(), minlength=V)
     assert stats.chisquare(counts, p * B * reps).pvalue > 1e-3
+
+
+# one block a row pair with one, two and four vectors a thread: the vocabularies around their lines
+@pytest.mark.parametrize("vocab", [4, 2044, 2048, 2052, 4096, 4100])
+def test_one_block_token_counts(vocab):
+    import paper_2410_05589_b200 as ps
+    s = synth.CONFIGS["mini32"].with_(hidden=64, n_heads=1, n_kv_heads=1, ffn=64, vocab=vocab, k_masks=3)
+    g = ps.drafter_from_shape(s, synth.weights(s), max_batch=2, max_ctx=8)
+    for T in (0.0, 0.7, 1.0):
+        tl = synth.zipf_logits(5, (vocab, T), 2, 5, vocab)
+        dl = synth.noisy_draft_logits(5, (vocab, T), tl[:, :4], 0.4)
+        tok = synth.sample_from_logits(5, (vocab, T), dl, T or 1.0)
+        out = g.verify(ps.to_device(tok), ps.to_device(dl), ps.to_device(tl), T, 3, 8)
+        assert_verify_same({k: v.cpu().numpy() for k, v in out.items()}, oracle.verify(tok, dl, tl, T, 3, 8))
