@@ -1160,6 +1160,10 @@ k_umma_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
 // accumulator row so that the finisher has all contributors' values in flight at once, and
 // what does not depend on the sums (who shares the tile, the residual rows) is fetched while
 // the MMAs still run.
+// MP: activation rows of the operands, 8 or 16.  Every weight box of 16 KB comes with the planes' boxes of 256 MP
+// bytes, all of them through L2, so that up to 8 rows take half of that traffic, one stage more fits the
+// ring, and the epilogue reads and adds half of the columns (13B, one sequence, 5 rows: 243.9 -> 242.5 us;
+// 128256 tokens 339.0 -> 336.7).
 constexpr int kChainMax = 4, kChainMaps = 13;
 struct ChainParams {
   int n;                                  // stages
@@ -1179,17 +1183,18 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
 }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
 
+template <int MP>
 __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_constant__ ChainParams p) {
   using namespace umma;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char* stages = smem_raw + (base - raw);
-  Ctl& ctl = *reinterpret_cast<Ctl*>(stages + kStages * kStageBytes);
+  Ctl& ctl = *reinterpret_cast<Ctl*>(stages + kRingBytes);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (tid == 0) {
-    for (int i = 0; i < kStages; ++i) { mbar_init(&ctl.full[i], 1); mbar_init(&ctl.empty[i], 1); }
+    for (int i = 0; i < n_stages<MP>(); ++i) { mbar_init(&ctl.full[i], 1); mbar_init(&ctl.empty[i], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&ctl.acc_full[i], 1); mbar_init(&ctl.acc_empty[i], kEpiThreads); }
     ctl.abort_flag = 0; ctl.is_last = 0; ctl.tile_last = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1208,8 +1213,8 @@ __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_c
 
   const int G = gridDim.x;
   volatile int* abort_flag = &ctl.abort_flag;
-  constexpr int MP = kMaxRows, sbytes = kStageBytes, nst = kStages, ksplit = kSplit, acols = kAccCols;
-  constexpr int plane_bytes = kBBytes;
+  constexpr int sbytes = stage_bytes<MP>(), nst = n_stages<MP>(), ksplit = kSplit, acols = kSplit * 2 * MP;
+  constexpr int plane_bytes = MP * kBK * 2;
   auto stage_segs = [&](const UArgs& a) {
     const int U = a.n_tiles * a.KB;
     return Segs(unit_begin(blockIdx.x, U, G), unit_begin(blockIdx.x + 1, U, G), a.KB);
@@ -1311,7 +1316,7 @@ __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_c
       for (int s = 0; s < p.n && alive; ++s) {
         const UArgs& a = p.a[s];
         const Segs segs = stage_segs(a);
-        const uint32_t id = a.lo ? idesc(2 * MP) : idesc(MP);
+        const uint32_t id = a.lo || MP == 8 ? idesc(2 * MP) : idesc(MP);   // (8 columns are too few for an instruction)
         for (int si = 0; si < segs.n && alive; ++si, ++segc) {
           int t, b, e;
           segs.get(si, t, b, e);
@@ -1415,39 +1420,41 @@ __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_c
         if (res_pre) {
           bool valid;
           const int n = tile_feature(a, t, r, valid);
-          float rvp[16];
+          float rvp[MP];
 #pragma unroll
-          for (int m = 0; m < 16; ++m) rvp[m] = (valid && m < mc) ? __ldcg(a.res + (size_t)m * a.ldr + n) : 0.f;
+          for (int m = 0; m < MP; ++m) rvp[m] = (valid && m < mc) ? __ldcg(a.res + (size_t)m * a.ldr + n) : 0.f;
 #pragma unroll
-          for (int m = 0; m < 16; ++m) ctl.land[m * 128 + r] = rvp[m];
+          for (int m = 0; m < MP; ++m) ctl.land[m * 128 + r] = rvp[m];
         }
         if (!whole) epi_sync();   // the contributor table is complete
         if (!dry && epi_any(!mbar_wait(&ctl.acc_full[buf], (segc >> 1) & 1, abort_flag))) { alive = false; break; }
         fence_after_sync();
         const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + buf * acols;
-        float v[16];
+        float v[MP];
 #pragma unroll
-        for (int m = 0; m < 16; ++m) v[m] = 0.f;
+        for (int m = 0; m < MP; ++m) v[m] = 0.f;
         if (!dry) {   // the tile's sums over this CTA's k-blocks: the accumulators and their hi / lo halves
           // (the ksplit accumulators, hi half then lo half each, are 2 ksplit MP consecutive columns:
-          // two loads bring them all, one wait)
-          static_assert(2 * ksplit * MP == 128, "accumulators of a tile span 128 columns");
+          // one or two loads bring them all, one wait)
+          static_assert(acols == (MP == 8 ? 64 : 128), "one or two loads");
           float w0[64], w1[64];
           tmem_ld64(ta, w0);
-          tmem_ld64(ta + 64, w1);
+          if constexpr (MP == 16) tmem_ld64(ta + 64, w1);
           tmem_ld_wait();
           const bool lo = a.lo != 0;
 #pragma unroll
-          for (int m = 0; m < 16; ++m) {
+          for (int m = 0; m < MP; ++m) {
             // same order of additions as one load per group: acc0.hi, acc0.lo, acc1.hi, ...
             float x = w0[m];
-            if (lo) x += w0[16 + m];
-            x += w0[32 + m];
-            if (lo) x += w0[48 + m];
-            x += w1[m];
-            if (lo) x += w1[16 + m];
-            x += w1[32 + m];
-            if (lo) x += w1[48 + m];
+            if (lo) x += w0[MP + m];
+            x += w0[2 * MP + m];
+            if (lo) x += w0[3 * MP + m];
+            const float (&w)[64] = MP == 16 ? w1 : w0;
+            constexpr int at = MP == 16 ? 0 : 4 * MP;
+            x += w[at + m];
+            if (lo) x += w[at + MP + m];
+            x += w[at + 2 * MP + m];
+            if (lo) x += w[at + 3 * MP + m];
             v[m] = x;
           }
           fence_before_sync();
@@ -1461,7 +1468,7 @@ __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_c
           if (blockIdx.x != c_last) {
             float4* d4 = reinterpret_cast<float4*>(P + r * 16);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < MP / 4; ++i)
               if (i < nvec) d4[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
             epi_sync();   // (orders the other threads' stores before the release below)
             if (et == 0) {
@@ -1488,11 +1495,11 @@ __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_c
             // up to four contributors' vectors in flight together
             const int nc = dry ? 1 : c_last - c_first;   // (the rehearsal reads this CTA's own slot)
             const float* Pr = a.partials + r * 16;
-            float own[16];
+            float own[MP];
 #pragma unroll
-            for (int m = 0; m < 16; ++m) { own[m] = v[m]; v[m] = 0.f; }
+            for (int m = 0; m < MP; ++m) { own[m] = v[m]; v[m] = 0.f; }
             const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (mc <= 8) {
+            if (MP == 8 || mc <= 8) {
 #pragma unroll 1
               for (int j0 = 0; j0 < nc; j0 += 4) {
                 float4 x[4][2];
@@ -1510,7 +1517,7 @@ __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_c
                     v[4 * i] += x[j][i].x; v[4 * i + 1] += x[j][i].y; v[4 * i + 2] += x[j][i].z; v[4 * i + 3] += x[j][i].w;
                   }
               }
-            } else {
+            } else if constexpr (MP == 16) {
 #pragma unroll 1
               for (int j0 = 0; j0 < nc; j0 += 2) {
                 float4 x[2][4];
@@ -1530,10 +1537,10 @@ __global__ void __launch_bounds__(umma::kThreads, 1) k_umma_chain(const __grid_c
               }
             }
 #pragma unroll
-            for (int m = 0; m < 16; ++m) v[m] += own[m];   // the finisher is the last in CTA order
+            for (int m = 0; m < MP; ++m) v[m] += own[m];   // the finisher is the last in CTA order
           }
 #pragma unroll
-          for (int m = 0; m < 16; ++m) ctl.acc[m * 128 + r] = v[m];
+          for (int m = 0; m < MP; ++m) ctl.acc[m * 128 + r] = v[m];
           if (epi == EPI_STORE) tile_epilogue<EPI_STORE>(a, ctl, t, r, q, lane, 0, mc, dry, res_pre);
           else if (epi == EPI_SWIGLU) tile_epilogue<EPI_SWIGLU>(a, ctl, t, r, q, lane, 0, mc, dry);
           else tile_epilogue<EPI_LMHEAD>(a, ctl, t, r, q, lane, 0, mc, dry);
@@ -1662,8 +1669,8 @@ __global__ void k_late_copy(uint32_t* dst, const uint32_t* src, size_t n, long l
 }
 
 // ---- host side: tensor maps of the operands -----------------------------------------------------
-struct PlaneMaps {   // one activation plane: boxes of 16 rows, and of every size the CTA-pair GEMM takes
-  CUtensorMap m16;
+struct PlaneMaps {   // one activation plane: boxes of 16 and 8 rows, and of every size the CTA-pair GEMM takes
+  CUtensorMap m16, m8;
   pg::PlaneMaps pair;
 };
 constexpr int kPlanSlots = 128;
@@ -1681,7 +1688,7 @@ struct UmmaMaps {
 };
 
 bool make_plane_maps(PlaneMaps* pm, const void* base, size_t rows, size_t cols) {
-  if (!make_map(&pm->m16, base, rows, cols, 16)) return false;
+  if (!make_map(&pm->m16, base, rows, cols, 16) || !make_map(&pm->m8, base, rows, cols, 8)) return false;
   for (int i = 0; i < pg::kMaxNp / pg::kNpStep; ++i) {
     if (i > 1 && (size_t)(i / 2) * pg::kNpStep >= rows) { pm->pair.m[i] = pm->pair.m[i - 1]; continue; }   // never that many rows
     if (!make_map(&pm->pair.m[i], base, rows, cols, (i + 1) * pg::kNpStep / 2)) return false;
@@ -1780,6 +1787,7 @@ ps_status run_stages(ps_ctx* c, StageDesc* d, int n, bool chain, int chain_id, c
     return PS_OK;
   }
   if (n > kChainMax) return fail(c, PS_ERR_INVALID_ARG, "too many chained stages");
+  const bool few = d[0].a.M <= 8;   // (see k_umma_chain)
   ChainParams p{};
   p.n = n;
   // (every chain of a step has counters of its own: a launch may start before the one two ahead of it has ended)
@@ -1800,11 +1808,11 @@ ps_status run_stages(ps_ctx* c, StageDesc* d, int n, bool chain, int chain_id, c
     }
     if (nm + 2 > kChainMaps + (x.a.lo ? 0 : 1)) return fail(c, PS_ERR_INVALID_ARG, "too many tensor maps in a chain");
     p.map_bh[i] = nm;
-    p.maps[nm++] = x.ph->m16;
+    p.maps[nm++] = few ? x.ph->m8 : x.ph->m16;
     p.map_bl[i] = p.map_bh[i];
-    if (x.a.lo) { p.map_bl[i] = nm; p.maps[nm++] = x.pl->m16; }
+    if (x.a.lo) { p.map_bl[i] = nm; p.maps[nm++] = few ? x.pl->m8 : x.pl->m16; }
   }
-  auto kern = k_umma_chain;
+  auto kern = few ? k_umma_chain<8> : k_umma_chain<16>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, umma::kSmemBytes);
   if (e != cudaSuccess) return cuda_check(c, e, "chain smem attribute");
   // A dependent launch like the others.  Its CTAs wait for one another: the grid is one CTA per

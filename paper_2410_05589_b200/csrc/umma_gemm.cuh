@@ -51,6 +51,7 @@ constexpr int kABytes = kTile * kBK * 2;          // 16 KB
 constexpr int kBBytes = kN * kBK * 2;             // 2 KB per plane at 16 rows
 constexpr int kStageBytes = kABytes + 2 * kBBytes;
 constexpr int kStages = 10;
+constexpr int kMaxStages = 12;
 constexpr int kRingBytes = kStages * kStageBytes;
 constexpr int kThreads = 192;
 constexpr int kEpiThreads = 128;
@@ -158,8 +159,8 @@ __device__ __forceinline__ bool epi_any(bool pred) {
 constexpr int kMaxCtas = 192;   // CTAs of one launch (one per SM)
 
 struct Ctl {
-  uint64_t full[kStages];     // a stage's boxes have landed
-  uint64_t empty[kStages];    // the MMAs that read a stage have completed
+  uint64_t full[kMaxStages];  // a stage's boxes have landed
+  uint64_t empty[kMaxStages]; // the MMAs that read a stage have completed
   uint64_t acc_full[2];       // an accumulator holds a finished segment
   uint64_t acc_empty[2];      // the epilogue warps have read it back
   uint32_t tmem_base;
@@ -178,6 +179,13 @@ struct Ctl {
   float land[kN * 128];       // partials of a shared tile on their way in: [pair of a batch][accumulator row]
   int coff[kMaxCtas];         // a shared tile's contributors: element offset of each one's partial, -1: none
 };
+
+// Rings of launches with up to MP = 8 or 16 activation rows: with 8 the planes' boxes are half as large.
+template <int MP>
+constexpr int stage_bytes() { return kABytes + 2 * MP * kBK * 2; }
+template <int MP>
+constexpr int n_stages() { return MP == 8 ? 11 : kStages; }
+static_assert(n_stages<8>() * stage_bytes<8>() <= kRingBytes && n_stages<8>() <= kMaxStages, "one control block serves both");
 
 constexpr int kSmemBytes = kStages * kStageBytes + (int)sizeof(Ctl) + 1024;   // + alignment slack
 

@@ -376,3 +376,16 @@ def test_mask_count_extremes(k, B):
     p = Pair(s, B)
     _compare_step(p, top_n=2)
     assert p.g.poll() == 0
+
+
+# the chained launches' operands of 8 and of 16 activation rows: the first, the last and the first beyond, a draft
+# step and an append of as many rows
+@pytest.mark.parametrize("B,k", [(1, 0), (1, 6), (1, 7), (2, 3), (3, 2), (1, 8), (8, 1)])
+def test_rows_around_the_operands(B, k):
+    s = synth.CONFIGS["mini"].with_(k_masks=k)
+    p = Pair(s, B, lens=[B * (k + 1)] + [3 + 5 * b for b in range(1, B)])
+    got = p.gpu_step(top_n=2)
+    for b in range(B):
+        want = p.oracle_step(b)
+        assert logits_close(got["logits"][b], want["logits"], s.dtype) <= 1.0, b     # the logits gate
+    assert p.g.check_guards() == 0 and p.g.poll() == 0
