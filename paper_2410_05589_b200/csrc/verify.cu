@@ -328,6 +328,7 @@ struct CluPart {       // one per block, read by the whole cluster
   int targ, bad;
   double st, sd;
   double wsum;         // weight held by this block
+  double turn[2];      // sums of successive exchanges (tree walk)
   int pick, lastp;     // token chosen inside this block / its last token with weight
 };
 
@@ -337,11 +338,32 @@ struct CluScratch {
   double d[kCluWarps], d2[kCluWarps];
 };
 
+// exp argument (t - m) / T with one rounding: in single precision with the rounding errors of the
+// difference and of the product carried along (i_hi + i_lo = 1 / T).  UNIT: T = 1.
+template <bool UNIT>
+__device__ __forceinline__ float exp_arg(float t, float m, float i_hi, float i_lo) {
+  const float d = t - m;
+  if (UNIT) return d;
+  const float bv = t - d, av = d + bv;
+  const float e = (t - av) + (bv - m);
+  const float p = d * i_hi;
+  const float r = p + (fmaf(d, i_hi, -p) + fmaf(e, i_hi, d * i_lo));
+  return d == -INFINITY ? d : r;   // (a NaN stays one)
+}
+
+// The same by way of double precision; at T = 1 that is the difference rounded once, which single precision
+// gives bit for bit without the conversions (the register-resident kernels, 8 or 16 tokens a thread and row: 13B, one
+// sequence 242.5 -> 241.4 us for draft + verify).
+template <bool UNIT>
+__device__ __forceinline__ float exp_arg_d(float t, float m, double inv_t) {
+  return UNIT ? t - m : (float)(((double)t - (double)m) * inv_t);
+}
+
 // (NCLU blocks per cluster: 8; 16 for vocabularies beyond 65536; 4 for batches of several waves.)
 // (V4: 16-byte vectors a thread holds per row: 4, or 2 when the row fits in half as many -- the
 // loops over a thread's tokens are unrolled, and this kernel runs its code once per launch, so
 // what it is not asked to execute it should not have to fetch.)
-template <int NCLU, int V4>
+template <int NCLU, int V4, bool UNIT>
 __device__ __forceinline__ void verify_cluster_body(const VerifyArgs& a) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
@@ -464,10 +486,10 @@ __device__ __forceinline__ void verify_cluster_body(const VerifyArgs& a) {
 #pragma unroll
     for (int e = 0; e < V4 * 4; ++e) {
       const bool in = e < C && v0 + e < V;
-      t[e] = in ? expf((float)(((double)t[e] - (double)tmax) * inv_t)) : 0.f;
+      t[e] = in ? expf(exp_arg_d<UNIT>(t[e], tmax, inv_t)) : 0.f;
       st += (double)t[e];
       if (drow) {
-        d[e] = in ? expf((float)(((double)d[e] - (double)dmax) * inv_t)) : 0.f;
+        d[e] = in ? expf(exp_arg_d<UNIT>(d[e], dmax, inv_t)) : 0.f;
         sd += (double)d[e];
       }
     }
@@ -616,30 +638,34 @@ __device__ __forceinline__ void verify_cluster_body(const VerifyArgs& a) {
 
 
 // The 8-block cluster is fixed at compile time; the 16-block one (an opt-in size) is a launch attribute.
+template <bool UNIT>
 __global__ void __cluster_dims__(kClu, 1, 1) __launch_bounds__(kCluThreads) k_verify_cluster(VerifyArgs a) {
-  verify_cluster_body<kClu, kCluV4>(a);
+  verify_cluster_body<kClu, kCluV4, UNIT>(a);
 }
 // (rows of up to 32768 tokens: 8 tokens per thread)
+template <bool UNIT>
 __global__ void __cluster_dims__(kClu, 1, 1) __launch_bounds__(kCluThreads) k_verify_cluster_v2(VerifyArgs a) {
-  verify_cluster_body<kClu, 2>(a);
+  verify_cluster_body<kClu, 2, UNIT>(a);
 }
 // (Rows of up to 8192 tokens: one block, whose barriers cost less than a cluster's; 1000 tokens, 5 row
 // pairs: 13.3 -> 11.1 us.  Rows of up to 2048 and 4096 tokens: a quarter and a half of the tokens a thread, for
 // the unrolled loops of a kernel that runs its code once: 1000 tokens, draft + verify 41.8 -> 39.0 us.)
 constexpr int kOneMaxVocab = kCluThreads * 4 * kCluV4;
-template <int V4>
+template <int V4, bool UNIT>
 __global__ void __launch_bounds__(kCluThreads) k_verify_block(VerifyArgs a) {
-  verify_cluster_body<1, V4>(a);
+  verify_cluster_body<1, V4, UNIT>(a);
 }
+template <bool UNIT>
 __global__ void __launch_bounds__(kCluThreads) k_verify_cluster16(VerifyArgs a) {
-  verify_cluster_body<16, kCluV4>(a);
+  verify_cluster_body<16, kCluV4, UNIT>(a);
 }
 // Four blocks per row pair: for batches whose 8-block clusters would not be resident at once
 // (one block fills an SM) while these are, and a thread can still hold its share of a row (16 tokens).
 constexpr int kCluSmall = 4;
 constexpr int kCluSmallMaxVocab = kCluSmall * kCluThreads * 4 * kCluV4;
+template <bool UNIT>
 __global__ void __cluster_dims__(kCluSmall, 1, 1) __launch_bounds__(kCluThreads) k_verify_cluster4(VerifyArgs a) {
-  verify_cluster_body<kCluSmall, kCluV4>(a);
+  verify_cluster_body<kCluSmall, kCluV4, UNIT>(a);
 }
 
 // ---- streaming variant: many row pairs --------------------------------------------------------
@@ -672,19 +698,6 @@ struct StreamScratch {
   double d[kStrWarps], d2[kStrWarps];
 };
 constexpr float kRefSlack = 60.f;   // exponent range left beside the reference before sums are formed again
-
-// exp argument (t - m) / T with one rounding: in single precision with the rounding errors of the
-// difference and of the product carried along (i_hi + i_lo = 1 / T).  UNIT: T = 1.
-template <bool UNIT>
-__device__ __forceinline__ float exp_arg(float t, float m, float i_hi, float i_lo) {
-  const float d = t - m;
-  if (UNIT) return d;
-  const float bv = t - d, av = d + bv;
-  const float e = (t - av) + (bv - m);
-  const float p = d * i_hi;
-  const float r = p + (fmaf(d, i_hi, -p) + fmaf(e, i_hi, d * i_lo));
-  return d == -INFINITY ? d : r;   // (a NaN stays one)
-}
 
 template <bool UNIT>
 __global__ void __launch_bounds__(kStrThreads, kStrPerSm) k_verify_stream(VerifyArgs a, VerifyRow* rows, VerifyDraw* draws) {
@@ -1227,25 +1240,28 @@ __global__ void __launch_bounds__(kStrThreads, kStrPerSm) k_row_softmax(const __
   cl.sync();   // no block leaves while the first one reads its part
 }
 
-// Sum over the cluster of one double per thread; every thread of every block gets the value.
+// Sum over the cluster of one double per thread; every thread of every block gets the value.  (One cluster
+// barrier and shuffle trees instead of two and a serial sum over the warps, here and in the draw: the walk
+// of 23 nodes, 128256 tokens, 29 -> 25 us.)
 __device__ double cluster_sum(cooperative_groups::cluster_group& cl, CluPart& part, CluScratch& s, double v,
-                              int tid, int warp, int lane) {
+                              int& turn, int warp, int lane) {
   v = warp_sum_d(v);
   __syncthreads();
   if (lane == 0) s.d[warp] = v;
   __syncthreads();
-  if (tid == 0) {
-    double x1 = 0.0;
-    for (int w = 0; w < kCluWarps; ++w) x1 += s.d[w];
-    part.wsum = x1;
+  if (warp == 0) {
+    double x1 = lane < kCluWarps ? s.d[lane] : 0.0;
+#pragma unroll
+    for (int o = kCluWarps / 2; o > 0; o >>= 1) x1 += __shfl_xor_sync(0xffffffffu, x1, o);
+    if (lane == 0) part.turn[turn] = x1;
   }
   cl.sync();
   // lane r fetches block r's sum (one remote round trip), a shuffle tree adds them
-  double tot = lane < (int)cl.num_blocks() ? cl.map_shared_rank(&part, lane)->wsum : 0.0;
+  double tot = lane < (int)cl.num_blocks() ? cl.map_shared_rank(&part, lane)->turn[turn] : 0.0;
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
   tot = __shfl_sync(0xffffffffu, tot, 0);
-  cl.sync();   // every block has read the partials before they are rewritten
+  turn ^= 1;   // (the other place next time: whoever rewrites this one has seen everyone past the next barrier)
   return tot;
 }
 
@@ -1272,11 +1288,17 @@ __device__ int cluster_draw(cooperative_groups::cluster_group& cl, CluPart& part
   __syncthreads();
   if (lane == 31) { s.d[warp] = incl; s.i[warp] = lastp; }
   __syncthreads();
-  if (tid == 0) {
-    double x1 = 0.0;
-    int lp = -1;
-    for (int k = 0; k < kCluWarps; ++k) { x1 += s.d[k]; lp = max(lp, s.i[k]); }
-    part.wsum = x1; part.lastp = lp; part.pick = -1;
+  // running sums over the warps, in order (every warp forms them: the one that holds the token needs its own)
+  double winc = lane < kCluWarps ? s.d[lane] : 0.0;
+  const double wown = winc;
+#pragma unroll
+  for (int o = 1; o < kCluWarps; o <<= 1) {
+    const double up = __shfl_up_sync(0xffffffffu, winc, o);
+    if (lane >= o) winc += up;
+  }
+  if (warp == 0) {
+    const int lp = __reduce_max_sync(0xffffffffu, lane < kCluWarps ? s.i[lane] : -1);
+    if (lane == kCluWarps - 1) { part.wsum = winc; part.lastp = lp; part.pick = -1; }
   }
   cl.sync();
   // lane r holds block r's weight; a shuffle scan gives every block's running sum
@@ -1299,13 +1321,10 @@ __device__ int cluster_draw(cooperative_groups::cluster_group& cl, CluPart& part
       base = __shfl_sync(0xffffffffu, binc - bw, sel);
     }
     if (sel == rank) {
-      double t2 = target - base, wrun = 0.0, wbase = 0.0;
-      int wsel = -1;
-      for (int k = 0; k < kCluWarps; ++k) {
-        const double nx = wrun + s.d[k];
-        if (wsel < 0 && nx > t2) { wsel = k; wbase = wrun; }
-        wrun = nx;
-      }
+      const double t2 = target - base;
+      const unsigned over_w = __ballot_sync(0xffffffffu, lane < kCluWarps && winc > t2);
+      const int wsel = over_w ? __ffs(over_w) - 1 : -1;
+      const double wbase = __shfl_sync(0xffffffffu, winc - wown, max(wsel, 0));
       if (warp == wsel) {
         const double t3 = t2 - wbase;
         const unsigned over = __ballot_sync(0xffffffffu, incl > t3);
@@ -1352,6 +1371,7 @@ struct TreeNodes {
 };
 
 // (The cluster size is a launch attribute: see launch_verify_tree.)
+template <bool UNIT>
 __global__ void __launch_bounds__(kCluThreads) k_tree_walk(const __grid_constant__ TreeArgs a) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
@@ -1392,7 +1412,7 @@ __global__ void __launch_bounds__(kCluThreads) k_tree_walk(const __grid_constant
     nd.r[tid] = (double)(ctr[0] >> 8) * (1.0 / 16777216.0);
   }
   __syncthreads();
-  int u = 0, len = 0, any_bad = 0, token = -1;
+  int u = 0, len = 0, any_bad = 0, token = -1, turn = 0;
   // every block takes the same branches below: the values they depend on are identical
   for (;;) {
     const int kid0 = a.topo.child_off[u], n_kids = a.topo.child_off[u + 1] - kid0;
@@ -1434,8 +1454,8 @@ __global__ void __launch_bounds__(kCluThreads) k_tree_walk(const __grid_constant
 #pragma unroll
         for (int e = 0; e < kCluV4 * 4; ++e) {
           const bool in = e < C && v0 + e < V;
-          t[e] = in ? expf((float)(((double)t[e] - (double)tmax) * inv_t)) : 0.f;
-          d[e] = (in && drow) ? expf((float)(((double)d[e] - (double)ds.max) * inv_t)) : 0.f;
+          t[e] = in ? expf(exp_arg_d<UNIT>(t[e], tmax, inv_t)) : 0.f;
+          d[e] = (in && drow) ? expf(exp_arg_d<UNIT>(d[e], ds.max, inv_t)) : 0.f;
         }
       };
       double st = ts.sum;
@@ -1497,7 +1517,7 @@ __global__ void __launch_bounds__(kCluThreads) k_tree_walk(const __grid_constant
           double mine = 0.0;
 #pragma unroll
           for (int e = 0; e < kCluV4 * 4; ++e) mine += (double)t[e];
-          st = cluster_sum(cl, part, s, mine, tid, warp, lane);
+          st = cluster_sum(cl, part, s, mine, turn, warp, lane);
         }
       }
       if (bad) {
@@ -1524,7 +1544,7 @@ __global__ void __launch_bounds__(kCluThreads) k_tree_walk(const __grid_constant
           double mine = 0.0;
 #pragma unroll
           for (int e = 0; e < kCluV4 * 4; ++e) mine += (double)fmaxf(t[e] * inv_st - cf * (d[e] * inv_sd), 0.f);
-          const double Z = cluster_sum(cl, part, s, mine, tid, warp, lane);
+          const double Z = cluster_sum(cl, part, s, mine, turn, warp, lane);
           if (Z > 0.0) { c = c_new; Zc = Z; } else { c = 0.0; Zc = 1.0; }   // nothing left: back to p
         }
         if (next < 0) {
@@ -1665,6 +1685,7 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
   a.rec = c->vrec; a.tickets = c->tickets; a.status = c->dev_status;
   const bool aligned = (((uintptr_t)target_logits | (uintptr_t)draft_logits) & 15u) == 0;
   const int nclu = a.V <= kCluMaxVocab ? kClu : 16, pairs = n_target * B;
+  const bool unit = temperature == 1.f || temperature == 0.f;   // (no exponentials at 0)
   // More row pairs than the register-resident clusters can take at once (each of their blocks fills
   // an SM): the streaming kernel, with as many blocks per pair as are resident together.  Below that
   // the register-resident ones win: one launch, and no second look at the rows.  Arg-max alone of many rows
@@ -1677,7 +1698,6 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
     while (per < 8 && 2 * pairs * per <= kStrPerSm * c->n_sm) per *= 2;
     const size_t bytes = (size_t)(((a.V + kDrawClu - 1) / kDrawClu + kSeg - 1) / kSeg) * sizeof(double);
     if (bytes <= 40 * 1024) {
-      const bool unit = temperature == 1.f;
       prof_mark(c, st, "begin");
       cudaError_t e = launch_cluster(unit ? k_verify_stream<true> : k_verify_stream<false>, dim3(n_target * per, B), per,
                                      kStrThreads, 0, st, false, a, c->vrow, c->vdraw);
@@ -1691,7 +1711,7 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
       return cuda_check(c, e, "k_verify_stream");
     }
   }
-  if (a.V % 4 == 0 && a.V <= kCluMaxVocab16 && aligned && (nclu == kClu || cluster_size_ok(c->cluster_ok[0], k_verify_cluster16, 16))) {
+  if (a.V % 4 == 0 && a.V <= kCluMaxVocab16 && aligned && (nclu == kClu || cluster_size_ok(c->cluster_ok[unit ? 0 : 2], unit ? k_verify_cluster16<true> : k_verify_cluster16<false>, 16))) {
     prof_mark(c, st, "begin");
     cudaError_t e;
     // (The 8-block clusters are plain launches: as dependents they start their loads earlier and run
@@ -1708,15 +1728,18 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
     if (a.V <= kOneMaxVocab && !share) {
       // (as few tokens a thread as hold the row: see verify_cluster_body)
       constexpr int kPer = kCluThreads * 4;
-      e = launch_after(a.V <= kPer ? k_verify_block<1> : a.V <= 2 * kPer ? k_verify_block<2> : k_verify_block<kCluV4>,
+      e = launch_after(a.V <= kPer       ? (unit ? k_verify_block<1, true> : k_verify_block<1, false>)
+                       : a.V <= 2 * kPer ? (unit ? k_verify_block<2, true> : k_verify_block<2, false>)
+                                         : (unit ? k_verify_block<kCluV4, true> : k_verify_block<kCluV4, false>),
                        dim3(n_target, B), dim3(kCluThreads), 0, st, pdl, a);
     } else if (nclu == kClu && a.V <= kCluSmallMaxVocab && n_target * B * kClu > c->n_sm) {   // half the waves
-      e = launch_after(k_verify_cluster4, dim3(n_target * kCluSmall, B), dim3(kCluThreads), 0, st, pdl, a);
+      e = launch_after(unit ? k_verify_cluster4<true> : k_verify_cluster4<false>, dim3(n_target * kCluSmall, B), dim3(kCluThreads), 0, st, pdl, a);
     } else if (nclu == kClu) {
-      e = launch_after(a.V <= kClu * kCluThreads * 4 * 2 ? k_verify_cluster_v2 : k_verify_cluster,
+      e = launch_after(a.V <= kClu * kCluThreads * 4 * 2 ? (unit ? k_verify_cluster_v2<true> : k_verify_cluster_v2<false>)
+                                                         : (unit ? k_verify_cluster<true> : k_verify_cluster<false>),
                        dim3(n_target * kClu, B), dim3(kCluThreads), 0, st, false, a);
     } else {
-      e = launch_cluster(k_verify_cluster16, dim3(n_target * 16, B), 16, kCluThreads, 0, st, false, a);
+      e = launch_cluster(unit ? k_verify_cluster16<true> : k_verify_cluster16<false>, dim3(n_target * 16, B), 16, kCluThreads, 0, st, false, a);
     }
     c->launches++;
     prof_mark(c, st, "verify");
@@ -1778,7 +1801,9 @@ ps_status launch_verify_tree(ps_ctx* c, int B, int n_nodes, const int* parent, c
   // not find room at once (16 trees of 23 nodes, 32000 tokens: 47.0 with clusters of 8, 34.8 with 4).
   const int want = a.V <= kOneMaxVocab / 2 ? 1 : a.V <= kOneMaxVocab ? kCluSmall : a.V <= kCluMaxVocab ? kClu : 16;
   const int nclu = 4 * B * want > 3 * c->n_sm ? least : want;
-  if (!cluster_size_ok(c->cluster_ok[1], k_tree_walk, nclu))
+  const bool unit = temperature == 1.f || temperature == 0.f;
+  auto walk = unit ? k_tree_walk<true> : k_tree_walk<false>;
+  if (!cluster_size_ok(c->cluster_ok[unit ? 1 : 3], walk, nclu))
     return fail(c, PS_ERR_UNSUPPORTED, "this device cannot run the 16-block clusters a vocabulary beyond 65536 needs");
   TreeRows list;
   list.n = 0;
@@ -1795,7 +1820,7 @@ ps_status launch_verify_tree(ps_ctx* c, int B, int n_nodes, const int* parent, c
                                  kStrThreads, 0, st, !c->prof, a, list);
   c->launches++;
   if (e == cudaSuccess) {
-    e = launch_cluster(k_tree_walk, dim3(nclu, B), nclu, kCluThreads, 0, st, !c->prof, a);
+    e = launch_cluster(walk, dim3(nclu, B), nclu, kCluThreads, 0, st, !c->prof, a);
     c->launches++;
   }
   prof_mark(c, st, "verify_tree");
