@@ -304,15 +304,18 @@ __global__ void __launch_bounds__(kThreads) k_logit_stats(const float* __restric
 ps_status launch_logit_stats(ps_ctx* c, const float* logits, int M, int V, int R, int top_n, int* top_ids,
                              float* top_logit, float* row_max, float* row_lse, const SampleArgs* sa, cudaStream_t st) {
   if (top_n <= 0 && !row_max && !row_lse && !sa) return PS_OK;
-  // Blocks per row (two are resident per SM): the count whose waves of 1 / nclu rows each are over first,
-  // with at least 2048 tokens a block (below that its fixed cost, about 2 us of reductions, outweighs
-  // what it takes off the pass).  144 rows of 32000 tokens: 2 blocks in one wave, 50 -> 30 us against 4
-  // in two; a single full wave is worth more than its share says (80 rows: 7 blocks in two waves 31 us).
+  // Blocks per row: the count whose waves are over first, with at least 2048 tokens a block (below that its
+  // fixed cost, about 2 us of reductions, outweighs what it takes off the pass).  With the sampler two blocks
+  // are resident per SM and its arithmetic is what takes time, so only the balance counts: 144 rows of
+  // 32000 tokens, 2 blocks in one wave, 50 -> 30 us against 4 in two; a single full wave is worth more
+  // than its share says (80 rows: 7 blocks in two waves 31 us).  Without it three are resident and a block
+  // is through 32000 tokens in about 5 us, so that many rows want few blocks: 640 rows 66 -> 33 us.
   int nclu = 1;
   double best = 1e30;
   for (int n = 1; n <= 8 && (n == 1 || V / n >= 2048); ++n) {
-    const long waves = ((long)M * n + 2 * c->n_sm - 1) / (2 * c->n_sm);
-    const double cost = (waves > 1 ? 1.15 : 1.0) * waves / n + 0.005 * n;
+    const long slots = (sa ? 2l : 3l) * c->n_sm, waves = ((long)M * n + slots - 1) / slots;
+    const double pass = 5.0 * V / 32000;
+    const double cost = sa ? (waves > 1 ? 1.15 : 1.0) * waves / n + 0.005 * n : waves * (2.5 + pass / n) + 0.05 * n;
     if (cost < best) { best = cost; nclu = n; }
   }
   cudaLaunchConfig_t cfg = {};
