@@ -458,10 +458,12 @@ k_pair_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
 }
 
 // Shared tiles of a MODE_STORE / MODE_SWIGLU stage: adds the contributors' slots in k order.
-// Block (tile, 8 rows); bound by the latency of its few loads, so a thread has all rows of a
-// contributor in flight together.
-constexpr int kFinRows = 8;
-template <bool ZIP>
+// Block (tile, kFinRows rows, and of a plain tile 256 of its columns); bound by the latency of its loads.  Where
+// the blocks of four rows find room at once, a thread has four rows of four contributors in flight (a tile of the
+// last wave has up to 18 contributors, each of which was a round trip with eight rows: 13B, 20 rows, q|k|v 7.1 -> 3.3
+// us; 33B, 144 rows 10 -> 4.7; 576 rows, LM head 10.2 -> 6.0); beyond that eight rows of two (of one, of gate and up)
+// move more per instruction (2048 appended rows 17.5 -> 15.0 us, 903 rows 24 -> 9.5; four of four 16.4).
+template <bool ZIP, int kFinRows, int kFinJ>
 __global__ void __launch_bounds__(256) k_finish_shared(const __grid_constant__ Args a) {
   pdl_launch_dependents();
   const Plan& p = a.p;
@@ -469,53 +471,50 @@ __global__ void __launch_bounds__(256) k_finish_shared(const __grid_constant__ A
   int w = t / p.n_rt;
   const int rt = t - w * p.n_rt, mi0 = blockIdx.y * kFinRows, m0 = rt * p.Np + mi0;
   const int rows = min(min(kFinRows, p.Np - mi0), p.M - m0);
+  const int TW = 256 * p.wt, c = blockIdx.z * 256 + threadIdx.x;   // (zipped: the second half are the up features)
+  const float* s = a.part + slot_row(p, 0, t, mi0) + c;
+  const size_t layer = (size_t)p.Np * TW;
+  constexpr int NS = ZIP ? 2 : 1;
+  float v[NS][kFinRows];
+#pragma unroll
+  for (int h = 0; h < NS; ++h)
+#pragma unroll
+    for (int i = 0; i < kFinRows; ++i) v[h][i] = 0.f;
   pdl_wait();
   if (cnt < 2 || rows <= 0) return;
-  const int TW = 256 * p.wt;
+  for (int j = 0; j < cnt; j += kFinJ) {
+    float x[kFinJ][NS][kFinRows];
+#pragma unroll
+    for (int b = 0; b < kFinJ; ++b)
+#pragma unroll
+      for (int h = 0; h < NS; ++h)
+#pragma unroll
+        for (int i = 0; i < kFinRows; ++i)
+          x[b][h][i] = j + b < cnt && i < rows ? __ldcg(s + (j + b) * layer + (size_t)i * TW + 256 * h) : 0.f;
+#pragma unroll
+    for (int b = 0; b < kFinJ; ++b)
+#pragma unroll
+      for (int h = 0; h < NS; ++h)
+#pragma unroll
+        for (int i = 0; i < kFinRows; ++i) v[h][i] += x[b][h][i];
+  }
   if (ZIP) {
-    const int n = w * 256 + threadIdx.x;
-    float g[kFinRows], u[kFinRows];
-#pragma unroll
-    for (int i = 0; i < kFinRows; ++i) g[i] = u[i] = 0.f;
-    for (int j = 0; j < cnt; ++j) {
-      const float* s = a.part + slot_row(p, j, t, mi0) + threadIdx.x;
-      float xg[kFinRows], xu[kFinRows];
-#pragma unroll
-      for (int i = 0; i < kFinRows; ++i) {
-        xg[i] = i < rows ? __ldcg(s + (size_t)i * TW) : 0.f;
-        xu[i] = i < rows ? __ldcg(s + (size_t)i * TW + 256) : 0.f;
-      }
-#pragma unroll
-      for (int i = 0; i < kFinRows; ++i) { g[i] += xg[i]; u[i] += xu[i]; }
-    }
+    const int n = w * 256 + c;
     if (n < p.mat_rows[0]) {
 #pragma unroll
       for (int i = 0; i < kFinRows; ++i) {
         const size_t at = (size_t)(m0 + i) * a.ld_plane + n;
-        if (i < rows) split1(silu_mul(g[i], u[i]), a.hi[at], a.lo[at]);
+        if (i < rows) split1(silu_mul(v[0][i], v[NS - 1][i]), a.hi[at], a.lo[at]);
       }
     }
   } else {
     int mat = 0;
     while (mat + 1 < p.n_mats && w >= p.mat_tiles[mat]) { w -= p.mat_tiles[mat]; ++mat; }
-    for (int c = threadIdx.x; c < TW; c += 256) {
-      const int n = w * TW + c;
-      float v[kFinRows];
+    const int n = w * TW + c;
+    if (n < p.mat_rows[mat]) {
 #pragma unroll
-      for (int i = 0; i < kFinRows; ++i) v[i] = 0.f;
-      for (int j = 0; j < cnt; ++j) {
-        const float* s = a.part + slot_row(p, j, t, mi0) + c;
-        float x[kFinRows];
-#pragma unroll
-        for (int i = 0; i < kFinRows; ++i) x[i] = i < rows ? __ldcg(s + (size_t)i * TW) : 0.f;
-#pragma unroll
-        for (int i = 0; i < kFinRows; ++i) v[i] += x[i];
-      }
-      if (n < p.mat_rows[mat]) {
-#pragma unroll
-        for (int i = 0; i < kFinRows; ++i)
-          if (i < rows) a.out[(size_t)(m0 + i) * a.ldo + p.mat_off[mat] + n] = v[i];
-      }
+      for (int i = 0; i < kFinRows; ++i)
+        if (i < rows) a.out[(size_t)(m0 + i) * a.ldo + p.mat_off[mat] + n] = v[0][i];
     }
   }
 }
@@ -743,9 +742,12 @@ ps_status launch_gemm(ps_ctx* c, const Weights& w, const PlaneMaps& hi, const Pl
 ps_status launch_finish_shared(ps_ctx* c, const Args& a, Mode mode, cudaStream_t st) {
   const Plan& p = a.p;
   if (!p.shared) return PS_OK;
-  const dim3 grid(p.rem, (std::min(p.Np, p.M) + kFinRows - 1) / kFinRows);
-  const cudaError_t e = mode == MODE_SWIGLU ? launch_after(k_finish_shared<true>, grid, dim3(256), 0, st, !c->prof, a)
-                                            : launch_after(k_finish_shared<false>, grid, dim3(256), 0, st, !c->prof, a);
+  const int np = std::min(p.Np, p.M), z = mode == MODE_SWIGLU ? 1 : p.wt;
+  const bool few = p.rem * ((np + 3) / 4) * z <= 3 * c->n_sm;   // (see k_finish_shared)
+  const int rows = few ? 4 : 8;
+  auto kern = mode == MODE_SWIGLU ? (few ? k_finish_shared<true, 4, 4> : k_finish_shared<true, 8, 1>)
+                                  : (few ? k_finish_shared<false, 4, 4> : k_finish_shared<false, 8, 2>);
+  const cudaError_t e = launch_after(kern, dim3(p.rem, (np + rows - 1) / rows, z), dim3(256), 0, st, !c->prof, a);
   c->launches++;
   return cuda_check(c, e, "k_finish_shared");
 }
