@@ -2171,6 +2171,35 @@ int fused_kv_rows(ps_ctx* c) {
   return fused_supported(c, most) && c->umma_maps ? most : 0;
 }
 
+// Rows of the passes that an append of `total` rows is made in.  A pass of n row tiles of 256 gives fc and k | v
+// so many tiles of 512 features, which the CTA pairs take in waves (those of either stage are as long as
+// one another).  A last wave that is nearly full counts whole; a small remainder is shared out with all
+// pairs, which costs its slots' way through memory, about a quarter of a wave; a pass about a tenth.
+// 13B: of 2048 rows fc has 80 tiles and k | v 160 on 74 pairs, of 1792 it is 70 and 140.  4999 rows in
+// passes of 2048 1414 us, of 1792 1328, of 1536 1414; 3900 rows 1091-1134 us and 998-1036, 3500 rows 901 and
+// 890; 7B shape (64 and 128 tiles) 958, 1042, 1043.  Splits that the count puts less than 4% ahead measured
+// even (33B shape, 4200 rows: 1876-1917 us in passes of 2048, 1914-1933 of 1536), so those stay with the most.
+int append_pass_rows(const ps_config& g, int n_sm, int total, int most) {
+  const int P = n_sm / 2, Hkv = g.n_kv_heads * g.head_dim, fc = (g.hidden + 511) / 512, kv = 2 * ((Hkv + 511) / 512);
+  auto waves = [&](int tiles) {
+    const int rem = tiles % P;
+    return tiles / P + (rem ? std::min(1.0, (double)rem / P + 0.25) : 0.0);
+  };
+  auto pass = [&](int rows) {
+    const int n = (rows + pg::kMaxNp - 1) / pg::kMaxNp;
+    return waves(fc * n) + waves(kv * n) + 0.1;
+  };
+  if (total <= pg::kMaxNp || most <= pg::kMaxNp) return most;
+  auto passes = [&](int rows) { return total / rows * pass(rows) + (total % rows ? pass(total % rows) : 0.0); };
+  int best = most;
+  double least = 0.96 * passes(most);
+  for (int rows = (most - 1) / pg::kMaxNp * pg::kMaxNp; rows >= pg::kMaxNp; rows -= pg::kMaxNp) {   // whole row tiles
+    const double cost = passes(rows);
+    if (cost < least - 1e-9) { least = cost; best = rows; }
+  }
+  return best;
+}
+
 ps_status fused_kv_append(ps_ctx* c, const SeqMap& sm, int rows, const void* hidden, const int* tokens,
                           cudaStream_t st) {
   return umma_kv_append(c, *static_cast<UmmaMaps*>(c->umma_maps), sm, rows, hidden, tokens, st);

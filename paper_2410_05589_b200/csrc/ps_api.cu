@@ -343,7 +343,8 @@ ps_status ps_poll(ps_ctx* c, void* stream) {
 // plain kernels.
 static ps_status append_rows(ps_ctx* c, SeqMap& sm, int total, const void* hidden, const int* tokens,
                              cudaStream_t st) {
-  const int fused_rows = fused_kv_rows(c), chunk = fused_rows > 0 ? fused_rows : kAppendChunk;
+  const int fused_rows = fused_kv_rows(c);
+  const int chunk = fused_rows > 0 ? append_pass_rows(c->cfg, c->n_sm, total, fused_rows) : kAppendChunk;
   for (int r0 = 0; r0 < total; r0 += chunk) {
     sm.row_base = r0;
     const int rows = std::min(chunk, total - r0);

@@ -206,7 +206,8 @@ bool make_map(CUtensorMap* m, const void* base, size_t rows, size_t cols, int bo
 bool make_halves_map(CUtensorMap* m, const void* base, size_t rows, int box_rows);
 // ---- fused bf16 kernels for small M ---------------------------------------------------------
 bool fused_supported(ps_ctx* c, int M);
-int fused_kv_rows(ps_ctx* c);     // rows per pass of fused_kv_append (0: not available)
+int fused_kv_rows(ps_ctx* c);     // most rows per pass of fused_kv_append (0: not available)
+int append_pass_rows(const ps_config& g, int n_sm, int total, int most);   // rows of an append's passes, at most `most`
 ps_status fused_kv_append(ps_ctx* c, const SeqMap& sm, int rows, const void* hidden, const int* tokens,
                           cudaStream_t st);
 // RoPE on the k half of fp32 kv rows [0, rows) and the store of k and v into the bf16 cache rows.

@@ -124,3 +124,28 @@ def test_hidden_sizes_beyond_the_row_norm():
     for b in (0, 4):
         assert logits_close(got["logits"][b], p.oracle_step(b)["logits"], s.dtype) <= 1.0, b     # the logits gate
     assert p.g.poll() == 0
+
+
+def test_append_in_passes_that_fill_their_waves():
+    """2304 new rows, hidden 5120, 40 kv heads: a pass of 1792 rows (70 and 140 tiles on 74 pairs) and one of 512
+    instead of 2048 and 256."""
+    import paper_2410_05589_b200 as ps
+    import torch
+    from harness import oracle_for
+    B, n = 128, 18
+    s = synth.CONFIGS["mini"].with_(hidden=5120, n_heads=40, n_kv_heads=40, ffn=64, vocab=200, k_masks=1)
+    W = synth.weights(s)
+    g = ps.drafter_from_shape(s, W, max_batch=B, max_ctx=40)
+    h, t = synth.hidden_states(s, "new", B * n), synth.token_ids(s, "new", B * n)
+    before = g.launch_count()
+    g.kv_append(list(range(B)), [n] * B, ps.to_device(h), ps.to_device(t))
+    torch.cuda.synchronize()
+    assert g.launch_count() - before >= 2 * 5          # two passes of gather, fc, norm, k | v, store
+    o = oracle_for(s, W, B, 40)
+    for b in (0, 99, 100, B - 1):                      # (99: its rows lie in both passes)
+        assert o.kv_append(b, h[b * n:(b + 1) * n], t[b * n:(b + 1) * n]) == 0
+        got = [x.float().cpu().numpy() for x in g.kv_export(b)]
+        for a, w in zip(got, o.kv_export(b)):
+            # values that agree to fp32 sums of 5120 and 10240 terms, rounded to bf16: one unit in the last place
+            assert (np.abs(a - w) <= 2.0 ** -7 * np.abs(w) + 1e-4).all(), b
+    assert g.poll() == 0 and g.check_guards() == 0
