@@ -1671,6 +1671,29 @@ bool cluster_size_ok(int* cache, void (*kern)(Args), int nclu) {
   return cache[nclu] > 0;
 }
 
+// Blocks of the streaming kernel that are resident at once in clusters of nclu (asked once per context and size).  A
+// cluster lies in one group of SMs, so that not all of kStrPerSm an SM can be filled: of 592, 560 blocks in
+// clusters of 4 or of 8 run together and 580 do not.
+static int stream_blocks_fit(ps_ctx* c, bool unit, int nclu) {
+  int& fit = c->stream_fit[unit ? 0 : 1][nclu];
+  if (fit == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nclu);
+    cfg.blockDim = dim3(kStrThreads);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = nclu; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, unit ? k_verify_stream<true> : k_verify_stream<false>, &cfg) != cudaSuccess || n <= 0)
+      n = kStrPerSm * c->n_sm * 9 / (10 * nclu);
+    (void)cudaGetLastError();
+    fit = n * nclu;
+  }
+  return fit;
+}
+
 ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* draft_tokens,
                         const float* draft_logits, const float* target_logits, float temperature,
                         uint64_t seed, uint64_t offset, int* accept_len, int* out_tokens,
@@ -1688,14 +1711,15 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
   const bool unit = temperature == 1.f || temperature == 0.f;   // (no exponentials at 0)
   // More row pairs than the register-resident clusters can take at once (each of their blocks fills
   // an SM): the streaming kernel, with as many blocks per pair as are resident together.  Below that
-  // the register-resident ones win: one launch, and no second look at the rows.  Arg-max alone of many rows
+  // the register-resident ones win: one launch, and no second look at the rows.  (144 pairs of 32000 tokens: clusters of
+  // 4, some of which wait for a second wave, 23.3 us, of 2 18.7.)  Arg-max alone of many rows
   // beyond 131072 tokens is one pass of k_verify's blocks (64 x 5 rows of 131076: 48 us, streamed 54; 16 x 6
   // rows: 20, streamed 13).
   const bool greedy_long = temperature == 0.f && a.V > kCluMaxVocab16 && 4 * pairs > 3 * c->n_sm;
   const int reg_blocks = a.V <= kOneMaxVocab ? 1 : nclu == kClu && a.V <= kCluSmallMaxVocab ? kCluSmall : nclu;
   if (a.V % 4 == 0 && aligned && !greedy_long && pairs * reg_blocks > c->n_sm) {
     int per = 1;
-    while (per < 8 && 2 * pairs * per <= kStrPerSm * c->n_sm) per *= 2;
+    while (per < 8 && 2 * pairs * per <= stream_blocks_fit(c, unit, 2 * per)) per *= 2;
     const size_t bytes = (size_t)(((a.V + kDrawClu - 1) / kDrawClu + kSeg - 1) / kSeg) * sizeof(double);
     if (bytes <= 40 * 1024) {
       prof_mark(c, st, "begin");

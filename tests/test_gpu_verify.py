@@ -165,3 +165,18 @@ def test_one_block_token_counts(vocab):
         tok = synth.sample_from_logits(5, (vocab, T), dl, T or 1.0)
         out = g.verify(ps.to_device(tok), ps.to_device(dl), ps.to_device(tl), T, 3, 8)
         assert_verify_same({k: v.cpu().numpy() for k, v in out.items()}, oracle.verify(tok, dl, tl, T, 3, 8))
+
+
+@pytest.mark.parametrize("B", [28, 29])
+def test_streamed_row_pairs_around_a_wave(B):
+    """140 and 145 row pairs: clusters of 4 blocks that are all resident, and of 2 where those of 4 are not."""
+    import paper_2410_05589_b200 as ps
+    V = 32000
+    s = synth.CONFIGS["mini32"].with_(hidden=64, n_heads=1, n_kv_heads=1, ffn=64, vocab=V, k_masks=4)
+    g = ps.drafter_from_shape(s, synth.weights(s), max_batch=B, max_ctx=8)
+    for T in (0.0, 0.7, 1.0):
+        tl = synth.zipf_logits(7, (B, T), B, 5, V)
+        dl = synth.noisy_draft_logits(7, (B, T), tl[:, :4], 0.4)
+        tok = synth.sample_from_logits(7, (B, T), dl, T or 1.0)
+        out = g.verify(ps.to_device(tok), ps.to_device(dl), ps.to_device(tl), T, 3, 8)
+        assert_verify_same({k: v.cpu().numpy() for k, v in out.items()}, oracle.verify(tok, dl, tl, T, 3, 8))
