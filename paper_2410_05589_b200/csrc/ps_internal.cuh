@@ -162,8 +162,8 @@ struct ps_ctx {
   int n_sm;                 // multiprocessors of the context's device
   int smem_optin;           // opt-in shared memory per block
   // answers asked of this context's device once (0 = not asked yet)
-  int cluster_ok[4][17] = {};     // [chain verify, tree verify, the same at other T than 0 and 1][cluster size]: 1 yes, -1 no
-  int stream_fit[2][9] = {};      // [T is 0 or 1, other][cluster size]: blocks of the streaming verify resident at once (0: not asked)
+  int clusters[4][17] = {};       // [chain verify, tree walk, the same at other T than 0 and 1][cluster size]: resident at once, -1 none
+  int stream_clusters[2][9] = {}; // streaming verify [T is 0 or 1, other][cluster size]
   int attn_blocks_per_sm[4][16] = {};   // [kernel variant][tile size / 16]: resident blocks, -1 none
   cudaStream_t copy_stream = nullptr;   // ps_round_host: carries the target logits beside the draft step
   cudaEvent_t copy_done = nullptr;

@@ -1646,52 +1646,29 @@ cudaError_t launch_cluster(void (*kern)(KArgs...), dim3 grid, int nclu, int thre
   return cudaLaunchKernelEx(&cfg, kern, a...);
 }
 
-// Whether the context's device can co-schedule nclu blocks of this kernel as one cluster (sizes
-// above 8 are an opt-in of the kernel, a per-device function attribute).  Asked once per context
-// and size; `cache` is the context's row for this kernel.
-template <class Args>
-bool cluster_size_ok(int* cache, void (*kern)(Args), int nclu) {
-  if (nclu <= 8) return true;
-  if (cache[nclu] == 0) {
-    cache[nclu] = -1;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+// Clusters of nclu blocks of this kernel that are resident on the context's device at once, -1 for none (sizes above 8
+// are an opt-in of the kernel, a per-device function attribute).  Asked once per context, kernel and size.  A
+// cluster lies in one group of SMs, so not every SM can be filled: with one block an SM 33 clusters of 4 (132
+// SMs), 15 of 8 (120), 7 of 16 (112); with four an SM 560 blocks in clusters of 4 or of 8, not 592.
+template <class... Args>
+int clusters_at_once(int& cache, void (*kern)(Args...), int threads, int nclu) {
+  if (cache == 0) {
+    cache = -1;
+    if (nclu <= 8 || cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(nclu);
-      cfg.blockDim = dim3(kCluThreads);
+      cfg.blockDim = dim3(threads);
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeClusterDimension;
       at[0].val.clusterDim.x = nclu; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
       cfg.attrs = at;
       cfg.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0) cache[nclu] = 1;
+      if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0) cache = n;
     }
     (void)cudaGetLastError();
   }
-  return cache[nclu] > 0;
-}
-
-// Blocks of the streaming kernel that are resident at once in clusters of nclu (asked once per context and size).  A
-// cluster lies in one group of SMs, so that not all of kStrPerSm an SM can be filled: of 592, 560 blocks in
-// clusters of 4 or of 8 run together and 580 do not.
-static int stream_blocks_fit(ps_ctx* c, bool unit, int nclu) {
-  int& fit = c->stream_fit[unit ? 0 : 1][nclu];
-  if (fit == 0) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nclu);
-    cfg.blockDim = dim3(kStrThreads);
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = nclu; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, unit ? k_verify_stream<true> : k_verify_stream<false>, &cfg) != cudaSuccess || n <= 0)
-      n = kStrPerSm * c->n_sm * 9 / (10 * nclu);
-    (void)cudaGetLastError();
-    fit = n * nclu;
-  }
-  return fit;
+  return cache;
 }
 
 ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* draft_tokens,
@@ -1710,16 +1687,35 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
   const int nclu = a.V <= kCluMaxVocab ? kClu : 16, pairs = n_target * B;
   const bool unit = temperature == 1.f || temperature == 0.f;   // (no exponentials at 0)
   // More row pairs than the register-resident clusters can take at once (each of their blocks fills
-  // an SM): the streaming kernel, with as many blocks per pair as are resident together.  Below that
-  // the register-resident ones win: one launch, and no second look at the rows.  (144 pairs of 32000 tokens: clusters of
-  // 4, some of which wait for a second wave, 23.3 us, of 2 18.7.)  Arg-max alone of many rows
-  // beyond 131072 tokens is one pass of k_verify's blocks (64 x 5 rows of 131076: 48 us, streamed 54; 16 x 6
-  // rows: 20, streamed 13).
+  // an SM): smaller clusters where those hold a row, then the streaming kernel, with as many blocks per pair as are
+  // resident together.  Below that the register-resident ones win: one launch, and no second look at the rows.
+  // (Draft + verify of 32000 tokens: 15 pairs in clusters of 8 253 us, streamed 256; 16 and 18 pairs, in two
+  // waves, 261 and 270, in clusters of 4 259 and 263; 32 pairs in clusters of 4 272, streamed 274; 36, in two
+  // waves, 297, streamed 293.  128256 tokens: 7 pairs in clusters of 16 328, streamed 336; 8, in two waves, 343,
+  // streamed 337.  144 pairs of 32000 tokens streamed by clusters of 4, in two waves, 23.3 us, of 2 18.7.)
+  // Arg-max alone of many rows beyond 131072 tokens is one pass of k_verify's blocks (64 x 5 rows of 131076:
+  // 48 us, streamed 54; 16 x 6 rows: 20, streamed 13).
   const bool greedy_long = temperature == 0.f && a.V > kCluMaxVocab16 && 4 * pairs > 3 * c->n_sm;
-  const int reg_blocks = a.V <= kOneMaxVocab ? 1 : nclu == kClu && a.V <= kCluSmallMaxVocab ? kCluSmall : nclu;
-  if (a.V % 4 == 0 && aligned && !greedy_long && pairs * reg_blocks > c->n_sm) {
+  int* const at_once = c->clusters[unit ? 0 : 2];
+  auto fits = [&](auto kern, int n) {
+    const int k = clusters_at_once(at_once[n], kern, kCluThreads, n);
+    return pairs <= (k > 0 ? k : c->n_sm / n);
+  };
+  int reg = 0;   // blocks per pair of the register-resident kernel, 0: they don't all find room
+  if (a.V <= kOneMaxVocab) reg = pairs <= c->n_sm ? 1 : 0;
+  else if (a.V > kCluMaxVocab16) reg = pairs * 16 <= c->n_sm ? 16 : 0;   // (k_verify's)
+  else if (nclu == 16) reg = fits(unit ? k_verify_cluster16<true> : k_verify_cluster16<false>, 16) ? 16 : 0;
+  else if (a.V <= kClu * kCluThreads * 4 * 2 ? fits(unit ? k_verify_cluster_v2<true> : k_verify_cluster_v2<false>, kClu)
+                                             : fits(unit ? k_verify_cluster<true> : k_verify_cluster<false>, kClu)) reg = kClu;
+  else if (a.V <= kCluSmallMaxVocab && fits(unit ? k_verify_cluster4<true> : k_verify_cluster4<false>, kCluSmall)) reg = kCluSmall;
+  if (a.V % 4 == 0 && aligned && !greedy_long && reg == 0) {
     int per = 1;
-    while (per < 8 && 2 * pairs * per <= stream_blocks_fit(c, unit, 2 * per)) per *= 2;
+    while (per < 8) {
+      const int k = clusters_at_once(c->stream_clusters[unit ? 0 : 1][2 * per], unit ? k_verify_stream<true> : k_verify_stream<false>,
+                                     kStrThreads, 2 * per);
+      if (pairs > (k > 0 ? k : kStrPerSm * c->n_sm / (2 * per))) break;
+      per *= 2;
+    }
     const size_t bytes = (size_t)(((a.V + kDrawClu - 1) / kDrawClu + kSeg - 1) / kSeg) * sizeof(double);
     if (bytes <= 40 * 1024) {
       prof_mark(c, st, "begin");
@@ -1735,7 +1731,7 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
       return cuda_check(c, e, "k_verify_stream");
     }
   }
-  if (a.V % 4 == 0 && a.V <= kCluMaxVocab16 && aligned && (nclu == kClu || cluster_size_ok(c->cluster_ok[unit ? 0 : 2], unit ? k_verify_cluster16<true> : k_verify_cluster16<false>, 16))) {
+  if (a.V % 4 == 0 && a.V <= kCluMaxVocab16 && aligned && (nclu == kClu || clusters_at_once(at_once[16], unit ? k_verify_cluster16<true> : k_verify_cluster16<false>, kCluThreads, 16) > 0)) {
     prof_mark(c, st, "begin");
     cudaError_t e;
     // (The 8-block clusters are plain launches: as dependents they start their loads earlier and run
@@ -1756,7 +1752,7 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
                        : a.V <= 2 * kPer ? (unit ? k_verify_block<2, true> : k_verify_block<2, false>)
                                          : (unit ? k_verify_block<kCluV4, true> : k_verify_block<kCluV4, false>),
                        dim3(n_target, B), dim3(kCluThreads), 0, st, pdl, a);
-    } else if (nclu == kClu && a.V <= kCluSmallMaxVocab && n_target * B * kClu > c->n_sm) {   // half the waves
+    } else if (nclu == kClu && a.V <= kCluSmallMaxVocab && (reg == kCluSmall || (reg != kClu && pairs * kClu > c->n_sm))) {   // half the waves
       e = launch_after(unit ? k_verify_cluster4<true> : k_verify_cluster4<false>, dim3(n_target * kCluSmall, B), dim3(kCluThreads), 0, st, pdl, a);
     } else if (nclu == kClu) {
       e = launch_after(a.V <= kClu * kCluThreads * 4 * 2 ? (unit ? k_verify_cluster_v2<true> : k_verify_cluster_v2<false>)
@@ -1827,7 +1823,7 @@ ps_status launch_verify_tree(ps_ctx* c, int B, int n_nodes, const int* parent, c
   const int nclu = 4 * B * want > 3 * c->n_sm ? least : want;
   const bool unit = temperature == 1.f || temperature == 0.f;
   auto walk = unit ? k_tree_walk<true> : k_tree_walk<false>;
-  if (!cluster_size_ok(c->cluster_ok[unit ? 1 : 3], walk, nclu))
+  if (nclu > 8 && clusters_at_once(c->clusters[unit ? 1 : 3][nclu], walk, kCluThreads, nclu) < 0)
     return fail(c, PS_ERR_UNSUPPORTED, "this device cannot run the 16-block clusters a vocabulary beyond 65536 needs");
   TreeRows list;
   list.n = 0;

@@ -167,16 +167,17 @@ def test_one_block_token_counts(vocab):
         assert_verify_same({k: v.cpu().numpy() for k, v in out.items()}, oracle.verify(tok, dl, tl, T, 3, 8))
 
 
-@pytest.mark.parametrize("B", [28, 29])
-def test_streamed_row_pairs_around_a_wave(B):
-    """140 and 145 row pairs: clusters of 4 blocks that are all resident, and of 2 where those of 4 are not."""
+@pytest.mark.parametrize("V,B,n", [(32000, 3, 5), (32000, 4, 4), (32000, 11, 3), (32000, 17, 2), (32000, 28, 5), (32000, 29, 5),
+                                   (65536, 5, 3), (65536, 8, 2), (128256, 1, 7), (128256, 4, 2)])
+def test_row_pairs_around_a_wave(V, B, n):
+    """B * n row pairs on both sides of the counts at which a kernel's clusters no longer find room at once: 15 | 16
+    of 8 blocks, 33 | 34 of 4, 7 | 8 of 16, and 140 | 145 of the streaming kernel's 4."""
     import paper_2410_05589_b200 as ps
-    V = 32000
-    s = synth.CONFIGS["mini32"].with_(hidden=64, n_heads=1, n_kv_heads=1, ffn=64, vocab=V, k_masks=4)
+    s = synth.CONFIGS["mini32"].with_(hidden=64, n_heads=1, n_kv_heads=1, ffn=64, vocab=V, k_masks=n - 1)
     g = ps.drafter_from_shape(s, synth.weights(s), max_batch=B, max_ctx=8)
     for T in (0.0, 0.7, 1.0):
-        tl = synth.zipf_logits(7, (B, T), B, 5, V)
-        dl = synth.noisy_draft_logits(7, (B, T), tl[:, :4], 0.4)
-        tok = synth.sample_from_logits(7, (B, T), dl, T or 1.0)
+        tl = synth.zipf_logits(7, (V, B, T), B, n, V)
+        dl = synth.noisy_draft_logits(7, (V, B, T), tl[:, :n - 1], 0.4)
+        tok = synth.sample_from_logits(7, (V, B, T), dl, T or 1.0)
         out = g.verify(ps.to_device(tok), ps.to_device(dl), ps.to_device(tl), T, 3, 8)
         assert_verify_same({k: v.cpu().numpy() for k, v in out.items()}, oracle.verify(tok, dl, tl, T, 3, 8))
