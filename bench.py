@@ -88,8 +88,8 @@ KERNEL_OF_STAGE_PAIR = {   # more than 16 rows
 
 
 def kernel_of_stage(stage, rows):
-    if stage == "verify" and rows > 18:
-        return "k_verify_cluster4" if rows <= 37 else "k_verify_stream + k_verify_draw"
+    if stage == "verify" and rows > 15:   # (15 clusters of 8 blocks and 33 of 4 find room at once)
+        return "k_verify_cluster4" if rows <= 33 else "k_verify_stream + k_verify_draw"
     if stage == "lm_head" and 6 < rows <= 16:
         return "k_umma_gemm<STORE> + k_logit_stats"
     if rows > 16 and stage in KERNEL_OF_STAGE_PAIR:
