@@ -83,7 +83,9 @@ constexpr int smem_bytes() { return n_slots(NR) * kSlotBytes + 4 * op_bytes(NR) 
 // What a (sequence, kv head) pair is to the kernel: the query rows of the kv head's group.  Sequences that read
 // the same cache rows (the groups of the training layout: one slot, each a position longer than the one before)
 // go several to a pair, so that their common keys are read and multiplied once: `subs` of them, whose
-// rows follow one another.  Sequence i of a pair sees len + i cached keys, where len is the first one's.
+// rows follow one another.  Sequence i of a pair sees len + i cached keys, where len is the first one's; the other
+// cached ones and the new ones of other sequences have probability 0 to it, and values that fit_row() made finite (told
+// apart in k_attn_tc, by the thread that issues the products, the attention of 128 groups of 300 keys took 30 us more).
 struct Work {
   SeqMap sm;
   int off[PS_MAX_BATCH + 1];   // units before bundle b of `subs` sequences (over all its kv heads)
@@ -325,6 +327,7 @@ __global__ void __launch_bounds__(256) k_attn_prep(const __grid_constant__ Work 
         v1.v[e] = __float2bfloat16_rn(vb[e]);
       }
     }
+    if (w.subs > 1) fit_row(k0, k1, v0, v1, 16);
     __nv_bfloat16* d = kv + ((size_t)(u * w.n_kv + hk) * 2 * kNewRows + sub * R + j) * kD + i;
     *reinterpret_cast<B4*>(d) = k0;
     *reinterpret_cast<B4*>(d + kD / 2) = k1;

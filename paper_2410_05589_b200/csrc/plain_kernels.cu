@@ -502,6 +502,7 @@ __global__ void __launch_bounds__(256) k_kv_store(SeqMap sm, const float* __rest
       v0.v[e] = __float2bfloat16_rn(va[e]);
       v1.v[e] = __float2bfloat16_rn(vb[e]);
     }
+    if (sm.fit) fit_row(k0, k1, v0, v1, per);
     const size_t at = ((slab + h) * max_ctx + pos) * d + i;
     *reinterpret_cast<B4*>(kcache + at) = k0;
     *reinterpret_cast<B4*>(kcache + at + half) = k1;

@@ -499,6 +499,7 @@ ps_status ps_group_forward(ps_ctx* c, int slot, int n_groups, const void* hidden
   SeqMap sm;
   std::memset(&sm, 0, sizeof(sm));
   sm.B = 1; sm.slot[0] = slot; sm.len[0] = L0; sm.row_off[0] = 0; sm.row_off[1] = n_groups;
+  sm.fit = 1;
   if ((s = append_rows(c, sm, n_groups, hidden, tokens, st)) != PS_OK) return s;
   // 2. the groups as a batch of draft steps on the same slot: group t sees cache rows
   //    [0, L0 + t), i.e. the prefix and the real rows before it, and its own k + 1 new rows

@@ -31,7 +31,27 @@ struct SeqMap {
   int slot[PS_MAX_BATCH];
   int len[PS_MAX_BATCH];
   int row_off[PS_MAX_BATCH + 1];
+  int fit;   // 1: the rows are stored as fit_row() has them
 };
+
+// A (position, head)'s key and value, of which each of `per` neighbouring lanes (a power of two) holds a part: if the
+// value is not finite the key becomes no number and the value zero.  A query that sees the key gets a score that is
+// none, and with it a result that is none; one that must not, and only gives it a probability of zero, is left alone (0 times
+// an infinite value is not 0).  For rows that queries of several positions meet in one product.
+template <class KV>
+__device__ __forceinline__ void fit_row(KV& k0, KV& k1, KV& v0, KV& v1, int per) {
+  constexpr int N = sizeof(KV) / 2;
+  auto *a = reinterpret_cast<unsigned short*>(&v0), *b = reinterpret_cast<unsigned short*>(&v1);
+  bool bad = false;
+#pragma unroll
+  for (int e = 0; e < N; ++e) bad |= (a[e] & 0x7F80) == 0x7F80 || (b[e] & 0x7F80) == 0x7F80;
+  const unsigned lane = threadIdx.x & 31, group = (0xFFFFFFFFu >> (32 - per)) << (lane & ~(per - 1));
+  if (__ballot_sync(group, bad)) {
+    auto *c = reinterpret_cast<unsigned short*>(&k0), *d = reinterpret_cast<unsigned short*>(&k1);
+#pragma unroll
+    for (int e = 0; e < N; ++e) { c[e] = d[e] = 0x7FFF; a[e] = b[e] = 0; }
+  }
+}
 
 __device__ __forceinline__ void seq_of_row(const SeqMap& s, int m, int& b, int& j) {
   int g = m + s.row_base;

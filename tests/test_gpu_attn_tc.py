@@ -151,3 +151,74 @@ def test_groups_of_one_slot(heads, kv_heads, k, L0, n, slots):
     assert g.check_guards() == 0 and g.poll() == 0
     again = g.group_forward(0, hid, tok, want_feat=True)
     assert torch.equal(out["logits"], again["logits"])
+
+
+# A bundle reads keys that only some of its groups see: what those hold must not reach the others.  Position `bad` of the
+# new ones is the first, the middle or the last of its bundle of 3 (5 rows a group), 8 (2), 2 (2 heads x 3) or 16 (1)
+# groups; the cached keys of the bundle end before, in and behind a tile's edge (128, 256)
+_BUNDLES = [(6, 6, 4, 201, 90, (30, 31, 32, 54, 55, 89)), (18, 18, 1, 125, 100, (0, 2, 3, 4, 7, 99)),
+            (6, 3, 2, 120, 131, (6, 7, 8, 130)), (18, 18, 0, 125, 100, (2, 3, 15))]
+
+
+def _tiles(L0, n):
+    return sum(max(1, -(-(L0 + t) // 128)) for t in range(n))
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("heads,kv_heads,k,L0,n,bad", _BUNDLES)
+def test_nonfinite_position_stays_out_of_the_groups_before_it(heads, kv_heads, k, L0, n, bad, value):
+    import torch
+    import paper_2410_05589_b200 as ps
+    s = synth.CONFIGS["mini"].with_(n_heads=heads, n_kv_heads=kv_heads, k_masks=k)
+    assert _tiles(L0, n) * heads >= 6 * 148         # the rule of the dispatch
+    g = ps.drafter_from_shape(s, synth.weights(s), max_batch=min(n, 128), max_ctx=L0 + n + k + 1)
+    g.kv_import(0, *(ps.to_device(x) for x in synth.kv_rows(s, "ctx", L0)))
+    hid, tok = ps.to_device(synth.hidden_states(s, "new", n)), ps.to_device(synth.token_ids(s, "new", n))
+    clean = g.group_forward(0, hid, tok)["logits"].double().cpu().numpy()
+    for t in bad:
+        h = hid.clone()
+        h[t, 100] = value
+        out = g.group_forward(0, h, tok)["logits"]
+        assert torch.isfinite(out[:t]).all() and torch.isnan(out[t:]).all(), t
+        if t:
+            assert logits_close(out[:t].double().cpu().numpy(), clean[:t], s.dtype) <= 1.0, t     # the logits gate
+    assert g.check_guards() == 0
+
+
+@pytest.mark.parametrize("heads,kv_heads,k,L0,n,bad", _BUNDLES)
+def test_value_that_overflows_stays_out_of_the_groups_before_it(heads, kv_heads, k, L0, n, bad):
+    """Finite keys, one channel of the value row infinite: channel 7 of the normalised row is 0 but at one position,
+    and a value channel is 3e38 times it.  (The channel's way into the output has weight 0, so that nothing else
+    changes.)"""
+    import torch
+    import paper_2410_05589_b200 as ps
+    s = synth.CONFIGS["mini"].with_(n_heads=heads, n_kv_heads=kv_heads, k_masks=k)
+    w = {name: ps.to_device(x) for name, x in synth.weights(s).items() if x is not None}
+    w["w_fc"][7] = 0.0
+    w["w_fc"][7, s.hidden + 3] = 8.0                # (fc reads embedding, then features)
+    w["w_fc"][7, 3] = 8.0
+    w["embed"][:, 3] = 0.0
+    w["mask_embed"][:, 3] = 0.0
+    w["mask_feat"][:, 3] = 0.0
+    w["w_v"][5] = 0.0
+    w["w_o"].view(s.hidden, heads, s.head_dim)[:, :heads // kv_heads, 5] = 0.0
+    kw = dict(dtype=s.dtype, hidden=s.hidden, n_heads=heads, n_kv_heads=kv_heads, head_dim=s.head_dim, ffn=s.ffn, vocab=s.vocab,
+              k_masks=k, max_batch=min(n, 128), max_ctx=L0 + n + k + 1)
+    ctx = [ps.to_device(x) for x in synth.kv_rows(s, "ctx", L0)]
+    hid, tok = ps.to_device(synth.hidden_states(s, "new", n)), ps.to_device(synth.token_ids(s, "new", n))
+    hid[:, 3] = 0.0
+    plain = ps.Drafter(weights=w, **kw)
+    w_v = w["w_v"].clone()
+    w_v[5, 7] = 3e38
+    huge = ps.Drafter(weights=dict(w, w_v=w_v), **kw)
+    for g in (plain, huge):
+        g.kv_import(0, *ctx)
+    for t in bad:
+        h = hid.clone()
+        h[t, 3] = 1.0
+        want = plain.group_forward(0, h, tok)["logits"]
+        out = huge.group_forward(0, h, tok)["logits"]
+        assert torch.isfinite(want).all() and torch.isfinite(out[:t]).all() and torch.isnan(out[t:]).all(), t
+        if t:
+            assert logits_close(out[:t].double().cpu().numpy(), want[:t].double().cpu().numpy(), s.dtype) <= 1.0, t     # the logits gate
+    assert huge.check_guards() == 0
