@@ -583,9 +583,9 @@ __device__ __forceinline__ void verify_cluster_body(const VerifyArgs& a) {
           const double target = u2 * total;
           const unsigned over_b = __ballot_sync(0xffffffffu, lane < nclu && binc > target);
           double base = 0.0;
-          if (over_b) {
+          if (over_b) {   // (the base is the sum that was compared: a rounded difference could lie above the target)
             sel = __ffs(over_b) - 1;
-            base = __shfl_sync(0xffffffffu, binc - bw, sel);
+            if (sel > 0) base = __shfl_sync(0xffffffffu, binc, sel - 1);
           }
           if (sel == rank) {
             // level 2: the warp, level 3: the lane, level 4: the token
@@ -1290,7 +1290,6 @@ __device__ int cluster_draw(cooperative_groups::cluster_group& cl, CluPart& part
   __syncthreads();
   // running sums over the warps, in order (every warp forms them: the one that holds the token needs its own)
   double winc = lane < kCluWarps ? s.d[lane] : 0.0;
-  const double wown = winc;
 #pragma unroll
   for (int o = 1; o < kCluWarps; o <<= 1) {
     const double up = __shfl_up_sync(0xffffffffu, winc, o);
@@ -1315,16 +1314,18 @@ __device__ int cluster_draw(cooperative_groups::cluster_group& cl, CluPart& part
   if (total > 0.0) {
     const double target = u * total;
     const unsigned over_b = __ballot_sync(0xffffffffu, lane < nb && binc > target);
+    // At every level what is taken off the target is the very sum before the one that exceeded it, so that nothing below
+    // is negative and the token has weight (a rounded difference, sum minus own, could lie above the target).
     double base = 0.0;
     if (over_b) {
       sel = __ffs(over_b) - 1;
-      base = __shfl_sync(0xffffffffu, binc - bw, sel);
+      if (sel > 0) base = __shfl_sync(0xffffffffu, binc, sel - 1);
     }
     if (sel == rank) {
       const double t2 = target - base;
       const unsigned over_w = __ballot_sync(0xffffffffu, lane < kCluWarps && winc > t2);
       const int wsel = over_w ? __ffs(over_w) - 1 : -1;
-      const double wbase = __shfl_sync(0xffffffffu, winc - wown, max(wsel, 0));
+      const double wbase = wsel > 0 ? __shfl_sync(0xffffffffu, winc, wsel - 1) : 0.0;
       if (warp == wsel) {
         const double t3 = t2 - wbase;
         const unsigned over = __ballot_sync(0xffffffffu, incl > t3);
