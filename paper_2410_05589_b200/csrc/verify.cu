@@ -348,7 +348,14 @@ __device__ __forceinline__ float exp_arg(float t, float m, float i_hi, float i_l
   const float e = (t - av) + (bv - m);
   const float p = d * i_hi;
   const float r = p + (fmaf(d, i_hi, -p) + fmaf(e, i_hi, d * i_lo));
-  return d == -INFINITY ? d : r;   // (a NaN stays one)
+  return d == -INFINITY ? d : fabsf(p) == INFINITY ? p : r;   // (a NaN stays one; what overflows has no errors to carry)
+}
+// 1 / T in two parts.  Temperatures below the smallest whose inverse is a float act like it: logits that differ
+// at all are then 1e31 apart.
+__device__ __forceinline__ void split_inverse(double inv_t, float& i_hi, float& i_lo) {
+  const double x = fmin(inv_t, (double)FLT_MAX);
+  i_hi = (float)x;
+  i_lo = (float)(x - (double)i_hi);
 }
 
 // The same by way of double precision; at T = 1 that is the difference rounded once, which single precision
@@ -714,7 +721,8 @@ __global__ void __launch_bounds__(kStrThreads, kStrPerSm) k_verify_stream(Verify
   const int share = ((V + nclu - 1) / nclu + kSeg - 1) / kSeg * kSeg;
   const int v_lo = min(V, rank * share), n_vec = (min(V, v_lo + share) - v_lo) / 4;   // V % 4 == 0
   const double inv_t = greedy ? 1.0 : 1.0 / (double)a.temperature;
-  const float i_hi = (float)inv_t, i_lo = (float)(inv_t - (double)i_hi);
+  float i_hi, i_lo;
+  split_inverse(inv_t, i_hi, i_lo);
   pdl_launch_dependents();
 
   // ---- one pass over both rows
@@ -929,7 +937,8 @@ k_verify_draw(VerifyArgs a, const VerifyDraw* draws) {
   const int share = ((V + kDrawClu - 1) / kDrawClu + kSeg - 1) / kSeg * kSeg;
   const int v_lo = min(V, rank * share), n_vec = (min(V, v_lo + share) - v_lo) / 4;   // V % 4 == 0
   const double inv_t = 1.0 / (double)a.temperature;
-  const float i_hi = (float)inv_t, i_lo = (float)(inv_t - (double)i_hi);
+  float i_hi, i_lo;
+  split_inverse(inv_t, i_hi, i_lo);
   const float4 none = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
   pdl_launch_dependents();
   pdl_wait();
@@ -1136,7 +1145,8 @@ __global__ void __launch_bounds__(kStrThreads, kStrPerSm) k_row_softmax(const __
   const int share = ((V + nclu - 1) / nclu + kSeg - 1) / kSeg * kSeg;
   const int v_lo = min(V, rank * share), n_vec = (min(V, v_lo + share) - v_lo) / 4;   // V % 4 == 0
   const double inv_t = greedy ? 1.0 : 1.0 / (double)a.temperature;
-  const float i_hi = (float)inv_t, i_lo = (float)(inv_t - (double)i_hi);
+  float i_hi, i_lo;
+  split_inverse(inv_t, i_hi, i_lo);
   pdl_launch_dependents();
   pdl_wait();
   constexpr int U = 4;

@@ -181,3 +181,19 @@ def test_row_pairs_around_a_wave(V, B, n):
         tok = synth.sample_from_logits(7, (V, B, T), dl, T or 1.0)
         out = g.verify(ps.to_device(tok), ps.to_device(dl), ps.to_device(tl), T, 3, 8)
         assert_verify_same({k: v.cpu().numpy() for k, v in out.items()}, oracle.verify(tok, dl, tl, T, 3, 8))
+
+
+# Temperatures whose inverse times a difference of logits, or whose inverse itself, is beyond single precision: as
+# good as arg-max, in clusters that hold their rows (5 pairs) and in those that stream them (36; 8 of 128256 tokens)
+@pytest.mark.parametrize("V,B,n", [(5000, 1, 4), (32000, 1, 5), (32000, 9, 4), (128256, 2, 4)])
+def test_vanishing_temperatures(V, B, n):
+    import paper_2410_05589_b200 as ps
+    s = synth.CONFIGS["mini32"].with_(hidden=64, n_heads=1, n_kv_heads=1, ffn=64, vocab=V, k_masks=n - 1)
+    g = ps.drafter_from_shape(s, synth.weights(s), max_batch=B, max_ctx=8)
+    tl = synth.zipf_logits(9, (V, B), B, n, V)
+    dl = synth.noisy_draft_logits(9, (V, B), tl, 0.4)
+    tok = dl.argmax(-1).astype(np.int32)
+    for T in (1e-30, 1e-37, 1e-38, 1e-42):
+        out = g.verify(ps.to_device(tok), ps.to_device(dl), ps.to_device(tl), T, 3, 8)
+        assert_verify_same({k: v.cpu().numpy() for k, v in out.items()}, oracle.verify(tok, dl, tl, float(np.float32(T)), 3, 8))
+    assert g.poll() == 0

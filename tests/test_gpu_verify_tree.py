@@ -197,3 +197,17 @@ def test_draft_step_build_tree_verify_tree_chain(sampled):
     with pytest.raises(ps.PsError):
         p.g.build_tree(list(range(-1, 6)), [0] * 7, out["top_ids"])  # deeper than k+1 rows
     assert p.g.poll() == 0
+
+
+def test_tree_at_vanishing_temperatures():
+    """1 / T times a difference of logits, or 1 / T itself, beyond single precision: as good as arg-max (a chain of
+    arg-max tokens; any other has probability 0 under both)."""
+    V, B, parent = 5000, 8, [-1, 0, 1, 2]
+    g = _ctx(V)
+    _, dl, tl = _case(parent, B, V, seed=11, T=0.5)
+    toks = dl.argmax(-1).astype(np.int32)
+    for T in (1e-30, 1e-37, 1e-38, 1e-42):
+        got, want = _run_both(g, parent, toks, dl, tl, float(np.float32(T)), seed=1, offset=5)
+        _assert_same(got, want)
+        assert want["accept_len"].max() > 0
+    assert g.poll() == 0
