@@ -123,10 +123,15 @@ def _iarr(xs):
     return (C.c_int * len(xs))(*map(int, xs))
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)   # (not a public name: a torch may lack it)
+
+
 def _stream(stream=None):
     if stream is not None:
         return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 _CUDA = torch.device("cuda")   # (the current device, like the name)

@@ -47,3 +47,15 @@ def test_no_oracle_in_product_path():
             if f.endswith((".py", ".cu", ".cuh", ".h")):
                 text = open(os.path.join(dp, f)).read()
                 assert "oracle" not in text.lower(), os.path.join(dp, f)
+
+
+def test_stream_handle_without_torchs_private_name(monkeypatch):
+    import torch
+    from paper_2410_05589_b200 import binding
+
+    class Stream:
+        cuda_stream = 77
+
+    monkeypatch.setattr(binding, "_raw_stream", None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    assert binding._stream() == 77 and binding._stream(Stream) == 77
