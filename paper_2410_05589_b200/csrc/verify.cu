@@ -1753,9 +1753,11 @@ ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* 
     // One block holds rows of up to 8192 tokens; from 6144 on, clusters that are resident together share a
     // row's exponentials to more gain than their barriers cost (8192 tokens, 5 pairs 11.2 -> 9.9 us, 30 pairs
     // 11.4 -> 10.2; 5000 tokens 9.9 against 10.0), unless an extra row's draw is among many (24: 12.6, 12.9).
-    // (Clusters of 8 that need most of the chip's SMs don't all find room at once: 16 pairs 15.1, one block 10.2.)
+    // (Clusters of 8 that need most of the chip's SMs don't all find room at once: 16 pairs 15.1, one block 10.2;
+    // nor do more than 33 of 4: 36 pairs of 8000 tokens 18.0, one block 12.5.)
     const bool share = a.V > 6144 && (4 * pairs * kClu <= 3 * c->n_sm ||
-                                      (n_target == n_draft && pairs * kClu > c->n_sm && pairs * kCluSmall <= c->n_sm));
+                                      (n_target == n_draft && pairs * kClu > c->n_sm &&
+                                       fits(unit ? k_verify_cluster4<true> : k_verify_cluster4<false>, kCluSmall)));
     if (a.V <= kOneMaxVocab && !share) {
       // (as few tokens a thread as hold the row: see verify_cluster_body)
       constexpr int kPer = kCluThreads * 4;

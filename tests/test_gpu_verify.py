@@ -183,6 +183,22 @@ def test_row_pairs_around_a_wave(V, B, n):
         assert_verify_same({k: v.cpu().numpy() for k, v in out.items()}, oracle.verify(tok, dl, tl, T, 3, 8))
 
 
+# as many target rows as drafts, rows that one block holds: 13 | 15 and 18 | 19 pairs are the ends of one block a pair,
+# 33 | 34 those of clusters of 4
+@pytest.mark.parametrize("V", [6148, 8192])
+@pytest.mark.parametrize("B,n", [(13, 1), (5, 3), (9, 2), (19, 1), (11, 3), (17, 2), (37, 1), (19, 2)])
+def test_row_pairs_of_short_rows(V, B, n):
+    import paper_2410_05589_b200 as ps
+    s = synth.CONFIGS["mini32"].with_(hidden=64, n_heads=1, n_kv_heads=1, ffn=64, vocab=V, k_masks=n - 1)
+    g = ps.drafter_from_shape(s, synth.weights(s), max_batch=B, max_ctx=8)
+    for T in (0.0, 0.7, 1.0):
+        tl = synth.zipf_logits(7, (V, B, T), B, n, V)
+        dl = synth.noisy_draft_logits(7, (V, B, T), tl, 0.4)
+        tok = synth.sample_from_logits(7, (V, B, T), dl, T or 1.0)
+        out = g.verify(ps.to_device(tok), ps.to_device(dl), ps.to_device(tl), T, 3, 8)
+        assert_verify_same({k: v.cpu().numpy() for k, v in out.items()}, oracle.verify(tok, dl, tl, T, 3, 8))
+
+
 # Temperatures whose inverse times a difference of logits, or whose inverse itself, is beyond single precision: as
 # good as arg-max, in clusters that hold their rows (5 pairs) and in those that stream them (36; 8 of 128256 tokens)
 @pytest.mark.parametrize("V,B,n", [(5000, 1, 4), (32000, 1, 5), (32000, 9, 4), (128256, 2, 4)])
