@@ -522,10 +522,9 @@ __global__ void __launch_bounds__(256) k_finish_shared(const __grid_constant__ A
 // Row m of a MODE_RAW stage: the row's slots added in k order, bias and residual, the row's sum
 // of squares, the planes of its RMS-normalised values.  One block per row, NV vectors of four features a
 // thread, held in registers from the loads to the stores.
-// Bound by the latency of its loads from L2, which are hidden in two ways: few rows (a block an SM) have two
-// vectors a thread and the slots of JB = 4 contributors in flight together; many rows one contributor, in
-// so few registers that several blocks share an SM.  The divisions that find a tile's slots are made once
-// per tile and block.
+// Bound by the latency of its loads from L2, which are hidden in two ways: the slots of JB = 4 contributors in flight
+// together, or one contributor's in so few registers that two blocks share an SM (see launch_row_norm).  The
+// divisions that find a tile's slots are made once per tile and block.
 template <int NV, int JB, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_row_norm(const __grid_constant__ Args a, int H, float eps,
                                                            const __nv_bfloat16* __restrict__ bias, const float* res,
@@ -755,11 +754,14 @@ ps_status launch_finish_shared(ps_ctx* c, const Args& a, Mode mode, cudaStream_t
 ps_status launch_row_norm(ps_ctx* c, const Args& a, int H, const __nv_bfloat16* bias, const float* res,
                           const __nv_bfloat16* gain, float* out, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t st) {
   if (H > kMaxNormWidth) return fail(c, PS_ERR_UNSUPPORTED, "hidden size beyond 32768");
-  // more rows than SMs: blocks that share an SM (see k_row_norm)
-  const bool many = H <= 8192 && a.p.M > c->n_sm;
-  const int per_thread = H > 8192 ? 0 : many && H > 5120 ? 16 : 8;   // features
-  const int threads = per_thread ? ((H + per_thread - 1) / per_thread + 31) / 32 * 32 : 512;
-  auto kern = many ? (H <= 5120 ? k_row_norm<2, 1, 640, 2> : k_row_norm<4, 1, 512, 2>)
+  // More rows than SMs, a second block on an SM: up to 4096 features the blocks of four contributors have 512 threads
+  // and share an SM as they are; of 640 threads two fit with one contributor in flight (5120 features, steps without a
+  // large vocabulary: 192 rows 333.0 -> 329.5 us, 512 rows 703 -> 691, 160 rows 298.0 and 297.7; 4096 features, 160 rows 223.5,
+  // with one contributor 227.3; 768 features 93.6 and 96.7).  Wider rows would not fit the registers of half an SM (6656
+  // features, 320 rows: 765, with 16 features a thread, spilled, 794; 8192 features 1158 and 1179).
+  const bool two = H > 4096 && H <= 5120 && a.p.M > c->n_sm;
+  const int threads = H <= 8192 ? (H / 8 + 31) / 32 * 32 : 512;
+  auto kern = two ? k_row_norm<2, 1, 640, 2>
               : H <= 8192 ? k_row_norm<2, 4, 1024, 1> : H <= 16384 ? k_row_norm<8, 1, 512, 1> : k_row_norm<16, 1, 512, 1>;
   const cudaError_t e = launch_after(kern, dim3(a.p.M), dim3(threads), 0, st, !c->prof, a, H, c->cfg.rms_eps, bias, res, gain,
                                      out, hi, lo);

@@ -149,3 +149,16 @@ def test_append_in_passes_that_fill_their_waves():
             # values that agree to fp32 sums of 5120 and 10240 terms, rounded to bf16: one unit in the last place
             assert (np.abs(a - w) <= 2.0 ** -7 * np.abs(w) + 1e-4).all(), b
     assert g.poll() == 0 and g.check_guards() == 0
+
+
+# 148 | 150 rows of 4224 features: the row norm with the slots of four contributors in flight, and with one and two
+# blocks an SM; 4096 and 5248 features stay with the first
+@pytest.mark.parametrize("heads,B", [(33, 74), (33, 75), (32, 75), (41, 75)])
+def test_row_norm_of_more_rows_than_sms(heads, B):
+    s = synth.CONFIGS["mini"].with_(hidden=128 * heads, n_heads=heads, n_kv_heads=heads, ffn=512, vocab=500, k_masks=1)
+    seqs = [0, B - 1]
+    p = Pair(s, B, lens=[1 + b % 7 for b in range(B)], oracle_seqs=seqs)
+    got = p.gpu_step(top_n=1)
+    for b in seqs:
+        assert logits_close(got["logits"][b], p.oracle_step(b)["logits"], s.dtype) <= 1.0, b     # the logits gate
+    assert p.g.check_guards() == 0 and p.g.poll() == 0
