@@ -57,6 +57,14 @@ def test_last_wave_of_a_long_append_keeps_the_pairs_busy():
     assert p["T"] * p["KB"] / (P * most) > 0.9, p
 
 
+@pytest.mark.parametrize("rows", [17, 160, 257, 1000, 2048])
+def test_row_norm_finds_the_slots_of_the_widest_rows(rows):
+    """Contributors in 6 bits, the first slot's place in vectors in the other 26."""
+    for k, planes in ((65536, 1), (32768, 2), (98304, 2)):
+        p = plan(rows, k, [32768], planes=planes, raw=1, slots=1 << 30)
+        assert 0 < p["most"] < 64 and p["slots"] * p["Np"] * 256 * p["wt"] // 4 < 1 << 26, p
+
+
 def test_workspace_beside_the_caches():
     """Scratch of a context, in MB beside its K/V slabs (13B: 123, 311 and 794 with the earlier slots;
     the bounds: as it is, and 2%)."""
