@@ -184,6 +184,7 @@ struct ps_ctx {
   // answers asked of this context's device once (0 = not asked yet)
   int clusters[4][17] = {};       // [chain verify, tree walk, the same at other T than 0 and 1][cluster size]: resident at once, -1 none
   int stream_clusters[2][9] = {}; // streaming verify [T is 0 or 1, other][cluster size]
+  int stats_clusters[9] = {};     // row statistics without the sampler [cluster size]
   int attn_blocks_per_sm[4][16] = {};   // [kernel variant][tile size / 16]: resident blocks, -1 none
   cudaStream_t copy_stream = nullptr;   // ps_round_host: carries the target logits beside the draft step
   cudaEvent_t copy_done = nullptr;
@@ -202,6 +203,31 @@ struct ps_ctx {
 };
 
 namespace ps {
+
+// Clusters of nclu blocks of this kernel that are resident on the context's device at once, -1 for none (sizes above 8
+// are an opt-in of the kernel, a per-device function attribute).  Asked once per context, kernel and size.  A
+// cluster lies in one group of SMs, so not every SM can be filled: with one block an SM 33 clusters of 4 (132
+// SMs), 15 of 8 (120), 7 of 16 (112); with four an SM 560 blocks in clusters of 4 or of 8, not 592.
+template <class... Args>
+int clusters_at_once(int& cache, void (*kern)(Args...), int threads, int nclu) {
+  if (cache == 0) {
+    cache = -1;
+    if (nclu <= 8 || cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(nclu);
+      cfg.blockDim = dim3(threads);
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = nclu; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0) cache = n;
+    }
+    (void)cudaGetLastError();
+  }
+  return cache;
+}
 
 ps_status fail(ps_ctx* c, ps_status s, const std::string& what);
 ps_status cuda_check(ps_ctx* c, cudaError_t e, const char* what);

@@ -309,13 +309,25 @@ ps_status launch_logit_stats(ps_ctx* c, const float* logits, int M, int V, int R
   // are resident per SM and its arithmetic is what takes time, so only the balance counts: 144 rows of
   // 32000 tokens, 2 blocks in one wave, 50 -> 30 us against 4 in two; a single full wave is worth more
   // than its share says (80 rows: 7 blocks in two waves 31 us).  Without it three are resident and a block
-  // is through 32000 tokens in about 5 us, so that many rows want few blocks: 640 rows 66 -> 33 us.
+  // is through 32000 tokens in about 5 us, so that many rows want few blocks: 640 rows 66 -> 33 us.  The clusters of
+  // a wave are as many as find room (444 blocks of their own, but 104 clusters of 4, 82 of 5, 48 of 8), where a wave
+  // that needs nearly every place takes as long as two, and a later wave begins before the one ahead of it has
+  // ended.  128256 tokens, 80 rows: 4 blocks (131 us for the step) instead of 5 (137), which fill 80 of 82 places; 32000
+  // tokens, 85 rows 90 -> 85.  Of 48 counts of rows and tokens the choice is 0.4% behind the best one, at most 2%.
   int nclu = 1;
   double best = 1e30;
   for (int n = 1; n <= 8 && (n == 1 || V / n >= 2048); ++n) {
-    const long slots = (sa ? 2l : 3l) * c->n_sm, waves = ((long)M * n + slots - 1) / slots;
-    const double pass = 5.0 * V / 32000;
-    const double cost = sa ? (waves > 1 ? 1.15 : 1.0) * waves / n + 0.005 * n : waves * (2.5 + pass / n) + 0.05 * n;
+    double cost;
+    if (sa) {
+      const long slots = 2l * c->n_sm, waves = ((long)M * n + slots - 1) / slots;
+      cost = (waves > 1 ? 1.15 : 1.0) * waves / n + 0.005 * n;
+    } else {
+      int places = clusters_at_once(c->stats_clusters[n], k_logit_stats<false>, kThreads, n);
+      if (places <= 0) places = std::max(1, 3 * c->n_sm / n);
+      const int room = n <= 2 ? places : places * 31 / 32;
+      const double waves = M <= room ? 1.0 : std::max(2, (M + places - 1) / places);
+      cost = 0.5 * (waves + std::max(1.0, (double)M / places)) * (4.0 + 5.0 * V / 32000 / n) + 0.05 * n;
+    }
     if (cost < best) { best = cost; nclu = n; }
   }
   cudaLaunchConfig_t cfg = {};

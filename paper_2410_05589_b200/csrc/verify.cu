@@ -1657,31 +1657,6 @@ cudaError_t launch_cluster(void (*kern)(KArgs...), dim3 grid, int nclu, int thre
   return cudaLaunchKernelEx(&cfg, kern, a...);
 }
 
-// Clusters of nclu blocks of this kernel that are resident on the context's device at once, -1 for none (sizes above 8
-// are an opt-in of the kernel, a per-device function attribute).  Asked once per context, kernel and size.  A
-// cluster lies in one group of SMs, so not every SM can be filled: with one block an SM 33 clusters of 4 (132
-// SMs), 15 of 8 (120), 7 of 16 (112); with four an SM 560 blocks in clusters of 4 or of 8, not 592.
-template <class... Args>
-int clusters_at_once(int& cache, void (*kern)(Args...), int threads, int nclu) {
-  if (cache == 0) {
-    cache = -1;
-    if (nclu <= 8 || cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(nclu);
-      cfg.blockDim = dim3(threads);
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = nclu; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0) cache = n;
-    }
-    (void)cudaGetLastError();
-  }
-  return cache;
-}
-
 ps_status launch_verify(ps_ctx* c, int B, int n_draft, int n_target, const int* draft_tokens,
                         const float* draft_logits, const float* target_logits, float temperature,
                         uint64_t seed, uint64_t offset, int* accept_len, int* out_tokens,

@@ -38,3 +38,22 @@ def test_row_stats_edges(vocab, B):
     got = out["sampled"].cpu().numpy().ravel()
     # single-precision noise: 2^-21 of values up to 17
     assert all(g == t or m < 2e-5 for g, t, m in zip(got, tok, margin))
+
+
+# Without the sampler the blocks a row takes depend on how many clusters find room: counts of rows on both sides of a
+# wave's last places (80 | 82 of clusters of 5, 100 | 102 of 4, 136 | 138 of 3, 222 | 224 of 2)
+@pytest.mark.parametrize("vocab", [10241, 32000])
+def test_row_stats_around_a_wave(vocab):
+    s = synth.CONFIGS["mini32"].with_(hidden=64, n_heads=1, n_kv_heads=1, ffn=64, vocab=vocab, k_masks=1)
+    W = synth.weights(s)
+    W["w_lm"] = W["w_lm"] * np.float32(20.0)
+    p = Pair(s, 112, lens=[3] * 112, weights=W, oracle_seqs=[])
+    h, t = p.to_device(p.hidden_last), p.to_device(p.token_last)
+    for B in (39, 40, 41, 50, 51, 68, 69, 111, 112):
+        out = p.g.draft_step(list(range(B)), h[:B], t[:B], top_n=3)
+        lg = out["logits"].double().cpu().numpy().reshape(-1, vocab)
+        order = np.argsort(-lg, axis=-1, kind="stable")[:, :3]
+        assert np.array_equal(out["top_ids"].cpu().numpy().reshape(-1, 3), order), B
+        assert np.array_equal(out["row_max"].cpu().numpy().ravel(), lg.max(-1).astype(np.float32)), B
+        lse = lg.max(-1) + np.log(np.exp(lg - lg.max(-1, keepdims=True)).sum(-1))
+        assert np.abs(out["row_lse"].cpu().numpy().ravel() - lse).max() < 2.0 ** -18 + 2.0 ** -23 * np.abs(lse).max(), B
