@@ -328,6 +328,10 @@ ps_status ps_debug_late_copy(ps_ctx* ctx, void* dst, const void* src, size_t byt
 ps_status ps_debug_gemm_plan(int rows, int k, int n_mats, const int* mat_rows, int zip, int planes, int raw,
                              size_t slot_floats, int n_sm, int* out);
 
+/* Test helper: rows of the passes that ps_kv_append makes of `total` new rows on the tensor cores of a device with
+ * n_sm multiprocessors, where a pass takes at most `most` (host only).  0: invalid arguments. */
+int ps_debug_append_pass_rows(const ps_config* cfg, int n_sm, int total, int most);
+
 /* Number of kernel launches the context has enqueued so far (host counter). */
 long long ps_launch_count(ps_ctx* ctx);
 

@@ -32,7 +32,7 @@ EXPORTS = (
     "ps_last_error", "ps_destroy", "ps_philox_fill", "ps_profile", "ps_profile_read",
     "ps_verify_static", "ps_debug_buffer", "ps_verify_tree", "ps_draft_step_sampled", "ps_group_forward",
     "ps_build_tree", "ps_debug_wait_expires", "ps_debug_check_guards", "ps_debug_late_copy",
-    "ps_debug_gemm_plan",
+    "ps_debug_gemm_plan", "ps_debug_append_pass_rows",
 )
 
 
@@ -86,6 +86,7 @@ def load_library(path: str | None = None) -> C.CDLL:
     lib.ps_debug_wait_expires.argtypes = [vp, C.c_longlong, vp]
     lib.ps_debug_check_guards.argtypes = [vp, vp, ip]
     lib.ps_debug_gemm_plan.argtypes = [C.c_int, C.c_int, C.c_int, ip, C.c_int, C.c_int, C.c_int, C.c_size_t, C.c_int, ip]
+    lib.ps_debug_append_pass_rows.argtypes = [C.POINTER(ps_config), C.c_int, C.c_int, C.c_int]
     lib.ps_debug_late_copy.argtypes = [vp, vp, vp, C.c_size_t, C.c_int, vp]
     lib.ps_kv_len.argtypes = [vp, C.c_int, ip]
     lib.ps_kv_reset.argtypes = [vp, C.c_int]

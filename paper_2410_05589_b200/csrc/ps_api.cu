@@ -299,6 +299,11 @@ ps_status ps_debug_gemm_plan(int rows, int k, int n_mats, const int* mat_rows, i
   return PS_OK;
 }
 
+int ps_debug_append_pass_rows(const ps_config* cfg, int n_sm, int total, int most) {
+  if (!cfg || cfg->hidden < 1 || cfg->n_kv_heads < 1 || cfg->head_dim < 1 || n_sm < 2 || total < 1 || most < 1) return 0;
+  return append_pass_rows(*cfg, n_sm, total, most);
+}
+
 ps_status ps_kv_len(ps_ctx* c, int slot, int* len) {
   if (!c || !len || slot < 0 || slot >= c->cfg.max_batch) return PS_ERR_INVALID_ARG;
   *len = c->len[slot];

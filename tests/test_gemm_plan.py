@@ -65,6 +65,31 @@ def test_row_norm_finds_the_slots_of_the_widest_rows(rows):
         assert 0 < p["most"] < 64 and p["slots"] * p["Np"] * 256 * p["wt"] // 4 < 1 << 26, p
 
 
+def pass_rows(hidden, kv_heads, total, most=2048, n_sm=148):
+    from paper_2410_05589_b200.binding import ps_config
+    cfg = ps_config(1, hidden, kv_heads, kv_heads, 128, 2 * hidden, 1000, 4, 1, 1024, 1e4, 1e-5, 0)
+    return load_library().ps_debug_append_pass_rows(C.byref(cfg), n_sm, total, most)
+
+
+def test_passes_of_an_append():
+    """13B: 1792 rows leave fc 70 tiles and k | v 140 on 74 pairs, 2048 rows 80 and 160; the others have no better pass
+    than the largest, nor has an append that one pass takes or that gains less than 4%."""
+    assert pass_rows(5120, 40, 4999) == pass_rows(5120, 40, 2304) == pass_rows(5120, 40, 2049) == 1792
+    assert pass_rows(5120, 40, 528, most=520) == 512
+    for total in (2049, 3000, 4999, 8000):
+        assert pass_rows(4096, 32, total) == pass_rows(6656, 52, total) == pass_rows(4096, 8, total) == 2048
+    assert pass_rows(5120, 40, 1792) == pass_rows(5120, 40, 3900) == 2048
+    for total in (1, 16, 255, 256):
+        assert pass_rows(5120, 40, total) == 2048 and pass_rows(5120, 40, total, most=128) == 128
+    for most in (128, 256, 300, 1000, 2048):
+        for total in range(1, 9000, 97):
+            for hidden, kv, n_sm in ((5120, 40, 148), (768, 6, 148), (8192, 8, 148), (5120, 40, 132), (4096, 32, 2)):
+                rows = pass_rows(hidden, kv, total, most, n_sm)
+                assert rows == most or (0 < rows < most and rows % 256 == 0), (most, total, hidden, n_sm)
+    from paper_2410_05589_b200.binding import load_library as lib
+    assert lib().ps_debug_append_pass_rows(None, 148, 100, 100) == 0
+
+
 def test_workspace_beside_the_caches():
     """Scratch of a context, in MB beside its K/V slabs (13B: 123, 311 and 794 with the earlier slots;
     the bounds: as it is, and 2%)."""

@@ -121,36 +121,37 @@ def test_both_sides_of_the_line(heads, kv_heads, B, L):
 
 
 # Training layout: groups of one slot share the query rows of a pair.  Rows of a sequence times sequences a
-# bundle: 5 x 3 (90 and 4 slots), 3 x 2 heads x 2, 9 x 1, 2 x 8 (from an empty context); contexts
-# that cross a tile within a bundle, a last bundle that is not full, more groups than slots
-@pytest.mark.parametrize("heads,kv_heads,k,L0,n,slots", [(6, 6, 4, 200, 90, 90), (18, 18, 4, 500, 16, 4), (6, 3, 2, 120, 131, 128),
-                                                         (6, 6, 8, 250, 80, 80), (18, 18, 1, 0, 100, 128)])
+# bundle: 5 x 3 (all full; 1 and 2 left over; four slots, so passes of 3 + 1), 3 x 2 heads x 2, 9 x 1, 2 x 8 (from an empty
+# context; 4 left over), 1 x 16; contexts that cross a tile within a bundle, more groups than slots
+@pytest.mark.parametrize("heads,kv_heads,k,L0,n,slots", [(6, 6, 4, 200, 90, 90), (6, 6, 4, 200, 91, 91), (6, 6, 4, 200, 92, 92),
+                                                         (18, 18, 4, 1600, 16, 4), (6, 3, 2, 120, 131, 128), (6, 6, 8, 250, 80, 80),
+                                                         (18, 18, 1, 0, 100, 128), (18, 18, 0, 100, 70, 70)])
 def test_groups_of_one_slot(heads, kv_heads, k, L0, n, slots):
     import torch
     import paper_2410_05589_b200 as ps
-    s = synth.CONFIGS["mini"].with_(n_heads=heads, n_kv_heads=kv_heads, k_masks=k)
+    from harness import oracle_for
+    s = synth.CONFIGS["mini"].with_(n_heads=heads, n_kv_heads=kv_heads, k_masks=k, vocab=600)
+    assert _tiles(L0, min(n, slots)) * heads >= 6 * 148         # the rule of the dispatch, for the first pass
     W = synth.weights(s)
-    K, V = (ps.to_device(x) for x in synth.kv_rows(s, "ctx", L0)) if L0 else (None, None)
-    hid, tok = ps.to_device(synth.hidden_states(s, "new", n)), ps.to_device(synth.token_ids(s, "new", n))
     g = ps.drafter_from_shape(s, W, max_batch=slots, max_ctx=L0 + n + k + 1)
+    o = oracle_for(s, W, 1, L0 + n + k + 1)
     if L0:
-        g.kv_import(0, K, V)
+        K, V = synth.kv_rows(s, "ctx", L0)
+        g.kv_import(0, ps.to_device(K), ps.to_device(V))
+        o.kv_import(0, as_f64(K, s.dtype), as_f64(V, s.dtype))
+    h, t = synth.hidden_states(s, "new", n), synth.token_ids(s, "new", n)
+    hid, tok = ps.to_device(h), ps.to_device(t)
     out = g.group_forward(0, hid, tok, want_feat=True)
-    # the same rows as draft steps of one sequence each
-    one = ps.drafter_from_shape(s, W, max_batch=1, max_ctx=L0 + n + k + 1)
-    for t in sorted({0, 1, 5, 6, 7, n // 2, 256 - L0 if 0 < 256 - L0 < n else 2, n - 2, n - 1}):
-        one.kv_reset(0)
-        if L0:
-            one.kv_import(0, K, V)
-        if t:
-            one.kv_append([0], [t], hid[:t].contiguous(), tok[:t].contiguous())
-        want = one.draft_step([0], hid[t:t + 1].contiguous(), tok[t:t + 1].contiguous(), want_feat=True)
-        for name in ("logits", "feat"):
-            got, ref = out[name][t].double().cpu().numpy(), want[name][0].double().cpu().numpy()
-            assert logits_close(got, ref, s.dtype) <= 1.0, (t, name)     # the logits gate
+    want = o.group_forward(0, h, t)
+    for name in ("logits", "feat"):
+        assert logits_close(out[name].double().cpu().numpy(), want[name], s.dtype) <= 1.0, name     # the logits gate
     assert g.check_guards() == 0 and g.poll() == 0
     again = g.group_forward(0, hid, tok, want_feat=True)
     assert torch.equal(out["logits"], again["logits"])
+
+
+def _tiles(L0, n):
+    return sum(max(1, -(-(L0 + t) // 128)) for t in range(n))
 
 
 # A bundle reads keys that only some of its groups see: what those hold must not reach the others.  Position `bad` of the
@@ -158,10 +159,6 @@ def test_groups_of_one_slot(heads, kv_heads, k, L0, n, slots):
 # groups; the cached keys of the bundle end before, in and behind a tile's edge (128, 256)
 _BUNDLES = [(6, 6, 4, 201, 90, (30, 31, 32, 54, 55, 89)), (18, 18, 1, 125, 100, (0, 2, 3, 4, 7, 99)),
             (6, 3, 2, 120, 131, (6, 7, 8, 130)), (18, 18, 0, 125, 100, (2, 3, 15))]
-
-
-def _tiles(L0, n):
-    return sum(max(1, -(-(L0 + t) // 128)) for t in range(n))
 
 
 @pytest.mark.parametrize("value", [np.nan, np.inf])

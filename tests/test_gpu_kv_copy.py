@@ -33,7 +33,7 @@ def test_copy_of_more_rows_than_one_launch_indexes():
     import paper_2410_05589_b200 as ps
     s = synth.CONFIGS["mini"].with_(vocab=64, ffn=64)
     width = s.n_kv_heads * s.head_dim
-    n = (1 << 30) // width + 5                        # single elements: 2^30 of them to a launch
+    n = (1 << 30) // width + 5                        # single elements, more than 2^30 of them
     d = ps.drafter_from_shape(s, synth.weights(s), max_batch=1, max_ctx=n + s.rows)
     flat = torch.empty(n * width + 1, dtype=torch.bfloat16, device="cuda").uniform_(-1, 1)
     K = flat[1:].view(n, width)

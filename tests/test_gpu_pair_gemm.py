@@ -126,23 +126,29 @@ def test_hidden_sizes_beyond_the_row_norm():
     assert p.g.poll() == 0
 
 
-def test_append_in_passes_that_fill_their_waves():
-    """2304 new rows, hidden 5120, 40 kv heads: a pass of 1792 rows (70 and 140 tiles on 74 pairs) and one of 512
-    instead of 2048 and 256."""
+# 2304 new rows, hidden 5120, 40 kv heads: a pass of 1792 rows (70 and 140 tiles on 74 pairs) and one of 512 instead of
+# 2048 and 256; where a pass takes 520 rows at most, 528 rows as one of 512 and one of 16, which runs as a chained launch
+@pytest.mark.parametrize("B,n,max_ctx,passes", [(128, 18, 40, (1792, 512)), (8, 66, 130, (512, 16))])
+def test_append_in_passes_that_fill_their_waves(B, n, max_ctx, passes):
+    import ctypes as C
     import paper_2410_05589_b200 as ps
     import torch
     from harness import oracle_for
-    B, n = 128, 18
     s = synth.CONFIGS["mini"].with_(hidden=5120, n_heads=40, n_kv_heads=40, ffn=64, vocab=200, k_masks=1)
     W = synth.weights(s)
-    g = ps.drafter_from_shape(s, W, max_batch=B, max_ctx=40)
+    g = ps.drafter_from_shape(s, W, max_batch=B, max_ctx=max_ctx)
+    most = min(2048, B * max_ctx // 2)
+    rows = g.lib.ps_debug_append_pass_rows(C.byref(g.cfg), torch.cuda.get_device_properties(0).multi_processor_count, B * n, most)
+    assert rows == passes[0] < most and sum(passes) == B * n
     h, t = synth.hidden_states(s, "new", B * n), synth.token_ids(s, "new", B * n)
     before = g.launch_count()
     g.kv_append(list(range(B)), [n] * B, ps.to_device(h), ps.to_device(t))
     torch.cuda.synchronize()
-    assert g.launch_count() - before >= 2 * 5          # two passes of gather, fc, norm, k | v, store
-    o = oracle_for(s, W, B, 40)
-    for b in (0, 99, 100, B - 1):                      # (99: its rows lie in both passes)
+    # a pass: gather, fc, norm, k | v, store, or gather, chain, store
+    assert g.launch_count() - before >= sum(5 if p > 16 else 3 for p in passes)
+    o = oracle_for(s, W, B, max_ctx)
+    edge = passes[0] // n
+    for b in sorted({0, edge, min(edge + 1, B - 1), B - 1}):       # (the edge's rows lie in both passes)
         assert o.kv_append(b, h[b * n:(b + 1) * n], t[b * n:(b + 1) * n]) == 0
         got = [x.float().cpu().numpy() for x in g.kv_export(b)]
         for a, w in zip(got, o.kv_export(b)):

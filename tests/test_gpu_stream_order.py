@@ -11,7 +11,7 @@ from harness import assert_verify_same
 pytestmark = pytest.mark.gpu
 
 
-# one block per row pair (vocabulary up to 8192), 8-block clusters, 4-block clusters (19 to 37 row
+# one block per row pair (vocabulary up to 8192), 8-block clusters, 4-block clusters (16 to 33 row
 # pairs), 16-block clusters, the streaming kernel, one block and three passes (odd vocabulary)
 @pytest.mark.parametrize("vocab,B,n_draft,bonus", [(1000, 1, 5, 0), (8192, 3, 5, 1), (32000, 1, 5, 0), (32000, 4, 5, 1),
                                                    (16384, 7, 5, 0), (128256, 1, 5, 0), (32000, 16, 4, 1), (1001, 2, 3, 0)])
