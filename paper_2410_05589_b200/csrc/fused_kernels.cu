@@ -2176,9 +2176,10 @@ int fused_kv_rows(ps_ctx* c) {
 // one another).  A last wave that is nearly full counts whole; a small remainder is shared out with all
 // pairs, which costs its slots' way through memory, about a quarter of a wave; a pass about a tenth.
 // 13B: of 2048 rows fc has 80 tiles and k | v 160 on 74 pairs, of 1792 it is 70 and 140.  4999 rows in
-// passes of 2048 1414 us, of 1792 1328, of 1536 1414; 3900 rows 1091-1134 us and 998-1036, 3500 rows 901 and
-// 890; 7B shape (64 and 128 tiles) 958, 1042, 1043.  Splits that the count puts less than 4% ahead measured
-// even (33B shape, 4200 rows: 1876-1917 us in passes of 2048, 1914-1933 of 1536), so those stay with the most.
+// passes of 2048 1408 us, of 1792 1324, of 1536 1485; 4200 rows 1202, 1109, 1257; 3500 rows 972, 875, 1015; 7B shape (64
+// and 128 tiles), 4999 rows 958, 1042, 1043.  Splits that the count puts less than 4% ahead stay with the most: some
+// measured even (33B shape, 4200 rows: 1876-1917 us in passes of 2048, 1914-1933 of 1536), some are better (13B, 3900
+// rows: 1111, of 1792 1033).
 int append_pass_rows(const ps_config& g, int n_sm, int total, int most) {
   const int P = n_sm / 2, Hkv = g.n_kv_heads * g.head_dim, fc = (g.hidden + 511) / 512, kv = 2 * ((Hkv + 511) / 512);
   auto waves = [&](int tiles) {

@@ -20,7 +20,7 @@
 // on the leader's barrier), warp 1 allocates tensor memory and, in the leader CTA, issues the
 // MMAs for both; warps 2..9 read the accumulators back and store them (two warps per lane
 // quadrant, alternating column chunks).  Accumulators are double buffered when two tiles' fit
-// tensor memory (wt * Np <= 256).
+// tensor memory (tiles of up to 256 columns: wt * Np, or twice that where the planes are one operand).
 //
 // A tile whose k range is shared by several pairs is left as partial sums in slots (see Plan) and
 // finished by a kernel of its own: no CTA waits for another cluster, the sums are added in k
@@ -625,14 +625,18 @@ __global__ void __launch_bounds__(NT, MINB) k_row_norm(const __grid_constant__ A
 
 // Modelled time of a launch and of what finishes it (microseconds), for the choice between plans
 // only; fitted to the stage times of plans with one and two sub-tiles and 1 to 16 k blocks, 7B to 33B
-// shapes, 20 to 640 rows (the plan chosen is 1.6% behind the best one on average; a model in which
+// shapes, 20 to 640 rows, with two MMAs a unit throughout (the plan chosen was 1.6% behind the best one on average; a model in which
 // each pair had a fixed share of HBM was 4.9% behind: 33B q|k|v at 20 rows 87 us, now 67; 13B LM head
 // at 20 rows 95 us, now 83; 33B q|k|v at 288 rows 158 us, now 139).
 //  - a unit of a pair (wt weight boxes and the planes beside them in both CTAs) takes the longer of
 //    its way through the ring and its MMAs; idle pairs leave their share of HBM to the others, so
 //    HBM bounds the launch as a whole;
 //  - two sub-tiles of more than 128 rows fill the tensor memory, so the MMAs of the next tile wait
-//    until this one is read: one sub-tile is the better one there unless a pair has one tile only;
+//    until this one is read: one sub-tile is the better one there unless a pair has one tile only.
+//    (Where the planes are one operand, two sub-tiles of more than 64 rows fill it too.  The count leaves
+//    that out: with it a few stages of 65 to 128 rows get other plans, which took as long for 33B, 8192 features and
+//    128256 tokens and made steps of the 7B shape 1.2% longer.  Nor does it matter that an MMA of a pair takes 95 cycles at
+//    least and not 58: such units wait for the ring.)
 //  - each contributor more costs a round trip, its slots the way through L2 twice, and a stage
 //    without a row norm a kernel that adds them.
 double stream_cost(const Plan& p, int planes, int units) {
