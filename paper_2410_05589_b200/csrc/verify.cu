@@ -1784,17 +1784,15 @@ ps_status launch_verify_tree(ps_ctx* c, int B, int n_nodes, const int* parent, c
     tp.depth[i] = (unsigned char)(parent[i] < 0 ? 0 : tp.depth[parent[i]] + 1);
     tp.max_depth = std::max(tp.max_depth, (int)tp.depth[i] + 1);
   }
-  int off = 0;
-  for (int u = 0; u <= n_nodes; ++u) {   // children of decision row u in increasing node id
-    tp.child_off[u] = (unsigned char)off;
-    for (int i = 0; i < n_nodes; ++i)
-      if (parent[i] == u - 1) {
-        tp.parent[i] = (signed char)parent[i];
-        tp.nth[i] = (unsigned char)(off - tp.child_off[u]);
-        tp.child_idx[off++] = (unsigned char)i;
-      }
+  // children of decision row u in increasing node id (comparing every node with every row was 1.5 us of a call with 60 nodes)
+  unsigned char count[PS_MAX_TREE_NODES + 1] = {};
+  for (int i = 0; i < n_nodes; ++i) {
+    tp.parent[i] = (signed char)parent[i];
+    tp.nth[i] = count[parent[i] + 1]++;
   }
-  tp.child_off[n_nodes + 1] = (unsigned char)off;
+  tp.child_off[0] = 0;
+  for (int u = 0; u <= n_nodes; ++u) tp.child_off[u + 1] = (unsigned char)(tp.child_off[u] + count[u]);
+  for (int i = 0; i < n_nodes; ++i) tp.child_idx[tp.child_off[parent[i] + 1] + tp.nth[i]] = (unsigned char)i;
   if (max_depth_out) *max_depth_out = tp.max_depth;
   if (temperature != 0.f && !draft_logits) return fail(c, PS_ERR_INVALID_ARG, "draft_logits needed at temperature > 0");
   const bool aligned = (((uintptr_t)target_logits | (uintptr_t)draft_logits) & 15u) == 0;
