@@ -23,10 +23,11 @@
 // Measured (attention alone, with the small kernel) against mma.sync blocks that stage a tile,
 // synchronise and compute: 33B shape, 16 sequences of 1024-4096 keys, 9 rows: 343 -> 210 us (973 MB:
 // 4.8 TB/s of K/V in the main kernel); 13B shape, 64 x 256-2048 keys, 9 rows: 459 -> 332 us (1.5 GB); 16
-// sequences, 5 rows: 94 -> 82 us; 128 training groups of 300-428 keys: 273 -> 198 us.  Then, at the clock that the
-// power limit leaves a long run (a step's cycles bound the kernel there), by the vector stores and by warps
-// that no longer meet at a barrier in every step: 64 sequences 338 -> 286 us, 33B shape 194 -> 184; by three groups a
-// pair, 128 training groups 200 -> 121 us.  What was worth
+// sequences, 5 rows: 94 -> 82 us; 128 training groups of 300-428 keys: 273 -> 198 us.  Then, by the vector
+// stores and by warps that no longer meet at a barrier in every step (both builds in turn on one GPU, events between the
+// stages): 64 sequences 393 -> 369 us, 33B shape 235 and 235, 16 sequences of 5 rows 95 -> 93; by three groups a
+// pair, 128 training groups 241 -> 134 us.  (The clock is what the power limit leaves: a call by itself has 334 us for the 64
+// sequences and 192 for the 33B shape.)  What was worth
 // most after the first version: one TMA instruction per tile (the producer thread issued sixteen:
 // 351 -> 318 us on the 64-sequence case, 282 -> 179 on the groups), two MMA issuers, eight softmax
 // warps.  Putting the new rows into the last cached tile was slower (more, smaller boxes).
