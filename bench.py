@@ -5,7 +5,7 @@
                     [--batch B] [--k-masks k]     # a point of the batch / mask-count sweep
                     [--flags F]                   # ps_config.flags (2: plain kernels, 4: mma.sync GEMMs)
                     [--no-configs]                # skip the other workloads' sub-records
-    python bench.py --impl reference ...      # the CPU checker timed on the host cores
+    python bench.py --impl reference ...      # the CPU oracle timed on the host cores
 
 One "step" = one parallel draft step (all k+1 rows, logits stored) followed by one verify
 call on synthetic target logits, for the workload's batch.  At temperature > 0 the drafts are
@@ -220,7 +220,7 @@ class ClockSampler(threading.Thread):
                 "samples": len(self.samples)}
 
 
-# ---- the CPU checker as a timed baseline ---------------------------------------------------------
+# ---- the CPU oracle as a timed baseline ---------------------------------------------------------
 def oracle_setup(s, B, lens):
     import oracle
     import synth
@@ -254,7 +254,7 @@ def oracle_time_step(o, s, b, k_use, hidden_last, token_last, target, T):
 
 
 def cpu_baseline(s, B, lens, hidden_last, token_last, target, T, budget_s):
-    """The CPU checker, as it stands, on a bounded sample of the same workload: on all host
+    """The CPU oracle, as it stands, on a bounded sample of the same workload: on all host
     cores, and (a shorter sample) on one."""
     import oracle
 
@@ -294,7 +294,7 @@ def cpu_baseline(s, B, lens, hidden_last, token_last, target, T, budget_s):
 
 
 def run_reference(args):
-    """--impl reference: the CPU checker timed on the host cores (rank 0 only)."""
+    """--impl reference: the CPU oracle timed on the host cores (rank 0 only)."""
     if int(os.environ.get("RANK", "0")) != 0:
         return
     import oracle
